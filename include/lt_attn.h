@@ -64,8 +64,9 @@ typedef unsigned short lt_bf16;
 /* Bytes of caller-owned device workspace the calls below need; 0 means the shape is
  * not supported.  The workspace must be 256-byte aligned.  Layout (backward), with S_pad = S
  * rounded up to a multiple of 128: a 256-byte status block (word 0: code of a wait that gave up;
- * words 1, 2, 4: the three maxima above as fp32 bits; word 3: work-item counter), -delta and -LSE/scale as 16-byte rows
- * of fp16 (hi, lo, 0 x 6) with 256*hi + lo = value, [B,Hq,S_pad] rows each, an fp32 dQ accumulator
+ * word 3: work-item counter), -delta and -LSE/scale as 16-byte rows
+ * of fp16 (hi, lo, 0 x 6) with 256*hi + lo = value, [B,Hq,S_pad] rows each (every 64th or 128th -LSE/scale row may
+ * carry partial maxima of the three quantities above in elements 4-6, which no product uses), an fp32 dQ accumulator
  * [B,Hq,S_pad,D], and, for the grouped-query shapes whose groups are split over work items (see
  * lt_attn_bwd_num_launches), fp32 dK and dV sums [B,Hkv,S_pad,D] each. */
 size_t lt_attn_fwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);

@@ -2,7 +2,7 @@
 //
 // Three kernels per call:
 //   bwd_preprocess_kernel : delta = rowsum(dO * O); writes -delta and -LSE/scale as fp16
-//                           (hi, lo) pairs, zeroes the fp32 dQ accumulator, records
+//                           (hi, lo) pairs, zeroes the fp32 dQ accumulator, records (one slot per block)
 //                           max |delta|, max ||dO_row||^2 and max ||V_row||^2 (together they bound |dS|)
 //   bwd_main_kernel       : per (batch, kv head, key tile j): loop over the group's
 //                           query heads and the visible query tiles i, recompute
@@ -62,9 +62,29 @@ enum {
 // warp works on kPreUnroll groups of rows at a time so that enough loads are in flight to
 // keep HBM busy.
 constexpr int kPreUnroll = 4;
+// Rows a block takes per trip, and the largest grid: three resident blocks on each of 148 multiprocessors.  The maxima a
+// block found go, as one 8-byte slot, into the -LSE/scale row that starts its first trip (elements 4-6 of that operand
+// row meet zero multipliers in the main kernel, so any finite 16-bit pattern is inert there): no memory has to be
+// cleared before this kernel, and nothing is reduced with atomics.  The main kernel's CTAs combine the slots.
+// Measured against a cleared status block and atomic maxima (one more operation on the stream): 16.2 -> 11.9 us for the
+// smallest backward, replayed from a graph.
+constexpr int kPreThreads = 256, kPreMaxBlocks = 444;
+template <int D>
+__host__ __device__ constexpr int pre_rows_per_block() { return (kPreThreads / 32) * (32 / (D / 8)) * kPreUnroll; }
+template <int D>
+__host__ __device__ constexpr int pre_blocks(long long n_rows) {
+    const long long want = (n_rows + pre_rows_per_block<D>() - 1) / pre_rows_per_block<D>();
+    return static_cast<int>(want < kPreMaxBlocks ? want : kPreMaxBlocks);
+}
+// A non-negative fp32 maximum as 16 bits: its upper half rounded up, so that it stays a bound; 0x7B00 (a finite
+// pattern in fp16 and bf16) stands for anything above 6e35, infinities and NaNs included.
+constexpr unsigned int kMaxSlotInf = 0x7B00u;
+__device__ __forceinline__ unsigned int max_slot_bits(unsigned int fp32_bits) {
+    return min((fp32_bits + 0xFFFFu) >> 16, kMaxSlotInf);
+}
 
 template <int D, bool kBf16>
-__global__ void __launch_bounds__(256, 3)  // three blocks per multiprocessor keep enough loads in flight
+__global__ void __launch_bounds__(kPreThreads, 3)  // three blocks per multiprocessor keep enough loads in flight
 bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ O, const float *__restrict__ lse,
                       uint4 *__restrict__ delta_ext, uint4 *__restrict__ lse_ext, float *__restrict__ dq_acc,
                       long long n_rows, int S, int S_pad, int Hq, lt_tensor_strides do_st, lt_tensor_strides o_st,
@@ -73,7 +93,12 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
                       lt_tensor_strides v_st, int v_plain) {
     // `n_rows` counts rows of the padded row space (every head rounded up to S_pad rows), the
     // indexing of delta_ext, lse_ext and dq_acc; padding rows get zeros everywhere.
+    grid_dependency_wait();    // launched under the tail of its predecessor, which may write O or read the workspace
     grid_launch_dependents();  // the main kernel sets itself up while this kernel's last blocks run
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        status[kStatusWordTimeout] = 0u;
+        status[kStatusWordItemCounter] = 0u;
+    }
     // fp32 dK/dV sums (only when key tiles are split over several work items): zero them
     for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < kv_acc_vec4;
          v += static_cast<long long>(gridDim.x) * blockDim.x)
@@ -155,7 +180,8 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
     // (kept as bit patterns: non-negative floats order like them, with inf above every finite value and
     // NaN above inf, so non-finite inputs saturate the bound)
     unsigned int max_v2 = 0u;
-    for (long long row0 = warp_global * kRowsPerTrip; row0 < v_rows; row0 += n_warps * kRowsPerTrip) {
+    // (from the other end of the grid, whose warps had the fewer rows above)
+    for (long long row0 = (n_warps - 1 - warp_global) * kRowsPerTrip; row0 < v_rows; row0 += n_warps * kRowsPerTrip) {
         uint4 a[kPreUnroll];
 #pragma unroll
         for (int u = 0; u < kPreUnroll; ++u) {
@@ -193,22 +219,21 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
         max_norm2 = fmaxf(max_norm2, __shfl_xor_sync(0xffffffffu, max_norm2, off));
         max_v2 = max(max_v2, __shfl_xor_sync(0xffffffffu, max_v2, off));
     }
-    // one set of atomics per block, and only when it would raise the stored maximum: thousands of
-    // atomics on the same words would otherwise queue up behind one another in L2
-    __shared__ float block_max[3][8];
+    __shared__ unsigned int block_max[3][kPreThreads / 32];
     if (lane == 0) {
-        block_max[0][threadIdx.x >> 5] = max_abs_delta;
-        block_max[1][threadIdx.x >> 5] = max_norm2;
-        block_max[2][threadIdx.x >> 5] = __uint_as_float(max_v2);
+        block_max[0][threadIdx.x >> 5] = __float_as_uint(max_abs_delta) & 0x7fffffffu;
+        block_max[1][threadIdx.x >> 5] = __float_as_uint(max_norm2) & 0x7fffffffu;
+        block_max[2][threadIdx.x >> 5] = max_v2;
     }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        unsigned int m = 0u;
+    __syncthreads();  // (also orders the slot after this block's own store of the row it lies in)
+    if (threadIdx.x == 0) {
+        unsigned int m[3] = {0u, 0u, 0u};
 #pragma unroll
-        for (int w = 0; w < 8; ++w) m = max(m, __float_as_uint(block_max[threadIdx.x][w]) & 0x7fffffffu);
-        unsigned int *word = status + (threadIdx.x == 0 ? kStatusWordMaxAbsDelta
-                                       : threadIdx.x == 1 ? kStatusWordMaxDoNorm2 : kStatusWordMaxVNorm2);
-        if (m > *reinterpret_cast<volatile unsigned int *>(word)) atomicMax(word, m);
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int w = 0; w < kPreThreads / 32; ++w) m[k] = max(m[k], block_max[k][w]);
+        uint2 *slot = reinterpret_cast<uint2 *>(lse_ext + static_cast<long long>(blockIdx.x) * pre_rows_per_block<D>()) + 1;
+        *slot = make_uint2(max_slot_bits(m[0]) | (max_slot_bits(m[1]) << 16), max_slot_bits(m[2]));
     }
 }
 
@@ -341,7 +366,7 @@ static_assert(128 * kRegsControl + kNumComputeWarps * 32 * kRegsCompute + kNumRe
 constexpr int kDqStageBufs = 3, kDqStageRows = 16;
 constexpr int kExtBytes = 2048;            // 128 rows x 16 bytes: one operand of the extra contraction step
 constexpr float kPScaleLog2Max = 14.f;     // P is kept as P * 2^c with c <= 14 so that fp16(P') <= 16384
-constexpr int kBarReduceWarps = 1;  // named barrier id
+constexpr int kBarReduceWarps = 1, kBarScale = 2;  // named barrier ids
 constexpr int kItemRing = 4;  // roles are never more than two items apart
 constexpr double kL2BatchBytes = 80.0e6;  // working set of one batch of work items (L2 holds 126 MB)
 
@@ -373,6 +398,7 @@ struct BwdSmem {
     uint64_t bar_s_full, bar_p_ready, bar_dp_full, bar_ds_ready, bar_ds_free, bar_dq_full, bar_dq_empty;
     uint32_t tmem_base;
     int abort_flag;
+    unsigned int call_max[3];  // the call's maxima (slot bits of max |delta|, max ||dO_row||^2, max ||V_row||^2)
 };
 
 static_assert(sizeof(BwdSmem<128>) <= 232448, "main kernel shared memory exceeds the 227 KB per-block limit");
@@ -464,14 +490,36 @@ __device__ __forceinline__ const __half *saved_p_tile(const BwdParams &p, const 
 // The exponent c of the power of two that P carries (P' = P * 2^c, c <= 14), and with it dS, so that
 // dS' uses fp16's normal range without overflow when it is rounded: chosen from a bound on
 // |dS| <= |dP| + |delta| <= max ||dO_row|| * max ||V_row|| + max |delta| over the whole call (the
-// three maxima come from the preprocess kernel).  dV and dQ / dK undo the factor exactly in their
-// epilogues.  Every thread that needs c computes it once per CTA from the status block.
-__device__ __forceinline__ int bwd_p_scale_log2(const unsigned int *status) {
-    const float do2 = __uint_as_float(__ldcg(status + kStatusWordMaxDoNorm2));
-    const float v2 = __uint_as_float(__ldcg(status + kStatusWordMaxVNorm2));
-    const float dmax = __uint_as_float(__ldcg(status + kStatusWordMaxAbsDelta));
-    const float bound = sqrtf(do2) * sqrtf(v2) + dmax;
-    if (!(bound < 3.0e38f)) return -14;                           // inf/NaN inputs: outputs are non-finite anyway
+// three maxima come from the preprocess kernel, one slot per block of it).  dV and dQ / dK undo the factor
+// exactly in their epilogues.  Run once per CTA by the softmax and reduction warps together.
+template <int D>
+__device__ __forceinline__ int bwd_p_scale_log2(const BwdParams &p, unsigned int *call_max) {
+    constexpr int kThreads = (kNumComputeWarps + kNumReduceWarps) * 32;
+    const long long n_rows = static_cast<long long>(p.B) * p.Hq * p.S_pad;
+    // (the -LSE/scale rows follow the -delta rows; the saved-P variant's lse_ext points elsewhere)
+    const uint2 *slots = reinterpret_cast<const uint2 *>(p.delta_ext + n_rows) + 1;
+    const int n = pre_blocks<D>(n_rows);
+    unsigned int m[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int u = 0; u < (kPreMaxBlocks + kThreads - 1) / kThreads; ++u) {
+        const int k = static_cast<int>(threadIdx.x) - kComputeWarp0 * 32 + u * kThreads;
+        if (k < n) {
+            const uint2 v = __ldcg(slots + static_cast<long long>(k) * (pre_rows_per_block<D>() * 2));
+            m[0] = max(m[0], v.x & 0xFFFFu);
+            m[1] = max(m[1], v.x >> 16);
+            m[2] = max(m[2], v.y);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+        if ((threadIdx.x & 31) == 0 && m[k]) atomicMax(call_max + k, m[k]);
+    }
+    named_barrier_sync(kBarScale, kThreads);
+    const unsigned int delta = call_max[0], do2 = call_max[1], v2 = call_max[2];
+    if (max(max(delta, do2), v2) >= kMaxSlotInf) return -14;  // inf/NaN inputs: outputs are non-finite anyway
+    const float bound = sqrtf(__uint_as_float(do2 << 16)) * sqrtf(__uint_as_float(v2 << 16)) + __uint_as_float(delta << 16);
+    if (!(bound < 3.0e38f)) return -14;
     if (!(bound > 1e-30f)) return static_cast<int>(kPScaleLog2Max);  // all-zero dO: any factor works
     return min(static_cast<int>(kPScaleLog2Max), max(-14, ilogbf(32768.f / bound)));
 }
@@ -507,7 +555,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const bool smem_ok = (smem_u32(smem_raw) & 1023u) == 0u;
     if (tid == 0) {
         sm.abort_flag = smem_ok ? 0 : 1;
-        if (!smem_ok) atomicCAS(p.status + kStatusWordTimeout, 0u, static_cast<unsigned int>(kBadSmemAlign));
+        sm.call_max[0] = sm.call_max[1] = sm.call_max[2] = 0u;
         mbar_init(&sm.bar_kv, 1);
         mbar_init(&sm.bar_dkv_full, 1);
         mbar_init(&sm.bar_acc_free, kNumReduceWarps);
@@ -550,6 +598,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // everything above ran while the preprocess kernel was finishing; its results (row operands, zeroed
     // accumulator, running maxima, item counter) are read only from here on
     grid_dependency_wait();
+    if (!smem_ok && tid == 0) atomicCAS(p.status + kStatusWordTimeout, 0u, static_cast<unsigned int>(kBadSmemAlign));
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
 #ifdef LT_BWD_TRACE
@@ -804,7 +853,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const float scale_log2 = p.scale * kLog2e;
         uint8_t *ds_tile = sm.ds + half_sel * kBoxBytesBwd;
         uint32_t pv[64];  // bits of this thread's 64 fp32 values of P' = P * 2^c for the current tile pair
-        const float p_scale_log2 = static_cast<float>(bwd_p_scale_log2(p.status));
+        const float p_scale_log2 = static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max));
         bool ok = smem_ok;
         int it = 0, ic = 0;
         LT_TRACE_BEGIN();
@@ -954,7 +1003,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         warpgroup_regs_set<kRegsReduce, kRegsAtLaunch>();
         const int quad = warp & 3;
         // P carried the factor 2^c through dS into the accumulators; the epilogues take it out again (exact)
-        const float inv_p_scale = exp2f(-static_cast<float>(bwd_p_scale_log2(p.status)));
+        const float inv_p_scale = exp2f(-static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max)));
         const float dq_mult = p.scale * inv_p_scale;
         bool ok = smem_ok;
         int it = 0, ic = 0;
@@ -1262,22 +1311,26 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     if ((rc = make_bhsd_map(&mk, K, B, Hkv, S, D, lay.k, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mv, V, B, Hkv, S, D, lay.v, 128, kBf16)) != LT_OK) return rc;
 
-    cudaError_t e = cudaMemsetAsync(status, 0, kStatusBytes, stream);
-    if (e != cudaSuccess) return record_cuda_error("cudaMemsetAsync(status)", e);
-
+    // programmatic stream serialisation: each kernel may start before its predecessor has finished and
+    // waits inside for it (grid_dependency_wait).  The conversion kernels do not let the next call's preprocess
+    // kernel start early: with that, a call on the LLaMA-2-7B shape took 453 us in a loop instead of 434.
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
     const int sms = sm_count();
-    constexpr int kRowsPerBlock = 8 * (32 / (D / 8)) * kPreUnroll;
-    const long long want = (n_rows + kRowsPerBlock - 1) / kRowsPerBlock;
-    const int pre_blocks = static_cast<int>(want < static_cast<long long>(sms) * 16 ? want : sms * 16);
-    bwd_preprocess_kernel<D, kBf16><<<pre_blocks, 256, 0, stream>>>(reinterpret_cast<const __half *>(dO),
-                                                             reinterpret_cast<const __half *>(O), LSE, delta_ext,
-                                                             lse_ext, dq_acc, n_rows, S, S_pad, Hq, lay.d_o, lay.o, plain_pre,
-                                                             1.f / scale, status, reinterpret_cast<float4 *>(dk_acc),
-                                                             parts > 1 ? static_cast<long long>(kv_floats / 2) : 0LL,
-                                                             reinterpret_cast<const __half *>(V),
-                                                             static_cast<long long>(B) * Hkv * S, Hkv, lay.v,
-                                                             is_contig(lay.v, Hkv) ? 1 : 0);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t cfg_pre = {};
+    cfg_pre.gridDim = dim3(pre_blocks<D>(n_rows));
+    cfg_pre.blockDim = dim3(kPreThreads);
+    cfg_pre.stream = stream;
+    cfg_pre.attrs = &pdl;
+    cfg_pre.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg_pre, bwd_preprocess_kernel<D, kBf16>, reinterpret_cast<const __half *>(dO),
+                                       reinterpret_cast<const __half *>(O), LSE, delta_ext, lse_ext, dq_acc, n_rows, S, S_pad,
+                                       Hq, lay.d_o, lay.o, plain_pre, 1.f / scale, status, reinterpret_cast<float4 *>(dk_acc),
+                                       parts > 1 ? static_cast<long long>(kv_floats / 2) : 0LL,
+                                       reinterpret_cast<const __half *>(V), static_cast<long long>(B) * Hkv * S, Hkv, lay.v,
+                                       is_contig(lay.v, Hkv) ? 1 : 0);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("bwd_preprocess_kernel launch", e);
 
     BwdParams prm;
@@ -1322,11 +1375,6 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     const int grid = n_items < sms ? n_items : sms;  // persistent: one CTA per SM walks the item list
     if (ev_main_begin && (e = cudaEventRecord(ev_main_begin, stream)) != cudaSuccess)
         return record_cuda_error("cudaEventRecord", e);
-    // programmatic stream serialisation: the kernel may start before its predecessor has finished and
-    // waits inside for it (grid_dependency_wait)
-    cudaLaunchAttribute pdl;
-    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg_main = {};
     cfg_main.gridDim = dim3(grid);
     cfg_main.blockDim = dim3(kBwdThreads);

@@ -137,7 +137,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
-
+    // the set-up above ran under the tail of the predecessor in the stream; from here on its results are used
+    grid_dependency_wait();
+    if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
 
     if (warp < kFwdSoftmaxWarp0) {
         warpgroup_regs_set<kFwdRegsControl, kFwdRegsAtLaunch>();
@@ -470,8 +472,6 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     if ((rc = make_bhsd_map(&mq, Q, B, Hq, S, D, lay.q, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mk, K, B, Hkv, S, D, lay.k, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mv, V, B, Hkv, S, D, lay.v, 128, kBf16)) != LT_OK) return rc;
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, stream);
-    if (e != cudaSuccess) return record_cuda_error("cudaMemsetAsync(status)", e);
     FwdParams prm;
     prm.O = reinterpret_cast<__half *>(O);
     prm.lse = LSE;
@@ -481,12 +481,22 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     prm.scale = scale;
     // at least 120 KB, so that one CTA (which takes all 512 tensor-memory columns) lives on an SM
     const size_t smem = std::max<size_t>(sizeof(FwdSmem<D>) + 1024, 120 * 1024);
-    e = cudaFuncSetAttribute(fwd_kernel<D, kBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = cudaFuncSetAttribute(fwd_kernel<D, kBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(fwd)", e);
     const int n_tiles = (S + kFwdTileRows - 1) / kFwdTileRows;
     const int grid = B * Hq * ((n_tiles + 1) / 2);
-    fwd_kernel<D, kBf16><<<grid, kFwdThreads, smem, stream>>>(mq, mk, mv, prm);
-    e = cudaGetLastError();
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kFwdThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, fwd_kernel<D, kBf16>, mq, mk, mv, prm);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("fwd_kernel launch", e);
     return LT_OK;
 }

@@ -13,14 +13,10 @@ namespace lt {
 
 // ----------------------------------------------------------------------------- status block
 // First 256 bytes of every workspace.  Word 0: 0 = ok, otherwise the code of the wait
-// that gave up.  Word 1: max |delta| bits, word 2: max ||dO_row||^2 bits, word 4: max ||V_row||^2
-// bits (backward).
+// that gave up.  Word 3: work-item counter (backward).  The other words are not used.
 constexpr int kStatusBytes = 256;
 constexpr int kStatusWordTimeout = 0;
-constexpr int kStatusWordMaxAbsDelta = 1;
-constexpr int kStatusWordMaxDoNorm2 = 2;
 constexpr int kStatusWordItemCounter = 3;  // next unclaimed work item of the backward main kernel
-constexpr int kStatusWordMaxVNorm2 = 4;
 
 // A wait gives up after this many clock cycles (about one second; the build of the give-up test
 // shortens it).
