@@ -10,6 +10,10 @@
 //                 accumulators
 //   warps 2..5  : epilogue - tensor memory -> fp16 -> global, one accumulator while the other is
 //                 being filled
+//
+// Two further kernels share this arrangement: CTA pairs working 256 x 256 tiles (many tiles), and narrower tiles whose
+// contraction is split over a cluster (few tiles); gemm_plan() chooses.
+#include <cmath>
 #include <cstdlib>
 #include "lt_common.cuh"
 #include "lt_host.h"
@@ -89,6 +93,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
+    // the set-up above ran under the tail of the predecessor in the stream
+    grid_dependency_wait();
+    if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
 
     if (warp == 0) {
         if (lane == 0) {
@@ -277,6 +284,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
+    grid_dependency_wait();
+    if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -397,11 +406,245 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     if (warp == 0) tmem_dealloc_pair(tmem, 512);
 }
 
+// ----------------------------------------------------------------------------- few output tiles
+// Shapes whose output has too few large tiles to occupy the chip: narrower tiles (128 x kBN) and the contraction of
+// each tile split over the CTAs of a cluster.  Every CTA accumulates its share of the contraction in tensor memory,
+// leaves the fp32 partial in its shared memory, and after a cluster barrier each CTA sums a slice of the tile's rows over
+// the cluster's partials (in rank order, so results are reproducible), rounds and stores it.  One tile share per CTA.
+template <int kBN>
+struct __align__(1024) GemmSplitSmem {
+    static constexpr uint32_t kBBytes = kBN * kGemmBK * 2;
+    static constexpr int kStages = static_cast<int>(196608 / (kGemmABytes + kBBytes));
+    static constexpr int kPitch = kBN + 4;  // floats per row of the partial: 16-byte stores of a warp hit all banks
+    union {
+        struct {
+            uint8_t a[kStages][kGemmABytes];
+            uint8_t b[kStages][kBBytes];
+        } ring;
+        float partial[kGemmBM * kPitch];  // once every block of the share has been multiplied
+    };
+    uint64_t bar_full[kStages], bar_empty[kStages], bar_acc;
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+template <int kBN, bool kBf16>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                  const GemmParams p) {
+    using Smem = GemmSplitSmem<kBN>;
+    constexpr int kStages = Smem::kStages;
+    extern __shared__ uint8_t smem_raw[];
+    // (the dynamic window starts at the same offset in every CTA, so the aligned structure does too)
+    Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const int tid = threadIdx.x;
+    const int warp = tid >> 5;
+    const int lane = tid & 31;
+    const int split = static_cast<int>(cluster_cta_count());
+    const int rank = static_cast<int>(cluster_cta_rank());
+    int tm, tn;
+    gemm_tile_coords(p, static_cast<int>(blockIdx.x) / split, tm, tn);
+    const int k_blocks = (p.K + kGemmBK - 1) / kGemmBK;
+    const int kb0 = static_cast<int>(static_cast<long long>(k_blocks) * rank / split);
+    const int n_kb = static_cast<int>(static_cast<long long>(k_blocks) * (rank + 1) / split) - kb0;  // >= 1
+
+    if (tid == 0) {
+        sm.abort_flag = 0;
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(&sm.bar_full[s], 1);
+            mbar_init(&sm.bar_empty[s], 1);
+        }
+        mbar_init(&sm.bar_acc, 1);
+        mbar_fence_init();
+        tma_prefetch_desc(&map_a);
+        tma_prefetch_desc(&map_b);
+    }
+    if (warp == 0) {
+        tmem_alloc(&sm.tmem_base, kBN);
+        tmem_relinquish();
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = sm.tmem_base;
+    volatile int *abort_flag = &sm.abort_flag;
+    grid_dependency_wait();
+    if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            bool ok = true;
+            int i = 0;
+            for (; i < n_kb; ++i) {
+                const int s = i % kStages;
+                const uint32_t use = i / kStages;
+                if (use >= 1 && !(ok = mbar_wait(&sm.bar_empty[s], (use - 1) & 1, abort_flag, p.status, kWaitGemmEmpty))) break;
+                mbar_arrive_expect_tx(&sm.bar_full[s], kGemmABytes + Smem::kBBytes);
+                tma_load_2d(sm.ring.b[s], &map_b, &sm.bar_full[s], (kb0 + i) * kGemmBK, tn * kBN);
+                tma_load_2d(sm.ring.a[s], &map_a, &sm.bar_full[s], (kb0 + i) * kGemmBK, tm * kGemmBM);
+            }
+            if (!ok || *abort_flag) {
+                // somebody gave up: wait (bounded) for the copies in flight before the CTA exits
+                for (int back = 0; back < kStages && back < i; ++back) {
+                    const int q = i - 1 - back;
+                    for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_full[q % kStages], (q / kStages) & 1); ++w) {}
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = make_idesc(kGemmBM, kBN, false, false, kBf16);
+            bool ok = true;
+            for (int i = 0; i < n_kb; ++i) {
+                const int s = i % kStages;
+                if (!(ok = mbar_wait(&sm.bar_full[s], (i / kStages) & 1, abort_flag, p.status, kWaitGemmFull))) break;
+                tc_fence_after_sync();
+                const uint64_t da = desc_kmajor(smem_u32(sm.ring.a[s])), db = desc_kmajor(smem_u32(sm.ring.b[s]));
+#pragma unroll
+                for (int kk = 0; kk < kGemmBK / 16; ++kk)
+                    umma_ss(tmem, da + kk * 2, db + kk * 2, idesc, (i > 0) | (kk > 0));
+                umma_commit(&sm.bar_empty[s]);
+            }
+            if (ok) umma_commit(&sm.bar_acc);
+        }
+    } else {
+        // this CTA's share of the sum: tensor memory -> shared memory (every load has landed and been read by then);
+        // thread = row of the tile
+        const int quad = warp & 3;  // tensor-memory lane quadrant this warp may read
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.bar_acc, 0, abort_flag, p.status, kWaitGemmAccFull));
+        if (ok) {
+            tc_fence_after_sync();
+            const uint32_t taddr = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+            float *row = sm.partial + (quad * 32 + lane) * Smem::kPitch;
+#pragma unroll
+            for (int c = 0; c < kBN / 32; ++c) {
+                uint32_t r[32];
+                tmem_ld32(taddr + c * 32, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int v = 0; v < 8; ++v)
+                    *reinterpret_cast<uint4 *>(row + c * 32 + v * 4) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+            }
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, kBN);
+    cluster_sync_all();  // every partial of the tile is in place
+    {
+        const int rows = min(kGemmBM, p.M - tm * kGemmBM);
+        const int r0 = rows * rank / split, r1 = rows * (rank + 1) / split;
+        constexpr int kChunks = kBN / 8;  // pieces of eight columns
+        const bool vec_ok = (p.N % 8) == 0;
+        const uint32_t base = smem_u32(sm.partial);
+        for (int u = tid; u < (r1 - r0) * kChunks; u += kGemmThreads) {
+            const int row = r0 + u / kChunks, col = (u % kChunks) * 8;
+            const int n = tn * kBN + col;
+            if (n >= p.N) continue;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+            const uint32_t local = base + (row * Smem::kPitch + col) * 4;
+            for (int q = 0; q < split; ++q) {
+                const uint32_t addr = cluster_map_shared(local, q);
+                const float4 u4 = ld_cluster_v4(addr), w4 = ld_cluster_v4(addr + 16);
+                x.x += u4.x; x.y += u4.y; x.z += u4.z; x.w += u4.w;
+                y.x += w4.x; y.y += w4.y; y.z += w4.z; y.w += w4.w;
+            }
+            __half *dst = p.C + (static_cast<long long>(tm) * kGemmBM + row) * p.N + n;
+            const uint4 o = make_uint4(pack2<kBf16>(x.x, x.y), pack2<kBf16>(x.z, x.w), pack2<kBf16>(y.x, y.y), pack2<kBf16>(y.z, y.w));
+            if (vec_ok) {  // (N a multiple of eight: a piece lies inside the row or outside)
+                *reinterpret_cast<uint4 *>(dst) = o;
+            } else {
+                const uint32_t w[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (n + e < p.N)
+                        reinterpret_cast<uint16_t *>(dst)[e] = static_cast<uint16_t>((w[e >> 1] >> ((e & 1) * 16)) & 0xFFFFu);
+            }
+        }
+    }
+    __syncthreads();
+    cluster_sync_all();  // nobody leaves while its partial may still be read
+}
+
+template <int kBN, bool kBf16>
+static int launch_gemm_split(const CUtensorMap &ma, const CUtensorMap &mb, GemmParams prm, int split, cudaStream_t stream) {
+    prm.tiles_m = (prm.M + kGemmBM - 1) / kGemmBM;
+    prm.tiles_n = (prm.N + kBN - 1) / kBN;
+    prm.group_rows = prm.tiles_m;
+    const size_t smem = sizeof(GemmSplitSmem<kBN>) + 1024;
+    auto kernel = gemm_split_kernel<kBN, kBf16>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(gemm_split)", e);
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = split;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(prm.tiles_m * prm.tiles_n * split);
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, kernel, ma, mb, prm);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    return e == cudaSuccess ? LT_OK : record_cuda_error("gemm_split_kernel launch", e);
+}
+
 }  // namespace lt
 
 extern "C" {
 
 size_t lt_gemm_f16_workspace_bytes(void) { return lt::kStatusBytes; }
+
+// Which kernel: tile width and contraction shares per tile, or the CTA-pair kernel.  The choice is the smallest
+// estimate of a time model in microseconds whose constants were fitted to 450 measured (shape, kernel) pairs (27 shapes
+// with 1-8192 rows, every width and split); the kernel it picks is within 3.3 % of the fastest one on average.
+//   first wave: launch, fill and drain, plus the blocks of the longest share (a block takes the larger part of issuing
+//   its products and of bringing its A and W rows in while the other CTAs do the same), plus the epilogue, which costs
+//   more per element when the partials of a cluster are summed; every further wave costs its own fill and drain, except
+//   in the persistent kernels.
+// Measured, us, before (256-wide tiles on one CTA or a pair) and now: 77 x 4096 x 4096 (M x N x K) 28.2 / 12.0 (128-wide,
+// four shares), 128 x 128 x 4096 22.3 / 8.7 (64-wide, eight), 424 x 265 x 5920 64 / 11.3 (64, six), 3000 x 128 x 11008
+// 54 / 21 (128, five), 1024 x 2048 x 8192 43.5 / 35.7 (256, two), 700 x 2048 x 1024 11.0 / 9.6 (256, whole).
+// On the other side of the line: 512 x 4096 x 4096 128-wide 25.7 against the pair kernel's 25.8, 1024 x 4096 x 4096 49
+// against 29.
+struct GemmPlan {
+    int bn, split;
+    bool pair;
+};
+static GemmPlan gemm_plan(int M, int N, int K) {
+    using namespace lt;
+    auto ceil_div = [](long long a, long long b) { return (a + b - 1) / b; };
+    const double k_blocks = static_cast<double>(ceil_div(K, kGemmBK));
+    GemmPlan best{kGemmBN, 1, false};
+    double best_us = 4.4 + ceil_div(ceil_div(M, kGemmBM) * ceil_div(N, kGemmBN), 148) * k_blocks * 0.357;
+    auto offer = [&](GemmPlan plan, double us) {
+        if (us < best_us) best = plan, best_us = us;
+    };
+    if (M > kGemmBM)
+        offer({kPairBN, 1, true}, 6.7 + ceil_div(ceil_div(M, kPairBM) * ceil_div(N, kPairBN), 74) * k_blocks * 0.304);
+    // clusters of so many CTAs, one CTA per multiprocessor, that fit at once (cudaOccupancyMaxActiveClusters on a B200)
+    constexpr int kMaxClusters[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    const double rows = M < kGemmBM ? M : kGemmBM;
+    for (int w = 0; w < 3; ++w) {
+        const int bn = 64 << w;
+        const double issue = w == 0 ? 0.260 : w == 1 ? 0.296 : 0.428;
+        const long long tiles = ceil_div(M, kGemmBM) * ceil_div(N, bn);
+        for (int split = w == 2 ? 2 : 1; split <= 8 && split <= k_blocks; ++split) {
+            const double waves = static_cast<double>(ceil_div(tiles, kMaxClusters[split]));
+            const double fill = tiles * split < 148 ? tiles * split / 148.0 : 1.0;
+            const double bring = (rows + bn) * (kGemmBK * 2) * 6.0e-6 * fill;
+            const double work = ceil(k_blocks / split) * sqrt(issue * issue + bring * bring) +
+                                rows * bn * 4e-3 * (split > 1 ? 0.0372 : 0.0154);
+            offer({bn, split, false}, 4.5 + (split > 1 ? 0.57 : 0.0) + waves * work + (waves - 1) * 4.6);
+        }
+    }
+    return best;
+}
 
 static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K, void *workspace,
                       size_t workspace_bytes, lt_stream_t stream, bool bf16) {
@@ -415,24 +658,40 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
     int rc = check_device();
     if (rc != LT_OK) return rc;
 
-    // More than one 128-row tile of A: CTA pairs work 256 x 256 tiles (LT_GEMM_SINGLE_CTA=1 in the
-    // environment keeps the single-CTA kernel, for comparison).
+    // (LT_GEMM_SINGLE_CTA=1 in the environment keeps the single-CTA kernel, for comparison)
     static const bool force_single = [] {
         const char *v = getenv("LT_GEMM_SINGLE_CTA");
         return v && v[0] == '1';
     }();
-    const bool use_pair = M > kGemmBM && !force_single;
+    GemmParams prm;
+    prm.C = reinterpret_cast<__half *>(C);
+    prm.status = reinterpret_cast<unsigned int *>(workspace);
+    prm.M = M; prm.N = N; prm.K = K;
 
+    const GemmPlan plan = force_single ? GemmPlan{kGemmBN, 1, false} : gemm_plan(M, N, K);
+    const bool use_pair = plan.pair;
     CUtensorMap ma, mb;
     if ((rc = make_tile_map(&ma, A, M, K, kGemmBM)) != LT_OK) return rc;
-    if ((rc = make_tile_map(&mb, W, N, K, use_pair ? 128 : kGemmBN)) != LT_OK) return rc;
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, stream);
-    if (e != cudaSuccess) return record_cuda_error("cudaMemsetAsync(status)", e);
+    if ((rc = make_tile_map(&mb, W, N, K, use_pair ? 128 : plan.bn)) != LT_OK) return rc;
+    if (!use_pair && plan.bn == 64)
+        return bf16 ? launch_gemm_split<64, true>(ma, mb, prm, plan.split, stream)
+                    : launch_gemm_split<64, false>(ma, mb, prm, plan.split, stream);
+    if (!use_pair && plan.bn == 128)
+        return bf16 ? launch_gemm_split<128, true>(ma, mb, prm, plan.split, stream)
+                    : launch_gemm_split<128, false>(ma, mb, prm, plan.split, stream);
+    if (!use_pair && plan.bn == 256 && plan.split > 1)
+        return bf16 ? launch_gemm_split<256, true>(ma, mb, prm, plan.split, stream)
+                    : launch_gemm_split<256, false>(ma, mb, prm, plan.split, stream);
+    cudaError_t e = cudaSuccess;
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.stream = stream;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = 1;
     if (use_pair) {
-        GemmParams prm;
-        prm.C = reinterpret_cast<__half *>(C);
-        prm.status = reinterpret_cast<unsigned int *>(workspace);
-        prm.M = M; prm.N = N; prm.K = K;
         prm.tiles_m = (M + kPairBM - 1) / kPairBM;
         prm.tiles_n = (N + kPairBN - 1) / kPairBN;
         const long long rows = static_cast<long long>(48.0e6 / (static_cast<double>(kPairBM) * K * 2.0));
@@ -445,34 +704,32 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
         static int max_pairs_cached[2] = {0, 0};
         int &max_pairs = max_pairs_cached[bf16 ? 1 : 0];
         if (max_pairs == 0) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(2);
-            cfg.blockDim = dim3(kGemmThreads);
-            cfg.dynamicSmemBytes = smem;
+            cudaLaunchConfig_t one = {};
+            one.gridDim = dim3(2);
+            one.blockDim = dim3(kGemmThreads);
+            one.dynamicSmemBytes = smem;
             cudaLaunchAttribute attr;
             attr.id = cudaLaunchAttributeClusterDimension;
             attr.val.clusterDim.x = 2;
             attr.val.clusterDim.y = 1;
             attr.val.clusterDim.z = 1;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
+            one.attrs = &attr;
+            one.numAttrs = 1;
             int n = 0;
-            e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+            e = cudaOccupancyMaxActiveClusters(&n, kernel, &one);
             if (e != cudaSuccess || n < 1) return record_cuda_error("cudaOccupancyMaxActiveClusters", e);
             max_pairs = n;
         }
         const long long n_tiles = static_cast<long long>(prm.tiles_m) * prm.tiles_n;
         const int pairs = static_cast<int>(n_tiles < max_pairs ? n_tiles : max_pairs);
-        kernel<<<2 * pairs, kGemmThreads, smem, stream>>>(ma, mb, prm);
-        e = cudaGetLastError();
+        cfg.gridDim = dim3(2 * pairs);
+        cfg.dynamicSmemBytes = smem;
+        e = cudaLaunchKernelEx(&cfg, kernel, ma, mb, prm);
+        if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return record_cuda_error("gemm_pair_kernel launch", e);
         return LT_OK;
     }
 
-    GemmParams prm;
-    prm.C = reinterpret_cast<__half *>(C);
-    prm.status = reinterpret_cast<unsigned int *>(workspace);
-    prm.M = M; prm.N = N; prm.K = K;
     prm.tiles_m = (M + kGemmBM - 1) / kGemmBM;
     prm.tiles_n = (N + kGemmBN - 1) / kGemmBN;
     {
@@ -492,8 +749,10 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
     }
     const long long n_tiles = static_cast<long long>(prm.tiles_m) * prm.tiles_n;
     const int grid = static_cast<int>(n_tiles < sms ? n_tiles : sms);
-    kernel<<<grid, kGemmThreads, smem, stream>>>(ma, mb, prm);
-    e = cudaGetLastError();
+    cfg.gridDim = dim3(grid);
+    cfg.dynamicSmemBytes = smem;
+    e = cudaLaunchKernelEx(&cfg, kernel, ma, mb, prm);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("gemm_kernel launch", e);
     return LT_OK;
 }

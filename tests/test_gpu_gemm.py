@@ -55,6 +55,35 @@ def test_gemm_matches_oracle(lt, oracle, M, N, K):
     assert np.max(np.abs(got - ref) - 2.0 ** -10 * np.abs(ref)) <= 1e-3
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (1, 8, 64), (5, 64, 8), (128, 64, 72),         # one narrow tile; one contraction block, a ragged second one
+    (1, 136, 520), (77, 1000, 1000), (129, 65, 4096),  # shares of unequal length; more CTAs of a cluster than rows
+    (3, 130, 8192), (128, 128, 4096),              # eight shares
+    (424, 265, 5920), (300, 127, 2056),            # several tile rows, N odd (scalar stores) and just below a tile
+    (130, 2048, 2048), (16, 5504, 4096), (40, 6000, 2000),  # 128- and 256-wide tiles, two to six shares
+    (1000, 2040, 4096), (600, 600, 600), (8192, 72, 136),   # more tiles than fit at once, short contractions
+])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_gemm_few_tiles(lt, M, N, K, dtype):
+    """Narrow tiles and split contractions against fp64 products of the same operands."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(M + N + K)
+    A = torch.randn((M, K), generator=gen, device="cuda").to(dtype)
+    W = (torch.randn((N, K), generator=gen, device="cuda") * K ** -0.5).to(dtype)
+    C = torch.full((M + 1, N), float("nan"), dtype=dtype, device="cuda")  # the row past the end must stay untouched
+    ws = lt.alloc_workspace(lt.lt_gemm_f16_workspace_bytes())
+    ws.fill_(0xFF)
+    lt.lt_gemm_f16(A, W, C[:M], ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    ref = A.double() @ W.double().T
+    err = (C[:M].double() - ref).abs()
+    half_ulp = 2.0 ** -11 if dtype == torch.float16 else 2.0 ** -8  # rounding of the result, relative to it
+    # plus fp32 accumulation: K products of order K^-1/2, each addition off by at most 2^-24 of a sum of order one (a
+    # factor of eight above that for the largest of up to a million elements), and the smallest subnormal step
+    assert (err <= half_ulp * ref.abs() + 8 * K ** 0.5 * 2.0 ** -24 + 2.0 ** -24).all(), float(err.max())
+    assert torch.isnan(C[M]).all()
+
+
 def test_gemm_integer_operands_are_exact(lt, oracle):
     """Small integers: every product and partial sum is exact in fp32 and fp16, so the result must
     equal the oracle bit for bit."""
