@@ -27,10 +27,12 @@ constexpr uint32_t kGemmBBytes = kGemmBN * kGemmBK * 2;   // 32 KB
 
 enum { kWaitGemmFull = 401, kWaitGemmEmpty = 402, kWaitGemmAccFull = 403, kWaitGemmAccEmpty = 404 };
 
+constexpr int kStagePitch = 33;
 struct __align__(1024) GemmSmem {
     uint8_t a[kGemmStages][kGemmABytes];
     uint8_t b[kGemmStages][kGemmBBytes];
     uint64_t bar_full[kGemmStages], bar_empty[kGemmStages], bar_acc_full[2], bar_acc_empty[2];
+    float stage[4][32 * kStagePitch];  // per epilogue warp: 32 x 32 of a tile on a ragged edge
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -56,6 +58,30 @@ __device__ __forceinline__ void gemm_tile_coords(const GemmParams &p, int tile, 
     const int r = tile - g * per_group;
     tm = first_m + r % rows;
     tn = r / rows;
+}
+
+// 32 rows x 32 columns of the output whose rows are not a whole number of 16-byte pieces (N % 8 != 0) or that stick out
+// past column N.  Each lane arrives with one row in registers; through shared memory the warp turns it so that
+// neighbouring lanes store neighbouring columns: 64 contiguous bytes per row and instruction, where a lane storing its own row
+// two bytes at a time touched a sector for every element (113 x 4051 x 208: 39 us).
+template <bool kBf16>
+__device__ __forceinline__ void gemm_store_ragged(float *stage, const uint32_t (&r)[32], const GemmParams &p,
+                                                  long long m0, int nc, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 32; ++e) stage[lane * kStagePitch + e] = __uint_as_float(r[e]);
+    __syncwarp();
+    const int rows = p.M - m0 < 32 ? static_cast<int>(p.M - m0) : 32;
+    if ((p.N & 1) == 0) {  // pairs of columns: half a warp per row
+        const int col = (lane & 15) * 2;
+        for (int q = lane >> 4; q < rows && nc + col < p.N; q += 2)
+            *reinterpret_cast<uint32_t *>(p.C + (m0 + q) * p.N + nc + col) =
+                pack2<kBf16>(stage[q * kStagePitch + col], stage[q * kStagePitch + col + 1]);
+    } else {
+        for (int q = 0; q < rows && nc + lane < p.N; ++q)
+            reinterpret_cast<uint16_t *>(p.C)[(m0 + q) * p.N + nc + lane] =
+                static_cast<uint16_t>(pack2<kBf16>(stage[q * kStagePitch + lane], 0.f) & 0xFFFFu);
+    }
 }
 
 template <bool kBf16>
@@ -195,9 +221,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sm.bar_acc_empty[acc]);
                 }
-                if (m < p.M) {
-                    const int nc = n0 + c * 32;
-                    if (vec_ok && nc + 32 <= p.N) {
+                const int nc = n0 + c * 32;
+                if (vec_ok && nc + 32 <= p.N) {
+                    if (m < p.M) {
 #pragma unroll
                         for (int v8 = 0; v8 < 4; ++v8) {
                             uint4 o;
@@ -207,13 +233,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                             o.w = pack2<kBf16>(__uint_as_float(r[8 * v8 + 6]), __uint_as_float(r[8 * v8 + 7]));
                             reinterpret_cast<uint4 *>(c_row + c * 32)[v8] = o;
                         }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (nc + e < p.N)
-                                reinterpret_cast<uint16_t *>(c_row)[c * 32 + e] =
-                                    static_cast<uint16_t>(pack2<kBf16>(__uint_as_float(r[e]), 0.f) & 0xFFFFu);
                     }
+                } else if (nc < p.N) {
+                    gemm_store_ragged<kBf16>(sm.stage[quad], r, p, m - lane, nc, lane);
                 }
             }
         }
@@ -239,6 +261,7 @@ struct __align__(1024) GemmPairSmem {
     uint8_t a[kPairStages][kPairABytes];
     uint8_t b[kPairStages][kPairBBytes];
     uint64_t bar_full[kPairStages], bar_empty[kPairStages], bar_acc_full[2], bar_acc_empty[2];
+    float stage[4][32 * kStagePitch];  // per epilogue warp: 32 x 32 of a tile on a ragged edge
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -374,9 +397,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(acc_empty0);
                 }
-                if (m < p.M) {
-                    const int nc = n0 + c * 32;
-                    if (vec_ok && nc + 32 <= p.N) {
+                const int nc = n0 + c * 32;
+                if (vec_ok && nc + 32 <= p.N) {
+                    if (m < p.M) {
 #pragma unroll
                         for (int v8 = 0; v8 < 4; ++v8) {
                             uint4 o;
@@ -386,13 +409,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                             o.w = pack2<kBf16>(__uint_as_float(r[8 * v8 + 6]), __uint_as_float(r[8 * v8 + 7]));
                             reinterpret_cast<uint4 *>(c_row + c * 32)[v8] = o;
                         }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (nc + e < p.N)
-                                reinterpret_cast<uint16_t *>(c_row)[c * 32 + e] =
-                                    static_cast<uint16_t>(pack2<kBf16>(__uint_as_float(r[e]), 0.f) & 0xFFFFu);
                     }
+                } else if (nc < p.N) {
+                    gemm_store_ragged<kBf16>(sm.stage[quad], r, p, m - lane, nc, lane);
                 }
             }
         }
@@ -554,6 +573,8 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
             if (vec_ok) {  // (N a multiple of eight: a piece lies inside the row or outside)
                 *reinterpret_cast<uint4 *>(dst) = o;
             } else {
+                // (one column per lane instead, with 4-byte reads of the partials, was slower: 274 x 3485 x 4424 56 us
+                // against 36)
                 const uint32_t w[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
