@@ -39,6 +39,7 @@
 #include <mutex>
 #include <stddef.h>
 #include <stdio.h>
+#include <type_traits>
 
 #include "lt_common.cuh"
 #include "lt_host.h"
@@ -871,7 +872,11 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 dst[4 * v] = u.x; dst[4 * v + 1] = u.y; dst[4 * v + 2] = u.z; dst[4 * v + 3] = u.w;
             }
         };
-        auto compute_p = [&](const BwdItem &w, int n, int t) -> bool {
+        // P' of running iteration t; masked: some keys of the tile are hidden.  D = 64 has an instantiation of its own for
+        // that: as selects behind a uniform flag the masks cost every tile 400 cycles of a pass that its tensor products
+        // wait for.  D = 128 is not bound by these warps, and a second copy of the pass cost it 3 %.
+        auto form_p = [&](const BwdItem &w, int t, bool diag, bool masked, auto masked_tag) -> bool {
+            constexpr bool kMasked = decltype(masked_tag)::value;
             if constexpr (kSavedP) {
                 // P'^T of the previous pair must have been read by its dV product before it is replaced
                 if (t > 0 && !LT_WAIT(&sm.bar_do_empty, (t - 1) & 1, kWaitDoEmpty)) return false;
@@ -894,8 +899,6 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             tc_fence_after_sync();
             LT_TL(tid == kComputeWarp0 * 32, 7, t);
             LT_TRACE_MARK(tp0);
-            const int hh = n / w.tiles_per_head;
-            const bool diag = p.causal && (w.i_first + (n - hh * w.tiles_per_head) == w.j);
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 // (one load at a time: asking for both halves before the first is used measured 2 % slower)
@@ -907,16 +910,14 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 for (int e = 0; e < 32; ++e)
                     pv[c * 32 + e] = __float_as_uint(fast_exp2(fmaf(__uint_as_float(sv[e]), scale_log2, p_scale_log2)));
             }
-            if (diag) {  // key row is hidden from query column q when row > q
+            if (kMasked || (D == 128 && masked)) {
+                // the key row is hidden from the query columns before it (causal diagonal), or it lies past the end of
+                // the sequence (ragged last tile): its zero-filled K row has score 0, which LSE does not bound, so its P
+                // is not a probability
+                const int first = w.j * kTileRows + row >= p.S ? 64 : diag ? row - static_cast<int>(cbase) : 0;
 #pragma unroll
                 for (int e = 0; e < 64; ++e)
-                    if (row > static_cast<int>(cbase) + e) pv[e] = 0u;
-            }
-            if (w.j * kTileRows + row >= p.S) {
-                // a key row past the end of the sequence (ragged last tile): its zero-filled K row has
-                // score 0, which LSE does not bound, so its P is not a probability; hide it
-#pragma unroll
-                for (int e = 0; e < 64; ++e) pv[e] = 0u;
+                    if (e < first) pv[e] = 0u;
             }
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -936,13 +937,23 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             return true;
         };
 
+        // tile: the query tile's index inside its head, counted from the first visible one
+        auto compute_p = [&](const BwdItem &w, int t, int tile) -> bool {
+            const bool diag = p.causal && tile == 0;
+            const bool masked = !kSavedP && (diag || (w.j + 1) * kTileRows > p.S);
+            if constexpr (D == 64 && !kSavedP)
+                if (masked) return form_p(w, t, diag, true, std::true_type{});
+            return form_p(w, t, diag, masked, std::false_type{});
+        };
+
         for (;; ++ic) {
             if (!ok || !LT_WAIT(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem)) break;
             const int item = sm.item_ring[ic % kItemRing];
             if (item < 0) break;
             const BwdItem w = bwd_item<kSplit>(p, item);
             if constexpr (kSavedP) load_saved_p(w, 0, ph);
-            ok = compute_p(w, 0, it);
+            ok = compute_p(w, it, 0);
+            int tile = 0;
             for (int n = 0; n < w.n_iter && ok; ++n, ++it) {
                 if constexpr (kSavedP)
                     if (n + 1 < w.n_iter) load_saved_p(w, n + 1, pn);
@@ -993,7 +1004,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
                     for (int e = 0; e < 32; ++e) ph[e] = pn[e];
                 }
-                if (n + 1 < w.n_iter) ok = compute_p(w, n + 1, it + 1);
+                if (++tile == w.tiles_per_head) tile = 0;
+                if (n + 1 < w.n_iter) ok = compute_p(w, it + 1, tile);
             }
 
         }
