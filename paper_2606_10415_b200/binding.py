@@ -123,18 +123,18 @@ def last_cuda_error() -> str:
 
 
 def _stream_ptr(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the current stream's handle, without building a Stream object (3.2 us of a call's host time)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream)
 
 
 def _ptr(t) -> int:
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def _dims(Q: torch.Tensor, K: torch.Tensor):
     B, Hq, S, D = Q.shape
-    return int(B), int(Hq), int(K.shape[1]), int(S), int(D)
+    return B, Hq, K.shape[1], S, D
 
 
 def _check_layout(*tensors):
@@ -178,7 +178,7 @@ def lt_attn_fwd(Q, K, V, O, LSE, causal, scale, workspace, stream=None) -> None:
     _check_layout(Q, K, V, O, LSE)
     B, Hq, Hkv, S, D = _dims(Q, K)
     rc = _lib.lt_attn_fwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), B, Hq, Hkv, S, D, int(bool(causal)),
-                          float(scale), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                          float(scale), _ptr(workspace), workspace.nbytes,
                           _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_fwd", rc)
@@ -190,7 +190,7 @@ def lt_attn_bwd(Q, K, V, O, dO, LSE, dQ, dK, dV, causal, scale, workspace, strea
     B, Hq, Hkv, S, D = _dims(Q, K)
     rc = _lib.lt_attn_bwd(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(dQ), _ptr(dK), _ptr(dV),
                           B, Hq, Hkv, S, D, int(bool(causal)), float(scale), _ptr(workspace),
-                          workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                          workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_bwd", rc)
 
@@ -208,7 +208,7 @@ def lt_attn_save_p(Q, K, LSE, P, causal, scale, workspace, stream=None) -> None:
     if P.numel() * P.element_size() < lt_attn_p_store_bytes(B, Hq, Hkv, S, D):
         raise ValueError("P is smaller than lt_attn_p_store_bytes()")
     rc = _lib.lt_attn_save_p(_ptr(Q), _ptr(K), _ptr(LSE), _ptr(P), B, Hq, Hkv, S, D, int(bool(causal)), float(scale),
-                             _ptr(workspace), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                             _ptr(workspace), workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_save_p", rc)
 
@@ -221,7 +221,7 @@ def lt_attn_bwd_saved_p(Q, K, V, O, dO, P, dQ, dK, dV, causal, scale, workspace,
         raise ValueError("P is smaller than lt_attn_p_store_bytes()")
     rc = _lib.lt_attn_bwd_saved_p(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(P), _ptr(dQ), _ptr(dK),
                                   _ptr(dV), B, Hq, Hkv, S, D, int(bool(causal)), float(scale), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                                  workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_bwd_saved_p", rc)
 
@@ -242,7 +242,7 @@ def lt_attn_fwd_strided(Q, K, V, O, LSE, causal, scale, workspace, stream=None) 
     lay.q, lay.k, lay.v, lay.o = (_strides_of(t) for t in (Q, K, V, O))
     rc = _lib.lt_attn_fwd_strided(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), ctypes.byref(lay), B, Hq, Hkv, S, D,
                                   int(bool(causal)), float(scale), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                                  workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_fwd_strided", rc)
 
@@ -256,7 +256,7 @@ def lt_attn_bwd_strided(Q, K, V, O, dO, LSE, dQ, dK, dV, causal, scale, workspac
         _strides_of(t) for t in (Q, K, V, O, dO, dQ, dK, dV))
     rc = _lib.lt_attn_bwd_strided(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(dQ), _ptr(dK),
                                   _ptr(dV), ctypes.byref(lay), B, Hq, Hkv, S, D, int(bool(causal)), float(scale),
-                                  _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                  _ptr(workspace), workspace.nbytes,
                                   _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_bwd_strided", rc)
@@ -277,7 +277,7 @@ def lt_gemm_f16(A, W, C, workspace, stream=None) -> None:
     if W.shape[1] != K or tuple(C.shape) != (M, N):
         raise ValueError("expected A [M, K], W [N, K], C [M, N]")
     rc = fn(_ptr(A), _ptr(W), _ptr(C), M, N, K, _ptr(workspace),
-                          workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                          workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_gemm_f16", rc)
 
@@ -297,7 +297,7 @@ def lt_attn_fwd_bf16(Q, K, V, O, LSE, causal, scale, workspace, stream=None) -> 
     lay.q, lay.k, lay.v, lay.o = (_strides_of(t) for t in (Q, K, V, O))
     rc = _lib.lt_attn_fwd_bf16(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(LSE), ctypes.byref(lay), B, Hq, Hkv, S, D,
                                int(bool(causal)), float(scale), _ptr(workspace),
-                               workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                               workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_fwd_bf16", rc)
 
@@ -312,7 +312,7 @@ def lt_attn_bwd_bf16(Q, K, V, O, dO, LSE, dQ, dK, dV, causal, scale, workspace, 
         _strides_of(t) for t in (Q, K, V, O, dO, dQ, dK, dV))
     rc = _lib.lt_attn_bwd_bf16(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(dQ), _ptr(dK), _ptr(dV),
                                ctypes.byref(lay), B, Hq, Hkv, S, D, int(bool(causal)), float(scale), _ptr(workspace),
-                               workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                               workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_bwd_bf16", rc)
 
@@ -327,7 +327,7 @@ def lt_attn_bwd_profiled(Q, K, V, O, dO, LSE, dQ, dK, dV, causal, scale, workspa
     e1 = 0 if main_end is None else int(main_end.cuda_event)
     rc = _lib.lt_attn_bwd_profiled(_ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(dO), _ptr(LSE), _ptr(dQ), _ptr(dK),
                                    _ptr(dV), B, Hq, Hkv, S, D, int(bool(causal)), float(scale), _ptr(workspace),
-                                   workspace.numel() * workspace.element_size(), _stream_ptr(stream), e0, e1)
+                                   workspace.nbytes, _stream_ptr(stream), e0, e1)
     if rc != LT_OK:
         raise LtError("lt_attn_bwd_profiled", rc)
 
@@ -362,7 +362,7 @@ def lt_attn_fwd_bwd_host(Q, K, V, dO, O, LSE, dQ, dK, dV, causal, scale, arena, 
     B, Hq, Hkv, S, D = _dims(Q, K)
     rc = _lib.lt_attn_fwd_bwd_host(_ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(O), _ptr(LSE), _ptr(dQ), _ptr(dK),
                                    _ptr(dV), B, Hq, Hkv, S, D, int(bool(causal)), float(scale), _ptr(arena),
-                                   arena.numel() * arena.element_size(), _stream_ptr(stream))
+                                   arena.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_attn_fwd_bwd_host", rc)
 
@@ -373,13 +373,13 @@ def lt_attn_check_status(workspace, stream=None) -> int:
 
 def lt_dbg_tile_gemm(A, B, C, mode, workspace, stream=None) -> None:
     rc = _lib.lt_dbg_tile_gemm(_ptr(A), _ptr(B), _ptr(C), int(mode), _ptr(workspace),
-                               workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+                               workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_dbg_tile_gemm", rc)
 
 
 def lt_dbg_wait_timeout(workspace, stream=None) -> None:
-    rc = _lib.lt_dbg_wait_timeout(_ptr(workspace), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+    rc = _lib.lt_dbg_wait_timeout(_ptr(workspace), workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_dbg_wait_timeout", rc)
 
