@@ -502,11 +502,12 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
 }
 
 // Internal streams and events of the host-buffer entry point, created on first use per device.
-constexpr int kHostMaxChunks = 8, kHostMaxDevices = 64;
+constexpr int kHostMaxChunks = 10, kHostMaxDevices = 64;
 struct HostPipe {
     bool ready = false;
     cudaStream_t s_in = nullptr, s_out = nullptr;
-    cudaEvent_t ev_start = nullptr, ev_out = nullptr, ev_in[kHostMaxChunks] = {}, ev_comp[kHostMaxChunks] = {};
+    cudaEvent_t ev_start = nullptr, ev_out = nullptr, ev_in[kHostMaxChunks] = {}, ev_do[kHostMaxChunks] = {}, ev_fwd[kHostMaxChunks] = {},
+                ev_comp[kHostMaxChunks] = {};
 };
 static HostPipe g_host_pipe[kHostMaxDevices];
 static std::mutex g_host_pipe_mu;
@@ -611,22 +612,31 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
     // previous one and the device-to-host copy of the one before run at the same time (two copy engines
     // and the SMs), on two internal streams beside the caller's.  A chunk is a contiguous slice of every
     // tensor and a problem of its own with B = 1.
+    // A chunk's forward starts when its Q, K, V are there (dO follows), and its O and LSE go back while its backward runs.
     const int G = Hq / Hkv;
     const int n_units = B * Hkv;
     const long long n_tiles = padded_rows(S) / 128;
     const long long unit_iters = static_cast<long long>(G) * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
-    // Few, large chunks (a copy of a few MB carries tens of microseconds of fixed cost, and a chunk's kernels take
-    // 0.2 ms however small it is); the last chunk is the smallest, because its kernels and its copy back are what is
-    // left to do when the input copy ends.
+    // Few chunks where a chunk's kernels are long however small it is (its longest work item is a serial walk of a group's
+    // tile pairs, about 2.1 us each) or copies would get small (beside copies in the other direction one of 3 MB costs
+    // 15 us on top of its bytes); otherwise ten, the first small, because the copies back are the longer queue and start
+    // with it, the last ones smaller still, because their kernels and copies back are what is left when the input copy
+    // ends.  Measured with O returned, ms, four / ten chunks: LLaMA-2-7B layer 3.74 / 3.54, 4 x 16 heads at S = 1024
+    // unmasked 1.97 / 1.94, Qwen2.5-32B layer (8 units) 2.98 / 3.81, 16 / 4 heads twice at S = 2048, D = 64 0.78 / 1.22.
     int bounds[kHostMaxChunks + 1];
     int n_chunks = 1;
     bounds[0] = 0;
     bounds[1] = n_units;
     if (unit_iters * n_units >= 3000 && n_units > 1) {  // otherwise not worth the extra streams
-        const int percent[4] = {30, 60, 85, 100};  // cumulative shares of the four chunks
+        constexpr int kFew[4] = {30, 60, 85, 100}, kMany[10] = {6, 18, 30, 42, 54, 66, 78, 88, 95, 100};  // cumulative shares, %
+        const double copy_us = static_cast<double>(2 * bq + 2 * bk) / 48.0e3;  // at 48 GB/s
+        const double chunk_us = 2.1 * G * n_tiles + 1.9 * n_tiles + 20.0;      // a small chunk's backward, forward, launches
+        const bool many = n_units >= 20 && copy_us > 15.0 * chunk_us;
+        const int *percent = many ? kMany : kFew;
+        const int np = many ? 10 : 4;
         n_chunks = 0;
-        for (int c = 0; c < 4; ++c) {
-            int end = c == 3 ? n_units : (n_units * percent[c] + 50) / 100;
+        for (int c = 0; c < np; ++c) {
+            const int end = c == np - 1 ? n_units : (n_units * percent[c] + 50) / 100;
             if (end <= bounds[n_chunks]) continue;  // fewer units than chunks
             bounds[++n_chunks] = end;
         }
@@ -647,6 +657,8 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
                       cudaEventCreateWithFlags(&pipe->ev_out, cudaEventDisableTiming) == cudaSuccess;
             for (int c = 0; c < kHostMaxChunks && ok; ++c)
                 ok = cudaEventCreateWithFlags(&pipe->ev_in[c], cudaEventDisableTiming) == cudaSuccess &&
+                     cudaEventCreateWithFlags(&pipe->ev_do[c], cudaEventDisableTiming) == cudaSuccess &&
+                     cudaEventCreateWithFlags(&pipe->ev_fwd[c], cudaEventDisableTiming) == cudaSuccess &&
                      cudaEventCreateWithFlags(&pipe->ev_comp[c], cudaEventDisableTiming) == cudaSuccess;
             if (!ok) return record_cuda_error("stream/event creation for the host pipeline", cudaGetLastError());
             pipe->ready = true;
@@ -671,14 +683,22 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
         LT_CUDA(cudaMemcpyAsync(d_Q + oq, Q + oq, cq, cudaMemcpyHostToDevice, s_in), "cudaMemcpyAsync");
         LT_CUDA(cudaMemcpyAsync(d_K + ok_, K + ok_, ck, cudaMemcpyHostToDevice, s_in), "cudaMemcpyAsync");
         LT_CUDA(cudaMemcpyAsync(d_V + ok_, V + ok_, ck, cudaMemcpyHostToDevice, s_in), "cudaMemcpyAsync");
-        LT_CUDA(cudaMemcpyAsync(d_dO + oq, dO + oq, cq, cudaMemcpyHostToDevice, s_in), "cudaMemcpyAsync");
         if (pipe) {
             LT_CUDA(cudaEventRecord(pipe->ev_in[c], s_in), "cudaEventRecord");
             LT_CUDA(cudaStreamWaitEvent(stream, pipe->ev_in[c], 0), "cudaStreamWaitEvent");
         }
+        LT_CUDA(cudaMemcpyAsync(d_dO + oq, dO + oq, cq, cudaMemcpyHostToDevice, s_in), "cudaMemcpyAsync");
+        if (pipe) LT_CUDA(cudaEventRecord(pipe->ev_do[c], s_in), "cudaEventRecord");
         rc = lt_attn_fwd(d_Q + oq, d_K + ok_, d_V + ok_, d_O + oq, d_lse + ol, 1, hq, hkv, S, D, causal, scale, fwd_ws,
                          kStatusBytes, stream);
         if (rc != LT_OK) return rc;
+        if (pipe) {
+            LT_CUDA(cudaEventRecord(pipe->ev_fwd[c], stream), "cudaEventRecord");
+            LT_CUDA(cudaStreamWaitEvent(stream, pipe->ev_do[c], 0), "cudaStreamWaitEvent");
+            LT_CUDA(cudaStreamWaitEvent(s_out, pipe->ev_fwd[c], 0), "cudaStreamWaitEvent");
+        }
+        if (O) LT_CUDA(cudaMemcpyAsync(O + oq, d_O + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
+        if (LSE) LT_CUDA(cudaMemcpyAsync(LSE + ol, d_lse + ol, cl, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         rc = lt_attn_bwd(d_Q + oq, d_K + ok_, d_V + ok_, d_O + oq, d_dO + oq, d_lse + ol, d_dQ + oq, d_dK + ok_,
                          d_dV + ok_, 1, hq, hkv, S, D, causal, scale, ws, ws_bytes, stream);
         if (rc != LT_OK) return rc;
@@ -686,8 +706,6 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
             LT_CUDA(cudaEventRecord(pipe->ev_comp[c], stream), "cudaEventRecord");
             LT_CUDA(cudaStreamWaitEvent(s_out, pipe->ev_comp[c], 0), "cudaStreamWaitEvent");
         }
-        if (O) LT_CUDA(cudaMemcpyAsync(O + oq, d_O + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
-        if (LSE) LT_CUDA(cudaMemcpyAsync(LSE + ol, d_lse + ol, cl, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         LT_CUDA(cudaMemcpyAsync(dQ + oq, d_dQ + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         LT_CUDA(cudaMemcpyAsync(dK + ok_, d_dK + ok_, ck, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         LT_CUDA(cudaMemcpyAsync(dV + ok_, d_dV + ok_, ck, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");

@@ -1,0 +1,38 @@
+"""The host-buffer call cut into many chunks (ten where copies outlast a chunk's kernels): every unit of every chunk
+against the device entry points on the whole problem, with and without the optional outputs, calls back to back."""
+import pytest
+import torch
+
+from paper_2606_10415_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(4, 16, 16, 1024, 128, False), (1, 24, 24, 3000, 128, True)])
+@pytest.mark.parametrize("with_o", [True, False])
+def test_many_chunks(B, Hq, Hkv, S, D, causal, with_o):
+    from paper_2606_10415_b200 import binding as lt
+    cfg = workloads.custom(B, Hq, Hkv, S, D, causal, seed=S)
+    host = [t.pin_memory() for t in workloads.make_inputs(cfg)]
+    Q, K, V, dO = (t.cuda() for t in host)
+    O, LSE = torch.empty_like(Q), torch.empty(Q.shape[:3], dtype=torch.float32, device="cuda")
+    want = [torch.empty_like(t) for t in (Q, K, V)]
+    dims = (B, Hq, Hkv, S, D)
+    ws = lt.alloc_workspace(lt.lt_attn_bwd_workspace_bytes(*dims))
+    lt.lt_attn_fwd(Q, K, V, O, LSE, causal, cfg.scale, ws)
+    lt.lt_attn_bwd(Q, K, V, O, dO, LSE, *want, causal, cfg.scale, ws)
+    h_O = torch.full(Q.shape, float("nan"), dtype=torch.float16, pin_memory=True) if with_o else None
+    h_L = torch.full(Q.shape[:3], float("nan"), dtype=torch.float32, pin_memory=True) if with_o else None
+    got = [torch.full(t.shape, float("nan"), dtype=torch.float16, pin_memory=True) for t in (Q, K, V)]
+    arena = lt.alloc_workspace(lt.lt_attn_host_arena_bytes(*dims))
+    for _ in range(3):  # later calls reuse the arena under the earlier ones' copies
+        lt.lt_attn_fwd_bwd_host(*host, h_O, h_L, *got, causal, cfg.scale, arena)
+    torch.cuda.synchronize()
+    if with_o:
+        assert torch.equal(h_O, O.cpu()) and torch.equal(h_L, LSE.cpu())
+    for name, g, w in zip(("dQ", "dK", "dV"), got, want):
+        g, w = g.double(), w.cpu().double()
+        assert torch.isfinite(g).all(), name
+        # a chunk picks its own power of two for dS, so roundings to fp16 may fall on the other side: half a unit
+        # in the last place of the operands and of the result, 2^-11 each
+        assert (g - w).norm() <= 2 * 2.0 ** -11 * w.norm(), name
