@@ -262,7 +262,8 @@ const char *lt_last_cuda_error(void);
 /* Number of kernels one call enqueues for this shape (for launch accounting by benchmarks): the
  * backward's preprocess, main and dQ-conversion kernels, plus the dK/dV conversion on grouped-query shapes
  * with fewer than about 1.5 key-tile work items per multiprocessor, where a group's query heads are split
- * over several items (4 instead of 3); 0 for an unsupported shape.  The forward enqueues one kernel. */
+ * over several items (4 instead of 3); sequences of at most 128 rows need 1 or 2 where that is faster; 0 for an unsupported
+ * shape.  The forward enqueues one kernel. */
 int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal);
 int lt_attn_fwd_num_launches(void);
 

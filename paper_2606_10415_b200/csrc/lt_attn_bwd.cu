@@ -84,35 +84,29 @@ __device__ __forceinline__ unsigned int max_slot_bits(unsigned int fp32_bits) {
     return min((fp32_bits + 0xFFFFu) >> 16, kMaxSlotInf);
 }
 
+// What the preprocess pass reads and writes.
+struct PreParams {
+    const __half *dO, *O, *V;
+    const float *lse;  // NULL in the saved-P variant
+    uint4 *delta_ext, *lse_ext;
+    float *dq_acc;  // zeroed; NULL when no accumulator is used
+    int S, S_pad, Hq, Hkv;
+    lt_tensor_strides do_st, o_st, v_st;
+    int plain, v_plain;  // contiguous tensors and no padding: a row's index is its place
+    float inv_scale;
+};
+
+// Rows [row_lo, row_hi) of the padded row space (every head rounded up to S_pad rows, the indexing of delta_ext, lse_ext
+// and dq_acc; padding rows get zeros everywhere), spread over `n_warps` warps of which this is number `warp`.
 template <int D, bool kBf16>
-__global__ void __launch_bounds__(kPreThreads, 3)  // three blocks per multiprocessor keep enough loads in flight
-bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ O, const float *__restrict__ lse,
-                      uint4 *__restrict__ delta_ext, uint4 *__restrict__ lse_ext, float *__restrict__ dq_acc,
-                      long long n_rows, int S, int S_pad, int Hq, lt_tensor_strides do_st, lt_tensor_strides o_st,
-                      int plain, float inv_scale, unsigned int *status, float4 *__restrict__ kv_acc,
-                      long long kv_acc_vec4, const __half *__restrict__ V, long long v_rows, int Hkv,
-                      lt_tensor_strides v_st, int v_plain) {
-    // `n_rows` counts rows of the padded row space (every head rounded up to S_pad rows), the
-    // indexing of delta_ext, lse_ext and dq_acc; padding rows get zeros everywhere.
-    grid_dependency_wait();    // launched under the tail of its predecessor, which may write O or read the workspace
-    grid_launch_dependents();  // the main kernel sets itself up while this kernel's last blocks run
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        status[kStatusWordTimeout] = 0u;
-        status[kStatusWordItemCounter] = 0u;
-    }
-    // fp32 dK/dV sums (only when key tiles are split over several work items): zero them
-    for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < kv_acc_vec4;
-         v += static_cast<long long>(gridDim.x) * blockDim.x)
-        kv_acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+__device__ __forceinline__ void pre_rows(const PreParams &p, long long row_lo, long long row_hi, long long warp,
+                                         long long n_warps, float &max_abs_delta, float &max_norm2) {
     constexpr int kLanesPerRow = D / 8;
     constexpr int kRowsPerWarp = 32 / kLanesPerRow;
     constexpr int kRowsPerTrip = kRowsPerWarp * kPreUnroll;
     const int lane = threadIdx.x & 31;
     const int sub = lane % kLanesPerRow;
-    const long long warp_global = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const long long n_warps = (static_cast<long long>(gridDim.x) * blockDim.x) >> 5;
-    float max_abs_delta = 0.f, max_norm2 = 0.f;
-    for (long long row0 = warp_global * kRowsPerTrip; row0 < n_rows; row0 += n_warps * kRowsPerTrip) {
+    for (long long row0 = row_lo + warp * kRowsPerTrip; row0 < row_hi; row0 += n_warps * kRowsPerTrip) {
         uint4 a[kPreUnroll], b[kPreUnroll];
         float l[kPreUnroll];
 #pragma unroll
@@ -120,27 +114,26 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
             const long long row = row0 + u * kRowsPerWarp + lane / kLanesPerRow;
             a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
             l[u] = 0.f;
-            // rows of dO, O and LSE behind padded row `row` (`plain`: contiguous tensors and no padding,
-            // so all three are row `row` itself)
+            // rows of dO, O and LSE behind padded row `row` (`plain`: all three are row `row` itself)
             long long src_do = row * D, src_o = row * D, src_lse = row;
-            bool valid = row < n_rows;
-            if (!plain && valid) {
-                const int bh = static_cast<int>(row / S_pad);
-                const int s_in = static_cast<int>(row - static_cast<long long>(bh) * S_pad);
-                const int bb = bh / Hq, hh = bh - bb * Hq;
-                valid = s_in < S;
-                src_do = bb * do_st.batch + hh * do_st.head + s_in * do_st.row;
-                src_o = bb * o_st.batch + hh * o_st.head + s_in * o_st.row;
-                src_lse = static_cast<long long>(bh) * S + s_in;
+            bool valid = row < row_hi;
+            if (!p.plain && valid) {
+                const int bh = static_cast<int>(row / p.S_pad);
+                const int s_in = static_cast<int>(row - static_cast<long long>(bh) * p.S_pad);
+                const int bb = bh / p.Hq, hh = bh - bb * p.Hq;
+                valid = s_in < p.S;
+                src_do = bb * p.do_st.batch + hh * p.do_st.head + s_in * p.do_st.row;
+                src_o = bb * p.o_st.batch + hh * p.o_st.head + s_in * p.o_st.row;
+                src_lse = static_cast<long long>(bh) * p.S + s_in;
             }
             if (valid) {
-                a[u] = __ldcs(reinterpret_cast<const uint4 *>(dO + src_do) + sub);
-                b[u] = __ldcs(reinterpret_cast<const uint4 *>(O + src_o) + sub);
-                if (sub == 0 && lse) l[u] = __ldg(lse + src_lse);  // (no LSE in the saved-P variant)
+                a[u] = __ldcs(reinterpret_cast<const uint4 *>(p.dO + src_do) + sub);
+                b[u] = __ldcs(reinterpret_cast<const uint4 *>(p.O + src_o) + sub);
+                if (sub == 0 && p.lse) l[u] = __ldg(p.lse + src_lse);  // (no LSE in the saved-P variant)
             }
-            if (row < n_rows) {
+            if (p.dq_acc && row < row_hi) {
                 // the zero fill does not depend on the loads: issue it while they are in flight
-                float4 *z = reinterpret_cast<float4 *>(dq_acc + row * D) + sub * 2;
+                float4 *z = reinterpret_cast<float4 *>(p.dq_acc + row * D) + sub * 2;
                 z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
                 z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
@@ -165,38 +158,46 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
                 acc += __shfl_xor_sync(0xffffffffu, acc, off);
                 n2 += __shfl_xor_sync(0xffffffffu, n2, off);
             }
-            if (row < n_rows) {
+            if (row < row_hi) {
                 if (sub == 0) {
                     // operand rows of the main kernel's extra contraction step: 256*hi + lo = value
-                    delta_ext[row] = split_ext<kBf16>(-acc);
-                    lse_ext[row] = split_ext<kBf16>(-l[u] * inv_scale);
+                    p.delta_ext[row] = split_ext<kBf16>(-acc);
+                    p.lse_ext[row] = split_ext<kBf16>(-l[u] * p.inv_scale);
                 }
                 max_abs_delta = fmaxf(max_abs_delta, fabsf(acc));
                 max_norm2 = fmaxf(max_norm2, n2);
             }
         }
     }
-    // largest squared row norm of V (rows of the logical [B,Hkv,S]): with the two maxima above it bounds
-    // |dS|, from which the main kernel picks the power of two that dS carries into fp16
-    // (kept as bit patterns: non-negative floats order like them, with inf above every finite value and
-    // NaN above inf, so non-finite inputs saturate the bound)
-    unsigned int max_v2 = 0u;
-    // (from the other end of the grid, whose warps had the fewer rows above)
-    for (long long row0 = (n_warps - 1 - warp_global) * kRowsPerTrip; row0 < v_rows; row0 += n_warps * kRowsPerTrip) {
+}
+
+// Largest squared norm of V's rows [row_lo, row_hi) (rows of the logical [B,Hkv,S]): with the two maxima above it bounds
+// |dS|, from which the main kernel picks the power of two that dS carries into fp16.  (Kept as a bit pattern:
+// non-negative floats order like them, with inf above every finite value and NaN above inf, so non-finite inputs
+// saturate the bound.)
+template <int D, bool kBf16>
+__device__ __forceinline__ void pre_v_rows(const PreParams &p, long long row_lo, long long row_hi, long long warp,
+                                           long long n_warps, unsigned int &max_v2) {
+    constexpr int kLanesPerRow = D / 8;
+    constexpr int kRowsPerWarp = 32 / kLanesPerRow;
+    constexpr int kRowsPerTrip = kRowsPerWarp * kPreUnroll;
+    const int lane = threadIdx.x & 31;
+    const int sub = lane % kLanesPerRow;
+    for (long long row0 = row_lo + warp * kRowsPerTrip; row0 < row_hi; row0 += n_warps * kRowsPerTrip) {
         uint4 a[kPreUnroll];
 #pragma unroll
         for (int u = 0; u < kPreUnroll; ++u) {
             const long long row = row0 + u * kRowsPerWarp + lane / kLanesPerRow;
             a[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (row < v_rows) {
+            if (row < row_hi) {
                 long long src = row * D;
-                if (!v_plain) {
-                    const int bg = static_cast<int>(row / S);
-                    const int s_in = static_cast<int>(row - static_cast<long long>(bg) * S);
-                    const int bb = bg / Hkv, gg = bg - bb * Hkv;
-                    src = bb * v_st.batch + gg * v_st.head + s_in * v_st.row;
+                if (!p.v_plain) {
+                    const int bg = static_cast<int>(row / p.S);
+                    const int s_in = static_cast<int>(row - static_cast<long long>(bg) * p.S);
+                    const int bb = bg / p.Hkv, gg = bg - bb * p.Hkv;
+                    src = bb * p.v_st.batch + gg * p.v_st.head + s_in * p.v_st.row;
                 }
-                a[u] = __ldg(reinterpret_cast<const uint4 *>(V + src) + sub);  // (the main kernel reads V again)
+                a[u] = __ldg(reinterpret_cast<const uint4 *>(p.V + src) + sub);  // (the main kernel reads V again)
             }
         }
 #pragma unroll
@@ -214,6 +215,30 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
             max_v2 = max(max_v2, __float_as_uint(n2) & 0x7fffffffu);
         }
     }
+}
+
+template <int D, bool kBf16>
+__global__ void __launch_bounds__(kPreThreads, 3)  // three blocks per multiprocessor keep enough loads in flight
+bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, unsigned int *status,
+                      float4 *__restrict__ kv_acc, long long kv_acc_vec4) {
+    grid_dependency_wait();    // launched under the tail of its predecessor, which may write O or read the workspace
+    grid_launch_dependents();  // the main kernel sets itself up while this kernel's last blocks run
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        status[kStatusWordTimeout] = 0u;
+        status[kStatusWordItemCounter] = 0u;
+    }
+    // fp32 dK/dV sums (only when key tiles are split over several work items): zero them
+    for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < kv_acc_vec4;
+         v += static_cast<long long>(gridDim.x) * blockDim.x)
+        kv_acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int lane = threadIdx.x & 31;
+    const long long warp_global = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const long long n_warps = (static_cast<long long>(gridDim.x) * blockDim.x) >> 5;
+    float max_abs_delta = 0.f, max_norm2 = 0.f;
+    unsigned int max_v2 = 0u;
+    pre_rows<D, kBf16>(p, 0, n_rows, warp_global, n_warps, max_abs_delta, max_norm2);
+    // (V from the other end of the grid, whose warps had the fewer rows above)
+    pre_v_rows<D, kBf16>(p, 0, v_rows, n_warps - 1 - warp_global, n_warps, max_v2);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         max_abs_delta = fmaxf(max_abs_delta, __shfl_xor_sync(0xffffffffu, max_abs_delta, off));
@@ -233,7 +258,7 @@ bwd_preprocess_kernel(const __half *__restrict__ dO, const __half *__restrict__ 
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int w = 0; w < kPreThreads / 32; ++w) m[k] = max(m[k], block_max[k][w]);
-        uint2 *slot = reinterpret_cast<uint2 *>(lse_ext + static_cast<long long>(blockIdx.x) * pre_rows_per_block<D>()) + 1;
+        uint2 *slot = reinterpret_cast<uint2 *>(p.lse_ext + static_cast<long long>(blockIdx.x) * pre_rows_per_block<D>()) + 1;
         *slot = make_uint2(max_slot_bits(m[0]) | (max_slot_bits(m[1]) << 16), max_slot_bits(m[2]));
     }
 }
@@ -404,6 +429,14 @@ struct BwdSmem {
 
 static_assert(sizeof(BwdSmem<128>) <= 232448, "main kernel shared memory exceeds the 227 KB per-block limit");
 
+// What the one-tile variant needs besides BwdParams: the preprocess pass's operands and the dQ output.
+struct BwdOneTileParams {
+    PreParams pre;
+    __half *dQ;
+    lt_tensor_strides dq_st;
+    int own_pre;  // run that pass in the main kernel
+};
+
 struct BwdParams {
     const uint4 *lse_ext;    // per query row: fp16 (hi, lo, 0 x 6) with 256*hi + lo = -LSE / scale
     const uint4 *delta_ext;  // per query row: fp16 (hi, lo, 0 x 6) with 256*hi + lo = -delta
@@ -493,13 +526,14 @@ __device__ __forceinline__ const __half *saved_p_tile(const BwdParams &p, const 
 // |dS| <= |dP| + |delta| <= max ||dO_row|| * max ||V_row|| + max |delta| over the whole call (the
 // three maxima come from the preprocess kernel, one slot per block of it).  dV and dQ / dK undo the factor
 // exactly in their epilogues.  Run once per CTA by the softmax and reduction warps together.
+// slots_used = false: the maxima are in call_max already.
 template <int D>
-__device__ __forceinline__ int bwd_p_scale_log2(const BwdParams &p, unsigned int *call_max) {
+__device__ __forceinline__ int bwd_p_scale_log2(const BwdParams &p, unsigned int *call_max, bool slots_used) {
     constexpr int kThreads = (kNumComputeWarps + kNumReduceWarps) * 32;
     const long long n_rows = static_cast<long long>(p.B) * p.Hq * p.S_pad;
     // (the -LSE/scale rows follow the -delta rows; the saved-P variant's lse_ext points elsewhere)
     const uint2 *slots = reinterpret_cast<const uint2 *>(p.delta_ext + n_rows) + 1;
-    const int n = pre_blocks<D>(n_rows);
+    const int n = slots_used ? pre_blocks<D>(n_rows) : 0;
     unsigned int m[3] = {0u, 0u, 0u};
 #pragma unroll
     for (int u = 0; u < (kPreMaxBlocks + kThreads - 1) / kThreads; ++u) {
@@ -530,11 +564,16 @@ __device__ __forceinline__ int bwd_p_scale_log2(const BwdParams &p, unsigned int
 // brought into L2 one iteration ahead and every softmax thread reads its own 128 bytes of the tile
 // straight into registers.  BwdParams::lse_ext, which this variant does not need, carries the
 // store's address (the parameter block keeps its size).
-template <int D, bool kBf16, bool kSplit, bool kSavedP = false>
+//
+// kOneTile: the variant for sequences of one tile (S <= 128).  A query tile then has one partial, so dQ leaves the
+// reduction warps rounded, without accumulator, zero fill and conversion kernel; and where a CTA has few heads to
+// go through (own_pre) it runs the preprocess pass over its own units' rows itself and picks its own factor 2^c, so that
+// the call is one launch.  Work items are dealt out by block number.  one_tile_launches() says when and what it measured.
+template <int D, bool kBf16, bool kSplit, bool kSavedP = false, bool kOneTile = false>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
-                const BwdParams p, const __grid_constant__ CUtensorMap map_dq) {
+                const BwdParams p, const __grid_constant__ CUtensorMap map_dq, const BwdOneTileParams one) {
     // map_dq (D = 64 only): the fp32 dQ accumulator as rows of 64 floats, boxes of 128 rows x 32 columns
     using Smem = BwdSmem<D>;
     constexpr int kBoxes = D / 64;
@@ -599,6 +638,9 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // The first work item of a CTA is its block number, and its first tiles are fetched while the preprocess kernel is
     // still running: they are the caller's tensors, complete before that kernel let this one start (it does so after
     // its own wait for its predecessor).  Saves the claim (800 cycles) and the tile latency (1 800) of every call.
+    // (A call of one launch has no such predecessor, and fetches after its wait.)
+    if constexpr (kOneTile)
+        if (one.own_pre) grid_dependency_wait();
     if (warp == 0 && lane == 0 && smem_ok) {
         const BwdItem w = bwd_item<kSplit>(p, static_cast<int>(blockIdx.x));
         const BwdQTile qt = bwd_q_tile(p, w, 0);
@@ -616,6 +658,29 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     // everything above ran while the preprocess kernel was finishing; its results (row operands, zeroed
     // accumulator, running maxima, item counter) are read only from here on
     grid_dependency_wait();
+    if constexpr (kOneTile) {
+        if (one.own_pre) {
+            if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
+            float max_abs_delta = 0.f, max_norm2 = 0.f;
+            unsigned int max_v2 = 0u;
+            __syncwarp();
+            for (int un = blockIdx.x; un < p.B * p.Hkv; un += gridDim.x) {
+                const long long rows = static_cast<long long>(p.Hq / p.Hkv) * p.S_pad;  // the group's heads are neighbours
+                pre_rows<D, kBf16>(one.pre, un * rows, (un + 1) * rows, warp, kBwdThreads / 32, max_abs_delta, max_norm2);
+                pre_v_rows<D, kBf16>(one.pre, static_cast<long long>(un) * p.S, static_cast<long long>(un + 1) * p.S,
+                                     kBwdThreads / 32 - 1 - warp, kBwdThreads / 32, max_v2);
+            }
+            const unsigned int m[3] = {__float_as_uint(max_abs_delta) & 0x7fffffffu, __float_as_uint(max_norm2) & 0x7fffffffu, max_v2};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const unsigned int v = __reduce_max_sync(0xffffffffu, m[k]);
+                if (lane == 0 && v) atomicMax(sm.call_max + k, max_slot_bits(v));
+            }
+            // the operand rows written above are read by bulk copies of this CTA
+            asm volatile("fence.proxy.async;" ::: "memory");
+            __syncthreads();
+        }
+    }
     if (!smem_ok && tid == 0) atomicCAS(p.status + kStatusWordTimeout, 0u, static_cast<unsigned int>(kBadSmemAlign));
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
@@ -641,7 +706,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 // first items) and publish it to the other roles; -1 tells everybody that the list is exhausted
                 auto claim = [&](int slot_ic) -> int {
                     unsigned int v = blockIdx.x;
-                    if (slot_ic > 0) v = atomicAdd(p.status + kStatusWordItemCounter, 1u) + gridDim.x;
+                    if constexpr (kOneTile) v += slot_ic * gridDim.x;
+                    else if (slot_ic > 0) v = atomicAdd(p.status + kStatusWordItemCounter, 1u) + gridDim.x;
                     const int item = v < static_cast<unsigned int>(n_items) ? static_cast<int>(v) : -1;
                     sm.item_ring[slot_ic % kItemRing] = item;
                     mbar_arrive(&sm.bar_item[slot_ic % kItemRing]);
@@ -878,7 +944,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const float scale_log2 = p.scale * kLog2e;
         uint8_t *ds_tile = sm.ds + half_sel * kBoxBytesBwd;
         uint32_t pv[64];  // bits of this thread's 64 fp32 values of P' = P * 2^c for the current tile pair
-        const float p_scale_log2 = static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max));
+        const float p_scale_log2 = static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max, !kOneTile || !one.own_pre));
         bool ok = smem_ok;
         int it = 0, ic = 0;
         LT_TRACE_BEGIN();
@@ -1039,7 +1105,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         warpgroup_regs_set<kRegsReduce, kRegsAtLaunch>();
         const int quad = warp & 3;
         // P carried the factor 2^c through dS into the accumulators; the epilogues take it out again (exact)
-        const float inv_p_scale = exp2f(-static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max)));
+        const float inv_p_scale = exp2f(-static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max, !kOneTile || !one.own_pre)));
         const float dq_mult = p.scale * inv_p_scale;
         bool ok = smem_ok;
         int it = 0, ic = 0;
@@ -1081,6 +1147,23 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 #pragma unroll
                         for (int e = 0; e < kDqStageRows; ++e) buf[e * 128 + d_idx] = __uint_as_float(r[e]) * dq_mult;
                     };
+                    // one tile: the group's rows are final; eight threads per row round sixteen elements each
+                    const BwdQTile qt = bwd_q_tile(p, w, n);
+                    auto put_rows = [&](int k) {
+                        const int rt = tid - kReduceWarp0 * 32, r_in = rt >> 3, c0 = (rt & 7) * 16;
+                        const int s_row = qt.s0 + k * kDqStageRows + r_in;
+                        if (s_row < p.S) {
+                            const float4 *src = reinterpret_cast<const float4 *>(sm.dq_stage[(gq + k) % kDqStageBufs] + r_in * 128 + c0);
+                            uint4 *dst = reinterpret_cast<uint4 *>(one.dQ + qt.b * one.dq_st.batch + qt.h * one.dq_st.head +
+                                                                   s_row * one.dq_st.row + c0);
+#pragma unroll
+                            for (int v = 0; v < 2; ++v) {
+                                const float4 x = src[2 * v], y = src[2 * v + 1];
+                                dst[v] = make_uint4(pack2<kBf16>(x.x, x.y), pack2<kBf16>(x.z, x.w), pack2<kBf16>(y.x, y.y),
+                                                    pack2<kBf16>(y.z, y.w));
+                            }
+                        }
+                    };
                     auto add_rows = [&](int k) {
                         bulk_reduce_add_f32(dq_tile + k * kDqStageRows * 128, sm.dq_stage[(gq + k) % kDqStageBufs],
                                             kDqStageRows * 128 * sizeof(float));
@@ -1108,7 +1191,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     // the buffer where group 1 goes was read by the last reduction but one of the previous pair
                     if (elected) bulk_wait_group_read<1>();
                     named_barrier_sync(kBarReduceWarps, kNumReduceWarps * 32);
-                    if (elected) add_rows(0);
+                    if constexpr (kOneTile) put_rows(0);
+                    else if (elected) add_rows(0);
                     // groups 1..7 rotate through the three buffers: before group k is issued, the bulk
                     // reduction of group k-2 has finished reading, which frees the buffer of group k+1
                     auto stage_rows = [&](int k, const uint32_t *r) {
@@ -1116,7 +1200,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                         fence_proxy_async_smem();
                         if (elected) bulk_wait_group_read<1>();
                         named_barrier_sync(kBarReduceWarps, kNumReduceWarps * 32);
-                        if (elected) add_rows(k);
+                        if constexpr (kOneTile) put_rows(k);
+                        else if (elected) add_rows(k);
                     };
                     stage_rows(1, r0b);
                     stage_rows(2, r1);
@@ -1143,6 +1228,23 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&sm.bar_dq_empty);
                     LT_TRACE_SINCE(12, tr0);
+                    if constexpr (kOneTile) {  // the rows are final
+                        const BwdQTile qt = bwd_q_tile(p, w, n);
+                        if (qt.s0 + q_row < p.S) {
+                            uint4 *dst = reinterpret_cast<uint4 *>(one.dQ + qt.b * one.dq_st.batch + qt.h * one.dq_st.head +
+                                                                   (qt.s0 + q_row) * one.dq_st.row);
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) {
+                                const uint32_t *x = &r[c >> 2][(c & 3) * 8];
+                                uint32_t o[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    o[e] = pack2<kBf16>(__uint_as_float(x[2 * e]) * dq_mult, __uint_as_float(x[2 * e + 1]) * dq_mult);
+                                dst[c] = make_uint4(o[0], o[1], o[2], o[3]);
+                            }
+                        }
+                        continue;
+                    }
                     // the buffer of this tile was last read by the reductions issued two tiles ago
                     if (elected) bulk_wait_group_read<1>();
                     named_barrier_sync(kBarReduceWarps, kNumReduceWarps * 32);
@@ -1311,6 +1413,21 @@ static int heads_per_item(int B, int Hq, int Hkv, int S, int D, int causal) {
     return G;
 }
 
+// Sequences of one tile: launches of a call in the one-tile variant, or 0 where the general path is the faster one.  With
+// one launch a CTA's rows are read by that CTA alone, about 1 us per head; with two the preprocess kernel spreads them over
+// the chip.  At D = 128 a partial that is rounded by the reduction warps themselves, not queued for the copy unit, holds up
+// the next head, so only short walks through a group gain.  Measured, us of device time, general / two launches / one
+// (batch, query / kv heads, S): D = 64: 1, 2/2, 128 11.2 / 9.4 / 8.8; 8, 16/16, 128 14.9 / 12.8 / 11.0; 2, 12/4, 128
+// 14.6 / 13.2 / 13.9; 8, 40/8, 64 22.7 / 19.9 / 21.5.  D = 128: 4, 32/32, 128 20.6 / 18.7 / 16.5; 8, 32/16, 64
+// 24.9 / 23.8 / 20.1; 8, 64/16, 128 40.8 / 37.8 / 36.2; 2, 8/4, 128 16.6 / 17.2 / 18.5; 1, 64/8, 128 29.8 / 35.5 / 47.4.
+static int one_tile_launches(int B, int Hq, int Hkv, int S, int D) {
+    if (S > kTileRows) return 0;
+    const long long sms = sm_count(), units = static_cast<long long>(B) * Hkv, G = Hq / Hkv;
+    const long long heads_per_cta = (units + sms - 1) / sms * G;
+    if (D == 64) return heads_per_cta <= 2 ? 1 : 2;
+    return heads_per_cta <= 4 && (G == 1 || units >= 96) ? 1 : 0;
+}
+
 template <int D, bool kBf16>
 static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
                       const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout &lay, int B,
@@ -1355,20 +1472,39 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl.val.programmaticStreamSerializationAllowed = 1;
     const int sms = sm_count();
-    cudaLaunchConfig_t cfg_pre = {};
-    cfg_pre.gridDim = dim3(pre_blocks<D>(n_rows));
-    cfg_pre.blockDim = dim3(kPreThreads);
-    cfg_pre.stream = stream;
-    cfg_pre.attrs = &pdl;
-    cfg_pre.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg_pre, bwd_preprocess_kernel<D, kBf16>, reinterpret_cast<const __half *>(dO),
-                                       reinterpret_cast<const __half *>(O), LSE, delta_ext, lse_ext, dq_acc, n_rows, S, S_pad,
-                                       Hq, lay.d_o, lay.o, plain_pre, 1.f / scale, status, reinterpret_cast<float4 *>(dk_acc),
-                                       parts > 1 ? static_cast<long long>(kv_floats / 2) : 0LL,
-                                       reinterpret_cast<const __half *>(V), static_cast<long long>(B) * Hkv * S, Hkv, lay.v,
-                                       is_contig(lay.v, Hkv) ? 1 : 0);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return record_cuda_error("bwd_preprocess_kernel launch", e);
+    cudaError_t e = cudaSuccess;
+    BwdOneTileParams one = {};
+    one.pre.dO = reinterpret_cast<const __half *>(dO);
+    one.pre.O = reinterpret_cast<const __half *>(O);
+    one.pre.V = reinterpret_cast<const __half *>(V);
+    one.pre.lse = LSE;
+    one.pre.delta_ext = delta_ext;
+    one.pre.lse_ext = lse_ext;
+    one.pre.dq_acc = dq_acc;
+    one.pre.S = S; one.pre.S_pad = S_pad; one.pre.Hq = Hq; one.pre.Hkv = Hkv;
+    one.pre.do_st = lay.d_o; one.pre.o_st = lay.o; one.pre.v_st = lay.v;
+    one.pre.plain = plain_pre;
+    one.pre.v_plain = is_contig(lay.v, Hkv) ? 1 : 0;
+    one.pre.inv_scale = 1.f / scale;
+    one.dQ = reinterpret_cast<__half *>(dQ);
+    one.dq_st = lay.dq;
+    const int tile_launches = saved_p || parts > 1 ? 0 : one_tile_launches(B, Hq, Hkv, S, D);
+    const bool one_tile = tile_launches > 0;
+    one.own_pre = tile_launches == 1 ? 1 : 0;
+    if (one_tile) one.pre.dq_acc = nullptr;
+    if (!one.own_pre) {
+        cudaLaunchConfig_t cfg_pre = {};
+        cfg_pre.gridDim = dim3(pre_blocks<D>(n_rows));
+        cfg_pre.blockDim = dim3(kPreThreads);
+        cfg_pre.stream = stream;
+        cfg_pre.attrs = &pdl;
+        cfg_pre.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg_pre, bwd_preprocess_kernel<D, kBf16>, one.pre, n_rows,
+                               static_cast<long long>(B) * Hkv * S, status, reinterpret_cast<float4 *>(dk_acc),
+                               parts > 1 ? static_cast<long long>(kv_floats / 2) : 0LL);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) return record_cuda_error("bwd_preprocess_kernel launch", e);
+    }
 
     BwdParams prm;
     prm.lse_ext = saved_p ? reinterpret_cast<const uint4 *>(saved_p) : lse_ext;
@@ -1406,6 +1542,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     auto main_kernel = parts > 1 ? bwd_main_kernel<D, kBf16, true> : bwd_main_kernel<D, kBf16, false>;
     if constexpr (!kBf16)
         if (saved_p) main_kernel = bwd_main_kernel<D, false, false, true>;
+    if (one_tile) main_kernel = bwd_main_kernel<D, kBf16, false, false, true>;
     e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(bwd_main)", e);
     const int n_items = B * Hkv * (S_pad / kTileRows) * parts;
@@ -1422,11 +1559,13 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     CUtensorMap mdq = mq;  // (D = 128 never touches it)
     if constexpr (D == 64)
         if ((rc = make_f32_tile_map(&mdq, dq_acc, static_cast<uint64_t>(n_rows), 64, 128)) != LT_OK) return rc;
-    e = cudaLaunchKernelEx(&cfg_main, main_kernel, mq, mk, mv, mdo, prm, mdq);
+    e = cudaLaunchKernelEx(&cfg_main, main_kernel, mq, mk, mv, mdo, prm, mdq, one);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("bwd_main_kernel launch", e);
     if (ev_main_end && (e = cudaEventRecord(ev_main_end, stream)) != cudaSuccess)
         return record_cuda_error("cudaEventRecord", e);
+
+    if (one_tile) return LT_OK;  // dQ is written
 
     const long long n_vec8 = static_cast<long long>(B) * Hq * S * D / 8;
     const long long fwant = (n_vec8 + 255) / 256;
@@ -1473,8 +1612,11 @@ size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D) {
 
 int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal) {
     if (lt::check_shape(B, Hq, Hkv, S, D, 1.0f) != LT_OK) return 0;
-    // preprocess, main, dQ conversion; plus the dK/dV conversion when groups are split over work items
-    return lt::heads_per_item(B, Hq, Hkv, S, D, causal) < Hq / Hkv ? 4 : 3;
+    // preprocess, main, dQ conversion; plus the dK/dV conversion when groups are split over work items; sequences of one
+    // tile need fewer
+    if (lt::heads_per_item(B, Hq, Hkv, S, D, causal) < Hq / Hkv) return 4;
+    const int tile_launches = lt::one_tile_launches(B, Hq, Hkv, S, D);
+    return tile_launches > 0 ? tile_launches : 3;
 }
 
 static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
