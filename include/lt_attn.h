@@ -118,8 +118,8 @@ int lt_attn_bwd_profiled(const lt_half *Q, const lt_half *K, const lt_half *V,
  * fixed array of LT_ATTN_BWD_NOALLOC_MAX_SCRATCH_BYTES inside the library itself, which every
  * GPU that loads the library holds until the process ends.  Inputs and outputs are still the
  * caller's device tensors, with the meaning and layout of lt_attn_bwd.
- *   - Shapes whose lt_attn_bwd_workspace_bytes() exceeds the built-in scratch (roughly
- *     B*Hq*S*D above four million elements) return LT_ERR_WORKSPACE; lt_last_cuda_error()
+ *   - Shapes whose workspace exceeds the built-in scratch (roughly B*Hq*S*D above four million elements;
+ *     the fp32 dK/dV sums of split groups do not count, without room for them groups stay whole) return LT_ERR_WORKSPACE; lt_last_cuda_error()
  *     then names both sizes.  Nothing is launched in that case.
  *   - The call allocates nothing: no cudaMalloc/cudaFree and no allocating library routine.
  *   - The first call on each device looks up the array's device address (one runtime query,
@@ -261,7 +261,7 @@ const char *lt_last_cuda_error(void);
 
 /* Number of kernels one call enqueues for this shape (for launch accounting by benchmarks): the
  * backward's preprocess, main and dQ-conversion kernels, plus the dK/dV conversion on grouped-query shapes
- * with fewer than about 1.5 key-tile work items per multiprocessor, where a group's query heads are split
+ * whose key-tile work items would be few or long, where a group's query heads are split
  * over several items (4 instead of 3); sequences of at most 128 rows need 1 or 2 where that is faster; 0 for an unsupported
  * shape.  The forward enqueues one kernel. */
 int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal);

@@ -36,6 +36,7 @@
 // heads over several work items (few, heavy items) and sums dK/dV in fp32 in the workspace; and a
 // variant that loads the probability tiles a forward pass saved (Section 4.1's own forward state,
 // written by lt_attn_save_p) instead of recomputing them.
+#include <math.h>
 #include <mutex>
 #include <stddef.h>
 #include <stdio.h>
@@ -267,10 +268,11 @@ bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, uns
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float *__restrict__ dq_acc, __half *__restrict__ dQ, long long n_vec8, int vec_per_head,
-                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain) {
+                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain, int kv_follows) {
     // n_vec8 groups of eight output elements, numbered over the logical [B,Hq,S,D]; the accumulator
     // is indexed in the padded row space (`plain`: contiguous dQ and no padding, so both are group v)
     grid_dependency_wait();  // launched while the main kernel drains: its reductions must have landed
+    if (kv_follows) grid_launch_dependents();  // the dK/dV conversion runs beside this one
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < n_vec8; v += stride) {
         long long src = v, dst = v * 8;
@@ -299,7 +301,7 @@ __global__ void __launch_bounds__(256)
 bwd_finalize_kv_kernel(const float *__restrict__ dk_acc, const float *__restrict__ dv_acc, __half *__restrict__ dK,
                        __half *__restrict__ dV, long long n_vec8, int vec_per_head, int vec_per_padded_head,
                        int vec_per_row, int Hkv, lt_tensor_strides dk_st, lt_tensor_strides dv_st) {
-    grid_dependency_wait();  // every share of the main kernel must have landed
+    // (started once every CTA of the dQ conversion has seen the main kernel complete, so every share has landed)
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < 2 * n_vec8; v += stride) {
         const bool second = v >= n_vec8;
@@ -321,6 +323,7 @@ bwd_finalize_kv_kernel(const float *__restrict__ dk_acc, const float *__restrict
         o.w = pack2<kBf16>(b.z, b.w);
         *reinterpret_cast<uint4 *>((second ? dV : dK) + dst) = o;
     }
+    grid_dependency_wait();  // what follows this kernel may rely on the dQ conversion having finished too
 }
 
 // ----------------------------------------------------------------------------- optional cycle trace
@@ -1387,19 +1390,34 @@ static int sm_count() {
 }
 static int heads_per_item(int B, int Hq, int Hkv, int S, int D, int causal) {
     const int sms = sm_count();
-    const long long split_below_items = sms + sms / 2;  // split when there are fewer than 1.5 whole-group items per SM
-    const long long split_target_items = 2 * sms;       // and then aim at two items per SM (every item pays a pipeline fill)
-    const long long split_min_iterations = 20 * sms;    // problems below this are launch-bound anyway
     const int G = Hq / Hkv;
     const long long n_tiles = padded_rows(S) / kTileRows;
     const long long n_base = static_cast<long long>(B) * Hkv * n_tiles;
-    const long long iters = static_cast<long long>(B) * Hq * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
-    if (G == 1 || iters < split_min_iterations) return G;
-    if (n_base < split_below_items) {
-        const long long split = (split_target_items + n_base - 1) / n_base;
-        const int hs = static_cast<int>(split < G ? split : G);
-        return (G + hs - 1) / hs;
+    if (G == 1) return 1;
+    // The heads per item with the shortest estimated makespan, in tile pairs (about 2.1 us each): the longest item or the
+    // average work of an SM, with what an item costs beside its pairs (pipeline fill and the epilogue, which adds to fp32
+    // sums when groups are split), and 3 for the zero fill and conversion of those sums.  Measured, us per call, whole
+    // groups / this choice: 8 / 1 heads at S = 2048 286 / 55; 16 / 4 at 1024 83 / 39; 4 x 16 / 2 at 1024, D = 64 112 / 51;
+    // 40 / 8 at 1024 108 / 64, at 2048 240 / 158; 2 x 40 / 8 at 1536 unmasked 391 / 357.  On the other side of the line:
+    // 8 x 20 / 4 at 512 79 whole, 81 split in two; 64 / 16 at 2048 237 whole, 269; 40 / 8 at 4096 525 whole, 525.
+    const double pairs = static_cast<double>(B) * Hq * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
+    int best = G;
+    double best_span = 0.;
+    for (int parts = 1; parts <= G; ++parts) {
+        const int hpi = (G + parts - 1) / parts;
+        if (parts > 1 && (G + hpi - 1) / hpi != parts) continue;  // the same items as with fewer parts
+        const double per_item = parts > 1 ? 6. : 2., items = static_cast<double>(n_base) * parts;
+        const double longest = static_cast<double>(hpi) * n_tiles + (parts > 1 ? 4. : 2.);
+        double span = pairs / sms + per_item * items / sms;
+        if (longest > span) span = longest;
+        if (!causal) {  // items of one length: whole rounds
+            const double rounds = ceil(items / sms) * (pairs / items + per_item);
+            if (rounds > span) span = rounds;
+        }
+        if (parts > 1) span += 3.;
+        if (parts == 1 || span < best_span) best = hpi, best_span = span;
     }
+    if (best < G) return best;
     // Enough whole-group items to fill the SMs, but too few to form L2-sized batches (a batch needs two items per
     // SM) while the working set is more than four times the L2: the accumulator rows of the heads in flight would be
     // fetched and written back again and again.  Two items per key tile make room for batches.  Measured, whole
@@ -1409,7 +1427,7 @@ static int heads_per_item(int B, int Hq, int Hkv, int S, int D, int causal) {
     // 1.52 / 1.59, the same with B = 2 at S = 4096 0.86 / 0.89, the Qwen2.5-32B layer (1.4 L2s) 0.53 / 0.56.
     const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
     const double working_set = unit_bytes * B * Hkv;
-    if (n_base < 4LL * sms && working_set > 4.0 * 126.0e6) return (G + 1) / 2;
+    if (n_base >= sms + sms / 2 && n_base < 4LL * sms && working_set > 4.0 * 126.0e6) return (G + 1) / 2;
     return G;
 }
 
@@ -1432,7 +1450,7 @@ template <int D, bool kBf16>
 static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
                       const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout &lay, int B,
                       int Hq, int Hkv, int S, int causal, float scale, void *workspace, cudaStream_t stream,
-                      cudaEvent_t ev_main_begin, cudaEvent_t ev_main_end, const lt_half *saved_p = nullptr) {
+                      cudaEvent_t ev_main_begin, cudaEvent_t ev_main_end, bool may_split, const lt_half *saved_p = nullptr) {
     // saved_p: the probability tiles of lt_attn_save_p; LSE is then not needed (fp16, whole groups only)
     const int S_pad = static_cast<int>(padded_rows(S));
     // fast addressing in the two streaming kernels when nothing is padded or strided
@@ -1449,7 +1467,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     uint4 *delta_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes);
     uint4 *lse_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes + ext_bytes);
     float *dq_acc = reinterpret_cast<float *>(ws + kStatusBytes + 2 * ext_bytes);
-    const int hpi = saved_p ? Hq / Hkv : heads_per_item(B, Hq, Hkv, S, D, causal);
+    const int hpi = saved_p || !may_split ? Hq / Hkv : heads_per_item(B, Hq, Hkv, S, D, causal);
     const int parts = (Hq / Hkv + hpi - 1) / hpi;
     const size_t kv_floats = static_cast<size_t>(B) * Hkv * S_pad * D;
     float *dk_acc = nullptr, *dv_acc = nullptr;
@@ -1578,7 +1596,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     cfg_fin.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg_fin, bwd_finalize_kernel<kBf16>, static_cast<const float *>(dq_acc),
                            reinterpret_cast<__half *>(dQ), n_vec8, S * (D / 8), S_pad * (D / 8), D / 8, Hq, lay.dq,
-                           plain_fin);
+                           plain_fin, parts > 1 ? 1 : 0);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("bwd_finalize_kernel launch", e);
     if (parts > 1) {
@@ -1599,12 +1617,16 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
 
 extern "C" {
 
+// the status block, the -delta and -LSE/scale rows and the fp32 dQ accumulator
+static size_t bwd_base_bytes(int B, int Hq, int S, int D) {
+    const size_t n_rows = static_cast<size_t>(B) * Hq * static_cast<size_t>(lt::padded_rows(S));
+    return lt::kStatusBytes + 2 * lt::round256(n_rows * 16) + lt::round256(n_rows * D * 4);
+}
+
 size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D) {
     if (lt::check_shape(B, Hq, Hkv, S, D, 1.0f) != LT_OK) return 0;
-    const size_t n_rows = static_cast<size_t>(B) * Hq * static_cast<size_t>(lt::padded_rows(S));
-    size_t bytes = lt::kStatusBytes + 2 * lt::round256(n_rows * 16) + lt::round256(n_rows * D * 4);
-    // fp32 dK / dV sums for shapes whose groups are split over work items (either mask; sized for the
-    // unmasked case, which splits no less often)
+    size_t bytes = bwd_base_bytes(B, Hq, S, D);
+    // fp32 dK / dV sums for shapes whose groups are split over work items (under either mask)
     if (lt::heads_per_item(B, Hq, Hkv, S, D, 1) < Hq / Hkv || lt::heads_per_item(B, Hq, Hkv, S, D, 0) < Hq / Hkv)
         bytes += 2 * lt::round256(static_cast<size_t>(B) * Hkv * static_cast<size_t>(lt::padded_rows(S)) * D * 4);
     return bytes;
@@ -1622,7 +1644,8 @@ int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal) {
 static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
                      const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout *layout, int B,
                      int Hq, int Hkv, int S, int D, int causal, float scale, void *workspace, size_t workspace_bytes,
-                     lt_stream_t stream, lt_event_t main_begin, lt_event_t main_end, bool bf16 = false) {
+                     lt_stream_t stream, lt_event_t main_begin, lt_event_t main_end, bool bf16 = false, bool fit = false) {
+    // fit: where the workspace holds no fp32 dK/dV sums, run with whole groups
     using namespace lt;
     if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
@@ -1633,21 +1656,22 @@ static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const
     for (const void *ptr : ptrs)
         if (!aligned16(ptr)) return LT_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(LSE) & 3u) != 0) return LT_ERR_UNSUPPORTED;  // fp32, read one at a time
-    if (!workspace || !aligned256(workspace) || workspace_bytes < lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D))
+    const bool may_split = workspace_bytes >= lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
+    if (!workspace || !aligned256(workspace) || (!may_split && !(fit && workspace_bytes >= bwd_base_bytes(B, Hq, S, D))))
         return LT_ERR_WORKSPACE;
     if ((rc = check_device()) != LT_OK) return rc;
     if (bf16) {
         if (D == 64)
             return launch_bwd<64, true>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                        stream, main_begin, main_end);
+                                        stream, main_begin, main_end, may_split);
         return launch_bwd<128, true>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     stream, main_begin, main_end);
+                                     stream, main_begin, main_end, may_split);
     }
     if (D == 64)
         return launch_bwd<64, false>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     stream, main_begin, main_end);
+                                     stream, main_begin, main_end, may_split);
     return launch_bwd<128, false>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                  stream, main_begin, main_end);
+                                  stream, main_begin, main_end, may_split);
 }
 
 int lt_attn_bwd_saved_p(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
@@ -1667,9 +1691,9 @@ int lt_attn_bwd_saved_p(const lt_half *Q, const lt_half *K, const lt_half *V, co
     const lt_attn_layout lay = contiguous_layout(Hq, Hkv, S, D);
     if (D == 64)
         return launch_bwd<64, false>(Q, K, V, O, dO, nullptr, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     static_cast<cudaStream_t>(stream), nullptr, nullptr, P);
+                                     static_cast<cudaStream_t>(stream), nullptr, nullptr, false, P);
     return launch_bwd<128, false>(Q, K, V, O, dO, nullptr, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                  static_cast<cudaStream_t>(stream), nullptr, nullptr, P);
+                                  static_cast<cudaStream_t>(stream), nullptr, nullptr, false, P);
 }
 
 int lt_attn_bwd_profiled(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
@@ -1705,6 +1729,15 @@ int lt_attn_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_h
 
 }  // extern "C"
 
+namespace lt {
+int bwd_in_any(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO, const float *LSE,
+               lt_half *dQ, lt_half *dK, lt_half *dV, int B, int Hq, int Hkv, int S, int D, int causal, float scale,
+               void *workspace, size_t workspace_bytes, lt_stream_t stream) {
+    return bwd_entry(Q, K, V, O, dO, LSE, dQ, dK, dV, nullptr, B, Hq, Hkv, S, D, causal, scale, workspace, workspace_bytes,
+                     stream, nullptr, nullptr, false, true);
+}
+}  // namespace lt
+
 // ----------------------------------------------------------------------------- backward without a caller workspace
 // Scratch for lt_attn_bwd_noalloc: lives in the library image, so every GPU that loads the
 // library carries these bytes until the process exits.  In host code the array's name is
@@ -1727,8 +1760,8 @@ int lt_attn_bwd_noalloc(const lt_half *Q, const lt_half *K, const lt_half *V, co
     if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
     if (rc != LT_OK) return rc;
-    const size_t need = lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
-    if (need == 0 || need > kNoAllocScratchBytes) {
+    const size_t need = bwd_base_bytes(B, Hq, S, D);
+    if (need > kNoAllocScratchBytes) {
         char msg[160];
         snprintf(msg, sizeof(msg), "this shape needs %zu bytes of scratch but the built-in scratch holds %zu; "
                  "use lt_attn_bwd with a caller workspace", need, kNoAllocScratchBytes);
@@ -1757,8 +1790,7 @@ int lt_attn_bwd_noalloc(const lt_half *Q, const lt_half *K, const lt_half *V, co
     }
     // lt_attn_bwd clears the status block and its preprocess kernel zeroes the dQ accumulator on
     // every call, so nothing left in the scratch by an earlier call is read
-    return lt_attn_bwd(Q, K, V, O, dO, LSE, dQ, dK, dV, B, Hq, Hkv, S, D, causal, scale, scratch,
-                       kNoAllocScratchBytes, stream);
+    return bwd_in_any(Q, K, V, O, dO, LSE, dQ, dK, dV, B, Hq, Hkv, S, D, causal, scale, scratch, kNoAllocScratchBytes, stream);
 }
 
 int lt_attn_bwd_noalloc_check_status(lt_stream_t stream) {
