@@ -9,6 +9,8 @@
 // pair while the other tile's scores are exponentiated.  S/P and O live in tensor memory.
 // The running row maximum is only raised when it grew by more than 2^8 since the output
 // was last rescaled, so most key tiles need no pass over O.
+#include <math.h>
+
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -45,7 +47,8 @@ struct __align__(1024) FwdSmem {
     uint8_t k[2][kTile];   // ring of key tiles
     uint8_t v[2][kTile];   // ring of value tiles
     uint64_t bar_q[2], bar_k_full[2], bar_k_empty[2], bar_v_full[2], bar_v_empty[2];
-    uint64_t bar_s_full[2], bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_done;
+    uint64_t bar_s_full[2], bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_done, bar_merge;
+    float2 merge[kFwdTileRows];  // (split keys) maximum and sum of the odd key tiles' half, per query row
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -75,7 +78,13 @@ __device__ unsigned long long g_fwd_trace[32];
 #endif
 
 // Registers are handed out per four warps, so ten warps get the 168-register cap of twelve.
-template <int D, bool kBf16>
+//
+// A CTA runs two chains S -> softmax -> P V -> S side by side (index t).  Normally they are the two query tiles of a pair
+// over the same key tiles; kSplitKeys: the even and the odd key tiles of one query tile, whose two softmaxes are put
+// together at the end (each chain has its own maximum, sum and O; a ring slot then belongs to one chain).  That is twice
+// the CTAs with half as long a walk, for grids that leave multiprocessors idle or wait for a few long walks:
+// splits_keys().
+template <int D, bool kBf16, bool kSplitKeys>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
            const __grid_constant__ CUtensorMap map_v, const FwdParams p) {
@@ -96,17 +105,21 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     const int n_tiles = (p.S + kFwdTileRows - 1) / kFwdTileRows;  // the last tile may be ragged
     const int n_pairs = (n_tiles + 1) / 2;
     const int n_bh = p.B * p.Hq;
-    const int pr = p.causal ? (n_pairs - 1 - blockIdx.x / n_bh) : (blockIdx.x / n_bh);
+    const int n_groups = kSplitKeys ? n_tiles : n_pairs;  // of query tiles, one to a CTA
+    const int pr = p.causal ? (n_groups - 1 - blockIdx.x / n_bh) : (blockIdx.x / n_bh);
     const int bh = blockIdx.x % n_bh;
     const int b = bh / p.Hq;
     const int h = bh % p.Hq;
     const int g = h / (p.Hq / p.Hkv);
-    const int i0 = 2 * pr;
-    const bool has_b = (i0 + 1) < n_tiles;
-    // last key tile of query tile t; -1 when the pair has no second tile
-    const int j_last0 = p.causal ? i0 : n_tiles - 1;
-    const int j_last1 = has_b ? (p.causal ? i0 + 1 : n_tiles - 1) : -1;
+    const int i0 = kSplitKeys ? pr : 2 * pr;
+    const int n_keys = p.causal ? i0 + 1 : n_tiles;  // key tiles of query tile i0
+    const bool has_b = kSplitKeys ? n_keys > 1 : (i0 + 1) < n_tiles;  // the second chain exists
+    // last step of chain t (a key tile; split keys: key tile 2 j + t); -1 when there is no second chain
+    const int j_last0 = kSplitKeys ? (n_keys + 1) / 2 - 1 : n_keys - 1;
+    const int j_last1 = kSplitKeys ? n_keys / 2 - 1 : has_b ? (p.causal ? i0 + 1 : n_tiles - 1) : -1;
     const int j_end = j_last0 > j_last1 ? j_last0 : j_last1;
+    const int key_end = kSplitKeys ? n_keys - 1 : j_end;         // last key tile to be loaded
+    const int n_q = kSplitKeys ? 1 : has_b ? 2 : 1;              // query tiles
 
     if (tid == 0) {
         sm.abort_flag = 0;
@@ -123,6 +136,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             mbar_init(&sm.bar_o_done[t], 1);
         }
         mbar_init(&sm.bar_done, 1);
+        mbar_init(&sm.bar_merge, 128);
         mbar_fence_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_k);
@@ -146,7 +160,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         if (warp == 0) {
             // ------------------------------------------------------------------ producer
             if (lane == 0) {
-                for (int t = 0; t < (has_b ? 2 : 1); ++t) {
+                for (int t = 0; t < n_q; ++t) {
                     mbar_arrive_expect_tx(&sm.bar_q[t], kTileBytes);
 #pragma unroll
                     for (int x = 0; x < kBoxes; ++x)
@@ -154,7 +168,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                 }
                 bool ok = true;
                 int armed = 0;  // key/value tiles whose loads were started
-                for (int j = 0; j <= j_end; ++j) {
+                for (int j = 0; j <= key_end; ++j) {
                     const int s = j & 1;
                     const uint32_t ph = (j >> 1) & 1;
                     const int kv_row0 = j * kFwdTileRows;  // inside the head; rows past S arrive as zeros
@@ -176,7 +190,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                 }
                 if (!ok || *abort_flag) {
                     // somebody gave up: wait (bounded) for the copies in flight before the CTA exits
-                    for (int t = 0; t < (has_b ? 2 : 1); ++t)
+                    for (int t = 0; t < n_q; ++t)
                         for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_q[t], 0); ++w) {}
                     for (int j = armed > 2 ? armed - 2 : 0; j < armed; ++j) {
                         for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_k_full[j & 1], (j >> 1) & 1); ++w) {}
@@ -205,7 +219,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     if (!leader) return;
 #pragma unroll
                     for (int kk = 0; kk < D / 16; ++kk)
-                        umma_ss(tmem + kColS + t * 128, dQ0 + t * kSlotStep + koff(kk), dK0 + s * kSlotStep + koff(kk), idesc_s, kk > 0);
+                        umma_ss(tmem + kColS + t * 128, dQ0 + (kSplitKeys ? 0 : t) * kSlotStep + koff(kk), dK0 + s * kSlotStep + koff(kk), idesc_s, kk > 0);
                     umma_commit(&sm.bar_s_full[t]);
                 };
                 // O_t (+)= P_t V, P_t read from tensor memory; the keys of a tile in two halves of 64, so that the
@@ -220,15 +234,46 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     if (half == 1) umma_commit(&sm.bar_o_done[t]);
                 };
                 bool ok = wait_all(&sm.bar_q[0], 0, kWaitFwdQ) &&
-                          (!has_b || wait_all(&sm.bar_q[1], 0, kWaitFwdQ)) &&
+                          (n_q < 2 || wait_all(&sm.bar_q[1], 0, kWaitFwdQ)) &&
                           wait_all(&sm.bar_k_full[0], 0, kWaitFwdK);
                 if (ok) {
                     tc_fence_after_sync();
                     issue_s(0, 0);
-                    if (has_b) issue_s(1, 0);
-                    if (leader) umma_commit(&sm.bar_k_empty[0]);
+                    if constexpr (kSplitKeys) {
+                        if (leader) umma_commit(&sm.bar_k_empty[0]);
+                        if (has_b && (ok = wait_all(&sm.bar_k_full[1], 0, kWaitFwdK))) {
+                            tc_fence_after_sync();
+                            issue_s(1, 1);
+                            if (leader) umma_commit(&sm.bar_k_empty[1]);
+                        }
+                    } else {
+                        if (has_b) issue_s(1, 0);
+                        if (leader) umma_commit(&sm.bar_k_empty[0]);
+                    }
                 }
                 LT_FT_DECL;
+                if constexpr (kSplitKeys) {
+                    for (int j = 0; j <= j_end && ok; ++j) {
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {  // chain t lives in ring slot t
+                            const int j_last_t = t == 0 ? j_last0 : j_last1;
+                            if (j > j_last_t) continue;
+                            if (!(ok = wait_all(&sm.bar_v_full[t], j & 1, kWaitFwdV) && wait_all(&sm.bar_p_half[t], j & 1, kWaitFwdP))) break;
+                            tc_fence_after_sync();
+                            issue_pv_half(t, t, j > 0, 0);
+                            if (!(ok = wait_all(&sm.bar_p_ready[t], j & 1, kWaitFwdP))) break;
+                            tc_fence_after_sync();
+                            issue_pv_half(t, t, j > 0, 1);
+                            if (leader) umma_commit(&sm.bar_v_empty[t]);
+                            if (j + 1 <= j_last_t) {
+                                if (!(ok = wait_all(&sm.bar_k_full[t], (j + 1) & 1, kWaitFwdK))) break;
+                                tc_fence_after_sync();
+                                issue_s(t, t);
+                                if (leader) umma_commit(&sm.bar_k_empty[t]);
+                            }
+                        }
+                    }
+                } else
                 for (int j = 0; j <= j_end && ok; ++j) {
                     const int s = j & 1, sn = s ^ 1;
                     LT_FT(0);
@@ -284,7 +329,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         const int quad = warp & 3;                      // tensor-memory lane quadrant of this warp
         const int row = quad * 32 + lane;               // query row inside the tile
         const int j_last = t == 0 ? j_last0 : j_last1;
-        const int i = i0 + t;
+        const int i = kSplitKeys ? i0 : i0 + t;
         const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
         const uint32_t tS = tmem + lane_base + kColS + t * 128;
         const uint32_t tO = tmem + lane_base + kColO + t * D;
@@ -400,7 +445,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     }
                 }
             };
-            if (p.causal ? (j == i) : (j == n_tiles - 1 && tail_keys < kFwdTileRows)) tile_softmax(std::true_type{});
+            const int key_tile = kSplitKeys ? 2 * j + t : j;
+            if (p.causal ? (key_tile == i) : (key_tile == n_tiles - 1 && tail_keys < kFwdTileRows)) tile_softmax(std::true_type{});
             else tile_softmax(std::false_type{});
             if (!ok) break;
             const float row_sum = (rs[0] + rs[1]) + (rs[2] + rs[3]);
@@ -422,9 +468,30 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             ok = mbar_wait(&sm.bar_o_done[t], j_last & 1, abort_flag, p.status, kWaitFwdO);
             ok = __all_sync(0xffffffffu, ok);
         }
-        if (ok && j_last >= 0) {
+        if constexpr (kSplitKeys) {
+            if (t == 1) {  // the other chain's warps put the two halves together
+                sm.merge[row] = make_float2(m_used, l);  // (no odd key tile: -inf and 0)
+                mbar_arrive(&sm.bar_merge);
+            } else if (ok) {
+                ok = mbar_wait(&sm.bar_merge, 0, abort_flag, p.status, kWaitFwdO) &&
+                     (j_last1 < 0 || mbar_wait(&sm.bar_o_done[1], j_last1 & 1, abort_flag, p.status, kWaitFwdO));
+                ok = __all_sync(0xffffffffu, ok);
+            }
+        }
+        if (ok && j_last >= 0 && !(kSplitKeys && t == 1)) {
             tc_fence_after_sync();
+            float w0 = 1.f, w1 = 0.f;  // weights of this chain's O and of the other's
+            if constexpr (kSplitKeys) {
+                const float2 o = sm.merge[row];
+                const float m = fmaxf(m_used, o.x);
+                w0 = fast_exp2(m_used - m);
+                w1 = fast_exp2(o.x - m);
+                l = l * w0 + o.y * w1;
+                m_used = m;
+            }
             const float inv_l = 1.f / l;
+            w0 *= inv_l;
+            w1 *= inv_l;
             const int s_row = i * kFwdTileRows + row;  // rows past S belong to nobody
             const long long q_row = static_cast<long long>(bh) * p.S + s_row;  // LSE is contiguous
             __half *o_row = p.O + b * p.o_st.batch + h * p.o_st.head + s_row * p.o_st.row;
@@ -432,14 +499,22 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t r[32];
                 tmem_ld32(tO + c * 32, r);
+                uint32_t r1[32];
+                if (kSplitKeys && j_last1 >= 0) tmem_ld32(tO + D + c * 32, r1);
                 tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    float x = __uint_as_float(r[e]) * w0;
+                    if (kSplitKeys && j_last1 >= 0) x = fmaf(__uint_as_float(r1[e]), w1, x);
+                    r[e] = __float_as_uint(x);
+                }
 #pragma unroll
                 for (int v8 = 0; v8 < 4; ++v8) {
                     uint4 o;
-                    o.x = pack2<kBf16>(__uint_as_float(r[8 * v8 + 0]) * inv_l, __uint_as_float(r[8 * v8 + 1]) * inv_l);
-                    o.y = pack2<kBf16>(__uint_as_float(r[8 * v8 + 2]) * inv_l, __uint_as_float(r[8 * v8 + 3]) * inv_l);
-                    o.z = pack2<kBf16>(__uint_as_float(r[8 * v8 + 4]) * inv_l, __uint_as_float(r[8 * v8 + 5]) * inv_l);
-                    o.w = pack2<kBf16>(__uint_as_float(r[8 * v8 + 6]) * inv_l, __uint_as_float(r[8 * v8 + 7]) * inv_l);
+                    o.x = pack2<kBf16>(__uint_as_float(r[8 * v8 + 0]), __uint_as_float(r[8 * v8 + 1]));
+                    o.y = pack2<kBf16>(__uint_as_float(r[8 * v8 + 2]), __uint_as_float(r[8 * v8 + 3]));
+                    o.z = pack2<kBf16>(__uint_as_float(r[8 * v8 + 4]), __uint_as_float(r[8 * v8 + 5]));
+                    o.w = pack2<kBf16>(__uint_as_float(r[8 * v8 + 6]), __uint_as_float(r[8 * v8 + 7]));
                     if (s_row < p.S) reinterpret_cast<uint4 *>(o_row + c * 32)[v8] = o;
                 }
             }
@@ -463,6 +538,28 @@ extern "C" int lt_dbg_fwd_trace(unsigned long long *out, int reset) {
 }
 #endif
 
+// Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
+// makespan in steps of both chains (about 1.9 us), with 1.5 for a CTA's fill and drain.  Of 22 shapes measured both ways
+// it picks the faster one every time.  us, pairs of tiles / split keys (heads, S): 8, 2048 33.9 / 21.5; 4, 8000
+// 112.8 / 64.7; 16, 512 13.4 / 10.0; 32, 1024 22.4 / 21.4; 16, 753 unmasked 17.5 / 12.5; on the other side 64, 640
+// 19.4 / 21.2; 40, 1920 53.9 / 60.0; 32, 4096 141.7 / 163.2.
+static bool splits_keys(int B, int Hq, int S, int causal) {
+    constexpr double kSms = 148., kFill = 1.5;
+    const double heads = static_cast<double>(B) * Hq;
+    const int n = (S + kFwdTileRows - 1) / kFwdTileRows, pairs = (n + 1) / 2;
+    if (n < 2) return false;
+    auto span = [&](double ctas, double steps, double longest) {
+        double t = (steps + kFill * ctas) / kSms;
+        if (!causal) t = ceil(ctas / kSms) * (longest + kFill);  // walks of one length: whole rounds
+        return t > longest + kFill ? t : longest + kFill;
+    };
+    // steps of all CTAs of a head; causal: a pair's walk is its later tile's, and a tile's chains have half its keys each
+    const double pair_steps = causal ? static_cast<double>(pairs) * (pairs + 1) - (n & 1 ? 1 : 0) : static_cast<double>(pairs) * n;
+    const double half = (n + 1) / 2, even = n / 2;
+    const double split_steps = causal ? half * (half + 1) / 2 + even * (even + 1) / 2 : n * half;
+    return span(heads * n, heads * split_steps, half) < span(heads * pairs, heads * pair_steps, n);
+}
+
 template <int D, bool kBf16>
 static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_half *O, float *LSE,
                       const lt_attn_layout &lay, int B, int Hq, int Hkv, int S, int causal, float scale,
@@ -481,10 +578,12 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     prm.scale = scale;
     // at least 120 KB, so that one CTA (which takes all 512 tensor-memory columns) lives on an SM
     const size_t smem = std::max<size_t>(sizeof(FwdSmem<D>) + 1024, 120 * 1024);
-    cudaError_t e = cudaFuncSetAttribute(fwd_kernel<D, kBf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    const bool split = splits_keys(B, Hq, S, causal);
+    auto kernel = split ? fwd_kernel<D, kBf16, true> : fwd_kernel<D, kBf16, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(fwd)", e);
     const int n_tiles = (S + kFwdTileRows - 1) / kFwdTileRows;
-    const int grid = B * Hq * ((n_tiles + 1) / 2);
+    const int grid = B * Hq * (split ? n_tiles : (n_tiles + 1) / 2);
     cudaLaunchAttribute pdl;
     pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl.val.programmaticStreamSerializationAllowed = 1;
@@ -495,7 +594,7 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     cfg.stream = stream;
     cfg.attrs = &pdl;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, fwd_kernel<D, kBf16>, mq, mk, mv, prm);
+    e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, prm);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("fwd_kernel launch", e);
     return LT_OK;

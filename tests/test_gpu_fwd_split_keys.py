@@ -1,0 +1,40 @@
+"""Forward whose CTAs take one query tile with its key tiles in two chains (few heads): one key tile (an empty second
+chain) to many, odd and even counts, ragged ends, both masks, head dimensions and types, a negative scale, maxima that
+rise late in one chain only, against fp64 softmax."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,Hkv,S,D", [(2, 1, 129, 64), (1, 1, 256, 128), (3, 3, 300, 128), (2, 2, 640, 64), (4, 2, 1153, 128),
+                                       (1, 1, 2048, 64)])
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype,scale_sign,ramp", [(torch.float16, 1, False), (torch.bfloat16, 1, False),
+                                                   (torch.float16, -1, False), (torch.float16, 1, True)])
+def test_split_keys(H, Hkv, S, D, causal, dtype, scale_sign, ramp):
+    from paper_2606_10415_b200 import binding as lt
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(S + D)
+    Q, K, V = (torch.randn((1, h, S, D), generator=gen, device="cuda") for h in (H, Hkv, Hkv))
+    if ramp:  # scores that grow along the keys, by far the most in the odd key tiles
+        tile = torch.arange(S, device="cuda") // 128
+        K = K * (0.2 + 0.8 * tile * (tile % 2)).view(1, 1, S, 1)
+    Q, K, V = (t.to(dtype) for t in (Q, K, V))
+    scale = scale_sign * D ** -0.5
+    O, LSE = torch.full_like(Q, float("nan")), torch.full((1, H, S), float("nan"), device="cuda")
+    ws = lt.alloc_workspace(256)
+    ws.fill_(0xFF)
+    fn = lt.lt_attn_fwd if dtype == torch.float16 else lt.lt_attn_fwd_bf16
+    fn(Q, K, V, O, LSE, causal, scale, ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    k, v = (t.double().repeat_interleave(H // Hkv, 1) for t in (K, V))
+    s = Q.double() @ k.transpose(-1, -2) * scale
+    if causal:
+        s.masked_fill_(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    ref = torch.exp(s - lse[..., None]) @ v
+    # the forward's gates: rounding of P and O, 2^-11 (fp16) or 2^-8 (bf16) each, in the 2-norm
+    assert (O.double() - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
+    # LSE is fp32: one unit of its own size besides the flat gate
+    assert ((LSE.double() - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
