@@ -29,10 +29,14 @@ def test_many_chunks(B, Hq, Hkv, S, D, causal, with_o):
         lt.lt_attn_fwd_bwd_host(*host, h_O, h_L, *got, causal, cfg.scale, arena)
     torch.cuda.synchronize()
     if with_o:
-        assert torch.equal(h_O, O.cpu()) and torch.equal(h_L, LSE.cpu())
+        # a chunk of few heads may take its keys in two chains: probabilities round to fp16 against another running
+        # maximum, and so does the result, 2^-11 each; S terms of the fp32 row sums are added in another order
+        g, w = h_O.double(), O.cpu().double()
+        assert torch.isfinite(g).all() and (g - w).norm() <= 2 * 2.0 ** -11 * w.norm()
+        assert (h_L.double() - LSE.cpu().double()).abs().max() <= S * 2.0 ** -24
     for name, g, w in zip(("dQ", "dK", "dV"), got, want):
         g, w = g.double(), w.cpu().double()
         assert torch.isfinite(g).all(), name
         # a chunk picks its own power of two for dS, so roundings to fp16 may fall on the other side: half a unit
-        # in the last place of the operands and of the result, 2^-11 each
-        assert (g - w).norm() <= 2 * 2.0 ** -11 * w.norm(), name
+        # in the last place of the operands, of the result and of the O that delta is formed from, 2^-11 each
+        assert (g - w).norm() <= 3 * 2.0 ** -11 * w.norm(), name
