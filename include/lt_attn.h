@@ -67,8 +67,8 @@ typedef unsigned short lt_bf16;
  * word 3: work-item counter), -delta and -LSE/scale as 16-byte rows
  * of fp16 (hi, lo, 0 x 6) with 256*hi + lo = value, [B,Hq,S_pad] rows each (every 64th or 128th -LSE/scale row may
  * carry partial maxima of the three quantities above in elements 4-6, which no product uses), an fp32 dQ accumulator
- * [B,Hq,S_pad,D], and, for the grouped-query shapes whose groups are split over work items (see
- * lt_attn_bwd_num_launches), fp32 dK and dV sums [B,Hkv,S_pad,D] each. */
+ * [B,Hq,S_pad,D], and, for shapes whose key tiles are split over work items (see lt_attn_bwd_num_launches), the items'
+ * fp32 shares of dK and dV, 2 x 128 x D floats each: two per multiprocessor, or two per key tile. */
 size_t lt_attn_fwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);
 size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);
 
@@ -90,9 +90,7 @@ int lt_attn_fwd(const lt_half *Q, const lt_half *K, const lt_half *V,
  *   in : Q, O, dO [B,Hq,S,D] fp16; K, V [B,Hkv,S,D] fp16; LSE [B,Hq,S] fp32
  *   out: dQ [B,Hq,S,D], dK, dV [B,Hkv,S,D] fp16 (overwritten, not accumulated into)
  * dQ is accumulated in fp32 in the workspace with atomic adds, so its last bits may
- * differ between runs; dK and dV are bitwise reproducible, except on the grouped-query shapes
- * whose groups are split over work items (see lt_attn_bwd_num_launches), where they are summed
- * the same way.  The main and conversion kernels are launched with programmatic stream
+ * differ between runs; dK and dV are bitwise reproducible.  The main and conversion kernels are launched with programmatic stream
  * serialisation (each starts under the tail of its predecessor and waits inside for it). */
 int lt_attn_bwd(const lt_half *Q, const lt_half *K, const lt_half *V,
                 const lt_half *O, const lt_half *dO, const float *LSE,
@@ -119,7 +117,7 @@ int lt_attn_bwd_profiled(const lt_half *Q, const lt_half *K, const lt_half *V,
  * GPU that loads the library holds until the process ends.  Inputs and outputs are still the
  * caller's device tensors, with the meaning and layout of lt_attn_bwd.
  *   - Shapes whose workspace exceeds the built-in scratch (roughly B*Hq*S*D above four million elements;
- *     the fp32 dK/dV sums of split groups do not count, without room for them groups stay whole) return LT_ERR_WORKSPACE; lt_last_cuda_error()
+ *     the fp32 shares of dK and dV do not count, without room for them key tiles stay whole) return LT_ERR_WORKSPACE; lt_last_cuda_error()
  *     then names both sizes.  Nothing is launched in that case.
  *   - The call allocates nothing: no cudaMalloc/cudaFree and no allocating library routine.
  *   - The first call on each device looks up the array's device address (one runtime query,
@@ -260,8 +258,8 @@ const char *lt_status_string(int status);
 const char *lt_last_cuda_error(void);
 
 /* Number of kernels one call enqueues for this shape (for launch accounting by benchmarks): the
- * backward's preprocess, main and dQ-conversion kernels, plus the dK/dV conversion on grouped-query shapes
- * whose key-tile work items would be few or long, where a group's query heads are split
+ * backward's preprocess, main and dQ-conversion kernels, plus one that adds shares of dK and dV on shapes
+ * whose key-tile work items would be few or long, where a key tile's query tiles are split
  * over several items (4 instead of 3); sequences of at most 128 rows need 1 or 2 where that is faster; 0 for an unsupported
  * shape.  The forward enqueues one kernel. */
 int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal);

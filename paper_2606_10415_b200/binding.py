@@ -156,7 +156,7 @@ def lt_attn_host_arena_bytes(B, Hq, Hkv, S, D) -> int:
 
 
 def lt_attn_bwd_num_launches(B, Hq, Hkv, S, D, causal) -> int:
-    """Kernels one backward call enqueues for this shape (3, or 4 when groups are split over work items)."""
+    """Kernels one backward call enqueues for this shape (3, or 4 when key tiles are split over work items, or fewer for short sequences)."""
     return int(_lib.lt_attn_bwd_num_launches(B, Hq, Hkv, S, D, int(bool(causal))))
 
 

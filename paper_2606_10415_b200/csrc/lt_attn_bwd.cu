@@ -9,6 +9,9 @@
 //                           P^T from LSE, and run the five tile contractions on
 //                           tcgen05 tensor cores with tensor-memory accumulators
 //   bwd_finalize_kernel   : dQ fp32 accumulator -> fp16
+// and, where key tiles are split over several CTAs, beside the last one
+//   bwd_shares_kernel     : fp32 shares of dK and dV -> fp16
+// (Sequences of one tile: one or two launches, see one_tile_launches.)
 //
 // Loop order differs from Algorithm 1 (which is query-outer and reduces dK/dV partials
 // across workers): here a CTA owns one key/value tile, keeps dK_j and dV_j resident in
@@ -32,8 +35,8 @@
 // extra 16-element contraction step whose operands are (256, 1, 0...) and the (hi, lo, 0...)
 // split of the term, so the softmax warps never touch LSE or delta.
 //
-// Instantiations of the main kernel: fp16 or bf16 operands; a variant that splits a group's query
-// heads over several work items (few, heavy items) and sums dK/dV in fp32 in the workspace; and a
+// Instantiations of the main kernel: fp16 or bf16 operands; a variant that splits a key tile's tile
+// pairs over several work items (see BwdDeal); one for sequences of one tile; and a
 // variant that loads the probability tiles a forward pass saved (Section 4.1's own forward state,
 // written by lt_attn_save_p) instead of recomputing them.
 #include <math.h>
@@ -220,18 +223,13 @@ __device__ __forceinline__ void pre_v_rows(const PreParams &p, long long row_lo,
 
 template <int D, bool kBf16>
 __global__ void __launch_bounds__(kPreThreads, 3)  // three blocks per multiprocessor keep enough loads in flight
-bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, unsigned int *status,
-                      float4 *__restrict__ kv_acc, long long kv_acc_vec4) {
+bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, unsigned int *status) {
     grid_dependency_wait();    // launched under the tail of its predecessor, which may write O or read the workspace
     grid_launch_dependents();  // the main kernel sets itself up while this kernel's last blocks run
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         status[kStatusWordTimeout] = 0u;
         status[kStatusWordItemCounter] = 0u;
     }
-    // fp32 dK/dV sums (only when key tiles are split over several work items): zero them
-    for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < kv_acc_vec4;
-         v += static_cast<long long>(gridDim.x) * blockDim.x)
-        kv_acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int lane = threadIdx.x & 31;
     const long long warp_global = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const long long n_warps = (static_cast<long long>(gridDim.x) * blockDim.x) >> 5;
@@ -268,11 +266,12 @@ bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, uns
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float *__restrict__ dq_acc, __half *__restrict__ dQ, long long n_vec8, int vec_per_head,
-                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain, int kv_follows) {
+                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain, int beside) {
     // n_vec8 groups of eight output elements, numbered over the logical [B,Hq,S,D]; the accumulator
     // is indexed in the padded row space (`plain`: contiguous dQ and no padding, so both are group v)
-    grid_dependency_wait();  // launched while the main kernel drains: its reductions must have landed
-    if (kv_follows) grid_launch_dependents();  // the dK/dV conversion runs beside this one
+    // launched while the main kernel drains: its reductions must have landed (beside: this kernel runs beside the one that
+    // adds the shares of dK and dV, whose CTAs have all seen that)
+    if (!beside) grid_dependency_wait();
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < n_vec8; v += stride) {
         long long src = v, dst = v * 8;
@@ -293,37 +292,114 @@ bwd_finalize_kernel(const float *__restrict__ dq_acc, __half *__restrict__ dQ, l
         o.w = pack2<kBf16>(b.z, b.w);
         *reinterpret_cast<uint4 *>(dQ + dst) = o;
     }
+    if (beside) grid_dependency_wait();  // what follows this kernel may rely on dK and dV too
 }
 
-// fp32 dK / dV sums [B,Hkv,S_pad,D] -> 16-bit outputs (only when key tiles were split over work items)
-template <bool kBf16>
-__global__ void __launch_bounds__(256)
-bwd_finalize_kv_kernel(const float *__restrict__ dk_acc, const float *__restrict__ dv_acc, __half *__restrict__ dK,
-                       __half *__restrict__ dV, long long n_vec8, int vec_per_head, int vec_per_padded_head,
-                       int vec_per_row, int Hkv, lt_tensor_strides dk_st, lt_tensor_strides dv_st) {
-    // (started once every CTA of the dQ conversion has seen the main kernel complete, so every share has landed)
-    const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-    for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < 2 * n_vec8; v += stride) {
-        const bool second = v >= n_vec8;
-        const long long u = second ? v - n_vec8 : v;
-        const int bh = static_cast<int>(u / vec_per_head);
-        const int rem = static_cast<int>(u - static_cast<long long>(bh) * vec_per_head);
-        const int s_in = rem / vec_per_row, c = rem - s_in * vec_per_row;
-        const int bb = bh / Hkv, hh = bh - bb * Hkv;
-        const long long src = static_cast<long long>(bh) * vec_per_padded_head + rem;
-        const lt_tensor_strides &st = second ? dv_st : dk_st;
-        const long long dst = bb * st.batch + hh * st.head + s_in * st.row + c * 8;
-        const float *acc = second ? dv_acc : dk_acc;
-        const float4 a = __ldcs(reinterpret_cast<const float4 *>(acc) + 2 * src);
-        const float4 b = __ldcs(reinterpret_cast<const float4 *>(acc) + 2 * src + 1);
-        uint4 o;
-        o.x = pack2<kBf16>(a.x, a.y);
-        o.y = pack2<kBf16>(a.z, a.w);
-        o.z = pack2<kBf16>(b.x, b.y);
-        o.w = pack2<kBf16>(b.z, b.w);
-        *reinterpret_cast<uint4 *>((second ? dV : dK) + dst) = o;
+// Two ways to spread the tile pairs of one key tile over several CTAs.  Each leaves fp32 shares of dK_j and dV_j in the
+// workspace, which bwd_shares_kernel adds in the order of the pairs (the same result from run to run).
+// Dealt out (ctas > 0), where the SMs would get only a few, or a few heavy, key tiles: the CTAs get consecutive stretches of
+// equal cost of one walk over all (unit, key tile, pair)s, where a unit is a (batch, kv head) with its group of query heads,
+// and a key tile costs its pairs plus kTileCost for filling the pipeline and storing dK_j and dV_j.  A CTA leaves at most
+// two shares: the end of its first key tile and the beginning of its last.
+// In halves (halves = 1): every key tile is two work items, claimed from the counter like whole ones.
+constexpr int kTileCost = 2;  // (measured with 2, 4, 6, 8: 2 is the best or within 1 % of it on 16 shapes)
+struct BwdDeal {
+    int ctas, halves;  // both 0: key tiles are whole
+    int n_units, G, n_tiles, causal;
+
+    __host__ __device__ __forceinline__ bool any() const { return ctas > 0 || halves; }
+    __host__ __device__ __forceinline__ int pairs(int j) const { return G * (causal ? n_tiles - j : n_tiles); }
+    // cost of a unit's key tiles before tile j
+    __host__ __device__ __forceinline__ int tile_start(int j) const {
+        return j * kTileCost + G * (causal ? j * n_tiles - j * (j - 1) / 2 : j * n_tiles);
     }
-    grid_dependency_wait();  // what follows this kernel may rely on the dQ conversion having finished too
+    // where CTA c's stretch begins
+    __host__ __device__ __forceinline__ int stretch(int c) const {
+        const int cost = n_units * tile_start(n_tiles), each = cost / ctas;
+        return each * c + (cost - each * ctas) * c / ctas;
+    }
+    // a stretch boundary x behind a key tile's start -> pairs of the tile before it
+    __host__ __device__ __forceinline__ int cut(int x, int n) const {
+        x -= kTileCost;
+        return x < 0 ? 0 : x > n ? n : x;
+    }
+    // key tile of a unit that holds cost x
+    __host__ __device__ __forceinline__ int tile_at(int x) const {
+        int lo = 0, hi = n_tiles - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (tile_start(mid) <= x) lo = mid;
+            else hi = mid - 1;
+        }
+        return lo;
+    }
+    // A share is a block of 2 x 128 x D floats: dK, then dV, each [D/4][128 rows][4], so that a warp stores or reads 512
+    // consecutive bytes.  Dealt out, they are numbered 2 c (the end of CTA c's first key tile) and 2 c + 1 (the beginning of
+    // its last); in halves, by key tile and half.
+    __host__ __device__ __forceinline__ int n_shares() const { return 2 * (halves ? n_units * n_tiles : ctas); }
+};
+
+// dK_j and dV_j of the key tiles that were dealt out to several CTAs: the fp32 shares, added in the order of the walk,
+// as 16-bit outputs.  Block (c, 32 columns of dK or dV) has the tile that CTA c's stretch ends in, if it began there
+// or before; it does nothing where the stretch ends with a tile or another CTA's does the beginning.  In halves: key tile c.
+// Launched before the dQ conversion, which runs beside it: 2-3 us less per call than behind it.
+template <int D, bool kBf16>
+__global__ void __launch_bounds__(256)
+bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __half *__restrict__ dV, const BwdDeal deal,
+                  int Hkv, int S, lt_tensor_strides dk_st, lt_tensor_strides dv_st) {
+    const int c = blockIdx.x, second = blockIdx.y & 1;
+    int parts = 0, unit, j = 0, first_share;
+    if (deal.halves) {
+        unit = c / deal.n_tiles;
+        j = c - unit * deal.n_tiles;
+        first_share = 2 * c;
+        parts = 2;
+    } else {
+        const int unit_cost = deal.tile_start(deal.n_tiles), end = deal.stretch(c + 1);
+        unit = end / unit_cost;
+        first_share = 2 * c + 1;
+        if (unit < deal.n_units) {
+            j = deal.tile_at(end - unit * unit_cost);
+            const int start = unit * unit_cost + deal.tile_start(j), n = deal.pairs(j);
+            int upto = deal.cut(end - start, n);
+            if (upto > 0 && upto < n && deal.cut(deal.stretch(c) - start, n) == 0)
+                for (parts = 1; upto < n; ++parts) upto = deal.cut(deal.stretch(c + parts + 1) - start, n);
+        }
+    }
+    grid_dependency_wait();    // launched while the main kernel drains: its shares must have landed
+    grid_launch_dependents();  // the dQ conversion runs beside this kernel
+    if (parts == 0) return;
+    constexpr int kShareVec = 128 * D / 4;  // float4s of dK or dV in a share
+    const int row = threadIdx.x & 127;
+    const int v8 = (blockIdx.y >> 1) * 4 + (threadIdx.x >> 7);
+    const float4 *src = shares + second * kShareVec + (2 * v8) * 128 + row;
+    const float4 *next = src + static_cast<long long>(first_share) * 2 * kShareVec;
+    float4 a[2][2];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) a[x >> 1][x & 1] = __ldcs(next + ((x >> 1) * 4 + (x & 1)) * 128);
+    next += 2 * kShareVec;  // the second share follows the first, further ones are two apart
+#pragma unroll 4
+    for (int k = 1; k < parts; ++k, next += 4 * kShareVec) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const float4 y = __ldcs(next + ((x >> 1) * 4 + (x & 1)) * 128);
+            float4 &t = a[x >> 1][x & 1];
+            t.x += y.x; t.y += y.y; t.z += y.z; t.w += y.w;
+        }
+    }
+    const int b = unit / Hkv, g = unit - b * Hkv, s_row = j * 128 + row;
+    const lt_tensor_strides &st = second ? dv_st : dk_st;
+    __half *dst = (second ? dV : dK) + b * st.batch + g * st.head + s_row * st.row + v8 * 8;
+    if (s_row >= S) return;
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        uint4 o;
+        o.x = pack2<kBf16>(a[x][0].x, a[x][0].y);
+        o.y = pack2<kBf16>(a[x][0].z, a[x][0].w);
+        o.z = pack2<kBf16>(a[x][1].x, a[x][1].y);
+        o.w = pack2<kBf16>(a[x][1].z, a[x][1].w);
+        *reinterpret_cast<uint4 *>(dst + x * 16) = o;
+    }
 }
 
 // ----------------------------------------------------------------------------- optional cycle trace
@@ -399,6 +475,29 @@ constexpr int kBarReduceWarps = 1, kBarScale = 2;  // named barrier ids
 constexpr int kItemRing = 4;  // roles are never more than two items apart
 constexpr double kL2BatchBytes = 80.0e6;  // working set of one batch of work items (L2 holds 126 MB)
 
+// A CTA's way through its stretch (in shared memory: the producer has few registers).
+struct BwdWalk {
+    int unit, j, start, begin, end;  // the next key tile and its place in the walk, the stretch
+
+    __device__ __forceinline__ void reset(const BwdDeal &d) {
+        const int unit_cost = d.tile_start(d.n_tiles);
+        begin = d.stretch(blockIdx.x);
+        end = d.stretch(blockIdx.x + 1);
+        unit = begin / unit_cost;
+        j = d.tile_at(begin - unit * unit_cost);
+        start = unit * unit_cost + d.tile_start(j);
+    }
+    __device__ __forceinline__ int4 next(const BwdDeal &d) {
+        while (start < end) {
+            const int n = d.pairs(j), tile = unit * d.n_tiles + j;
+            const int from = d.cut(begin - start, n), to = d.cut(end - start, n);
+            start += kTileCost + n;
+            if (++j == d.n_tiles) j = 0, ++unit;
+            if (to > from) return make_int4(tile, from, to, from == 0 && to == n ? -1 : 2 * blockIdx.x + (from == 0));
+        }
+        return make_int4(-1, 0, 0, 0);
+    }
+};
 template <int D>
 struct BwdSmem {
     static constexpr int kBoxes = D / 64;
@@ -421,10 +520,12 @@ struct BwdSmem {
     uint64_t bar_kv, bar_dkv_full, bar_acc_free;
     // work items are claimed from a global counter by the producer and published to the other roles
     uint64_t bar_item[kItemRing];
-    int item_ring[kItemRing];
+    int4 item_ring[kItemRing];  // (x alone where key tiles are whole)
     // per (query head, query tile) iteration
     uint64_t bar_q_full[kQStages], bar_q_empty[kQStages], bar_do_full, bar_do_empty;
     uint64_t bar_s_full, bar_p_ready, bar_dp_full, bar_ds_ready, bar_ds_free, bar_dq_full, bar_dq_empty;
+    BwdWalk walk;
+    int4 first_item;
     uint32_t tmem_base;
     int abort_flag;
     unsigned int call_max[3];  // the call's maxima (slot bits of max |delta|, max ||dO_row||^2, max ||V_row||^2)
@@ -448,56 +549,58 @@ struct BwdParams {
     __half *dV;
     unsigned int *status;
     int B, Hq, Hkv, S, S_pad, causal;  // S_pad: S rounded up to whole 128-row tiles
-    // (batch, kv head) units per L2-sized batch of work items.  In the variant that splits a group of
-    // query heads over several items the word also carries, above bit 16, the items per (unit, key
-    // tile) and, above bit 24, the query heads per item; dK and dV then point at the fp32 sums
-    // [B,Hkv,S_pad,D] of the parts.  (The structure keeps its size: the main kernel's register
-    // allocation is sensitive to it.)
-    int units_per_batch;
+    int units_per_batch;  // (batch, kv head) units per L2-sized batch of work items
+    BwdDeal deal;         // of the variant that splits key tiles
+    float4 *shares;
     float scale;
     lt_tensor_strides dk_st, dv_st;  // element strides of dK and dV
 };
 
-// One work item = key tile j of (batch b, kv head g).  Items are numbered so that the heavy
-// ones (small j under a causal mask) come first; CTA c takes items c, c + gridDim.x, ...
+// One work item = key tile j of (batch b, kv head g): the flattened (query head of the group, query tile) loop, or a
+// stretch of it.
 struct BwdItem {
     int j, b, g, i_first, tiles_per_head, n_iter;
-    int h_first;  // first query head of the group this item covers (0 unless the group is split)
+    int n_first;  // first iteration of the flattened loop this item covers
+    int share;    // where its dK_j and dV_j go: a share, or (-1) the outputs
 };
-template <bool kSplit>
-__device__ __forceinline__ BwdItem bwd_item(const BwdParams &p, int item) {
-    BwdItem w;
-    const int parts = kSplit ? ((p.units_per_batch >> 16) & 0xFF) : 1;
-    const int units_per_batch = kSplit ? (p.units_per_batch & 0xFFFF) : p.units_per_batch;
-    const int heads_per_item = kSplit ? ((p.units_per_batch >> 24) & 0xFF) : 0;
+// Items are numbered batch of (batch, kv head) units by batch; inside a batch key tile by key tile (heavy tiles
+// first), all units of the batch per key tile.  A batch is sized so that everything its items touch (K, V, the
+// group's Q and dO, the fp32 dQ rows) stays in L2 while the CTAs work through it; with one batch this is the plain
+// heavy-first order.
+__device__ __forceinline__ void bwd_item_place(const BwdParams &p, int item, int &j, int &bg) {
     const int n_tiles = (p.S + kTileRows - 1) / kTileRows;  // the last tile may be ragged
-    const int n_bg = p.B * p.Hkv;
-    // Items are numbered batch of (batch, kv head) units by batch; inside a batch key tile by key tile
-    // (heavy tiles first), all units of the batch per key tile.  A batch is sized so that everything its
-    // items touch (K, V, the group's Q and dO, the fp32 dQ rows) stays in L2 while the CTAs work
-    // through it; with one batch this is the plain heavy-first order.
-    const int batch = item / (units_per_batch * n_tiles * parts);
-    const int first_unit = batch * units_per_batch;
-    const int units = min(units_per_batch, n_bg - first_unit);
-    // A group of query heads may be split into `parts` items per key tile (shapes with few, heavy
-    // items); the parts of one key tile are neighbours in the numbering.
-    const int within = item - first_unit * n_tiles * parts;
-    w.j = within / (units * parts);
-    const int rem = within - w.j * units * parts;
-    const int unit_local = rem / parts;
-    const int part = rem - unit_local * parts;
-    const int bg = first_unit + unit_local;
+    const int batch = item / (p.units_per_batch * n_tiles);
+    const int first_unit = batch * p.units_per_batch;
+    const int units = min(p.units_per_batch, p.B * p.Hkv - first_unit);
+    const int within = item - first_unit * n_tiles;
+    j = within / units;
+    bg = first_unit + within - j * units;
+}
+// half `item & 1` of item `item >> 1`, as the producer publishes parts of key tiles: {unit * key tiles + j, first pair, end, share}
+__device__ __forceinline__ int4 bwd_half_item(const BwdParams &p, int item) {
+    int j, bg;
+    bwd_item_place(p, item >> 1, j, bg);
+    const int n = p.deal.pairs(j), tile = bg * p.deal.n_tiles + j, mid = (n + 1) >> 1, half = item & 1;
+    return make_int4(tile, half ? mid : 0, half ? n : mid, 2 * tile + half);
+}
+template <bool kSplit>
+__device__ __forceinline__ BwdItem bwd_item(const BwdParams &p, const int4 &rec) {
+    BwdItem w;
+    const int n_tiles = (p.S + kTileRows - 1) / kTileRows;
+    int bg;
+    if constexpr (kSplit) {
+        bg = rec.x / n_tiles;
+        w.j = rec.x - bg * n_tiles;
+    } else {
+        bwd_item_place(p, rec.x, w.j, bg);
+    }
     w.b = bg / p.Hkv;
     w.g = bg - w.b * p.Hkv;
     w.i_first = p.causal ? w.j : 0;
     w.tiles_per_head = n_tiles - w.i_first;
-    if constexpr (kSplit) {
-        w.h_first = part * heads_per_item;
-        w.n_iter = min(heads_per_item, p.Hq / p.Hkv - w.h_first) * w.tiles_per_head;
-    } else {
-        w.h_first = 0;
-        w.n_iter = (p.Hq / p.Hkv) * w.tiles_per_head;  // flattened (query head of the group, query tile) loop
-    }
+    w.n_first = kSplit ? rec.y : 0;
+    w.n_iter = kSplit ? rec.z - rec.y : (p.Hq / p.Hkv) * w.tiles_per_head;
+    w.share = kSplit ? rec.w : -1;
     return w;
 }
 // Iteration n of an item -> its query tile: batch, query head, first row inside the head, and the tile's first row in the padded row space of the workspace arrays
@@ -507,11 +610,12 @@ struct BwdQTile {
     long long padded_row0;
 };
 __device__ __forceinline__ BwdQTile bwd_q_tile(const BwdParams &p, const BwdItem &w, int n) {
+    n += w.n_first;
     const int hh = n / w.tiles_per_head;
     const int i = w.i_first + (n - hh * w.tiles_per_head);
     BwdQTile q;
     q.b = w.b;
-    q.h = w.g * (p.Hq / p.Hkv) + w.h_first + hh;
+    q.h = w.g * (p.Hq / p.Hkv) + hh;
     q.s0 = i * kTileRows;
     q.padded_row0 = (static_cast<long long>(w.b) * p.Hq + q.h) * p.S_pad + q.s0;
     return q;
@@ -592,7 +696,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-    const int n_items = (p.S_pad / kTileRows) * p.B * p.Hkv * (kSplit ? ((p.units_per_batch >> 16) & 0xFF) : 1);
+    const int n_items = p.B * p.Hkv * (p.S_pad / kTileRows) * (kSplit ? 2 : 1);  // (split: in halves)
 
     // the swizzled tiles need 1024-byte alignment; the shared window is expected to give it
     const bool smem_ok = (smem_u32(smem_raw) & 1023u) == 0u;
@@ -645,17 +749,29 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     if constexpr (kOneTile)
         if (one.own_pre) grid_dependency_wait();
     if (warp == 0 && lane == 0 && smem_ok) {
-        const BwdItem w = bwd_item<kSplit>(p, static_cast<int>(blockIdx.x));
-        const BwdQTile qt = bwd_q_tile(p, w, 0);
-        mbar_arrive_expect_tx(&sm.bar_q_full[0], kSavedP ? kTileBytes : kTileBytes + kExtBytes);
-        mbar_arrive_expect_tx(&sm.bar_kv, 2 * kTileBytes);
-        mbar_arrive_expect_tx(&sm.bar_do_full, kTileBytes + kExtBytes);
+        int4 rec = make_int4(static_cast<int>(blockIdx.x), 0, 0, 0);
+        if constexpr (kSplit) {
+            if (p.deal.halves) {
+                rec = bwd_half_item(p, static_cast<int>(blockIdx.x));
+            } else {
+                sm.walk.reset(p.deal);
+                rec = sm.walk.next(p.deal);
+            }
+            sm.first_item = rec;
+        }
+        if (!kSplit || rec.x >= 0) {
+            const BwdItem w = bwd_item<kSplit>(p, rec);
+            const BwdQTile qt = bwd_q_tile(p, w, 0);
+            mbar_arrive_expect_tx(&sm.bar_q_full[0], kSavedP ? kTileBytes : kTileBytes + kExtBytes);
+            mbar_arrive_expect_tx(&sm.bar_kv, 2 * kTileBytes);
+            mbar_arrive_expect_tx(&sm.bar_do_full, kTileBytes + kExtBytes);
 #pragma unroll
-        for (int x = 0; x < kBoxes; ++x) {
-            tma_load_4d(sm.q[0] + x * kBoxBytesBwd, &map_q, &sm.bar_q_full[0], x * 64, qt.s0, qt.h, qt.b);
-            tma_load_4d(sm.k + x * kBoxBytesBwd, &map_k, &sm.bar_kv, x * 64, w.j * kTileRows, w.g, w.b);
-            tma_load_4d(sm.d_o + x * kBoxBytesBwd, &map_do, &sm.bar_do_full, x * 64, qt.s0, qt.h, qt.b);
-            tma_load_4d(sm.v + x * kBoxBytesBwd, &map_v, &sm.bar_kv, x * 64, w.j * kTileRows, w.g, w.b);
+            for (int x = 0; x < kBoxes; ++x) {
+                tma_load_4d(sm.q[0] + x * kBoxBytesBwd, &map_q, &sm.bar_q_full[0], x * 64, qt.s0, qt.h, qt.b);
+                tma_load_4d(sm.k + x * kBoxBytesBwd, &map_k, &sm.bar_kv, x * 64, w.j * kTileRows, w.g, w.b);
+                tma_load_4d(sm.d_o + x * kBoxBytesBwd, &map_do, &sm.bar_do_full, x * 64, qt.s0, qt.h, qt.b);
+                tma_load_4d(sm.v + x * kBoxBytesBwd, &map_v, &sm.bar_kv, x * 64, w.j * kTileRows, w.g, w.b);
+            }
         }
     }
     // everything above ran while the preprocess kernel was finishing; its results (row operands, zeroed
@@ -707,19 +823,30 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 int last_q = -1, last_do = -1, kv_loads = 0;  // for the cleanup after an abandoned wait
                 // claim the next unclaimed item (heavy ones have the low numbers; the grid's first ones are the CTAs'
                 // first items) and publish it to the other roles; -1 tells everybody that the list is exhausted
-                auto claim = [&](int slot_ic) -> int {
-                    unsigned int v = blockIdx.x;
-                    if constexpr (kOneTile) v += slot_ic * gridDim.x;
-                    else if (slot_ic > 0) v = atomicAdd(p.status + kStatusWordItemCounter, 1u) + gridDim.x;
-                    const int item = v < static_cast<unsigned int>(n_items) ? static_cast<int>(v) : -1;
-                    sm.item_ring[slot_ic % kItemRing] = item;
+                auto claim = [&](int slot_ic) -> int4 {
+                    int4 rec = make_int4(-1, 0, 0, 0);
+                    if (kSplit && slot_ic == 0) {
+                        rec = sm.first_item;
+                    } else if (kSplit && !p.deal.halves) {
+                        rec = sm.walk.next(p.deal);
+                    } else {
+                        unsigned int v = blockIdx.x;
+                        if constexpr (kOneTile) v += slot_ic * gridDim.x;
+                        else if (slot_ic > 0) v = atomicAdd(p.status + kStatusWordItemCounter, 1u) + gridDim.x;
+                        if (v < static_cast<unsigned int>(n_items)) {
+                            rec.x = static_cast<int>(v);
+                            if constexpr (kSplit) rec = bwd_half_item(p, rec.x);
+                        }
+                    }
+                    if constexpr (kSplit) sm.item_ring[slot_ic % kItemRing] = rec;
+                    else sm.item_ring[slot_ic % kItemRing].x = rec.x;
                     mbar_arrive(&sm.bar_item[slot_ic % kItemRing]);
-                    return item;
+                    return rec;
                 };
-                int item = claim(0);
-                while (item >= 0 && ok) {
+                int4 item = claim(0);
+                while (item.x >= 0 && ok) {
                     const BwdItem w = bwd_item<kSplit>(p, item);
-                    int next_item = -1;
+                    int4 next_item = make_int4(-1, 0, 0, 0);
                     for (int n = 0; n < w.n_iter && ok; ++n, ++it) {
                         const int s = it & 1, k = it >> 1;
                         const BwdQTile qt = bwd_q_tile(p, w, n);
@@ -762,7 +889,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                             // with the last query tile of this item on its way, claim the next item and ask for
                             // its K/V tiles to be brought into L2 while this item finishes
                             next_item = claim(ic + 1);
-                            if (next_item >= 0) {
+                            if (next_item.x >= 0) {
                                 const BwdItem wn = bwd_item<kSplit>(p, next_item);
 #pragma unroll
                                 for (int x = 0; x < kBoxes; ++x) {
@@ -842,8 +969,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 int it = 0, ic = 0;
                 for (;; ++ic) {
                     if (!(ok = LT_WAIT_ALL(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem))) break;
-                    const int item = sm.item_ring[ic % kItemRing];
-                    if (item < 0) break;
+                    const int4 item = sm.item_ring[ic % kItemRing];
+                    if (item.x < 0) break;
                     const BwdItem w = bwd_item<kSplit>(p, item);
                     ok = LT_WAIT_ALL(&sm.bar_kv, ic & 1, kWaitKV) &&
                          LT_WAIT_ALL(&sm.bar_q_full[it & 1], (it >> 1) & 1, kWaitStageFull);
@@ -1041,12 +1168,12 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
         for (;; ++ic) {
             if (!ok || !LT_WAIT(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem)) break;
-            const int item = sm.item_ring[ic % kItemRing];
-            if (item < 0) break;
+            const int4 item = sm.item_ring[ic % kItemRing];
+            if (item.x < 0) break;
             const BwdItem w = bwd_item<kSplit>(p, item);
             if constexpr (kSavedP) load_saved_p(w, 0, ph);
-            ok = compute_p(w, it, 0);
-            int tile = 0;
+            int tile = kSplit ? w.n_first % w.tiles_per_head : 0;
+            ok = compute_p(w, it, tile);
             for (int n = 0; n < w.n_iter && ok; ++n, ++it) {
                 if constexpr (kSavedP)
                     if (n + 1 < w.n_iter) load_saved_p(w, n + 1, pn);
@@ -1120,8 +1247,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             ok = ok && LT_WAIT(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem);
             ok = named_barrier_and(kBarReduceWarps, kNumReduceWarps * 32, ok);
             if (!ok) break;
-            const int item = sm.item_ring[ic % kItemRing];
-            if (item < 0) break;
+            const int4 item = sm.item_ring[ic % kItemRing];
+            if (item.x < 0) break;
             const BwdItem w = bwd_item<kSplit>(p, item);
             for (int n = 0; n < w.n_iter; ++n, ++it) {
                 ok = LT_WAIT(&sm.bar_dq_full, it & 1, kWaitDqFull);
@@ -1300,18 +1427,13 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                             if (lane == 0) mbar_arrive(&sm.bar_acc_free);
                             LT_TL(tid == kReduceWarp0 * 32, 15, it);
                         }
-                        if constexpr (kSplit) {
-                            // the group's heads are spread over several items: add this item's share to
-                            // the fp32 sums; a separate pass rounds them once all shares are in
-                            float *acc = reinterpret_cast<float *>(which == 0 ? p.dK : p.dV) +
-                                         ((static_cast<long long>(w.b) * p.Hkv + w.g) * p.S_pad + s_row) * D + c * 32;
-                            if (s_row < p.S) {
+                        if (kSplit && w.share >= 0) {
+                            // (rows past S come from zero-filled key rows: finite, never read)
+                            float4 *share = p.shares + (static_cast<long long>(w.share) * 2 + which) * (kTileRows * D / 4) + c * 8 * kTileRows + row;
 #pragma unroll
-                                for (int v4 = 0; v4 < 8; ++v4)
-                                    red_add_v4(acc + 4 * v4, __uint_as_float(r[4 * v4 + 0]) * mult,
-                                               __uint_as_float(r[4 * v4 + 1]) * mult, __uint_as_float(r[4 * v4 + 2]) * mult,
-                                               __uint_as_float(r[4 * v4 + 3]) * mult);
-                            }
+                            for (int v4 = 0; v4 < 8; ++v4)
+                                share[v4 * kTileRows] = make_float4(__uint_as_float(r[4 * v4 + 0]) * mult, __uint_as_float(r[4 * v4 + 1]) * mult,
+                                                                    __uint_as_float(r[4 * v4 + 2]) * mult, __uint_as_float(r[4 * v4 + 3]) * mult);
                             continue;
                         }
 #pragma unroll
@@ -1375,10 +1497,6 @@ extern "C" int lt_dbg_bwd_trace(unsigned long long *out, int reset) {
 }
 #endif
 
-// Query heads of a group per work item.  A (batch, kv head, key tile) item normally covers the whole
-// group (dK_j, dV_j of all its heads accumulate in one CTA's tensor memory).  Shapes that would give
-// the 148 SMs only a few, heavy items get the group split over several items instead; their shares of
-// dK_j, dV_j are then summed in fp32 in the workspace and rounded by a small extra kernel.
 // Multiprocessors of the current device (148 on a B200; that figure is also the answer when the query fails,
 // so that the sizes derived from it never depend on an error path).
 static int sm_count() {
@@ -1388,47 +1506,53 @@ static int sm_count() {
         return 148;
     return sms;
 }
-static int heads_per_item(int B, int Hq, int Hkv, int S, int D, int causal) {
+// Whether and how key tiles are split (BwdDeal), with at most `room` bytes of shares.  Not at all: every key tile is one
+// work item, claimed from a counter, its dK_j and dV_j accumulated in one CTA's tensor memory.
+static size_t share_bytes(const BwdDeal &deal, int D) {
+    return static_cast<size_t>(deal.any() ? deal.n_shares() : 0) * (2 * kTileRows * 4) * D;
+}
+static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size_t room = ~static_cast<size_t>(0)) {
     const int sms = sm_count();
-    const int G = Hq / Hkv;
-    const long long n_tiles = padded_rows(S) / kTileRows;
-    const long long n_base = static_cast<long long>(B) * Hkv * n_tiles;
-    if (G == 1) return 1;
-    // The heads per item with the shortest estimated makespan, in tile pairs (about 2.1 us each): the longest item or the
-    // average work of an SM, with what an item costs beside its pairs (pipeline fill and the epilogue, which adds to fp32
-    // sums when groups are split), and 3 for the zero fill and conversion of those sums.  Measured, us per call, whole
-    // groups / this choice: 8 / 1 heads at S = 2048 286 / 55; 16 / 4 at 1024 83 / 39; 4 x 16 / 2 at 1024, D = 64 112 / 51;
-    // 40 / 8 at 1024 108 / 64, at 2048 240 / 158; 2 x 40 / 8 at 1536 unmasked 391 / 357.  On the other side of the line:
-    // 8 x 20 / 4 at 512 79 whole, 81 split in two; 64 / 16 at 2048 237 whole, 269; 40 / 8 at 4096 525 whole, 525.
-    const double pairs = static_cast<double>(B) * Hq * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
-    int best = G;
-    double best_span = 0.;
-    for (int parts = 1; parts <= G; ++parts) {
-        const int hpi = (G + parts - 1) / parts;
-        if (parts > 1 && (G + hpi - 1) / hpi != parts) continue;  // the same items as with fewer parts
-        const double per_item = parts > 1 ? 6. : 2., items = static_cast<double>(n_base) * parts;
-        const double longest = static_cast<double>(hpi) * n_tiles + (parts > 1 ? 4. : 2.);
-        double span = pairs / sms + per_item * items / sms;
-        if (longest > span) span = longest;
-        if (!causal) {  // items of one length: whole rounds
-            const double rounds = ceil(items / sms) * (pairs / items + per_item);
-            if (rounds > span) span = rounds;
+    BwdDeal deal{0, 0, B * Hkv, Hq / Hkv, static_cast<int>(padded_rows(S) / kTileRows), causal ? 1 : 0};
+    const double n_tiles = deal.n_tiles, G = deal.G, items = deal.n_units * n_tiles;
+    const double pairs = B * G * Hkv * (causal ? 0.5 * n_tiles * (n_tiles + 1.) : n_tiles * n_tiles);
+    const double cost = pairs + kTileCost * items;
+    if (G * n_tiles < 2. || cost > 1.0e9) return deal;  // (nothing to split; costs are 32-bit numbers)
+    // (small walks: stretches of two; a small workspace: as many as have room for their shares)
+    int ctas = cost < 2. * sms ? static_cast<int>(cost / 2.) : sms;
+    const size_t two_shares = static_cast<size_t>(2) * (2 * kTileRows * 4) * D;
+    if (room / two_shares < static_cast<size_t>(ctas)) ctas = static_cast<int>(room / two_shares);
+    // Estimated makespans, in tile pairs (2-3 us each): whole key tiles, the longest one or the average work of an SM, in
+    // whole rounds where all are equal; dealt out, the average plus what the parts cost: the shares stored and added (they
+    // grow with the CTAs), and a second pipeline filled in the CTAs whose stretch crosses into another key tile.  Measured, us per call, whole / dealt
+    // out (batch, query / kv heads, S; D = 128 under the causal mask unless noted): 1, 40/8, 2048 244 / 149; 1, 40/8, 1024
+    // 108 / 56; 1, 2/1, 3566 131 / 39; 1, 1/1, 4135, D = 64 60 / 26; 1, 2/2, 2999 unmasked 66 / 43; 8, 5/1, 2572, D = 64
+    // unmasked 399 / 221; 1, 16/8, 208 22.0 / 19.1.  On the other side of the line: 1, 64/16, 2048 244 / 257; 1, 8/8, 4096
+    // 105 / 127; 1, 32/32, 1024 45 / 61; 2, 8/8, 384 unmasked 19.0 / 22.6; near it: 8, 20/4, 512 81 / 78; 1, 8/8, 2048
+    // 51 / 48; 1, 40/8, 4096 and 1, 32/8, 4096 equal.  One tile: 1, 32/8, 128 20.7 / 17.8; 8, 40/8, 128 32.0 / 35.6.
+    double whole = cost / sms;
+    if (whole < G * n_tiles + kTileCost) whole = G * n_tiles + kTileCost;
+    if (!causal && whole < ceil(items / sms) * (G * n_tiles + kTileCost)) whole = ceil(items / sms) * (G * n_tiles + kTileCost);
+    if (n_tiles == 1. && D == 64) whole -= 1.;  // (the one-tile variant has fewer launches)
+    if (ctas > 0) {
+        const double crossings = items < ctas ? items / ctas : 1.;
+        const double dealt = cost / ctas + 1.6 + 0.028 * ctas + 3.0 * crossings * crossings;
+        if (dealt < 0.95 * whole) {
+            deal.ctas = ctas;
+            return deal;
         }
-        if (parts > 1) span += 3.;
-        if (parts == 1 || span < best_span) best = hpi, best_span = span;
     }
-    if (best < G) return best;
-    // Enough whole-group items to fill the SMs, but too few to form L2-sized batches (a batch needs two items per
-    // SM) while the working set is more than four times the L2: the accumulator rows of the heads in flight would be
-    // fetched and written back again and again.  Two items per key tile make room for batches.  Measured, whole
-    // against split, ms per call: LLaMA-2-70B layer with B = 2 1.78 / 1.69 (3.6 -> 1.45 GB of DRAM traffic), the
-    // same at S = 8192 with B = 1 3.38 / 3.02, 32 / 4 heads at S = 16384 6.06 / 5.76.  Smaller working sets lose
-    // more to the second pipeline fill and the fp32 epilogue than they gain: 32 / 8 heads at S = 8192 (2.4 L2s)
-    // 1.52 / 1.59, the same with B = 2 at S = 4096 0.86 / 0.89, the Qwen2.5-32B layer (1.4 L2s) 0.53 / 0.56.
-    const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
-    const double working_set = unit_bytes * B * Hkv;
-    if (n_base >= sms + sms / 2 && n_base < 4LL * sms && working_set > 4.0 * 126.0e6) return (G + 1) / 2;
-    return G;
+    if (G > 1. && items >= sms + sms / 2 && items < 4. * sms) {
+        // Enough key tiles to fill the SMs, but too few to form L2-sized batches (a batch needs two items per SM) while the
+        // working set is more than four times the L2: the accumulator rows of the heads in flight would be fetched and
+        // written back again and again.  Halves make room for batches.
+        // Measured, ms per call, halves / whole, medians of 7 or 9 whose single values spread by 10 % (the power limit): 2, 64/8,
+        // 4096 1.74-1.78 / 1.82-1.84 in two comparisons, 1.76 / 1.66 in a third; 1, 64/8, 8192 3.19 / 3.24.
+        const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
+        if (unit_bytes * deal.n_units > 4.0 * 126.0e6) deal.halves = 1;
+    }
+    if (share_bytes(deal, D) > room) deal.halves = 0;
+    return deal;
 }
 
 // Sequences of one tile: launches of a call in the one-tile variant, or 0 where the general path is the faster one.  With
@@ -1449,8 +1573,8 @@ static int one_tile_launches(int B, int Hq, int Hkv, int S, int D) {
 template <int D, bool kBf16>
 static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
                       const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout &lay, int B,
-                      int Hq, int Hkv, int S, int causal, float scale, void *workspace, cudaStream_t stream,
-                      cudaEvent_t ev_main_begin, cudaEvent_t ev_main_end, bool may_split, const lt_half *saved_p = nullptr) {
+                      int Hq, int Hkv, int S, int causal, float scale, void *workspace, size_t workspace_bytes, cudaStream_t stream,
+                      cudaEvent_t ev_main_begin, cudaEvent_t ev_main_end, const lt_half *saved_p = nullptr) {
     // saved_p: the probability tiles of lt_attn_save_p; LSE is then not needed (fp16, whole groups only)
     const int S_pad = static_cast<int>(padded_rows(S));
     // fast addressing in the two streaming kernels when nothing is padded or strided
@@ -1467,14 +1591,10 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     uint4 *delta_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes);
     uint4 *lse_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes + ext_bytes);
     float *dq_acc = reinterpret_cast<float *>(ws + kStatusBytes + 2 * ext_bytes);
-    const int hpi = saved_p || !may_split ? Hq / Hkv : heads_per_item(B, Hq, Hkv, S, D, causal);
-    const int parts = (Hq / Hkv + hpi - 1) / hpi;
-    const size_t kv_floats = static_cast<size_t>(B) * Hkv * S_pad * D;
-    float *dk_acc = nullptr, *dv_acc = nullptr;
-    if (parts > 1) {
-        dk_acc = reinterpret_cast<float *>(ws + kStatusBytes + 2 * ext_bytes + round256(static_cast<size_t>(n_rows) * D * 4));
-        dv_acc = dk_acc + kv_floats;  // kv_floats * 4 is a multiple of 256 bytes
-    }
+    const size_t base_bytes = kStatusBytes + 2 * ext_bytes + round256(static_cast<size_t>(n_rows) * D * 4);
+    BwdDeal deal{};
+    if (!saved_p) deal = deal_pairs(B, Hq, Hkv, S, D, causal, workspace_bytes - base_bytes);
+    const bool split = deal.any();
 
     CUtensorMap mq, mk, mv, mdo;
     int rc;
@@ -1506,7 +1626,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     one.pre.inv_scale = 1.f / scale;
     one.dQ = reinterpret_cast<__half *>(dQ);
     one.dq_st = lay.dq;
-    const int tile_launches = saved_p || parts > 1 ? 0 : one_tile_launches(B, Hq, Hkv, S, D);
+    const int tile_launches = saved_p || split ? 0 : one_tile_launches(B, Hq, Hkv, S, D);
     const bool one_tile = tile_launches > 0;
     one.own_pre = tile_launches == 1 ? 1 : 0;
     if (one_tile) one.pre.dq_acc = nullptr;
@@ -1518,8 +1638,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
         cfg_pre.attrs = &pdl;
         cfg_pre.numAttrs = 1;
         e = cudaLaunchKernelEx(&cfg_pre, bwd_preprocess_kernel<D, kBf16>, one.pre, n_rows,
-                               static_cast<long long>(B) * Hkv * S, status, reinterpret_cast<float4 *>(dk_acc),
-                               parts > 1 ? static_cast<long long>(kv_floats / 2) : 0LL);
+                               static_cast<long long>(B) * Hkv * S, status);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return record_cuda_error("bwd_preprocess_kernel launch", e);
     }
@@ -1542,28 +1661,21 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
         const int n_units = B * Hkv;
         int n_batches = static_cast<int>(unit_bytes * n_units / kL2BatchBytes) + 1;
         // CTAs flow from one batch into the next, but the last batch should still offer every SM two items
-        const int max_batches = (n_units * (S_pad / kTileRows) * parts) / (2 * sms);
+        const int max_batches = static_cast<int>(static_cast<long long>(n_units) * (S_pad / kTileRows) * (deal.halves ? 2 : 1) / (2 * sms));
         if (n_batches > max_batches) n_batches = max_batches;
         if (n_batches < 1) n_batches = 1;
         prm.units_per_batch = (n_units + n_batches - 1) / n_batches;
-        if (parts > 1) {
-            if (prm.units_per_batch > 0xFFFF || parts > 0xFF || hpi > 0x7F) {
-                set_last_error("lt_attn_bwd", "shape too large for the split-group variant");
-                return LT_ERR_UNSUPPORTED;
-            }
-            prm.units_per_batch |= (parts << 16) | (hpi << 24);
-            prm.dK = reinterpret_cast<__half *>(dk_acc);
-            prm.dV = reinterpret_cast<__half *>(dv_acc);
-        }
     }
+    prm.deal = deal;
+    prm.shares = reinterpret_cast<float4 *>(ws + base_bytes);
     const size_t smem = sizeof(BwdSmem<D>);
-    auto main_kernel = parts > 1 ? bwd_main_kernel<D, kBf16, true> : bwd_main_kernel<D, kBf16, false>;
+    auto main_kernel = split ? bwd_main_kernel<D, kBf16, true> : bwd_main_kernel<D, kBf16, false>;
     if constexpr (!kBf16)
         if (saved_p) main_kernel = bwd_main_kernel<D, false, false, true>;
     if (one_tile) main_kernel = bwd_main_kernel<D, kBf16, false, false, true>;
     e = cudaFuncSetAttribute(main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(bwd_main)", e);
-    const int n_items = B * Hkv * (S_pad / kTileRows) * parts;
+    const int n_items = deal.ctas > 0 ? deal.ctas : B * Hkv * (S_pad / kTileRows) * (deal.halves ? 2 : 1);
     const int grid = n_items < sms ? n_items : sms;  // persistent: one CTA per SM walks the item list
     if (ev_main_begin && (e = cudaEventRecord(ev_main_begin, stream)) != cudaSuccess)
         return record_cuda_error("cudaEventRecord", e);
@@ -1594,22 +1706,20 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     cfg_fin.stream = stream;
     cfg_fin.attrs = &pdl;
     cfg_fin.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg_fin, bwd_finalize_kernel<kBf16>, static_cast<const float *>(dq_acc),
-                           reinterpret_cast<__half *>(dQ), n_vec8, S * (D / 8), S_pad * (D / 8), D / 8, Hq, lay.dq,
-                           plain_fin, parts > 1 ? 1 : 0);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return record_cuda_error("bwd_finalize_kernel launch", e);
-    if (parts > 1) {
-        const long long kv_vec8 = static_cast<long long>(B) * Hkv * S * D / 8;
-        const long long kwant = (2 * kv_vec8 + 255) / 256;
-        cfg_fin.gridDim = dim3(static_cast<int>(kwant < static_cast<long long>(sms) * 16 ? kwant : sms * 16));
-        e = cudaLaunchKernelEx(&cfg_fin, bwd_finalize_kv_kernel<kBf16>, static_cast<const float *>(dk_acc),
-                               static_cast<const float *>(dv_acc), reinterpret_cast<__half *>(dK),
-                               reinterpret_cast<__half *>(dV), kv_vec8, S * (D / 8), S_pad * (D / 8), D / 8, Hkv, lay.dk,
+    if (split) {
+        cfg_fin.gridDim = dim3(deal.n_shares() / 2, 2 * (D / 32));
+        e = cudaLaunchKernelEx(&cfg_fin, bwd_shares_kernel<D, kBf16>, static_cast<const float4 *>(prm.shares),
+                               reinterpret_cast<__half *>(dK), reinterpret_cast<__half *>(dV), deal, Hkv, S, lay.dk,
                                lay.dv);
         if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return record_cuda_error("bwd_finalize_kv_kernel launch", e);
+        if (e != cudaSuccess) return record_cuda_error("bwd_shares_kernel launch", e);
+        cfg_fin.gridDim = dim3(fin_blocks);
     }
+    e = cudaLaunchKernelEx(&cfg_fin, bwd_finalize_kernel<kBf16>, static_cast<const float *>(dq_acc),
+                           reinterpret_cast<__half *>(dQ), n_vec8, S * (D / 8), S_pad * (D / 8), D / 8, Hq, lay.dq,
+                           plain_fin, split ? 1 : 0);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return record_cuda_error("bwd_finalize_kernel launch", e);
     return LT_OK;
 }
 
@@ -1626,9 +1736,10 @@ static size_t bwd_base_bytes(int B, int Hq, int S, int D) {
 size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D) {
     if (lt::check_shape(B, Hq, Hkv, S, D, 1.0f) != LT_OK) return 0;
     size_t bytes = bwd_base_bytes(B, Hq, S, D);
-    // fp32 dK / dV sums for shapes whose groups are split over work items (under either mask)
-    if (lt::heads_per_item(B, Hq, Hkv, S, D, 1) < Hq / Hkv || lt::heads_per_item(B, Hq, Hkv, S, D, 0) < Hq / Hkv)
-        bytes += 2 * lt::round256(static_cast<size_t>(B) * Hkv * static_cast<size_t>(lt::padded_rows(S)) * D * 4);
+    // fp32 shares of dK and dV for shapes whose tile pairs are dealt out (under either mask)
+    const size_t masked = lt::share_bytes(lt::deal_pairs(B, Hq, Hkv, S, D, 1), D);
+    const size_t full = lt::share_bytes(lt::deal_pairs(B, Hq, Hkv, S, D, 0), D);
+    bytes += masked > full ? masked : full;
     return bytes;
 }
 
@@ -1636,7 +1747,7 @@ int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal) {
     if (lt::check_shape(B, Hq, Hkv, S, D, 1.0f) != LT_OK) return 0;
     // preprocess, main, dQ conversion; plus the dK/dV conversion when groups are split over work items; sequences of one
     // tile need fewer
-    if (lt::heads_per_item(B, Hq, Hkv, S, D, causal) < Hq / Hkv) return 4;
+    if (lt::deal_pairs(B, Hq, Hkv, S, D, causal).any()) return 4;
     const int tile_launches = lt::one_tile_launches(B, Hq, Hkv, S, D);
     return tile_launches > 0 ? tile_launches : 3;
 }
@@ -1645,7 +1756,7 @@ static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const
                      const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout *layout, int B,
                      int Hq, int Hkv, int S, int D, int causal, float scale, void *workspace, size_t workspace_bytes,
                      lt_stream_t stream, lt_event_t main_begin, lt_event_t main_end, bool bf16 = false, bool fit = false) {
-    // fit: where the workspace holds no fp32 dK/dV sums, run with whole groups
+    // fit: where the workspace has no room for the shares of dK and dV, run with whole key tiles
     using namespace lt;
     if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
@@ -1656,22 +1767,22 @@ static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const
     for (const void *ptr : ptrs)
         if (!aligned16(ptr)) return LT_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(LSE) & 3u) != 0) return LT_ERR_UNSUPPORTED;  // fp32, read one at a time
-    const bool may_split = workspace_bytes >= lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
-    if (!workspace || !aligned256(workspace) || (!may_split && !(fit && workspace_bytes >= bwd_base_bytes(B, Hq, S, D))))
+    const size_t needed = fit ? bwd_base_bytes(B, Hq, S, D) : lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
+    if (!workspace || !aligned256(workspace) || workspace_bytes < needed)
         return LT_ERR_WORKSPACE;
     if ((rc = check_device()) != LT_OK) return rc;
     if (bf16) {
         if (D == 64)
             return launch_bwd<64, true>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                        stream, main_begin, main_end, may_split);
+                                        workspace_bytes, stream, main_begin, main_end);
         return launch_bwd<128, true>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     stream, main_begin, main_end, may_split);
+                                     workspace_bytes, stream, main_begin, main_end);
     }
     if (D == 64)
         return launch_bwd<64, false>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     stream, main_begin, main_end, may_split);
+                                     workspace_bytes, stream, main_begin, main_end);
     return launch_bwd<128, false>(Q, K, V, O, dO, LSE, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                  stream, main_begin, main_end, may_split);
+                                  workspace_bytes, stream, main_begin, main_end);
 }
 
 int lt_attn_bwd_saved_p(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
@@ -1691,9 +1802,9 @@ int lt_attn_bwd_saved_p(const lt_half *Q, const lt_half *K, const lt_half *V, co
     const lt_attn_layout lay = contiguous_layout(Hq, Hkv, S, D);
     if (D == 64)
         return launch_bwd<64, false>(Q, K, V, O, dO, nullptr, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                     static_cast<cudaStream_t>(stream), nullptr, nullptr, false, P);
+                                     workspace_bytes, static_cast<cudaStream_t>(stream), nullptr, nullptr, P);
     return launch_bwd<128, false>(Q, K, V, O, dO, nullptr, dQ, dK, dV, lay, B, Hq, Hkv, S, causal, scale, workspace,
-                                  static_cast<cudaStream_t>(stream), nullptr, nullptr, false, P);
+                                  workspace_bytes, static_cast<cudaStream_t>(stream), nullptr, nullptr, P);
 }
 
 int lt_attn_bwd_profiled(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,

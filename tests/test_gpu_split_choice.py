@@ -1,6 +1,7 @@
-"""Groups of query heads split over work items on small problems: one tile and several, parts of unequal size, as many
-parts as heads, both head dimensions, types and masks, against the oracle; and the entry points that run with whole
-groups because their scratch has no room for the split groups' fp32 sums."""
+"""Key tiles split over several CTAs: dealt out (one tile and several, one query head per key/value head and many, stretches
+of a single pair, tiles of many parts, both head dimensions, types and masks) and in halves, against the oracle; dK and dV
+the same from run to run; and the entry points that run with whole key tiles because their scratch has no room for the fp32
+shares."""
 import pytest
 import torch
 
@@ -21,9 +22,11 @@ def _forward(lt, cfg, dt=torch.float16):
 
 @pytest.mark.parametrize("B,Hq,Hkv,S,D,causal,launches", [
     (1, 8, 1, 64, 64, True, 4), (1, 64, 8, 128, 128, True, 4), (2, 8, 1, 200, 64, False, 4), (1, 10, 2, 500, 128, False, 4),
-    (1, 5, 1, 129, 128, True, 4), (1, 20, 4, 640, 128, True, 4),   # five heads: parts of unequal size
+    (1, 5, 1, 129, 128, True, 4), (1, 20, 4, 640, 128, True, 4),   # five heads: tiles cut at unequal places
     (4, 8, 1, 300, 64, True, 4),
-    (1, 4, 2, 256, 64, True, 3), (2, 8, 4, 256, 128, False, 3),    # short groups stay whole
+    (1, 1, 1, 407, 128, True, 4), (1, 2, 2, 1000, 128, False, 4), (3, 2, 2, 1500, 64, True, 4),  # one head per kv head
+    (1, 4, 2, 256, 64, True, 4), (2, 8, 4, 256, 128, False, 4),    # stretches of one or two pairs
+    (1, 4, 4, 144, 64, True, 3), (2, 8, 8, 384, 128, False, 3),    # short walks stay whole
 ])
 @pytest.mark.parametrize("dtype", ["fp16", "bf16"])
 def test_split_on_small_problems(oracle, B, Hq, Hkv, S, D, causal, launches, dtype):
@@ -37,12 +40,38 @@ def test_split_on_small_problems(oracle, B, Hq, Hkv, S, D, causal, launches, dty
         ws[:256].fill_(0xFF)
         bwd(*ins, *outs, causal, cfg.scale, ws)
         bwd(*ins, *outs, causal, cfg.scale, ws)
+        again = [t.clone() for t in outs[1:]]
+        bwd(*ins, *outs, causal, cfg.scale, ws)
+        assert all(torch.equal(x, y) for x, y in zip(again, outs[1:])), "dK, dV differ between runs"
     assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
     ref = oracle.attn_bwd(*(t.double().numpy() for t in host), causal, cfg.scale)
     check_grads(outs, ref, f"split {cfg}", dtype=dtype, absolute=False)
 
 
-def test_noalloc_without_room_for_the_sums(oracle):
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_halves(oracle, dtype):
+    # 256 key tiles of up to 256 pairs on a working set of 1.1 GB: too few for batches, so each is two items
+    from paper_2606_10415_b200 import binding as lt
+    B, Hq, Hkv, S, D = 32, 32, 1, 900, 128
+    assert lt.lt_attn_bwd_num_launches(B, Hq, Hkv, S, D, True) == 4
+    dt, scale = torch.float16 if dtype == "fp16" else torch.bfloat16, D ** -0.5
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    Q, K, V, dO = (torch.randn((B, h, S, D), generator=gen, device="cuda").to(dt) for h in (Hq, Hkv, Hkv, Hq))
+    O, LSE = torch.empty_like(Q), torch.empty((B, Hq, S), dtype=torch.float32, device="cuda")
+    fwd, bwd = (lt.lt_attn_fwd, lt.lt_attn_bwd) if dtype == "fp16" else (lt.lt_attn_fwd_bf16, lt.lt_attn_bwd_bf16)
+    fwd(Q, K, V, O, LSE, True, scale, lt.alloc_workspace(256))
+    outs = [torch.full_like(t, float("nan")) for t in (Q, K, V)]
+    ws = lt.alloc_workspace(lt.lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D))
+    ws.fill_(0xFF)
+    bwd(Q, K, V, O, dO, LSE, *outs, True, scale, ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    assert all(torch.isfinite(t).all() for t in outs)
+    for b in (0, 13, 31):
+        ref = oracle.attn_bwd(*(t[b:b + 1].cpu().double().numpy() for t in (Q, K, V, dO)), True, scale)
+        check_grads([t[b:b + 1] for t in outs], ref, f"halves, batch {b}", dtype=dtype, absolute=False)
+
+
+def test_noalloc_without_room_for_the_shares(oracle):
     from paper_2606_10415_b200 import binding as lt
     cfg = workloads.custom(1, 8, 1, 4096, 128, True, seed=5)
     dims = (cfg.B, cfg.Hq, cfg.Hkv, cfg.S, cfg.D)
@@ -51,4 +80,4 @@ def test_noalloc_without_room_for_the_sums(oracle):
     lt.lt_attn_bwd_noalloc(*ins, *outs, cfg.causal, cfg.scale)
     assert lt.lt_attn_bwd_noalloc_check_status() == lt.LT_OK
     ref = oracle.attn_bwd(*(t.double().numpy() for t in host), cfg.causal, cfg.scale)
-    check_grads(outs, ref, "noalloc, whole groups")
+    check_grads(outs, ref, "noalloc, whole key tiles")
