@@ -601,7 +601,7 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
 }
 
 // Internal streams and events of the host-buffer entry point, created on first use per device.
-constexpr int kHostMaxChunks = 10, kHostMaxDevices = 64;
+constexpr int kHostMaxChunks = 6, kHostMaxDevices = 64;
 struct HostPipe {
     bool ready = false;
     cudaStream_t s_in = nullptr, s_out = nullptr;
@@ -716,23 +716,25 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
     const int n_units = B * Hkv;
     const long long n_tiles = padded_rows(S) / 128;
     const long long unit_iters = static_cast<long long>(G) * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
-    // Few chunks where a chunk's kernels are long however small it is (its longest work item is a serial walk of a group's
-    // tile pairs, about 2.1 us each) or copies would get small (beside copies in the other direction one of 3 MB costs
-    // 15 us on top of its bytes); otherwise ten, the first small, because the copies back are the longer queue and start
-    // with it, the last ones smaller still, because their kernels and copies back are what is left when the input copy
-    // ends.  Measured with O returned, ms, four / ten chunks: LLaMA-2-7B layer 3.74 / 3.54, 4 x 16 heads at S = 1024
-    // unmasked 1.97 / 1.94, Qwen2.5-32B layer (8 units) 2.98 / 3.81, 16 / 4 heads twice at S = 2048, D = 64 0.78 / 1.22.
+    // The copies in one direction take as long as those in the other, so chunks of equal size keep both copy engines busy:
+    // a chunk's results go back while the next one comes in.  More chunks leave less to do before the first and after the
+    // last, and pay more for copies that get small (beside copies in the other direction one of 3 MB costs 15 us on top
+    // of its bytes).  Six, where the kernels of one take little of its copies' time; four, the last ones smaller, where
+    // they take more of it or units are few.  Measured with O returned, ms, four / six / ten chunks (six beside ten in one
+    // comparison, four in both): LLaMA-2-7B layer 3.68 / 3.47 / 3.64; 24 heads of 3 000 2.16 / 1.94 / 1.98; 4 x 16 heads at
+    // S = 1024 unmasked 1.95 / 1.87 / 1.96; Qwen2.5-32B layer (8 units) 2.77 / 2.82 / 3.09; 8 x 8 heads at S = 2048
+    // unmasked 3.67 / 3.85 / 3.56; six of exactly a sixth, or five, seven, eight equal ones are 1-3 % behind on average.
     int bounds[kHostMaxChunks + 1];
     int n_chunks = 1;
     bounds[0] = 0;
     bounds[1] = n_units;
     if (unit_iters * n_units >= 3000 && n_units > 1) {  // otherwise not worth the extra streams
-        constexpr int kFew[4] = {30, 60, 85, 100}, kMany[10] = {6, 18, 30, 42, 54, 66, 78, 88, 95, 100};  // cumulative shares, %
+        constexpr int kFew[4] = {30, 60, 85, 100}, kMany[6] = {17, 34, 51, 68, 85, 100};  // cumulative shares, %
         const double copy_us = static_cast<double>(2 * bq + 2 * bk) / 48.0e3;  // at 48 GB/s
         const double chunk_us = 2.1 * G * n_tiles + 1.9 * n_tiles + 20.0;      // a small chunk's backward, forward, launches
         const bool many = n_units >= 20 && copy_us > 15.0 * chunk_us;
         const int *percent = many ? kMany : kFew;
-        const int np = many ? 10 : 4;
+        const int np = many ? 6 : 4;
         n_chunks = 0;
         for (int c = 0; c < np; ++c) {
             const int end = c == np - 1 ? n_units : (n_units * percent[c] + 50) / 100;

@@ -1,4 +1,4 @@
-"""The host-buffer call cut into many chunks (ten where copies outlast a chunk's kernels): every unit of every chunk
+"""The host-buffer call cut into many chunks (six where copies outlast a chunk's kernels): every unit of every chunk
 against the device entry points on the whole problem, with and without the optional outputs, calls back to back."""
 import pytest
 import torch
