@@ -395,8 +395,8 @@ def run_ours(args, cfg):
     if lt.lt_attn_check_status(ws) != lt.LT_OK:
         raise SystemExit("backward kernel reported: " + lt.last_cuda_error())
     main_ms = [a.elapsed_time(b) for _, a, b, _ in kernel_events]
-    # what runs before the main kernel (status clear + preprocess kernel) and after it (dQ conversion, and the
-    # dK/dV conversion on split-group shapes), from the same profiled calls
+    # what runs before the main kernel (preprocess kernel) and after it (dQ conversion, and the
+    # dK/dV shares where key tiles are split), from the same profiled calls
     pre_ms = [c0.elapsed_time(a) for c0, a, _, _ in kernel_events]
     post_ms = [b.elapsed_time(c1) for _, _, b, c1 in kernel_events]
 
@@ -518,7 +518,7 @@ def run_ours(args, cfg):
                          "other_kernels": {"preprocess_ms": sum(pre_ms) / len(pre_ms),
                                            "finalize_ms": sum(post_ms) / len(post_ms),
                                            "how": "CUDA events around the profiled calls: call begin to main "
-                                                  "kernel begin (status clear + preprocess kernel), main kernel "
+                                                  "kernel begin (preprocess kernel), main kernel "
                                                   "end to call end (conversion kernels); with the events in "
                                                   "place the kernels do not overlap, so the three add up to a "
                                                   "little more than ms_per_step"},
