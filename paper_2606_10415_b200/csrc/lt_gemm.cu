@@ -42,6 +42,7 @@ struct GemmParams {
     unsigned int *status;
     int M, N, K;
     int tiles_m, tiles_n;
+    uint32_t a_bytes;  // a block of A's rows as it is brought into shared memory
     int group_rows;  // tile rows of A kept hot in L2 while the W column blocks stream past them
 };
 
@@ -135,7 +136,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                     const uint32_t use = kb_total / kGemmStages;
                     if (use >= 1 && !(ok = mbar_wait(&sm.bar_empty[s], (use - 1) & 1, abort_flag, p.status, kWaitGemmEmpty)))
                         break;
-                    mbar_arrive_expect_tx(&sm.bar_full[s], kGemmABytes + kGemmBBytes);
+                    mbar_arrive_expect_tx(&sm.bar_full[s], p.a_bytes + kGemmBBytes);
                     tma_load_2d(sm.a[s], &map_a, &sm.bar_full[s], kb * kGemmBK, tm * kGemmBM);
                     tma_load_2d(sm.b[s], &map_b, &sm.bar_full[s], kb * kGemmBK, tn * kGemmBN);
                 }
@@ -498,7 +499,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                 const int s = i % kStages;
                 const uint32_t use = i / kStages;
                 if (use >= 1 && !(ok = mbar_wait(&sm.bar_empty[s], (use - 1) & 1, abort_flag, p.status, kWaitGemmEmpty))) break;
-                mbar_arrive_expect_tx(&sm.bar_full[s], kGemmABytes + Smem::kBBytes);
+                mbar_arrive_expect_tx(&sm.bar_full[s], p.a_bytes + Smem::kBBytes);
                 tma_load_2d(sm.ring.b[s], &map_b, &sm.bar_full[s], (kb0 + i) * kGemmBK, tn * kBN);
                 tma_load_2d(sm.ring.a[s], &map_a, &sm.bar_full[s], (kb0 + i) * kGemmBK, tm * kGemmBM);
             }
@@ -688,11 +689,19 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
     prm.C = reinterpret_cast<__half *>(C);
     prm.status = reinterpret_cast<unsigned int *>(workspace);
     prm.M = M; prm.N = N; prm.K = K;
+    // A of up to 64 rows: only those are brought in (whole swizzle atoms of eight), not a box of 128 whose other rows the
+    // copy fills with zeros.  The products read whatever lies behind them in shared memory, and write it to accumulator
+    // rows that nobody stores.  Measured, us, box of 128 / of the rows: 1 x 4096 x 4096 (M x N x K) 11.6 / 9.8, 12 rows
+    // 12.9 / 10.8, 40 rows 11.8 / 11.7; 1 x 11008 x 4096 21.8 / 19.1; 1 x 2048 x 8192 15.2 / 12.1; 24 x 1024 x 1024 6.3 /
+    // 5.9; 8 x 32768 x 512 9.3 / 7.9.  On the other side of the line nothing is gained: 77 x 4096 x 4096 12.7 / 12.8,
+    // 100 rows 13.9 / 14.1, 100 x 32768 x 512 10.3 / 10.5.
+    const uint32_t a_rows = M <= 64 ? (M + 7) / 8 * 8 : kGemmBM;
+    prm.a_bytes = a_rows * kGemmBK * 2;
 
     const GemmPlan plan = force_single ? GemmPlan{kGemmBN, 1, false} : gemm_plan(M, N, K);
     const bool use_pair = plan.pair;
     CUtensorMap ma, mb;
-    if ((rc = make_tile_map(&ma, A, M, K, kGemmBM)) != LT_OK) return rc;
+    if ((rc = make_tile_map(&ma, A, M, K, a_rows)) != LT_OK) return rc;
     if ((rc = make_tile_map(&mb, W, N, K, use_pair ? 128 : plan.bn)) != LT_OK) return rc;
     if (!use_pair && plan.bn == 64)
         return bf16 ? launch_gemm_split<64, true>(ma, mb, prm, plan.split, stream)

@@ -86,6 +86,30 @@ def test_gemm_few_tiles(lt, M, N, K, dtype):
     assert torch.isnan(C[M]).all()
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (1, 4096, 1024), (7, 512, 4096), (8, 1024, 1024), (9, 72, 72), (33, 2048, 2048), (57, 11008, 512), (64, 4096, 1024),
+    (65, 4096, 1024), (5, 40960, 256), (64, 40000, 128),  # the last two: several tiles per CTA
+])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_gemm_few_rows(lt, M, N, K, dtype):
+    """Few rows of A: the rest of a tile's operand rows are whatever shared memory holds, here NaN from the call before."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(M + N + K)
+    A = torch.randn((M, K), generator=gen, device="cuda").to(dtype)
+    W = (torch.randn((N, K), generator=gen, device="cuda") * K ** -0.5).to(dtype)
+    C = torch.full((M + 1, N), float("nan"), dtype=dtype, device="cuda")  # the row past the end must stay untouched
+    ws = lt.alloc_workspace(lt.lt_gemm_f16_workspace_bytes())
+    full = torch.full((128, K), float("nan"), dtype=dtype, device="cuda")
+    lt.lt_gemm_f16(full, W, torch.empty((128, N), dtype=dtype, device="cuda"), ws)
+    lt.lt_gemm_f16(A, W, C[:M], ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    ref = A.double() @ W.double().T
+    err = (C[:M].double() - ref).abs()
+    half_ulp = 2.0 ** -11 if dtype == torch.float16 else 2.0 ** -8  # (the bound of test_gemm_few_tiles)
+    assert (err <= half_ulp * ref.abs() + 8 * K ** 0.5 * 2.0 ** -24 + 2.0 ** -24).all(), float(err.max())
+    assert torch.isnan(C[M]).all()
+
+
 def test_gemm_integer_operands_are_exact(lt, oracle):
     """Small integers: every product and partial sum is exact in fp32 and fp16, so the result must
     equal the oracle bit for bit."""
