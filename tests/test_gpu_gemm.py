@@ -110,6 +110,56 @@ def test_gemm_few_rows(lt, M, N, K, dtype):
     assert torch.isnan(C[M]).all()
 
 
+@pytest.mark.parametrize("M,N", [(77, 512), (256, 640), (600, 2048), (40, 24000)])
+def test_gemm_back_to_back(lt, M, N):
+    """Each product reads what the one before wrote and overwrites what that one read: calls in a row, whose kernels start
+    under each other's tails, give what calls with a synchronisation between them give."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(M)
+    W = (torch.randn((N, 256), generator=gen, device="cuda") / 16).half()
+    Wt = (torch.randn((256, N), generator=gen, device="cuda") * N ** -0.5).half()
+    X0 = torch.randn((M, 256), generator=gen, device="cuda").half()
+    ws = lt.alloc_workspace(lt.lt_gemm_f16_workspace_bytes())
+    results = []
+    for sync in (True, False):
+        X, Y = X0.clone(), torch.empty((M, N), dtype=torch.float16, device="cuda")
+        torch.cuda.synchronize()
+        for _ in range(12):
+            lt.lt_gemm_f16(X, W, Y, ws)
+            if sync:
+                torch.cuda.synchronize()
+            lt.lt_gemm_f16(Y, Wt, X, ws)
+            if sync:
+                torch.cuda.synchronize()
+        results.append(X)
+    assert torch.isfinite(results[0]).all() and torch.equal(*results)
+
+
+def test_gemm_before_attention(lt):
+    """Attention calls behind the products that make their operands, with nothing between them, and a product behind them."""
+    S, D = 384, 64
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    X, W = (torch.randn(shape, generator=gen, device="cuda").half() for shape in ((S, 256), (4, D, 256)))
+    W /= 16
+    ws = lt.alloc_workspace(lt.lt_attn_bwd_workspace_bytes(1, 1, 1, S, D))
+    results = []
+    for sync in (True, False):
+        Q, K, V, dO, O, dQ, dK, dV = (torch.full((1, 1, S, D), float("nan"), dtype=torch.float16, device="cuda") for _ in range(8))
+        LSE, Y = torch.empty((1, 1, S), device="cuda"), torch.empty((S, 256), dtype=torch.float16, device="cuda")
+        calls = [lambda t=t, w=w: lt.lt_gemm_f16(X, w, t[0, 0], ws) for t, w in zip((Q, K, V, dO), W)]
+        calls += [lambda: lt.lt_attn_fwd(Q, K, V, O, LSE, True, 0.125, ws),
+                  lambda: lt.lt_attn_bwd(Q, K, V, O, dO, LSE, dQ, dK, dV, True, 0.125, ws),
+                  lambda: lt.lt_gemm_f16(dV[0, 0], W[0].T.contiguous(), Y, ws)]
+        torch.cuda.synchronize()
+        for call in calls:
+            call()
+            if sync:
+                torch.cuda.synchronize()
+        results.append((O, LSE, dK, dV, Y))
+    assert all(torch.isfinite(a).all() and torch.equal(a, b) for a, b in zip(*results))
+
+
 def test_gemm_integer_operands_are_exact(lt, oracle):
     """Small integers: every product and partial sum is exact in fp32 and fp16, so the result must
     equal the oracle bit for bit."""
