@@ -124,7 +124,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     grid_dependency_wait();
     // The next kernel of the stream may be scheduled as this one's CTAs exit and set itself up (it waits for the whole grid
     // before it touches memory); all CTAs of this grid are running by then, so none is kept out.  Measured, us per call in
-    // a loop, without / with: 16 x 1024 x 1024 (M x N x K) 5.8 / 4.8, 77 x 4096 x 4096 12.9 / 11.9, 300 x 1000 x 1000 8.1 /
+    // a graph of calls, without / with: 16 x 1024 x 1024 (M x N x K) 5.8 / 4.8, 77 x 4096 x 4096 12.9 / 11.9, 300 x 1000 x 1000 8.1 /
     // 7.0, 512 x 4096 x 4096 24.2 / 22.4, 2048 x 11008 x 4096 159 / 156, 8192 x 1024 x 512 13.2 / 12.9.
     grid_launch_dependents();
     if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
