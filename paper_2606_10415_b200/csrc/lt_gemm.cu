@@ -651,6 +651,11 @@ static GemmPlan gemm_plan(int M, int N, int K) {
     const double k_blocks = static_cast<double>(ceil_div(K, kGemmBK));
     GemmPlan best{kGemmBN, 1, false};
     double best_us = 4.4 + ceil_div(ceil_div(M, kGemmBM) * ceil_div(N, kGemmBN), 148) * k_blocks * 0.357;
+    // A short contraction does not hide the fill and the 256-wide drain, which take this much by themselves.  Measured, us,
+    // without this line (256-wide) / with it (64- or 128-wide): 150 x 1408 x 152 8.3 / 5.0, 404 x 1152 x 272 8.1 / 5.3, 266 x
+    // 685 x 224 14.2 / 7.2; 150 drawn shapes 1.05x, none slower.  Longer contractions on one wave are right at 256:
+    // 700 x 2048 x 1024 9.7 against 10.3.
+    if (best_us < 7.2) best_us = 7.2;
     auto offer = [&](GemmPlan plan, double us) {
         if (us < best_us) best = plan, best_us = us;
     };

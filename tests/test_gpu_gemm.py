@@ -61,6 +61,7 @@ def test_gemm_matches_oracle(lt, oracle, M, N, K):
     (3, 130, 8192), (128, 128, 4096),              # eight shares
     (424, 265, 5920), (300, 127, 2056),            # several tile rows, N odd (scalar stores) and just below a tile
     (130, 2048, 2048), (16, 5504, 4096), (40, 6000, 2000),  # 128- and 256-wide tiles, two to six shares
+    (150, 1408, 152), (404, 1152, 272), (266, 685, 224), (129, 600, 456),  # short contractions on several tile rows
     (1000, 2040, 4096), (600, 600, 600), (8192, 72, 136),   # more tiles than fit at once, short contractions
     (700, 2047, 136), (260, 2046, 136), (129, 2008, 64),    # 256-wide tiles whose edge is odd, even, in eights
     (2000, 3999, 2048), (2048, 3998, 2048), (1900, 4040, 2048),  # the same on CTA pairs
