@@ -9,6 +9,7 @@
 // pair while the other tile's scores are exponentiated.  S/P and O live in tensor memory.
 // The running row maximum is only raised when it grew by more than 2^8 since the output
 // was last rescaled, so most key tiles need no pass over O.
+#include <float.h>
 #include <math.h>
 
 #include <algorithm>
@@ -418,7 +419,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                 }
                 LT_FT(4);
                 // P = exp2(score - m_used) as fp16 over the first 64 columns of the S region
-                const float neg_m = -m_used;
+                // (split keys: a chain may begin with a tile whose scores are all -inf, keys hidden by -inf in K; such a tile
+                // gets zeros here, as it does where a tile with a finite maximum came before it)
+                const float neg_m = kSplitKeys ? fminf(-m_used, FLT_MAX) : -m_used;
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
 #pragma unroll

@@ -38,3 +38,33 @@ def test_split_keys(H, Hkv, S, D, causal, dtype, scale_sign, ramp):
     assert (O.double() - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
     # LSE is fp32: one unit of its own size besides the flat gate
     assert ((LSE.double() - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
+
+
+@pytest.mark.parametrize("H,Hkv,S,D,hidden", [(1, 1, 256, 128, (1,)), (4, 2, 300, 64, (1,)), (2, 2, 640, 128, (1,)),
+                                              (2, 1, 640, 64, (1, 3)), (1, 1, 1100, 128, (1, 2, 3, 5, 7))])
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_hidden_key_tiles(H, Hkv, S, D, hidden, causal, dtype):
+    """Keys hidden by a channel of ones in Q against -inf in K: score -inf, weight zero, also where that is every key of the
+    tile a chain starts with, or of all its tiles."""
+    from paper_2606_10415_b200 import binding as lt
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(S + D)
+    Q, K, V = (torch.randn((1, h, S, D), generator=gen, device="cuda").to(dtype) for h in (H, Hkv, Hkv))
+    Q[..., 0] = 1.0
+    gone = torch.isin(torch.arange(S, device="cuda") // 128, torch.tensor(hidden, device="cuda"))
+    K[:, :, gone, 0] = float("-inf")
+    O, LSE = torch.full_like(Q, float("nan")), torch.full((1, H, S), float("nan"), device="cuda")
+    ws = lt.alloc_workspace(256)
+    fn = lt.lt_attn_fwd if dtype == torch.float16 else lt.lt_attn_fwd_bf16
+    fn(Q, K, V, O, LSE, causal, D ** -0.5, ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    k, v = (t.double().repeat_interleave(H // Hkv, 1) for t in (K, V))
+    s = Q.double() @ k.transpose(-1, -2) * D ** -0.5
+    if causal:
+        s.masked_fill_(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    ref = torch.exp(s - lse[..., None]) @ v
+    assert torch.isfinite(O).all()  # (the gates of test_split_keys)
+    assert (O.double() - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
+    assert ((LSE.double() - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
