@@ -9,7 +9,7 @@
 //                           P^T from LSE, and run the five tile contractions on
 //                           tcgen05 tensor cores with tensor-memory accumulators
 //   bwd_finalize_kernel   : dQ fp32 accumulator -> fp16
-// and, where key tiles are split over several CTAs, beside the last one
+// and, where key tiles are split over several CTAs, before the last one
 //   bwd_shares_kernel     : fp32 shares of dK and dV -> fp16
 // (Sequences of one tile: one or two launches, see one_tile_launches.)
 //
@@ -266,12 +266,10 @@ bwd_preprocess_kernel(const PreParams p, long long n_rows, long long v_rows, uns
 template <bool kBf16>
 __global__ void __launch_bounds__(256)
 bwd_finalize_kernel(const float *__restrict__ dq_acc, __half *__restrict__ dQ, long long n_vec8, int vec_per_head,
-                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain, int beside) {
+                    int vec_per_padded_head, int vec_per_row, int Hq, lt_tensor_strides dq_st, int plain) {
     // n_vec8 groups of eight output elements, numbered over the logical [B,Hq,S,D]; the accumulator
     // is indexed in the padded row space (`plain`: contiguous dQ and no padding, so both are group v)
-    // launched while the main kernel drains: its reductions must have landed (beside: this kernel runs beside the one that
-    // adds the shares of dK and dV, whose CTAs have all seen that)
-    if (!beside) grid_dependency_wait();
+    grid_dependency_wait();  // launched while its predecessor drains: the main kernel's reductions must have landed
     const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
     for (long long v = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; v < n_vec8; v += stride) {
         long long src = v, dst = v * 8;
@@ -292,7 +290,6 @@ bwd_finalize_kernel(const float *__restrict__ dq_acc, __half *__restrict__ dQ, l
         o.w = pack2<kBf16>(b.z, b.w);
         *reinterpret_cast<uint4 *>(dQ + dst) = o;
     }
-    if (beside) grid_dependency_wait();  // what follows this kernel may rely on dK and dV too
 }
 
 // Two ways to spread the tile pairs of one key tile over several CTAs.  Each leaves fp32 shares of dK_j and dV_j in the
@@ -342,7 +339,9 @@ struct BwdDeal {
 // dK_j and dV_j of the key tiles that were dealt out to several CTAs: the fp32 shares, added in the order of the walk,
 // as 16-bit outputs.  Block (c, 32 columns of dK or dV) has the tile that CTA c's stretch ends in, if it began there
 // or before; it does nothing where the stretch ends with a tile or another CTA's does the beginning.  In halves: key tile c.
-// Launched before the dQ conversion, which runs beside it: 2-3 us less per call than behind it.
+// The dQ conversion behind it is launched early and waits for all of it: that wait is also the one for the main kernel's
+// reductions.  Reading the accumulator under this kernel, on the strength of this kernel's own wait, saved 1-1.8 us per
+// call (16 query heads on 4, 777 rows, D = 64: 24.4 against 26.2), but nothing promises a grid what another one waited for.
 template <int D, bool kBf16>
 __global__ void __launch_bounds__(256)
 bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __half *__restrict__ dV, const BwdDeal deal,
@@ -366,8 +365,8 @@ bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __
                 for (parts = 1; upto < n; ++parts) upto = deal.cut(deal.stretch(c + parts + 1) - start, n);
         }
     }
-    grid_dependency_wait();    // launched while the main kernel drains: its shares must have landed
-    grid_launch_dependents();  // the dQ conversion runs beside this kernel
+    grid_launch_dependents();
+    grid_dependency_wait();  // launched while the main kernel drains: its shares must have landed
     if (parts == 0) return;
     constexpr int kShareVec = 128 * D / 4;  // float4s of dK or dV in a share
     const int row = threadIdx.x & 127;
@@ -1717,7 +1716,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     }
     e = cudaLaunchKernelEx(&cfg_fin, bwd_finalize_kernel<kBf16>, static_cast<const float *>(dq_acc),
                            reinterpret_cast<__half *>(dQ), n_vec8, S * (D / 8), S_pad * (D / 8), D / 8, Hq, lay.dq,
-                           plain_fin, split ? 1 : 0);
+                           plain_fin);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("bwd_finalize_kernel launch", e);
     return LT_OK;

@@ -48,6 +48,39 @@ def test_split_on_small_problems(oracle, B, Hq, Hkv, S, D, causal, launches, dty
     check_grads(outs, ref, f"split {cfg}", dtype=dtype, absolute=False)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(1, 8, 1, 300, 64, False), (1, 40, 8, 1024, 128, True), (1, 2, 2, 1000, 64, True),
+                                                 (1, 2, 1, 3566, 128, True)])
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+def test_split_calls_on_changing_data(B, Hq, Hkv, S, D, causal, dtype):
+    """The kernels of a call start under one another's tails, and two calls share a workspace: what a call adds up and
+    converts has to be its own.  Two problems in turn without a synchronisation, each call into outputs of its own, against the
+    same calls made alone on a workspace full of NaN."""
+    from paper_2606_10415_b200 import binding as lt
+    dt = torch.float16 if dtype == "fp16" else torch.bfloat16
+    bwd = lt.lt_attn_bwd if dtype == "fp16" else lt.lt_attn_bwd_bf16
+    assert lt.lt_attn_bwd_num_launches(B, Hq, Hkv, S, D, causal) == 4
+    scale = D ** -0.5
+    problems = [_forward(lt, workloads.custom(B, Hq, Hkv, S, D, causal, seed=seed), dt)[1:] for seed in (1, 2)]
+    ws = lt.alloc_workspace(lt.lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D))
+    for ins, outs in problems:
+        ws.fill_(0xFF)
+        bwd(*ins, *outs, causal, scale, ws)
+        torch.cuda.synchronize()
+        assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+        assert all(torch.isfinite(t).all() for t in outs)
+    ws.fill_(0xFF)
+    calls = [(k, [torch.full_like(t, float("nan")) for t in problems[k][1]]) for k in (0, 1) * 6]
+    torch.cuda.synchronize()
+    for k, outs in calls:
+        bwd(*problems[k][0], *outs, causal, scale, ws)
+    assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+    for k, outs in calls:
+        want = problems[k][1]
+        assert torch.equal(outs[1], want[1]) and torch.equal(outs[2], want[2])
+        # dQ's fp32 partials arrive in any order, so a result may round to the other neighbour: 2^-11 (2^-8) of it
+        assert (outs[0].double() - want[0].double()).norm() <= (2.0 ** -11 if dtype == "fp16" else 2.0 ** -8) * want[0].double().norm()
+
+
 @pytest.mark.parametrize("dtype", ["fp16", "bf16"])
 def test_halves(oracle, dtype):
     # 256 key tiles of up to 256 pairs on a working set of 1.1 GB: too few for batches, so each is two items
