@@ -68,7 +68,9 @@ typedef unsigned short lt_bf16;
  * of fp16 (hi, lo, 0 x 6) with 256*hi + lo = value, [B,Hq,S_pad] rows each (every 64th or 128th -LSE/scale row may
  * carry partial maxima of the three quantities above in elements 4-6, which no product uses), an fp32 dQ accumulator
  * [B,Hq,S_pad,D], and, for shapes whose key tiles are split over work items (see lt_attn_bwd_num_launches), the items'
- * fp32 shares of dK and dV, 2 x 128 x D floats each: two per multiprocessor, or two per key tile. */
+ * fp32 shares of dK and dV, 2 x 128 x D floats each: two per multiprocessor, or two per key tile.  A workspace (or arena)
+ * without room for all shares, down to one that ends with the accumulator, is accepted by every backward call: key tiles
+ * are then shared by fewer CTAs, or stay whole, which is slower and changes the order in which dK and dV are summed. */
 size_t lt_attn_fwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);
 size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);
 
@@ -117,7 +119,7 @@ int lt_attn_bwd_profiled(const lt_half *Q, const lt_half *K, const lt_half *V,
  * GPU that loads the library holds until the process ends.  Inputs and outputs are still the
  * caller's device tensors, with the meaning and layout of lt_attn_bwd.
  *   - Shapes whose workspace exceeds the built-in scratch (roughly B*Hq*S*D above four million elements;
- *     the fp32 shares of dK and dV do not count, without room for them key tiles stay whole) return LT_ERR_WORKSPACE; lt_last_cuda_error()
+ *     the fp32 shares of dK and dV do not count) return LT_ERR_WORKSPACE; lt_last_cuda_error()
  *     then names both sizes.  Nothing is launched in that case.
  *   - The call allocates nothing: no cudaMalloc/cudaFree and no allocating library routine.
  *   - The first call on each device looks up the array's device address (one runtime query,
@@ -200,7 +202,7 @@ int lt_attn_bwd_bf16(const lt_bf16 *Q, const lt_bf16 *K, const lt_bf16 *V,
  * lt_attn_bwd_saved_p computes dQ, dK, dV as lt_attn_bwd does, with `P` (the store above, same shape
  * arguments and mask) in place of LSE: the main kernel issues no S = Q K^T product and no exponentials;
  * it reads each tile of P once (32 KB per tile pair, B*Hq*nT*(nT+1)/2 tile pairs under a causal mask).
- * Contiguous fp16 tensors only; workspace of lt_attn_bwd_workspace_bytes() bytes; three launches; status
+ * Contiguous fp16 tensors only; workspace as for lt_attn_bwd (no shares are used); three launches; status
  * and error behaviour as lt_attn_bwd.  P carries fp16 rounding (and flushes probabilities below 2^-24
  * to zero), which the recompute path does not, so its gradients are slightly less accurate. */
 size_t lt_attn_p_store_bytes(int B, int Hq, int Hkv, int S, int D);
@@ -233,7 +235,7 @@ int lt_gemm_bf16(const lt_bf16 *A, const lt_bf16 *W, lt_bf16 *C, int M, int N, i
 
 /* Same computation as lt_attn_fwd followed by lt_attn_bwd, but every tensor pointer is
  * a HOST pointer (pinned memory makes the copies asynchronous).  `arena` is a caller-
- * owned DEVICE buffer of at least lt_attn_host_arena_bytes() bytes, 256-byte aligned,
+ * owned DEVICE buffer of lt_attn_host_arena_bytes() bytes (less, as far as a smaller workspace allows), 256-byte aligned,
  * that holds the device copies and the workspace.  The call enqueues the host-to-device
  * copies of Q, K, V, dO, the two kernels' work and the device-to-host copies of
  * O, LSE, dQ, dK, dV on `stream`; the host outputs are valid once the stream is

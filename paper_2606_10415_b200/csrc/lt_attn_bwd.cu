@@ -1590,7 +1590,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     uint4 *delta_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes);
     uint4 *lse_ext = reinterpret_cast<uint4 *>(ws + kStatusBytes + ext_bytes);
     float *dq_acc = reinterpret_cast<float *>(ws + kStatusBytes + 2 * ext_bytes);
-    const size_t base_bytes = kStatusBytes + 2 * ext_bytes + round256(static_cast<size_t>(n_rows) * D * 4);
+    const size_t base_bytes = bwd_least_bytes(B, Hq, S, D);
     BwdDeal deal{};
     if (!saved_p) deal = deal_pairs(B, Hq, Hkv, S, D, causal, workspace_bytes - base_bytes);
     const bool split = deal.any();
@@ -1724,17 +1724,18 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
 
 }  // namespace lt
 
-extern "C" {
-
-// the status block, the -delta and -LSE/scale rows and the fp32 dQ accumulator
-static size_t bwd_base_bytes(int B, int Hq, int S, int D) {
-    const size_t n_rows = static_cast<size_t>(B) * Hq * static_cast<size_t>(lt::padded_rows(S));
-    return lt::kStatusBytes + 2 * lt::round256(n_rows * 16) + lt::round256(n_rows * D * 4);
+namespace lt {
+size_t bwd_least_bytes(int B, int Hq, int S, int D) {
+    const size_t n_rows = static_cast<size_t>(B) * Hq * static_cast<size_t>(padded_rows(S));
+    return kStatusBytes + 2 * round256(n_rows * 16) + round256(n_rows * D * 4);
 }
+}  // namespace lt
+
+extern "C" {
 
 size_t lt_attn_bwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D) {
     if (lt::check_shape(B, Hq, Hkv, S, D, 1.0f) != LT_OK) return 0;
-    size_t bytes = bwd_base_bytes(B, Hq, S, D);
+    size_t bytes = lt::bwd_least_bytes(B, Hq, S, D);
     // fp32 shares of dK and dV for shapes whose tile pairs are dealt out (under either mask)
     const size_t masked = lt::share_bytes(lt::deal_pairs(B, Hq, Hkv, S, D, 1), D);
     const size_t full = lt::share_bytes(lt::deal_pairs(B, Hq, Hkv, S, D, 0), D);
@@ -1754,8 +1755,7 @@ int lt_attn_bwd_num_launches(int B, int Hq, int Hkv, int S, int D, int causal) {
 static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO,
                      const float *LSE, lt_half *dQ, lt_half *dK, lt_half *dV, const lt_attn_layout *layout, int B,
                      int Hq, int Hkv, int S, int D, int causal, float scale, void *workspace, size_t workspace_bytes,
-                     lt_stream_t stream, lt_event_t main_begin, lt_event_t main_end, bool bf16 = false, bool fit = false) {
-    // fit: where the workspace has no room for the shares of dK and dV, run with whole key tiles
+                     lt_stream_t stream, lt_event_t main_begin, lt_event_t main_end, bool bf16 = false) {
     using namespace lt;
     if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
@@ -1766,8 +1766,7 @@ static int bwd_entry(const lt_half *Q, const lt_half *K, const lt_half *V, const
     for (const void *ptr : ptrs)
         if (!aligned16(ptr)) return LT_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(LSE) & 3u) != 0) return LT_ERR_UNSUPPORTED;  // fp32, read one at a time
-    const size_t needed = fit ? bwd_base_bytes(B, Hq, S, D) : lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
-    if (!workspace || !aligned256(workspace) || workspace_bytes < needed)
+    if (!workspace || !aligned256(workspace) || workspace_bytes < bwd_least_bytes(B, Hq, S, D))
         return LT_ERR_WORKSPACE;
     if ((rc = check_device()) != LT_OK) return rc;
     if (bf16) {
@@ -1795,7 +1794,7 @@ int lt_attn_bwd_saved_p(const lt_half *Q, const lt_half *K, const lt_half *V, co
     for (const void *ptr : ptrs)
         if (!aligned16(ptr)) return LT_ERR_UNSUPPORTED;
     if (!aligned256(P)) return LT_ERR_UNSUPPORTED;
-    if (!workspace || !aligned256(workspace) || workspace_bytes < lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D))
+    if (!workspace || !aligned256(workspace) || workspace_bytes < bwd_least_bytes(B, Hq, S, D))
         return LT_ERR_WORKSPACE;
     if ((rc = check_device()) != LT_OK) return rc;
     const lt_attn_layout lay = contiguous_layout(Hq, Hkv, S, D);
@@ -1839,15 +1838,6 @@ int lt_attn_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_h
 
 }  // extern "C"
 
-namespace lt {
-int bwd_in_any(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO, const float *LSE,
-               lt_half *dQ, lt_half *dK, lt_half *dV, int B, int Hq, int Hkv, int S, int D, int causal, float scale,
-               void *workspace, size_t workspace_bytes, lt_stream_t stream) {
-    return bwd_entry(Q, K, V, O, dO, LSE, dQ, dK, dV, nullptr, B, Hq, Hkv, S, D, causal, scale, workspace, workspace_bytes,
-                     stream, nullptr, nullptr, false, true);
-}
-}  // namespace lt
-
 // ----------------------------------------------------------------------------- backward without a caller workspace
 // Scratch for lt_attn_bwd_noalloc: lives in the library image, so every GPU that loads the
 // library carries these bytes until the process exits.  In host code the array's name is
@@ -1870,7 +1860,7 @@ int lt_attn_bwd_noalloc(const lt_half *Q, const lt_half *K, const lt_half *V, co
     if (!Q || !K || !V || !O || !dO || !LSE || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
     if (rc != LT_OK) return rc;
-    const size_t need = bwd_base_bytes(B, Hq, S, D);
+    const size_t need = bwd_least_bytes(B, Hq, S, D);
     if (need > kNoAllocScratchBytes) {
         char msg[160];
         snprintf(msg, sizeof(msg), "this shape needs %zu bytes of scratch but the built-in scratch holds %zu; "
@@ -1898,9 +1888,9 @@ int lt_attn_bwd_noalloc(const lt_half *Q, const lt_half *K, const lt_half *V, co
         }
         scratch = g_noalloc_scratch_addr[dev];
     }
-    // lt_attn_bwd clears the status block and its preprocess kernel zeroes the dQ accumulator on
-    // every call, so nothing left in the scratch by an earlier call is read
-    return bwd_in_any(Q, K, V, O, dO, LSE, dQ, dK, dV, B, Hq, Hkv, S, D, causal, scale, scratch, kNoAllocScratchBytes, stream);
+    // every call clears the status words and zeroes the dQ accumulator itself where it uses them, so nothing left in the
+    // scratch by an earlier call is read
+    return lt_attn_bwd(Q, K, V, O, dO, LSE, dQ, dK, dV, B, Hq, Hkv, S, D, causal, scale, scratch, kNoAllocScratchBytes, stream);
 }
 
 int lt_attn_bwd_noalloc_check_status(lt_stream_t stream) {

@@ -673,14 +673,18 @@ int lt_attn_fwd_bf16(const lt_bf16 *Q, const lt_bf16 *K, const lt_bf16 *V, lt_bf
                      true);
 }
 
-size_t lt_attn_host_arena_bytes(int B, int Hq, int Hkv, int S, int D) {
-    const size_t wb = lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
-    if (wb == 0) return 0;
+// the arena with `workspace_bytes` for the backward
+static size_t host_arena_bytes(int B, int Hq, int Hkv, int S, int D, size_t workspace_bytes) {
     const size_t nq = lt::round256(static_cast<size_t>(B) * Hq * S * D * 2);
     const size_t nk = lt::round256(static_cast<size_t>(B) * Hkv * S * D * 2);
     const size_t nl = lt::round256(static_cast<size_t>(B) * Hq * S * 4);
     // Q, dO, O, dQ | K, V, dK, dV | LSE | forward status block | backward workspace
-    return 4 * nq + 4 * nk + nl + lt::kStatusBytes + wb;
+    return 4 * nq + 4 * nk + nl + lt::kStatusBytes + workspace_bytes;
+}
+
+size_t lt_attn_host_arena_bytes(int B, int Hq, int Hkv, int S, int D) {
+    const size_t wb = lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D);
+    return wb == 0 ? 0 : host_arena_bytes(B, Hq, Hkv, S, D, wb);
 }
 
 int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *dO, lt_half *O,
@@ -690,7 +694,7 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
     if (!Q || !K || !V || !dO || !dQ || !dK || !dV) return LT_ERR_INVALID_ARG;
     int rc = check_shape(B, Hq, Hkv, S, D, scale);
     if (rc != LT_OK) return rc;
-    const size_t need = lt_attn_host_arena_bytes(B, Hq, Hkv, S, D);
+    const size_t need = host_arena_bytes(B, Hq, Hkv, S, D, bwd_least_bytes(B, Hq, S, D));
     if (!arena || !aligned256(arena) || arena_bytes < need) return LT_ERR_WORKSPACE;
     const size_t bq = static_cast<size_t>(B) * Hq * S * D * 2, bk = static_cast<size_t>(B) * Hkv * S * D * 2;
     const size_t bl = static_cast<size_t>(B) * Hq * S * 4;
@@ -803,7 +807,7 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
         }
         if (O) LT_CUDA(cudaMemcpyAsync(O + oq, d_O + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         if (LSE) LT_CUDA(cudaMemcpyAsync(LSE + ol, d_lse + ol, cl, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
-        rc = bwd_in_any(d_Q + oq, d_K + ok_, d_V + ok_, d_O + oq, d_dO + oq, d_lse + ol, d_dQ + oq, d_dK + ok_,
+        rc = lt_attn_bwd(d_Q + oq, d_K + ok_, d_V + ok_, d_O + oq, d_dO + oq, d_lse + ol, d_dQ + oq, d_dK + ok_,
                          d_dV + ok_, 1, hq, hkv, S, D, causal, scale, ws, ws_bytes, stream);
         if (rc != LT_OK) return rc;
         if (pipe) {

@@ -51,9 +51,8 @@ int check_layout(const lt_attn_layout &lay, int D);
 // sequence length rounded up to whole 128-row tiles
 inline long long padded_rows(int S) { return (static_cast<long long>(S) + 127) / 128 * 128; }
 
-// lt_attn_bwd in a workspace that need not hold the fp32 dK/dV sums of split groups (the groups then stay whole).
-int bwd_in_any(const lt_half *Q, const lt_half *K, const lt_half *V, const lt_half *O, const lt_half *dO, const float *LSE,
-               lt_half *dQ, lt_half *dK, lt_half *dV, int B, int Hq, int Hkv, int S, int D, int causal, float scale,
-               void *workspace, size_t workspace_bytes, lt_stream_t stream);
+// The least workspace of a backward call: the status block, the -delta and -LSE/scale rows and the fp32 dQ accumulator.
+// What lies behind them holds shares of dK and dV; with less room for those fewer CTAs share key tiles, or none.
+size_t bwd_least_bytes(int B, int Hq, int S, int D);
 
 }  // namespace lt

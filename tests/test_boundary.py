@@ -55,6 +55,36 @@ def test_workspace_sizes(binding):
     assert binding.lt_attn_host_arena_bytes(1, 2, 2, 128, 64) > binding.lt_attn_bwd_workspace_bytes(1, 2, 2, 128, 64)
 
 
+def _least_workspace(B, Hq, S, D):
+    rows = B * Hq * -(-S // 128) * 128
+    return 256 + 2 * rows * 16 + rows * D * 4
+
+
+# shapes whose key tiles are shared by several CTAs; the shares of dK and dV are room that a call can do without
+SHARED_KEY_TILES = [(1, 4, 4, 938, 128), (1, 2, 2, 1000, 64), (1, 40, 8, 2048, 128), (2, 64, 8, 4096, 128)]
+
+
+@pytest.mark.parametrize("dims", SHARED_KEY_TILES)
+def test_workspace_without_room_for_shares_is_accepted(binding, dims):
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("a device is present: the calls would be launched")
+    b = binding
+    B, Hq, Hkv, S, D = dims
+    least = _least_workspace(B, Hq, S, D)
+    assert b.lt_attn_bwd_workspace_bytes(*dims) > least
+    shape = dict(B=B, Hq=Hq, Hkv=Hkv, S=S, D=D)
+    past_the_check = (b.LT_ERR_CUDA, b.LT_ERR_UNSUPPORTED)  # no device here
+    assert b.lt_attn_bwd_raw(*_bwd_args(ws_bytes=least, **shape)) in past_the_check
+    assert b.lt_attn_bwd_raw(*_bwd_args(ws_bytes=least - 1, **shape)) == b.LT_ERR_WORKSPACE
+    lib = b._lib
+    saved = lambda n: lib.lt_attn_bwd_saved_p(*[0x1000] * 9, *dims, 1, 0.125, 0x10000, n, 0)
+    assert saved(least) in past_the_check and saved(least - 1) == b.LT_ERR_WORKSPACE
+    arena = b.lt_attn_host_arena_bytes(*dims) - b.lt_attn_bwd_workspace_bytes(*dims) + least
+    host = lambda n: lib.lt_attn_fwd_bwd_host(*[0x1000] * 9, *dims, 1, 0.125, 0x10000, n, 0)
+    assert host(arena) in past_the_check and host(arena - 1) == b.LT_ERR_WORKSPACE
+
+
 def test_launch_counts(binding):
     # three kernels per backward call; four on grouped-query shapes with few, heavy work items
     assert binding.lt_attn_bwd_num_launches(1, 32, 32, 4096, 128, True) == 3

@@ -114,3 +114,22 @@ def test_noalloc_without_room_for_the_shares(oracle):
     assert lt.lt_attn_bwd_noalloc_check_status() == lt.LT_OK
     ref = oracle.attn_bwd(*(t.double().numpy() for t in host), cfg.causal, cfg.scale)
     check_grads(outs, ref, "noalloc, whole key tiles")
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(1, 4, 4, 938, 128, True), (1, 2, 2, 1000, 64, False), (1, 20, 4, 640, 128, True)])
+@pytest.mark.parametrize("room", [0, 3, 40])
+def test_workspace_with_room_for_few_shares(oracle, B, Hq, Hkv, S, D, causal, room):
+    """`room`: shares that fit behind the accumulator.  Nothing past the size given is touched."""
+    from paper_2606_10415_b200 import binding as lt
+    cfg = workloads.custom(B, Hq, Hkv, S, D, causal, seed=S)
+    host, ins, outs = _forward(lt, cfg)
+    rows = B * Hq * -(-S // 128) * 128
+    n = 256 + 2 * rows * 16 + rows * D * 4 + room * 2 * 128 * D * 4
+    assert n < lt.lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D)
+    buf = lt.alloc_workspace(lt.lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D))
+    buf.fill_(0xFF)
+    lt.lt_attn_bwd(*ins, *outs, causal, cfg.scale, buf[:n])
+    assert lt.lt_attn_check_status(buf) == lt.LT_OK, lt.last_cuda_error()
+    assert (buf[n:] == 0xFF).all()
+    ref = oracle.attn_bwd(*(t.double().numpy() for t in host), causal, cfg.scale)
+    check_grads(outs, ref, f"room for {room} shares {cfg}", absolute=False)
