@@ -1544,9 +1544,13 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
     if (G > 1. && items >= sms + sms / 2 && items < 4. * sms) {
         // Enough key tiles to fill the SMs, but too few to form L2-sized batches (a batch needs two items per SM) while the
         // working set is more than four times the L2: the accumulator rows of the heads in flight would be fetched and
-        // written back again and again.  Halves make room for batches.
-        // Measured, ms per call, halves / whole, medians of 7 or 9 whose single values spread by 10 % (the power limit): 2, 64/8,
-        // 4096 1.74-1.78 / 1.82-1.84 in two comparisons, 1.76 / 1.66 in a third; 1, 64/8, 8192 3.19 / 3.24.
+        // written back again and again.  Halves make room for batches and even out the end of the walk; each costs a share
+        // stored and added, and a pipeline filled.  What decides is how the GPU is driven: less DRAM traffic draws less power
+        // (2, 64/8, 4096: 728 W against 852), which a long run gets back as clock and a single call does not.  us per call, whole
+        // / halves, 0.6 s of calls on end (median of five in turn) and, in brackets, single calls on an idle GPU: 2, 64/8, 4096
+        // 1760 / 1692 (1530 / 1499); 1, 64/8, 8192 3158 / 3010 (2779 / 2677); 4, 64/4, 2000 1136 / 1054 (983 / 904);
+        // 4, 64/8, 2048 1033 / 1004 (895 / 903); 8, 64/8, 1024 658 / 663 (586 / 609).  Where both kinds of call alternate every
+        // 3 ms and so share one clock, even grids of short key tiles lose: 986 / 1037 and 640 / 679 for the last two.
         const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
         if (unit_bytes * deal.n_units > 4.0 * 126.0e6) deal.halves = 1;
     }
