@@ -68,7 +68,8 @@ typedef unsigned short lt_bf16;
  * of fp16 (hi, lo, 0 x 6) with 256*hi + lo = value, [B,Hq,S_pad] rows each (every 64th or 128th -LSE/scale row may
  * carry partial maxima of the three quantities above in elements 4-6, which no product uses), an fp32 dQ accumulator
  * [B,Hq,S_pad,D], and, for shapes whose key tiles are split over work items (see lt_attn_bwd_num_launches), the items'
- * fp32 shares of dK and dV, 2 x 128 x D floats each: two per multiprocessor, or two per key tile.  A workspace (or arena)
+ * fp32 shares of dK and dV, 2 x 128 x D floats each: one per multiprocessor and one per key tile where key tiles are
+ * fewer, otherwise two per multiprocessor; or two per key tile.  A workspace (or arena)
  * without room for all shares, down to one that ends with the accumulator, is accepted by every backward call: key tiles
  * are then shared by fewer CTAs, or stay whole, which is slower and changes the order in which dK and dV are summed. */
 size_t lt_attn_fwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D);

@@ -331,9 +331,16 @@ struct BwdDeal {
         return lo;
     }
     // A share is a block of 2 x 128 x D floats: dK, then dV, each [D/4][128 rows][4], so that a warp stores or reads 512
-    // consecutive bytes.  Dealt out, they are numbered 2 c (the end of CTA c's first key tile) and 2 c + 1 (the beginning of
-    // its last); in halves, by key tile and half.
-    __host__ __device__ __forceinline__ int n_shares() const { return 2 * (halves ? n_units * n_tiles : ctas); }
+    // consecutive bytes.  In halves they are numbered by key tile and half; dealt out, 2 c (the end of CTA c's first key
+    // tile) and 2 c + 1 (the beginning of its last), or, where that takes fewer, c + key tile, which grows along the walk.
+    __host__ __device__ __forceinline__ int tiles() const { return n_units * n_tiles; }
+    __host__ __device__ __forceinline__ bool few_tiles() const { return tiles() <= ctas; }
+    __host__ __device__ __forceinline__ int share(int c, int tile, bool begins) const {
+        return few_tiles() ? c + tile : 2 * c + begins;
+    }
+    __host__ __device__ __forceinline__ int n_shares() const {
+        return halves ? 2 * tiles() : few_tiles() ? ctas + tiles() - 1 : 2 * ctas;
+    }
 };
 
 // dK_j and dV_j of the key tiles that were dealt out to several CTAs: the fp32 shares, added in the order of the walk,
@@ -347,7 +354,7 @@ __global__ void __launch_bounds__(256)
 bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __half *__restrict__ dV, const BwdDeal deal,
                   int Hkv, int S, lt_tensor_strides dk_st, lt_tensor_strides dv_st) {
     const int c = blockIdx.x, second = blockIdx.y & 1;
-    int parts = 0, unit, j = 0, first_share;
+    int parts = 0, unit, j = 0, first_share = 0;
     if (deal.halves) {
         unit = c / deal.n_tiles;
         j = c - unit * deal.n_tiles;
@@ -356,9 +363,9 @@ bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __
     } else {
         const int unit_cost = deal.tile_start(deal.n_tiles), end = deal.stretch(c + 1);
         unit = end / unit_cost;
-        first_share = 2 * c + 1;
         if (unit < deal.n_units) {
             j = deal.tile_at(end - unit * unit_cost);
+            first_share = deal.share(c, unit * deal.n_tiles + j, true);
             const int start = unit * unit_cost + deal.tile_start(j), n = deal.pairs(j);
             int upto = deal.cut(end - start, n);
             if (upto > 0 && upto < n && deal.cut(deal.stretch(c) - start, n) == 0)
@@ -376,9 +383,10 @@ bwd_shares_kernel(const float4 *__restrict__ shares, __half *__restrict__ dK, __
     float4 a[2][2];
 #pragma unroll
     for (int x = 0; x < 4; ++x) a[x >> 1][x & 1] = __ldcs(next + ((x >> 1) * 4 + (x & 1)) * 128);
-    next += 2 * kShareVec;  // the second share follows the first, further ones are two apart
+    next += 2 * kShareVec;  // the second share follows the first, further ones are one or two apart
+    const int apart = (deal.few_tiles() ? 2 : 4) * kShareVec;
 #pragma unroll 4
-    for (int k = 1; k < parts; ++k, next += 4 * kShareVec) {
+    for (int k = 1; k < parts; ++k, next += apart) {
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const float4 y = __ldcs(next + ((x >> 1) * 4 + (x & 1)) * 128);
@@ -492,7 +500,7 @@ struct BwdWalk {
             const int from = d.cut(begin - start, n), to = d.cut(end - start, n);
             start += kTileCost + n;
             if (++j == d.n_tiles) j = 0, ++unit;
-            if (to > from) return make_int4(tile, from, to, from == 0 && to == n ? -1 : 2 * blockIdx.x + (from == 0));
+            if (to > from) return make_int4(tile, from, to, from == 0 && to == n ? -1 : d.share(blockIdx.x, tile, from == 0));
         }
         return make_int4(-1, 0, 0, 0);
     }
@@ -1519,8 +1527,9 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
     if (G * n_tiles < 2. || cost > 1.0e9) return deal;  // (nothing to split; costs are 32-bit numbers)
     // (small walks: stretches of two; a small workspace: as many as have room for their shares)
     int ctas = cost < 2. * sms ? static_cast<int>(cost / 2.) : sms;
-    const size_t two_shares = static_cast<size_t>(2) * (2 * kTileRows * 4) * D;
-    if (room / two_shares < static_cast<size_t>(ctas)) ctas = static_cast<int>(room / two_shares);
+    const size_t in_room = room / (static_cast<size_t>(2 * kTileRows * 4) * D), tiles = static_cast<size_t>(deal.tiles());
+    const size_t most = in_room / 2 + 1 > tiles ? in_room + 1 - tiles : in_room / 2;  // (few_tiles() or not)
+    if (most < static_cast<size_t>(ctas)) ctas = static_cast<int>(most);
     // Estimated makespans, in tile pairs (2-3 us each): whole key tiles, the longest one or the average work of an SM, in
     // whole rounds where all are equal; dealt out, the average plus what the parts cost: the shares stored and added (they
     // grow with the CTAs), and a second pipeline filled in the CTAs whose stretch crosses into another key tile.  Measured, us per call, whole / dealt
@@ -1710,7 +1719,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     cfg_fin.attrs = &pdl;
     cfg_fin.numAttrs = 1;
     if (split) {
-        cfg_fin.gridDim = dim3(deal.n_shares() / 2, 2 * (D / 32));
+        cfg_fin.gridDim = dim3(deal.halves ? deal.tiles() : deal.ctas, 2 * (D / 32));
         e = cudaLaunchKernelEx(&cfg_fin, bwd_shares_kernel<D, kBf16>, static_cast<const float4 *>(prm.shares),
                                reinterpret_cast<__half *>(dK), reinterpret_cast<__half *>(dV), deal, Hkv, S, lay.dk,
                                lay.dv);

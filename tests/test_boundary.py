@@ -85,6 +85,14 @@ def test_workspace_without_room_for_shares_is_accepted(binding, dims):
     assert host(arena) in past_the_check and host(arena - 1) == b.LT_ERR_WORKSPACE
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,S,D", [(1, 4, 4, 938, 128), (1, 2, 2, 1000, 64), (1, 1, 1, 4135, 64), (1, 40, 8, 2048, 128)])
+def test_room_for_shares_follows_the_key_tiles(binding, B, Hq, Hkv, S, D):
+    # fewer key tiles than the 148 multiprocessors: a share begins with a multiprocessor or with a key tile
+    tiles = B * Hkv * -(-S // 128)
+    shares = (binding.lt_attn_bwd_workspace_bytes(B, Hq, Hkv, S, D) - _least_workspace(B, Hq, S, D)) / (2 * 128 * D * 4)
+    assert tiles < 148 and 0 < shares <= 148 + tiles - 1
+
+
 def test_launch_counts(binding):
     # three kernels per backward call; four on grouped-query shapes with few, heavy work items
     assert binding.lt_attn_bwd_num_launches(1, 32, 32, 4096, 128, True) == 3
