@@ -44,6 +44,10 @@ int lt_dbg_tile_gemm(const lt_half *A, const lt_half *B, float *C, int mode,
  * every wait inside the attention kernels takes. */
 int lt_dbg_wait_timeout(void *workspace, size_t workspace_bytes, lt_stream_t stream);
 
+/* The kernel lt_gemm_f16 and lt_gemm_bf16 choose for these sizes: columns of an output tile, CTAs of a cluster that share
+ * a tile's contraction (1: nobody does), and whether CTA pairs share tiles.  Nothing is launched, no device is needed. */
+int lt_dbg_gemm_plan(int M, int N, int K, int *tile_columns, int *shares, int *pairs);
+
 /* Development builds only (not exported by the product library, hence described, not declared):
  *   -DLT_BWD_TIMELINE=<cta>: `int lt_dbg_bwd_timeline(long long *out)` copies 20 x 256 clock stamps to the
  *     host buffer `out` ([event][tile pair] of that CTA's first 256 tile pairs in the last backward call;

@@ -30,7 +30,7 @@ EXPORTS = (
     "lt_last_cuda_error", "lt_attn_bwd_num_launches", "lt_attn_fwd_num_launches", "lt_attn_bwd_noalloc_check_status",
 )
 # test-support entry points (include/lt_attn_debug.h)
-DEBUG_EXPORTS = ("lt_dbg_tile_gemm", "lt_dbg_wait_timeout")
+DEBUG_EXPORTS = ("lt_dbg_tile_gemm", "lt_dbg_wait_timeout", "lt_dbg_gemm_plan")
 
 
 class TensorStrides(ctypes.Structure):
@@ -108,6 +108,8 @@ def _load() -> ctypes.CDLL:
     lib.lt_dbg_tile_gemm.restype = i
     lib.lt_dbg_wait_timeout.argtypes = [vp, sz, vp]
     lib.lt_dbg_wait_timeout.restype = i
+    lib.lt_dbg_gemm_plan.argtypes = [i, i, i] + [ctypes.POINTER(i)] * 3
+    lib.lt_dbg_gemm_plan.restype = i
     return lib
 
 
@@ -382,6 +384,15 @@ def lt_dbg_wait_timeout(workspace, stream=None) -> None:
     rc = _lib.lt_dbg_wait_timeout(_ptr(workspace), workspace.nbytes, _stream_ptr(stream))
     if rc != LT_OK:
         raise LtError("lt_dbg_wait_timeout", rc)
+
+
+def lt_dbg_gemm_plan(M, N, K) -> tuple[int, int, bool]:
+    """(columns of a tile, CTAs that share its contraction, CTA pairs) of the kernel lt_gemm_f16 chooses."""
+    out = [ctypes.c_int() for _ in range(3)]
+    rc = _lib.lt_dbg_gemm_plan(M, N, K, *(ctypes.byref(o) for o in out))
+    if rc != LT_OK:
+        raise LtError("lt_dbg_gemm_plan", rc)
+    return out[0].value, out[1].value, bool(out[2].value)
 
 
 def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:

@@ -15,6 +15,7 @@
 // contraction is split over a cluster (few tiles); gemm_plan() chooses.
 #include <cmath>
 #include <cstdlib>
+#include "../../include/lt_attn_debug.h"
 #include "lt_common.cuh"
 #include "lt_host.h"
 
@@ -631,7 +632,11 @@ size_t lt_gemm_f16_workspace_bytes(void) { return lt::kStatusBytes; }
 
 // Which kernel: tile width and contraction shares per tile, or the CTA-pair kernel.  The choice is the smallest
 // estimate of a time model in microseconds whose constants were fitted to 450 measured (shape, kernel) pairs (27 shapes
-// with 1-8192 rows, every width and split); the kernel it picks is within 3.3 % of the fastest one on average.
+// with 1-8192 rows, every width and split), before the kernels were launched under one another's tails.  Measured since
+// with all plans on 90 drawn shapes, calls back to back in a graph: the kernel it picks takes 4.9 % more than the fastest
+// one on average, 52 % at worst (397 x 3773 x 648 19.5 us, 128-wide 12.8).  On 300 drawn shapes against the two kernels that
+// came before (256-wide on one CTA up to 128 rows, on pairs above): 0.42 of the time in the geometric mean, one shape
+// slower by more than 2 % (1812 x 2880 x 1176 29.1 / 31.1).
 //   first wave: launch, fill and drain, plus the blocks of the longest share (a block takes the larger part of issuing
 //   its products and of bringing its A and W rows in while the other CTAs do the same), plus the epilogue, which costs
 //   more per element when the partials of a cluster are summed; every further wave costs its own fill and drain, except
@@ -680,6 +685,24 @@ static GemmPlan gemm_plan(int M, int N, int K) {
     return best;
 }
 
+// the plan, or the single-CTA kernel where LT_GEMM_SINGLE_CTA=1 in the environment keeps it, for comparison
+static GemmPlan gemm_choice(int M, int N, int K) {
+    static const bool force_single = [] {
+        const char *v = getenv("LT_GEMM_SINGLE_CTA");
+        return v && v[0] == '1';
+    }();
+    return force_single ? GemmPlan{lt::kGemmBN, 1, false} : gemm_plan(M, N, K);
+}
+
+int lt_dbg_gemm_plan(int M, int N, int K, int *tile_columns, int *shares, int *pairs) {
+    if (M <= 0 || N <= 0 || K <= 0 || !tile_columns || !shares || !pairs) return LT_ERR_INVALID_ARG;
+    const GemmPlan plan = gemm_choice(M, N, K);
+    *tile_columns = plan.bn;
+    *shares = plan.split;
+    *pairs = plan.pair ? 1 : 0;
+    return LT_OK;
+}
+
 static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K, void *workspace,
                       size_t workspace_bytes, lt_stream_t stream, bool bf16) {
     using namespace lt;
@@ -692,11 +715,6 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
     int rc = check_device();
     if (rc != LT_OK) return rc;
 
-    // (LT_GEMM_SINGLE_CTA=1 in the environment keeps the single-CTA kernel, for comparison)
-    static const bool force_single = [] {
-        const char *v = getenv("LT_GEMM_SINGLE_CTA");
-        return v && v[0] == '1';
-    }();
     GemmParams prm;
     prm.C = reinterpret_cast<__half *>(C);
     prm.status = reinterpret_cast<unsigned int *>(workspace);
@@ -710,7 +728,7 @@ static int gemm_entry(const void *A, const void *W, void *C, int M, int N, int K
     const uint32_t a_rows = M <= 64 ? (M + 7) / 8 * 8 : kGemmBM;
     prm.a_bytes = a_rows * kGemmBK * 2;
 
-    const GemmPlan plan = force_single ? GemmPlan{kGemmBN, 1, false} : gemm_plan(M, N, K);
+    const GemmPlan plan = gemm_choice(M, N, K);
     const bool use_pair = plan.pair;
     CUtensorMap ma, mb;
     if ((rc = make_tile_map(&ma, A, M, K, a_rows)) != LT_OK) return rc;

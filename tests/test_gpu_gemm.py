@@ -41,8 +41,8 @@ def run_gemm(lt, A, W):
     (1, 8, 8), (100, 200, 72), (129, 257, 136), (300, 1000, 520),  # ragged in every dimension
     (384, 250, 64), (77, 36, 1024),                                # N not a multiple of 8: scalar stores
     (2048, 1024, 768),                                             # more tiles than SMs would need twice
-    (128, 40000, 128),   # one tile row: the single-CTA kernel, 157 tiles over 148 CTAs (accumulator ring reused)
-    (520, 20000, 192),   # CTA pairs: 3 x 79 tiles of 256 x 256 over 74 pairs (both accumulators reused), ragged M and N
+    (128, 40000, 128),   # one tile row: 157 tiles of the 256-wide kernel over 148 CTAs
+    (520, 20000, 192),   # 5 x 79 tiles of the 256-wide kernel, ragged M and N
 ])
 def test_gemm_matches_oracle(lt, oracle, M, N, K):
     A, W = make_operands(M, N, K, seed=M + N + K)
@@ -63,7 +63,7 @@ def test_gemm_matches_oracle(lt, oracle, M, N, K):
     (130, 2048, 2048), (16, 5504, 4096), (40, 6000, 2000),  # 128- and 256-wide tiles, two to six shares
     (150, 1408, 152), (404, 1152, 272), (266, 685, 224), (129, 600, 456),  # short contractions on several tile rows
     (1000, 2040, 4096), (600, 600, 600), (8192, 72, 136),   # more tiles than fit at once, short contractions
-    (700, 2047, 136), (260, 2046, 136), (129, 2008, 64),    # 256-wide tiles whose edge is odd, even, in eights
+    (700, 2047, 136), (260, 2046, 136), (129, 2008, 64),    # narrow tiles whose edge is odd, even, in eights
     (2000, 3999, 2048), (2048, 3998, 2048), (1900, 4040, 2048),  # the same on CTA pairs
 ])
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
@@ -85,6 +85,45 @@ def test_gemm_few_tiles(lt, M, N, K, dtype):
     # factor of eight above that for the largest of up to a million elements), and the smallest subnormal step
     assert (err <= half_ulp * ref.abs() + 8 * K ** 0.5 * 2.0 ** -24 + 2.0 ** -24).all(), float(err.max())
     assert torch.isnan(C[M]).all()
+
+
+@pytest.mark.parametrize("M,N,K,plan", [
+    # the 256-wide kernel on single CTAs: edges that are odd, even, in eights; the last with up to four tiles per CTA
+    (570, 2427, 344, (256, 1, False)), (560, 2430, 344, (256, 1, False)), (570, 2424, 344, (256, 1, False)),
+    (4000, 4001, 256, (256, 1, False)),
+    # on CTA pairs, up to four tiles per pair, so that both accumulators are used again
+    (4000, 4001, 1024, (256, 1, True)), (3970, 4002, 1024, (256, 1, True)), (4000, 4008, 1024, (256, 1, True)),
+    # narrow tiles, whole and split contractions
+    (260, 2046, 136, (64, 1, False)), (700, 2047, 136, (128, 1, False)), (424, 265, 5920, (64, 6, False)),
+    (130, 2048, 2048, (128, 4, False)), (40, 6000, 2000, (256, 5, False)), (1000, 2040, 4096, (256, 2, False)),
+])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_gemm_each_kernel(lt, M, N, K, plan, dtype):
+    """Each kernel of the choice, every element of its result, and that the sizes do select it."""
+    assert lt.lt_dbg_gemm_plan(M, N, K) == plan
+    test_gemm_few_tiles(lt, M, N, K, dtype)
+
+
+def test_gemm_pairs_on_two_streams(lt):
+    """Two products of the CTA-pair kernel on two streams at once: clusters of both launches share the SMs."""
+    shapes = [(1024, 4096, 4096), (1900, 4040, 2048)]
+    streams, calls = [torch.cuda.Stream() for _ in shapes], []
+    for k, (M, N, K) in enumerate(shapes):
+        assert lt.lt_dbg_gemm_plan(M, N, K) == (256, 1, True)
+        A, W = (t.cuda() for t in make_operands(M, N, K, seed=30 + k))
+        calls.append((A, -A, W, [torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda") for _ in range(4)],
+                      lt.alloc_workspace(256)))
+    torch.cuda.synchronize()
+    for i in range(4):
+        for stream, (A, minus_A, W, C, ws) in zip(streams, calls):
+            lt.lt_gemm_f16(minus_A if i % 2 else A, W, C[i], ws, stream)
+    torch.cuda.synchronize()
+    for A, _, W, C, ws in calls:
+        assert lt.lt_attn_check_status(ws) == lt.LT_OK, lt.last_cuda_error()
+        ref = A.double() @ W.double().T
+        for i in range(4):
+            err = (C[i].double() - (ref if i % 2 == 0 else -ref)).abs()  # (the bound of test_gemm_few_tiles)
+            assert (err <= 2.0 ** -11 * ref.abs() + 8 * A.shape[1] ** 0.5 * 2.0 ** -24 + 2.0 ** -24).all()
 
 
 @pytest.mark.parametrize("M,N,K", [
@@ -203,8 +242,8 @@ def test_gemm_bf16_matches_oracle(lt, oracle, M, N, K):
 
 @pytest.mark.parametrize("seed", [0, 1])
 def test_gemm_random_shapes(lt, oracle, seed):
-    """Seeded sweep over ragged shapes on both kernels (one tile row: single CTA; more: CTA pairs):
-    integer operands, so every result is exact and compared bit for bit."""
+    """Seeded sweep over ragged shapes of up to 1 100 rows (narrow tiles, whole and split contractions): integer operands, so
+    every result is exact and compared bit for bit."""
     rng = np.random.default_rng(1000 + seed)
     for case in range(12):
         M = int(rng.choice([1, 64, 127, 128, 129, 255, 256, 257, 384, 513, 700, 1100]))
@@ -220,8 +259,7 @@ def test_gemm_random_shapes(lt, oracle, seed):
 
 
 def test_gemm_pair_kernel_on_two_streams(lt, oracle):
-    """Two products on two streams at once (clusters of both launches share the SMs); each has its own
-    status block and result."""
+    """Two products on two streams at once, whose CTAs share the SMs; each has its own status block and result."""
     s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
     A1, W1 = make_operands(1024, 2048, 512, seed=21)
     A2, W2 = make_operands(768, 1536, 1024, seed=22)
