@@ -521,7 +521,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     if (s_row < p.S) reinterpret_cast<uint4 *>(o_row + c * 32)[v8] = o;
                 }
             }
-            if (s_row < p.S) p.lse[q_row] = (m_used + log2f(l)) * kFwdLn2;
+            // (split keys: the weight of one half, an approximate exponential, adds 1e-7 to LSE's error; two roundings fewer
+            // here take off more)
+            if (s_row < p.S) p.lse[q_row] = kSplitKeys ? fmaf(m_used, kFwdLn2, logf(l)) : (m_used + log2f(l)) * kFwdLn2;
         }
     }
 

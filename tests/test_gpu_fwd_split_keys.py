@@ -68,3 +68,29 @@ def test_hidden_key_tiles(H, Hkv, S, D, hidden, causal, dtype):
     assert torch.isfinite(O).all()  # (the gates of test_split_keys)
     assert (O.double() - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
     assert ((LSE.double() - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
+
+
+@pytest.mark.parametrize("H,S,D,causal", [(32, 1024, 128, True), (8, 700, 64, True), (4, 1500, 64, False)])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+def test_no_further_from_64_bits_than_query_pairs(H, S, D, causal, dtype):
+    """The same heads alone (their keys in two chains) and many times over (pairs of query tiles): putting two chains
+    together costs neither O nor LSE any precision."""
+    from paper_2606_10415_b200 import binding as lt
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(S)
+    Q, K, V = (torch.randn((1, H, S, D), generator=gen, device="cuda").to(dtype) for _ in range(3))
+    s = Q.double() @ K.double().transpose(-1, -2) * D ** -0.5
+    if causal:
+        s.masked_fill_(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
+    lse = torch.logsumexp(s, -1)
+    ref = torch.exp(s - lse[..., None]) @ V.double()
+    fn = lt.lt_attn_fwd if dtype == torch.float16 else lt.lt_attn_fwd_bf16
+    off, last = [], None
+    for B in (1, 512 // H):
+        q, k, v = (t.expand(B, -1, -1, -1).contiguous() for t in (Q, K, V))
+        O, LSE = torch.empty_like(q), torch.empty((B, H, S), device="cuda")
+        fn(q, k, v, O, LSE, causal, D ** -0.5, lt.alloc_workspace(256))
+        assert last is None or not torch.equal(last, O[0])  # the two forms do differ
+        last = O[0]
+        off.append(((O[0].double() - ref[0]).norm(), (LSE[0].double() - lse[0]).norm()))
+    assert off[0][0] <= off[1][0] and off[0][1] <= off[1][1], off
