@@ -725,23 +725,21 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
     const int n_units = B * Hkv;
     const long long n_tiles = padded_rows(S) / 128;
     const long long unit_iters = static_cast<long long>(G) * (causal ? n_tiles * (n_tiles + 1) / 2 : n_tiles * n_tiles);
-    // The copies in one direction take as long as those in the other, so chunks of equal size keep both copy engines busy:
-    // a chunk's results go back while the next one comes in.  More chunks leave less to do before the first and after the
-    // last, and pay more for copies that get small (beside copies in the other direction one of 3 MB costs 15 us on top
-    // of its bytes).  Six, where the kernels of one take little of its copies' time; four, the last ones smaller, where
-    // they take more of it or units are few.  Measured with O returned, ms, four / six / ten chunks (six beside ten in one
-    // comparison, four in both): LLaMA-2-7B layer 3.68 / 3.47 / 3.64; 24 heads of 3 000 2.16 / 1.94 / 1.98; 4 x 16 heads at
-    // S = 1024 unmasked 1.95 / 1.87 / 1.96; Qwen2.5-32B layer (8 units) 2.77 / 2.82 / 3.09; 8 x 8 heads at S = 2048
-    // unmasked 3.67 / 3.85 / 3.56; six of exactly a sixth, or five, seven, eight equal ones are 1-3 % behind on average.
+    // The copies in one direction take as long as those in the other, and the copies back can only begin when the first
+    // chunk has come in and been worked on: the smaller that chunk, the better, but every copy beside others in the other
+    // direction costs about 15 us on top of its bytes.  Four chunks, the last ones smaller, or six of about equal size.
+    // Measured with O returned on 100 shapes (four / six, ratio of the times, and ms for some): one query head per key/value
+    // head and 20 to 34 units 0.99-1.15, median 1.02 (LLaMA-2-7B layer, 32 units, 3.80 / 3.51; 24 heads of 3 000 2.26 / 2.05); 36 to 64
+    // units 0.94-1.04, median 0.96, at every S from 1 500 to 4 096 (40 heads of 4 096 4.65 / 4.77; of 2 048 2.40 / 2.54; 8 x 8 heads of 2 048
+    // unmasked 3.76 / 3.96); fewer than 20 units, for which six chunks get uneven, 0.97-1.06; grouped queries 0.96-0.99 (Qwen2.5-32B
+    // layer 2.83 / 2.86; 40 / 20 heads of 4 096 3.51 / 3.61).
     int bounds[kHostMaxChunks + 1];
     int n_chunks = 1;
     bounds[0] = 0;
     bounds[1] = n_units;
     if (unit_iters * n_units >= 3000 && n_units > 1) {  // otherwise not worth the extra streams
         constexpr int kFew[4] = {30, 60, 85, 100}, kMany[6] = {17, 34, 51, 68, 85, 100};  // cumulative shares, %
-        const double copy_us = static_cast<double>(2 * bq + 2 * bk) / 48.0e3;  // at 48 GB/s
-        const double chunk_us = 2.1 * G * n_tiles + 1.9 * n_tiles + 20.0;      // a small chunk's backward, forward, launches
-        const bool many = n_units >= 20 && copy_us > 15.0 * chunk_us;
+        const bool many = G == 1 && n_units >= 20 && n_units <= 34;
         const int *percent = many ? kMany : kFew;
         const int np = many ? 6 : 4;
         n_chunks = 0;

@@ -1,4 +1,4 @@
-"""The host-buffer call cut into many chunks (six where copies outlast a chunk's kernels): every unit of every chunk
+"""The host-buffer call cut into chunks (four of them, or six: 24 heads of 3 000): every unit of every chunk
 against the device entry points on the whole problem, with and without the optional outputs, calls back to back."""
 import pytest
 import torch
@@ -42,7 +42,7 @@ def test_many_chunks(B, Hq, Hkv, S, D, causal, with_o):
         assert (g - w).norm() <= 3 * 2.0 ** -11 * w.norm(), name
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(4, 16, 16, 1024, 128, False), (1, 16, 8, 3000, 128, True)])
+@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(4, 16, 16, 1024, 128, False), (1, 16, 8, 3000, 128, True), (1, 24, 24, 3000, 128, True)])
 def test_calls_on_changing_data(B, Hq, Hkv, S, D, causal):
     """Calls in a row on one arena, each with other inputs and into outputs of its own: a copy that overtook the kernels it
     waits for, or a chunk that was overwritten under a copy, would leave another call's values."""
