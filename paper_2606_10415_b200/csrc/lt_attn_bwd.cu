@@ -1542,10 +1542,19 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
     if (whole < G * n_tiles + kTileCost) whole = G * n_tiles + kTileCost;
     if (!causal && whole < ceil(items / sms) * (G * n_tiles + kTileCost)) whole = ceil(items / sms) * (G * n_tiles + kTileCost);
     if (n_tiles == 1. && D == 64) whole -= 1.;  // (the one-tile variant has fewer launches)
+    // Everything the items touch (K, V, Q, dO and the fp32 dQ rows), in L2s of 126 MB.  Dealt out, all units are walked at once,
+    // whole key tiles batch by batch (launch_bwd), so the gain has to be the larger, the more there is.  380 shapes with
+    // estimates of 0.6 and above, dealt against the faster of whole and halved key tiles: without that term the choice took
+    // 2.0 % more than the faster one on average, up to 28 %, with it 0.7 %, up to 15 %.  us, dealt / whole, unmasked: 2, 64/16,
+    // 1439 (1.8 L2s, estimate 0.92) 1.28 of the time; 8, 20/4, 3328 (4.8, 0.95) 1.26; 8, 32/4, 1472 (3.4, 0.90) 1244 / 1020; on the other
+    // side 8, 8/2, 5009 (3.0, 0.88) 2355 / 2673; 4, 64/16, 1685, D = 64 (2.1, 0.89) 804 / 874; not told apart: 8, 32/4, 1472,
+    // D = 64 (1.7, 0.90) 674 / 596.
+    const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
+    const double working_set = unit_bytes * deal.n_units / 126.0e6;
     if (ctas > 0) {
         const double crossings = items < ctas ? items / ctas : 1.;
         const double dealt = cost / ctas + 1.6 + 0.028 * ctas + 3.0 * crossings * crossings;
-        if (dealt < 0.95 * whole) {
+        if (dealt < (0.95 - 0.02 * working_set) * whole) {
             deal.ctas = ctas;
             return deal;
         }
@@ -1560,8 +1569,7 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
         // 1760 / 1692 (1530 / 1499); 1, 64/8, 8192 3158 / 3010 (2779 / 2677); 4, 64/4, 2000 1136 / 1054 (983 / 904);
         // 4, 64/8, 2048 1033 / 1004 (895 / 903); 8, 64/8, 1024 658 / 663 (586 / 609).  Where both kinds of call alternate every
         // 3 ms and so share one clock, even grids of short key tiles lose: 986 / 1037 and 640 / 679 for the last two.
-        const double unit_bytes = static_cast<double>(padded_rows(S)) * D * (2.0 * 2 + G * (2.0 * 2 + 4));
-        if (unit_bytes * deal.n_units > 4.0 * 126.0e6) deal.halves = 1;
+        if (working_set > 4.0) deal.halves = 1;
     }
     if (share_bytes(deal, D) > room) deal.halves = 0;
     return deal;
