@@ -545,15 +545,14 @@ extern "C" int lt_dbg_fwd_trace(unsigned long long *out, int reset) {
 
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
 // makespan in steps of both chains (about 1.9 us), with kFill for a CTA's start, fill and drain, and a margin for the second
-// softmax's merge.  On 260 shapes near the line, both ways measured, it picks the faster one or one within 3 % of it every
-// time (0.02 % behind on average; without the margin and the second round 0.9 %, up to 30 %: 64 heads of 267 12.3 / 16.0); on
-// 600 others it is 0.06 % behind on average, 7 % at worst.
+// softmax's merge.  On 860 shapes near the line, both ways measured, it is 0.04 % behind the faster one on average and 7 % at
+// worst (without the margin and the second round 0.9 % and 30 %: 64 heads of 267 12.3 / 16.0).
 // us, pairs of tiles / split keys (heads, S): 8, 2048 33.9 / 21.5; 4, 8000
 // 112.8 / 64.7; 16, 512 13.4 / 10.0; 32, 1024 22.4 / 21.4; 16, 753 unmasked 17.5 / 12.5; on the other side 64, 640
 // 19.4 / 21.2; 40, 1920 53.9 / 60.0; 32, 4096 141.7 / 163.2; 16, 3743 60.4 / 70.3; 64 of 442, D = 64 13.1 / 15.6.
 static bool splits_keys(int B, int Hq, int S, int causal) {
     constexpr int kSms = 148;
-    constexpr double kFill = 2.2, kMargin = 0.92;
+    constexpr double kFill = 2.2;
     const double heads = static_cast<double>(B) * Hq;
     const int n = (S + kFwdTileRows - 1) / kFwdTileRows, pairs = (n + 1) / 2;
     if (n < 2) return false;
@@ -575,7 +574,7 @@ static bool splits_keys(int B, int Hq, int S, int causal) {
     const double split_steps = half * (half + 1) / 2 + even * (even + 1) / 2;
     const double split = span(n, split_steps, [&](int q) { return static_cast<double>(causal ? (n - q + 1) / 2 : (n + 1) / 2); });
     const double whole = span(pairs, pair_steps, [&](int q) { return static_cast<double>(causal && q > 0 ? 2 * (pairs - q) : n); });
-    return split < kMargin * whole;
+    return split < (causal ? 0.92 : 0.95) * whole;
 }
 
 template <int D, bool kBf16>
