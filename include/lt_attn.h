@@ -26,7 +26,7 @@
  *     allocate no device memory.  Two calls may overlap on the GPU only if they use
  *     different workspaces.
  *   - Value range of the backward: dS is rounded to fp16 (bf16) after multiplication by a power of two
- *     picked per call from max ||dO_row||, max |delta| and max ||V_row|| (their product bounds |dS|), so
+ *     picked per call (where a call is one launch, per thread block over its own heads) from max ||dO_row||, max |delta| and max ||V_row|| (their product bounds |dS|), so
  *     gradients keep their relative accuracy for upstream gradients and values of any usual magnitude.
  *     Non-finite inputs make that bound infinite; the most cautious factor is then used.
  *   - Return value: LT_OK or an lt_status error.  Errors found on the host launch

@@ -78,7 +78,8 @@ __device__ unsigned long long g_fwd_trace[32];
 #define LT_FT_COUNT(slot, n)
 #endif
 
-// Registers are handed out per four warps, so ten warps get the 168-register cap of twelve.
+// Twelve warps: a producer, an issuer (and two idle ones, so that registers can be resized by groups of four), and four
+// softmax warps for each of the two chains.
 //
 // A CTA runs two chains S -> softmax -> P V -> S side by side (index t).  Normally they are the two query tiles of a pair
 // over the same key tiles; kSplitKeys: the even and the odd key tiles of one query tile, whose two softmaxes are put
