@@ -1532,7 +1532,9 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
     if (most < static_cast<size_t>(ctas)) ctas = static_cast<int>(most);
     // Estimated makespans, in tile pairs (2-3 us each): whole key tiles, the longest one or the average work of an SM, in
     // whole rounds where all are equal; dealt out, the average plus what the parts cost: the shares stored and added (they
-    // grow with the CTAs), and a second pipeline filled in the CTAs whose stretch crosses into another key tile.  Measured, us per call, whole / dealt
+    // grow with the CTAs) by a kernel that the dQ conversion waits for, and a second pipeline filled in the CTAs whose stretch
+    // crosses into another key tile.  Constants fitted to 240 short calls near the line, both ways in graphs: on those and on 240
+    // others 0.2 % behind the faster one on average, 6 % at worst.  Measured, us per call, whole / dealt
     // out (batch, query / kv heads, S; D = 128 under the causal mask unless noted): 1, 40/8, 2048 244 / 149; 1, 40/8, 1024
     // 108 / 56; 1, 2/1, 3566 131 / 39; 1, 1/1, 4135, D = 64 60 / 26; 1, 2/2, 2999 unmasked 66 / 43; 8, 5/1, 2572, D = 64
     // unmasked 399 / 221; 1, 16/8, 208 22.0 / 19.1.  On the other side of the line: 1, 64/16, 2048 244 / 257; 1, 8/8, 4096
@@ -1553,8 +1555,8 @@ static BwdDeal deal_pairs(int B, int Hq, int Hkv, int S, int D, int causal, size
     const double working_set = unit_bytes * deal.n_units / 126.0e6;
     if (ctas > 0) {
         const double crossings = items < ctas ? items / ctas : 1.;
-        const double dealt = cost / ctas + 1.6 + 0.028 * ctas + 3.0 * crossings * crossings;
-        if (dealt < (0.95 - 0.02 * working_set) * whole) {
+        const double dealt = cost / ctas + 2.75 + 0.016 * ctas + 0.8 * crossings * crossings;
+        if (dealt < (0.94 - 0.02 * working_set) * whole) {
             deal.ctas = ctas;
             return deal;
         }
