@@ -3,10 +3,10 @@
 // takes saved probability tiles; this library keeps LSE and rebuilds P in the backward).
 //
 // One CTA per (batch, query head, pair of neighbouring 128-row query tiles).  Warp 0 streams
-// K_j / V_j tiles with TMA through two-stage rings, warp 1 issues S = Q_i K_j^T and
-// O += P V_j on the tcgen05 tensor cores, and each query tile has its own group of four
-// softmax warps (one thread per query row), so that the tensor cores work on one tile of the
-// pair while the other tile's scores are exponentiated.  S/P and O live in tensor memory.
+// K_j / V_j tiles with TMA through one ring, warp 1 issues S = Q_i K_j^T and O += P V_j on the
+// tcgen05 tensor cores, and each query tile has its own group of four softmax warps (one thread
+// per query row), so that the tensor cores work on one tile of the pair while the other tile's
+// scores are exponentiated.  S, P and O live in tensor memory.
 // The running row maximum is only raised when it grew by more than 2^8 since the output
 // was last rescaled, so most key tiles need no pass over O.
 #include <float.h>
@@ -36,8 +36,8 @@ static_assert(kFwdRegsAtLaunch * kFwdThreads <= 65536 && 128 * kFwdRegsControl +
 constexpr float kFwdRescaleLog2 = 8.f;        // P <= 2^8 stays far inside fp16 range
 
 enum {
-    kWaitFwdQ = 301, kWaitFwdK = 302, kWaitFwdV = 303, kWaitFwdS = 304, kWaitFwdP = 305,
-    kWaitFwdO = 306, kWaitFwdKEmpty = 307, kWaitFwdVEmpty = 308, kWaitFwdDone = 309
+    kWaitFwdQ = 301, kWaitFwdKV = 302, kWaitFwdEmpty = 303, kWaitFwdS = 304, kWaitFwdP = 305,
+    kWaitFwdO = 306, kWaitFwdSFree = 307, kWaitFwdDone = 309
 };
 
 template <int D>
@@ -45,57 +45,54 @@ struct __align__(1024) FwdSmem {
     static constexpr int kBoxes = D / 64;
     static constexpr int kTile = kBoxes * kFwdBoxBytes;
     uint8_t q[2][kTile];   // the pair's two query tiles
-    uint8_t k[2][kTile];   // ring of key tiles
-    uint8_t v[2][kTile];   // ring of value tiles
-    uint64_t bar_q[2], bar_k_full[2], bar_k_empty[2], bar_v_full[2], bar_v_empty[2];
-    uint64_t bar_s_full[2], bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_done, bar_merge;
+    static constexpr int kSlots = D == 128 ? 5 : 8;
+    uint8_t kv[kSlots][kTile];   // ring of key and value tiles, in the order of their use
+    uint64_t bar_q[2], bar_kv_full[kSlots], bar_kv_empty[kSlots];
+    uint64_t bar_s_full[2], bar_s_free, bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_done, bar_merge;
     float2 merge[kFwdTileRows];  // (split keys) maximum and sum of the odd key tiles' half, per query row
     uint32_t tmem_base;
     int abort_flag;
 };
 
 struct FwdParams {
-    __half *O;
     float *lse;
     unsigned int *status;
     int B, Hq, Hkv, S, causal;
     float scale;
-    lt_tensor_strides o_st;  // element strides of O
 };
-
-#ifdef LT_FWD_TRACE
-// Development build only: summed clock() intervals.  [0..7] issuer, [8..15] softmax lane 0 of
-// every warp, [16] tiles processed by softmax warps, [17] key tiles seen by issuers, [18] CTA cycles.
-__device__ unsigned long long g_fwd_trace[32];
-#define LT_FT_DECL uint32_t ft_acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}; uint32_t ft_t = clock()
-#define LT_FT(slot) do { const uint32_t ft_n = clock(); ft_acc[slot] += ft_n - ft_t; ft_t = ft_n; } while (0)
-#define LT_FT_FLUSH(base) do { for (int ft_i = 0; ft_i < 8; ++ft_i) if (ft_acc[ft_i]) atomicAdd(&g_fwd_trace[(base) + ft_i], static_cast<unsigned long long>(ft_acc[ft_i])); } while (0)
-#define LT_FT_COUNT(slot, n) atomicAdd(&g_fwd_trace[slot], static_cast<unsigned long long>(n))
-#else
-#define LT_FT_DECL
-#define LT_FT(slot)
-#define LT_FT_FLUSH(base)
-#define LT_FT_COUNT(slot, n)
-#endif
 
 // Twelve warps: a producer, an issuer (and two idle ones, so that registers can be resized by groups of four), and four
 // softmax warps for each of the two chains.
 //
 // A CTA runs two chains S -> softmax -> P V -> S side by side (index t).  Normally they are the two query tiles of a pair
 // over the same key tiles; kSplitKeys: the even and the odd key tiles of one query tile, whose two softmaxes are put
-// together at the end (each chain has its own maximum, sum and O; a ring slot then belongs to one chain).  That is twice
-// the CTAs with half as long a walk, for grids that leave multiprocessors idle or wait for a few long walks:
-// splits_keys().
+// together at the end (each chain has its own maximum, sum and O).  That is twice the CTAs with half as long a walk, for
+// grids that leave multiprocessors idle or wait for a few long walks: splits_keys().
+//
+// What bounds it: the exponential unit, 1 024 cycles per tile of 128 x 128 scores, with the softmax warps' other work (load,
+// maximum, store, hand-offs: about 1 300 cycles a tile) that two warps per scheduler hide only in part; a step of both
+// chains takes about 3 100 cycles, the exponential unit and the tensor cores (2 048 cycles a step at D = 128) are each
+// busy for two thirds of it, and in long runs the power limit.  Hence the layout of tensor memory: the softmax warps hold
+// a tile's scores in registers as soon as they are there, so the chains share one region of scores and P has columns of its
+// own; a chain's next scores are formed under its softmax instead of behind its product P V.  (With S and P of a chain in one
+// region a step took 3 600 cycles, most of it the chain softmax -> P V -> S.)  Measured, us, a region per chain / this
+// (heads, S, D; causal unless noted; single calls): 32, 4096, 128 145 / 131; 32, 1024, 128 22.4 / 20.1; 32, 3000, 128 92.5 / 82;
+// 64 of 1531, 64 unmasked 79.4 / 77.7; 64/8 heads of 8192 unmasked 1740 / 1690.
+// Tried: two warps per row and tile, 16 softmax warps with a vote on the maximum (11 % slower: they wait for each other);
+// the maximum found during the first quarter's exponentials (3 % slower); both chains started at once (2 %
+// slower: they stay in step and want the exponential unit together); a fifth of the exponentials as polynomials (no gain at
+// this share of the unit's time).
 template <int D, bool kBf16, bool kSplitKeys>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-           const __grid_constant__ CUtensorMap map_v, const FwdParams p) {
+           const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const FwdParams p) {
     using Smem = FwdSmem<D>;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kTileBytes = Smem::kTile;
     constexpr uint32_t kTmemCols = 512;
-    constexpr uint32_t kColS = 0;     // tile t: S / P at columns [128 t, 128 t + 128)
-    constexpr uint32_t kColO = 256;   // tile t: O at columns [256 + D t, 256 + D t + D)
+    constexpr uint32_t kColS = 0;     // scores of one chain at a time
+    constexpr uint32_t kColP = 128;   // chain t: P at columns [128 + 64 t, 192 + 64 t)
+    constexpr uint32_t kColO = 256;   // chain t: O at columns [256 + D t, 256 + D t + D)
 
     extern __shared__ uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -120,7 +117,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     const int j_last0 = kSplitKeys ? (n_keys + 1) / 2 - 1 : n_keys - 1;
     const int j_last1 = kSplitKeys ? n_keys / 2 - 1 : has_b ? (p.causal ? i0 + 1 : n_tiles - 1) : -1;
     const int j_end = j_last0 > j_last1 ? j_last0 : j_last1;
-    const int key_end = kSplitKeys ? n_keys - 1 : j_end;         // last key tile to be loaded
     const int n_q = kSplitKeys ? 1 : has_b ? 2 : 1;              // query tiles
 
     if (tid == 0) {
@@ -128,21 +124,23 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             mbar_init(&sm.bar_q[t], 1);
-            mbar_init(&sm.bar_k_full[t], 1);
-            mbar_init(&sm.bar_k_empty[t], 1);
-            mbar_init(&sm.bar_v_full[t], 1);
-            mbar_init(&sm.bar_v_empty[t], 1);
             mbar_init(&sm.bar_s_full[t], 1);
-            mbar_init(&sm.bar_p_ready[t], 128);
-            mbar_init(&sm.bar_p_half[t], 128);
+            mbar_init(&sm.bar_p_ready[t], 4);
+            mbar_init(&sm.bar_p_half[t], 4);
             mbar_init(&sm.bar_o_done[t], 1);
         }
+        for (int x = 0; x < Smem::kSlots; ++x) {
+            mbar_init(&sm.bar_kv_full[x], 1);
+            mbar_init(&sm.bar_kv_empty[x], 1);
+        }
+        mbar_init(&sm.bar_s_free, 4);
         mbar_init(&sm.bar_done, 1);
         mbar_init(&sm.bar_merge, 128);
         mbar_fence_init();
         tma_prefetch_desc(&map_q);
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
+        tma_prefetch_desc(&map_o);
     }
     if (warp == 0) {
         tmem_alloc(&sm.tmem_base, kTmemCols);
@@ -153,176 +151,135 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     tc_fence_after_sync();
     const uint32_t tmem = sm.tmem_base;
     volatile int *abort_flag = &sm.abort_flag;
-    // the set-up above ran under the tail of the predecessor in the stream; from here on its results are used
-    grid_dependency_wait();
-    if (blockIdx.x == 0 && tid == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
+    // (The set-up above, and the softmax warps' first pass below, run under the tail of the predecessor in the stream; its
+    // results are read, and O and LSE written, only behind grid_dependency_wait().)
 
+    // The tensor-core work in its order: score products are numbered by (step, chain); number m is issued when the softmax
+    // warps hold the scores of number m - 1 in registers, the products with V of number m - 2 come behind it.  on_s and
+    // on_pv get (step, chain, whether it is the first and the last to use the step's key or value tile) and return false to leave.
+    auto walk = [&](auto on_s, auto on_pv) -> bool {
+        auto first = [&](int j, int t) { return kSplitKeys || t == (j <= j_last0 ? 0 : 1); };
+        auto last = [&](int j, int t) { return kSplitKeys || t == (j <= j_last1 ? 1 : 0); };
+        int m = 0, j1 = 0, t1 = 0, j2 = 0, t2 = 0;  // numbers m - 1 and m - 2
+        for (int j = 0; j <= j_end; ++j) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (j > (t == 0 ? j_last0 : j_last1)) continue;
+                // (behind the end of the first chain, its last product with V goes ahead, so that its output can be stored)
+                const bool ahead = !kSplitKeys && j > j_last0;
+                if (ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+                if (!on_s(m, j, t, first(j, t), last(j, t))) return false;
+                if (!ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+                j2 = j1; t2 = t1;
+                j1 = j; t1 = t;
+                ++m;
+            }
+        }
+        if (m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+        return on_pv(j1, t1, first(j1, t1), last(j1, t1));
+    };
     if (warp < kFwdSoftmaxWarp0) {
         warpgroup_regs_set<kFwdRegsControl, kFwdRegsAtLaunch>();
         if (warp == 0) {
             // ------------------------------------------------------------------ producer
             if (lane == 0) {
+                grid_dependency_wait();
+                if (blockIdx.x == 0) p.status[kStatusWordTimeout] = 0u;  // (a wait gives up after a second at the earliest)
                 for (int t = 0; t < n_q; ++t) {
                     mbar_arrive_expect_tx(&sm.bar_q[t], kTileBytes);
 #pragma unroll
                     for (int x = 0; x < kBoxes; ++x)
                         tma_load_4d(sm.q[t] + x * kFwdBoxBytes, &map_q, &sm.bar_q[t], x * 64, (i0 + t) * kFwdTileRows, h, b);
                 }
-                bool ok = true;
-                int armed = 0;  // key/value tiles whose loads were started
-                for (int j = 0; j <= key_end; ++j) {
-                    const int s = j & 1;
-                    const uint32_t ph = (j >> 1) & 1;
-                    const int kv_row0 = j * kFwdTileRows;  // inside the head; rows past S arrive as zeros
-                    if (j >= 2 && !(ok = mbar_wait(&sm.bar_k_empty[s], ph ^ 1, abort_flag, p.status, kWaitFwdKEmpty))) break;
-                    mbar_arrive_expect_tx(&sm.bar_k_full[s], kTileBytes);
+                int fill = 0, slot = 0, round = 0;  // fill = round * kSlots + slot: tiles whose loads were started
+                auto load = [&](const CUtensorMap *map, int j, int t) -> bool {
+                    const int row0 = (kSplitKeys ? 2 * j + t : j) * kFwdTileRows;  // inside the head; rows past S arrive as zeros
+                    if (round > 0 && !mbar_wait(&sm.bar_kv_empty[slot], (round - 1) & 1, abort_flag, p.status, kWaitFwdEmpty)) return false;
+                    mbar_arrive_expect_tx(&sm.bar_kv_full[slot], kTileBytes);
 #pragma unroll
                     for (int x = 0; x < kBoxes; ++x)
-                        tma_load_4d(sm.k[s] + x * kFwdBoxBytes, &map_k, &sm.bar_k_full[s], x * 64, kv_row0, g, b);
-                    if (j >= 2 && !(ok = mbar_wait(&sm.bar_v_empty[s], ph ^ 1, abort_flag, p.status, kWaitFwdVEmpty))) {
-                        // the key tile just started still has to land before shared memory is given up
-                        for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_k_full[s], ph); ++w) {}
-                        break;
-                    }
-                    mbar_arrive_expect_tx(&sm.bar_v_full[s], kTileBytes);
-#pragma unroll
-                    for (int x = 0; x < kBoxes; ++x)
-                        tma_load_4d(sm.v[s] + x * kFwdBoxBytes, &map_v, &sm.bar_v_full[s], x * 64, kv_row0, g, b);
-                    armed = j + 1;
-                }
+                        tma_load_4d(sm.kv[slot] + x * kFwdBoxBytes, map, &sm.bar_kv_full[slot], x * 64, row0, g, b);
+                    ++fill;
+                    if (++slot == Smem::kSlots) slot = 0, ++round;
+                    return true;
+                };
+                const bool ok = walk([&](int, int j, int t, bool first, bool) { return !first || load(&map_k, j, t); },
+                                     [&](int j, int t, bool first, bool) { return !first || load(&map_v, j, t); });
                 if (!ok || *abort_flag) {
                     // somebody gave up: wait (bounded) for the copies in flight before the CTA exits
                     for (int t = 0; t < n_q; ++t)
                         for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_q[t], 0); ++w) {}
-                    for (int j = armed > 2 ? armed - 2 : 0; j < armed; ++j) {
-                        for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_k_full[j & 1], (j >> 1) & 1); ++w) {}
-                        for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_v_full[j & 1], (j >> 1) & 1); ++w) {}
-                    }
+                    for (int f = fill > Smem::kSlots ? fill - Smem::kSlots : 0; f < fill; ++f)
+                        for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_kv_full[f % Smem::kSlots], (f / Smem::kSlots) & 1); ++w) {}
                 }
             }
         } else if (warp == 1) {
             // ------------------------------------------------------------------ MMA issuer
             // The whole warp walks the loop, so that counters, wait results (voted) and descriptor arithmetic are
             // warp-uniform; one elected lane issues the products and commits.
-            {
-                const bool leader = elect_one();
-                auto wait_all = [&](uint64_t *bar, uint32_t parity, int code) {
-                    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, p.status, code));
-                };
-                // descriptors of slot 0; slot 1 of each ring follows one tile later
-                const uint64_t dQ0 = desc_kmajor(smem_u32(sm.q[0])), dK0 = desc_kmajor(smem_u32(sm.k[0]));
-                const uint64_t dV0 = desc_mnmajor(smem_u32(sm.v[0]), kFwdBoxBytes);
-                constexpr uint64_t kSlotStep = static_cast<uint64_t>(kTileBytes) >> 4;
-                auto koff = [](int kk) -> uint64_t { return static_cast<uint64_t>((kk >> 2) * (kFwdBoxBytes >> 4) + (kk & 3) * 2); };
-                auto roff = [](int kk) -> uint64_t { return static_cast<uint64_t>(kk * (2048 >> 4)); };
-                constexpr uint32_t idesc_s = make_idesc(128, 128, false, false, kBf16);
-                constexpr uint32_t idesc_o = make_idesc(128, D, false, true, kBf16);
-                auto issue_s = [&](int t, int s) {  // S_t = Q_t K^T with the key tile in ring slot s
-                    if (!leader) return;
+            const bool leader = elect_one();
+            auto wait_all = [&](uint64_t *bar, uint32_t parity, uint64_t *bar_b, uint32_t parity_b, int code) {
+                return mbar_wait_warp(bar, parity, bar_b, parity_b, abort_flag, p.status, code);
+            };
+            constexpr uint64_t kSlotStep = static_cast<uint64_t>(kTileBytes) >> 4;
+            int slot = 0, round = 0;  // the ring's next tile
+            int k_slot = 0, k_round = 0, v_slot = 0, v_round = 0;  // the tiles in use
+            auto next_tile = [&](bool first, int &mine, int &mine_round) {
+                if (!first) return;
+                mine = slot;
+                mine_round = round;
+                if (++slot == Smem::kSlots) slot = 0, ++round;
+            };
+            // descriptors of slot 0; the next slot follows one tile later
+            const uint64_t dQ0 = desc_kmajor(smem_u32(sm.q[0])), dK0 = desc_kmajor(smem_u32(sm.kv[0]));
+            const uint64_t dV0 = desc_mnmajor(smem_u32(sm.kv[0]), kFwdBoxBytes);
+            auto koff = [](int kk) -> uint64_t { return static_cast<uint64_t>((kk >> 2) * (kFwdBoxBytes >> 4) + (kk & 3) * 2); };
+            auto roff = [](int kk) -> uint64_t { return static_cast<uint64_t>(kk * (2048 >> 4)); };
+            constexpr uint32_t idesc_s = make_idesc(128, 128, false, false, kBf16);
+            constexpr uint32_t idesc_o = make_idesc(128, D, false, true, kBf16);
+            if (wait_all(&sm.bar_q[0], 0, n_q < 2 ? nullptr : &sm.bar_q[1], 0, kWaitFwdQ))
+                walk(
+                    [&](int m, int j, int t, bool first, bool last) -> bool {
+                        // chain t's scores, in the one score region
+                        next_tile(first, k_slot, k_round);
+                        if (!wait_all(&sm.bar_kv_full[k_slot], k_round & 1, m > 0 ? &sm.bar_s_free : nullptr, (m - 1) & 1, kWaitFwdSFree)) return false;
+                        tc_fence_after_sync();
+                        if (leader) {
+                            const uint64_t dQ = dQ0 + (kSplitKeys ? 0 : t) * kSlotStep, dK = dK0 + k_slot * kSlotStep;
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)
-                        umma_ss(tmem + kColS + t * 128, dQ0 + (kSplitKeys ? 0 : t) * kSlotStep + koff(kk), dK0 + s * kSlotStep + koff(kk), idesc_s, kk > 0);
-                    umma_commit(&sm.bar_s_full[t]);
-                };
-                // O_t (+)= P_t V, P_t read from tensor memory; the keys of a tile in two halves of 64, so that the
-                // first half's products run while the softmax warps exponentiate the second half (quarters were
-                // measured too and lost to the extra hand-offs)
-                auto issue_pv_half = [&](int t, int s, bool acc, int half) {
-                    if (!leader) return;
-#pragma unroll
-                    for (int kk = 4 * half; kk < 4 * half + 4; ++kk)
-                        umma_ts(tmem + kColO + t * D, tmem + kColS + t * 128 + kk * 8, dV0 + s * kSlotStep + roff(kk), idesc_o,
-                                acc | (kk > 0));
-                    if (half == 1) umma_commit(&sm.bar_o_done[t]);
-                };
-                bool ok = wait_all(&sm.bar_q[0], 0, kWaitFwdQ) &&
-                          (n_q < 2 || wait_all(&sm.bar_q[1], 0, kWaitFwdQ)) &&
-                          wait_all(&sm.bar_k_full[0], 0, kWaitFwdK);
-                if (ok) {
-                    tc_fence_after_sync();
-                    issue_s(0, 0);
-                    if constexpr (kSplitKeys) {
-                        if (leader) umma_commit(&sm.bar_k_empty[0]);
-                        if (has_b && (ok = wait_all(&sm.bar_k_full[1], 0, kWaitFwdK))) {
-                            tc_fence_after_sync();
-                            issue_s(1, 1);
-                            if (leader) umma_commit(&sm.bar_k_empty[1]);
+                            for (int kk = 0; kk < D / 16; ++kk) umma_ss(tmem + kColS, dQ + koff(kk), dK + koff(kk), idesc_s, kk > 0);
+                            umma_commit(&sm.bar_s_full[t]);
+                            if (last) umma_commit(&sm.bar_kv_empty[k_slot]);
                         }
-                    } else {
-                        if (has_b) issue_s(1, 0);
-                        if (leader) umma_commit(&sm.bar_k_empty[0]);
-                    }
-                }
-                LT_FT_DECL;
-                if constexpr (kSplitKeys) {
-                    for (int j = 0; j <= j_end && ok; ++j) {
+                        return true;
+                    },
+                    [&](int j, int t, bool first, bool last) -> bool {
+                        // O_t (+)= P_t V, P_t read from tensor memory; the keys of a tile in two halves of 64, so that the
+                        // first half's products run while the softmax warps exponentiate the second half (quarters were
+                        // measured too and lost to the extra hand-offs)
+                        next_tile(first, v_slot, v_round);
+                        const uint64_t dV = dV0 + v_slot * kSlotStep;
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {  // chain t lives in ring slot t
-                            const int j_last_t = t == 0 ? j_last0 : j_last1;
-                            if (j > j_last_t) continue;
-                            if (!(ok = wait_all(&sm.bar_v_full[t], j & 1, kWaitFwdV) && wait_all(&sm.bar_p_half[t], j & 1, kWaitFwdP))) break;
+                        for (int half = 0; half < 2; ++half) {
+                            if (!wait_all(half == 0 ? &sm.bar_p_half[t] : &sm.bar_p_ready[t], j & 1, half == 0 ? &sm.bar_kv_full[v_slot] : nullptr,
+                                          v_round & 1, kWaitFwdP)) return false;
                             tc_fence_after_sync();
-                            issue_pv_half(t, t, j > 0, 0);
-                            if (!(ok = wait_all(&sm.bar_p_ready[t], j & 1, kWaitFwdP))) break;
-                            tc_fence_after_sync();
-                            issue_pv_half(t, t, j > 0, 1);
-                            if (leader) umma_commit(&sm.bar_v_empty[t]);
-                            if (j + 1 <= j_last_t) {
-                                if (!(ok = wait_all(&sm.bar_k_full[t], (j + 1) & 1, kWaitFwdK))) break;
-                                tc_fence_after_sync();
-                                issue_s(t, t);
-                                if (leader) umma_commit(&sm.bar_k_empty[t]);
+                            if (leader) {
+#pragma unroll
+                                for (int kk = 4 * half; kk < 4 * half + 4; ++kk)
+                                    umma_ts(tmem + kColO + t * D, tmem + kColP + t * 64 + kk * 8, dV + roff(kk), idesc_o, (j > 0) | (kk > 0));
+                                if (half == 1) {
+                                    umma_commit(&sm.bar_o_done[t]);
+                                    if (last) umma_commit(&sm.bar_kv_empty[v_slot]);
+                                }
                             }
                         }
-                    }
-                } else
-                for (int j = 0; j <= j_end && ok; ++j) {
-                    const int s = j & 1, sn = s ^ 1;
-                    LT_FT(0);
-                    if (!(ok = wait_all(&sm.bar_v_full[s], (j >> 1) & 1, kWaitFwdV))) break;
-                    LT_FT(1);
-                    bool k_next_ready = false;
-#pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        const int j_last_t = t == 0 ? j_last0 : j_last1;
-                        if (j > j_last_t) continue;
-                        LT_FT(0);
-                        if (!(ok = wait_all(&sm.bar_p_half[t], j & 1, kWaitFwdP))) break;
-                        tc_fence_after_sync();
-                        issue_pv_half(t, s, j > 0, 0);
-                        if (!(ok = wait_all(&sm.bar_p_ready[t], j & 1, kWaitFwdP))) break;
-                        LT_FT(2 + t);
-                        tc_fence_after_sync();
-                        LT_FT(0);
-                        issue_pv_half(t, s, j > 0, 1);
-                        LT_FT(5);
-                        // the second tile of the pair, when it uses this key tile, uses it last
-                        const int last_user = (j <= j_last1) ? 1 : 0;
-                        if (t == last_user && leader) umma_commit(&sm.bar_v_empty[s]);
-                        if (j + 1 <= j_last_t) {
-                            if (!k_next_ready) {
-                                LT_FT(0);
-                                if (!(ok = wait_all(&sm.bar_k_full[sn], ((j + 1) >> 1) & 1, kWaitFwdK))) break;
-                                LT_FT(4);
-                                tc_fence_after_sync();
-                                k_next_ready = true;
-                            }
-                            LT_FT(0);
-                            issue_s(t, sn);
-                            LT_FT(6);
-                            const int last_user_next = (j + 1 <= j_last1) ? 1 : 0;
-                            if (t == last_user_next && leader) umma_commit(&sm.bar_k_empty[sn]);
-                        }
-                    }
-                }
-                LT_FT(0);
-                LT_FT_FLUSH(0);
-                LT_FT_COUNT(17, j_end + 1);
-                // every product issued above has finished before tensor memory is released
-                if (leader) umma_commit(&sm.bar_done);
-                if (!wait_all(&sm.bar_done, 0, kWaitFwdDone))
-                    for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_done, 0); ++w) {}
-            }
+                        return true;
+                    });
+            // every product issued above has finished before tensor memory is released
+            if (leader) umma_commit(&sm.bar_done);
+            if (!wait_all(&sm.bar_done, 0, nullptr, 0, kWaitFwdDone))
+                for (int w = 0; w < (1 << 16) && !mbar_try_wait(&sm.bar_done, 0); ++w) {}
         }
     } else {
         // ------------------------------------------------------------------ softmax warps
@@ -333,7 +290,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         const int j_last = t == 0 ? j_last0 : j_last1;
         const int i = kSplitKeys ? i0 : i0 + t;
         const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
-        const uint32_t tS = tmem + lane_base + kColS + t * 128;
+        const uint32_t tS = tmem + lane_base + kColS;
+        const uint32_t tP = tmem + lane_base + kColP + t * 64;
         const uint32_t tO = tmem + lane_base + kColO + t * D;
         const float scale_log2 = p.scale * kFwdLog2e;
         // last visible key of a masked tile: the row's own index on a causal diagonal tile, the end of
@@ -343,134 +301,121 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         float m_used = -INFINITY;  // the maximum the stored P, l and O are relative to
         float l = 0.f;             // running sum of exp2(score - m_used)
         bool ok = true;
-        LT_FT_DECL;
-        for (int j = 0; j <= j_last; ++j) {
-            LT_FT(0);
-            ok = mbar_wait(&sm.bar_s_full[t], j & 1, abort_flag, p.status, kWaitFwdS);
-            LT_FT(1);
-            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        // Pass -1 works on whatever tensor memory holds and leaves nothing behind: it brings the loop's instructions into the
+        // instruction cache while the first tiles are on their way (a first tile took 3 400 cycles instead of 1 450).
+        for (int j = t == 0 ? -1 : 0; j <= j_last; ++j) {
+            if (j >= 0 && !(ok = mbar_wait_warp(&sm.bar_s_full[t], j & 1, nullptr, 0, abort_flag, p.status, kWaitFwdS))) break;
             tc_fence_after_sync();
             // the whole score row of this key tile stays in registers
             uint32_t sc[128];
 #pragma unroll
             for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sc[c * 32]));
             tmem_wait_ld();
-            LT_FT(2);
-            float rs[4] = {0.f, 0.f, 0.f, 0.f};  // independent partial row sums
-            auto tile_softmax = [&](auto diag_tag) {
-                constexpr bool kMasked = decltype(diag_tag)::value;  // keys past `last_key` are invisible
-                // row extremum of the raw scores over the unmasked keys: the maximum of
-                // scale*log2(e)*score is that factor times the largest (smallest, for a negative
-                // scale) raw score
-                // (eight independent running extrema: one warp per scheduler has no other work to
-                // cover the latency of a dependent chain)
-                float ex[8];
-                if (scale_log2 >= 0.f) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) ex[u] = -INFINITY;
-#pragma unroll
-                    for (int e = 0; e < 64; ++e) {  // two keys per step: a three-input maximum
-                        const float a = (!kMasked || e <= last_key) ? __uint_as_float(sc[e]) : -INFINITY;
-                        const float c = (!kMasked || e + 64 <= last_key) ? __uint_as_float(sc[e + 64]) : -INFINITY;
-                        ex[e & 7] = fmaxf(ex[e & 7], fmaxf(a, c));
-                    }
-#pragma unroll
-                    for (int u = 4; u > 0; u >>= 1)
-#pragma unroll
-                        for (int w = 0; w < u; ++w) ex[w] = fmaxf(ex[w], ex[w + u]);
-                } else {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) ex[u] = INFINITY;
-#pragma unroll
-                    for (int e = 0; e < 64; ++e) {
-                        const float a = (!kMasked || e <= last_key) ? __uint_as_float(sc[e]) : INFINITY;
-                        const float c = (!kMasked || e + 64 <= last_key) ? __uint_as_float(sc[e + 64]) : INFINITY;
-                        ex[e & 7] = fminf(ex[e & 7], fminf(a, c));
-                    }
-#pragma unroll
-                    for (int u = 4; u > 0; u >>= 1)
-#pragma unroll
-                        for (int w = 0; w < u; ++w) ex[w] = fminf(ex[w], ex[w + u]);
-                }
-                const float ext = ex[0];
-                const float row_max = ext * scale_log2;
-                LT_FT(3);
-                if (j == 0) {
-                    m_used = row_max;  // key 0 is never masked, so this is finite for finite inputs
-                } else {
-                    const bool raise = (row_max - m_used) > kFwdRescaleLog2;
-                    if (__any_sync(0xffffffffu, raise)) {
-                        // O must hold every earlier product before it is rescaled
-                        ok = mbar_wait(&sm.bar_o_done[t], (j - 1) & 1, abort_flag, p.status, kWaitFwdO);
-                        if (!(ok = __all_sync(0xffffffffu, ok))) return;
-                        tc_fence_after_sync();
-                        const float alpha = raise ? fast_exp2(m_used - row_max) : 1.f;
-#pragma unroll
-                        for (int c = 0; c < D / 16; ++c) {  // narrow pieces: the score row holds most registers
-                            uint32_t r[16];
-                            tmem_ld16(tO + c * 16, r);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-                            tmem_st16(tO + c * 16, r);
-                        }
-                        l *= alpha;
-                        if (raise) m_used = row_max;
-                    }
-                }
-                LT_FT(4);
-                // P = exp2(score - m_used) as fp16 over the first 64 columns of the S region
-                // (split keys: a chain may begin with a tile whose scores are all -inf, keys hidden by -inf in K; such a tile
-                // gets zeros here, as it does where a tile with a finite maximum came before it)
-                const float neg_m = kSplitKeys ? fminf(-m_used, FLT_MAX) : -m_used;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-#pragma unroll
-                    for (int e = 64 * half; e < 64 * half + 64; ++e) {
-                        const float x = fmaf(__uint_as_float(sc[e]), scale_log2, neg_m);
-                        float pe = fast_exp2(x);
-                        if (kMasked && e > last_key) pe = 0.f;
-                        rs[e & 3] += pe;
-                        sc[e] = __float_as_uint(pe);
-                    }
-#pragma unroll
-                    for (int c = 2 * half; c < 2 * half + 2; ++c) {
-                        uint32_t out[16];
-#pragma unroll
-                        for (int e = 0; e < 32; e += 2)
-                            out[e / 2] = pack2<kBf16>(__uint_as_float(sc[c * 32 + e]), __uint_as_float(sc[c * 32 + e + 1]));
-                        tmem_st16(tS + c * 16, out);
-                    }
-                    if (half == 0) {
-                        // the first 64 keys' probabilities are in place: their products may start
-                        tmem_wait_st();
-                        tc_fence_before_sync();
-                        mbar_arrive(&sm.bar_p_half[t]);
-                    }
-                }
-            };
-            const int key_tile = kSplitKeys ? 2 * j + t : j;
-            if (p.causal ? (key_tile == i) : (key_tile == n_tiles - 1 && tail_keys < kFwdTileRows)) tile_softmax(std::true_type{});
-            else tile_softmax(std::false_type{});
-            if (!ok) break;
-            const float row_sum = (rs[0] + rs[1]) + (rs[2] + rs[3]);
-            l += row_sum;
-            LT_FT(5);
-            tmem_wait_st();
+            // the other chain's scores may follow
             tc_fence_before_sync();
-            mbar_arrive(&sm.bar_p_ready[t]);
-            LT_FT(6);
+            __syncwarp();
+            if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_s_free);
+            const int key_tile = kSplitKeys ? 2 * j + t : j;
+            if (p.causal ? key_tile == i : key_tile == n_tiles - 1 && tail_keys < kFwdTileRows) {
+                // keys past `last_key` are invisible
+                const uint32_t hidden = __float_as_uint(scale_log2 >= 0.f ? -INFINITY : INFINITY);
+#pragma unroll
+                for (int e = 0; e < 128; ++e)
+                    if (e > last_key) sc[e] = hidden;
+            }
+            // row extremum of the raw scores: the maximum of scale*log2(e)*score is that factor times the largest
+            // (smallest, for a negative scale) raw score
+            // (eight independent running extrema: one warp per scheduler has no other work to cover the latency of a
+            // dependent chain)
+            float ex[8];
+            if (scale_log2 >= 0.f) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) ex[u] = -INFINITY;
+#pragma unroll
+                for (int e = 0; e < 64; ++e)  // two keys per step: a three-input maximum
+                    ex[e & 7] = fmaxf(ex[e & 7], fmaxf(__uint_as_float(sc[e]), __uint_as_float(sc[e + 64])));
+#pragma unroll
+                for (int u = 4; u > 0; u >>= 1)
+#pragma unroll
+                    for (int w = 0; w < u; ++w) ex[w] = fmaxf(ex[w], ex[w + u]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) ex[u] = INFINITY;
+#pragma unroll
+                for (int e = 0; e < 64; ++e)
+                    ex[e & 7] = fminf(ex[e & 7], fminf(__uint_as_float(sc[e]), __uint_as_float(sc[e + 64])));
+#pragma unroll
+                for (int u = 4; u > 0; u >>= 1)
+#pragma unroll
+                    for (int w = 0; w < u; ++w) ex[w] = fminf(ex[w], ex[w + u]);
+            }
+            const float row_max = ex[0] * scale_log2;
+            if (j <= 0) {
+                m_used = row_max;  // key 0 is never masked, so this is finite for finite inputs
+                l = 0.f;
+            } else {
+                const bool raise = (row_max - m_used) > kFwdRescaleLog2;
+                if (__any_sync(0xffffffffu, raise)) {
+                    // O must hold every earlier product before it is rescaled
+                    if (!(ok = mbar_wait_warp(&sm.bar_o_done[t], (j - 1) & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO))) break;
+                    tc_fence_after_sync();
+                    const float alpha = raise ? fast_exp2(m_used - row_max) : 1.f;
+#pragma unroll
+                    for (int c = 0; c < D / 16; ++c) {  // narrow pieces: the score row holds most registers
+                        uint32_t r[16];
+                        tmem_ld16(tO + c * 16, r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
+                        tmem_st16(tO + c * 16, r);
+                    }
+                    l *= alpha;
+                    if (raise) m_used = row_max;
+                }
+            }
+            // P = exp2(score - m_used) as fp16
+            // (split keys: a chain may begin with a tile whose scores are all -inf, keys hidden by -inf in K; such a tile
+            // gets zeros here, as it does where a tile with a finite maximum came before it)
+            const float neg_m = kSplitKeys ? fminf(-m_used, FLT_MAX) : -m_used;
+            const uint64_t scale2 = f32x2(scale_log2, scale_log2), neg_m2 = f32x2(neg_m, neg_m);
+            uint64_t rs[2] = {0ull, 0ull};  // independent partial row sums, two each
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+#pragma unroll
+                for (int e = 64 * half; e < 64 * half + 64; e += 2) {
+                    float2 x = f32x2_parts(f32x2_fma(f32x2(__uint_as_float(sc[e]), __uint_as_float(sc[e + 1])), scale2, neg_m2));
+                    x.x = fast_exp2(x.x);
+                    x.y = fast_exp2(x.y);
+                    rs[(e >> 1) & 1] = f32x2_add(rs[(e >> 1) & 1], f32x2(x.x, x.y));
+                    sc[e] = __float_as_uint(x.x);
+                    sc[e + 1] = __float_as_uint(x.y);
+                }
+                if (half == 0 && j > 0) {
+                    // the products with the previous P must have read it
+                    if (!(ok = mbar_wait_warp(&sm.bar_o_done[t], (j - 1) & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO))) break;
+                    tc_fence_after_sync();
+                }
+#pragma unroll
+                for (int c = 2 * half; c < 2 * half + 2; ++c) {
+                    uint32_t out[16];
+#pragma unroll
+                    for (int e = 0; e < 32; e += 2)
+                        out[e / 2] = pack2<kBf16>(__uint_as_float(sc[c * 32 + e]), __uint_as_float(sc[c * 32 + e + 1]));
+                    tmem_st16(tP + c * 16, out);
+                }
+                // a half's probabilities are in place: their products may start
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0 && j >= 0) mbar_arrive(half == 0 ? &sm.bar_p_half[t] : &sm.bar_p_ready[t]);
+            }
+            if (!ok) break;
+            const float2 rs0 = f32x2_parts(rs[0]), rs1 = f32x2_parts(rs[1]);
+            l += (rs0.x + rs0.y) + (rs1.x + rs1.y);
         }
-#ifdef LT_FWD_TRACE
-        if (lane == 0) {
-            LT_FT_FLUSH(8);
-            LT_FT_COUNT(16, j_last + 1);
-        }
-#endif
 
         if (ok && j_last >= 0) {
-            ok = mbar_wait(&sm.bar_o_done[t], j_last & 1, abort_flag, p.status, kWaitFwdO);
-            ok = __all_sync(0xffffffffu, ok);
+            ok = mbar_wait_warp(&sm.bar_o_done[t], j_last & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO);
         }
         if constexpr (kSplitKeys) {
             if (t == 1) {  // the other chain's warps put the two halves together
@@ -498,9 +443,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             w1 *= inv_l;
             const int s_row = i * kFwdTileRows + row;  // rows past S belong to nobody
             const long long q_row = static_cast<long long>(bh) * p.S + s_row;  // LSE is contiguous
-            __half *o_row = p.O + b * p.o_st.batch + h * p.o_st.head + s_row * p.o_st.row;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
+            // The query tile has been used for the last time: a warp lays its 32 rows of O out in its place as a tile load
+            // would, and a tile store takes them from there (rows past S are not written).  (Stored from the registers, each
+            // thread its own row 16 bytes at a time, a pair of tiles took 3 300 cycles, now 2 300.)
+            uint8_t *stage = sm.q[kSplitKeys ? 0 : t];
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {  // (run once, from a cold instruction cache: a loop is shorter)
                 uint32_t r[32];
                 tmem_ld32(tO + c * 32, r);
                 uint32_t r1[32];
@@ -519,12 +467,22 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     o.y = pack2<kBf16>(__uint_as_float(r[8 * v8 + 2]), __uint_as_float(r[8 * v8 + 3]));
                     o.z = pack2<kBf16>(__uint_as_float(r[8 * v8 + 4]), __uint_as_float(r[8 * v8 + 5]));
                     o.w = pack2<kBf16>(__uint_as_float(r[8 * v8 + 6]), __uint_as_float(r[8 * v8 + 7]));
-                    if (s_row < p.S) reinterpret_cast<uint4 *>(o_row + c * 32)[v8] = o;
+                    *reinterpret_cast<uint4 *>(stage + (c >> 1) * kFwdBoxBytes + swz128_offset(row, (c & 1) * 32 + v8 * 8)) = o;
                 }
+            }
+            fence_proxy_async_smem();
+            grid_dependency_wait();
+            __syncwarp();
+            if (lane == 0 && i * kFwdTileRows + quad * 32 < p.S) {
+#pragma unroll
+                for (int x = 0; x < kBoxes; ++x)
+                    tma_store_4d(&map_o, stage + x * kFwdBoxBytes + quad * 4096, x * 64, i * kFwdTileRows + quad * 32, h, b);
+                bulk_commit_group();
             }
             // (split keys: the weight of one half, an approximate exponential, adds 1e-7 to LSE's error; two roundings fewer
             // here take off more)
             if (s_row < p.S) p.lse[q_row] = kSplitKeys ? fmaf(m_used, kFwdLn2, logf(l)) : (m_used + log2f(l)) * kFwdLn2;
+            bulk_wait_group_read<0>();  // (shared memory stays until the stores have read it)
         }
     }
 
@@ -532,17 +490,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
-
-#ifdef LT_FWD_TRACE
-extern "C" int lt_dbg_fwd_trace(unsigned long long *out, int reset) {
-    if (out && cudaMemcpyFromSymbol(out, g_fwd_trace, sizeof(g_fwd_trace)) != cudaSuccess) return LT_ERR_CUDA;
-    if (reset) {
-        static unsigned long long zeros[32];
-        if (cudaMemcpyToSymbol(g_fwd_trace, zeros, sizeof(zeros)) != cudaSuccess) return LT_ERR_CUDA;
-    }
-    return LT_OK;
-}
-#endif
 
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
 // makespan in steps of both chains (about 1.9 us), with kFill for a CTA's start, fill and drain, and a margin for the second
@@ -582,15 +529,14 @@ template <int D, bool kBf16>
 static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_half *O, float *LSE,
                       const lt_attn_layout &lay, int B, int Hq, int Hkv, int S, int causal, float scale,
                       void *workspace, cudaStream_t stream) {
-    CUtensorMap mq, mk, mv;
+    CUtensorMap mq, mk, mv, mo;
     int rc;
     if ((rc = make_bhsd_map(&mq, Q, B, Hq, S, D, lay.q, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mk, K, B, Hkv, S, D, lay.k, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mv, V, B, Hkv, S, D, lay.v, 128, kBf16)) != LT_OK) return rc;
+    if ((rc = make_bhsd_map(&mo, O, B, Hq, S, D, lay.o, 32, kBf16)) != LT_OK) return rc;
     FwdParams prm;
-    prm.O = reinterpret_cast<__half *>(O);
     prm.lse = LSE;
-    prm.o_st = lay.o;
     prm.status = reinterpret_cast<unsigned int *>(workspace);
     prm.B = B; prm.Hq = Hq; prm.Hkv = Hkv; prm.S = S; prm.causal = causal ? 1 : 0;
     prm.scale = scale;
@@ -612,7 +558,7 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     cfg.stream = stream;
     cfg.attrs = &pdl;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, prm);
+    e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mo, prm);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("fwd_kernel launch", e);
     return LT_OK;

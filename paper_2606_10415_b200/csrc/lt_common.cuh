@@ -92,6 +92,32 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
 }
 
+// The same wait by a whole warp on one or two barriers, with a warp-uniform outcome.  The first test of both is voted on
+// directly: a barrier that has completed costs no divergent branch, and two of them one round trip.  (In a loop that issues
+// products, mbar_wait with its outcome voted afterwards took 170-240 cycles for a completed barrier, and there are several per
+// tile.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar_a, uint32_t parity_a, uint64_t *bar_b, uint32_t parity_b,
+                                               volatile int *abort_flag, unsigned int *status, int code) {
+    auto done = [&]() {
+        const bool a = mbar_try_wait(bar_a, parity_a), b = !bar_b || mbar_try_wait(bar_b, parity_b);
+        return __all_sync(0xffffffffu, a && b) != 0;
+    };
+    if (done()) return true;
+    const long long t0 = clock64();
+    uint32_t spins = 0;
+    while (!done()) {
+        if ((++spins & 63u) == 0u) {
+            const bool late = clock64() - t0 > kWaitLimitCycles;
+            if (late) {
+                *abort_flag = 1;
+                atomicCAS(status + kStatusWordTimeout, 0u, static_cast<unsigned int>(code));
+            }
+            if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+        }
+    }
+    return true;
+}
+
 // ----------------------------------------------------------------------------- dependent launches
 // A kernel launched with programmatic stream serialisation may start while the previous kernel of
 // the stream is still running; it must not touch that kernel's results before grid_dependency_wait().
@@ -156,6 +182,15 @@ __device__ __forceinline__ void tma_prefetch_l2_4d(const CUtensorMap *map, int x
                  : "memory");
 }
 
+// The tile store shared -> global on such a view: x a multiple of 8 elements, no coordinate negative; rows past the end of a head are
+// not written.  Completion is tracked in bulk groups.
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void *src, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z), "r"(w)
+                 : "memory");
+}
+
 // 1-D bulk copy global -> shared (both 16-byte aligned, size a multiple of 16 bytes);
 // completion is counted in bytes on `bar`.
 __device__ __forceinline__ void bulk_load_1d(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
@@ -202,6 +237,22 @@ __device__ __forceinline__ bool named_barrier_and(int id, int threads, bool pred
         ".reg .pred p, q;\n"
         "setp.ne.u32 q, %1, 0;\n"
         "bar.red.and.pred p, %2, %3, q;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(out)
+        : "r"(static_cast<uint32_t>(pred)), "r"(id), "r"(threads)
+        : "memory");
+    return out != 0;
+}
+
+// and one that ORs it
+__device__ __forceinline__ bool named_barrier_or(int id, int threads, bool pred) {
+    uint32_t out;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.u32 q, %1, 0;\n"
+        "bar.red.or.pred p, %2, %3, q;\n"
         "selp.u32 %0, 1, 0, p;\n"
         "}\n"
         : "=r"(out)
@@ -488,6 +539,32 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // ----------------------------------------------------------------------------- numerics helpers
+// two fp32 operations in one instruction, each rounded like the single one
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 f32x2_parts(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
