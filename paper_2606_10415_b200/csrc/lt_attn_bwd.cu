@@ -444,15 +444,25 @@ __device__ __forceinline__ bool traced_wait(Trace &tr, uint64_t *bar, uint32_t p
     tr.acc[code - 200] += static_cast<unsigned int>(clock()) - t0;
     return r;
 }
+#define LT_WAIT_BOTH(bar_a, parity_a, bar_b, parity_b, code) \
+    traced_wait_warp(trace_, bar_a, parity_a, bar_b, parity_b, abort_flag, p.status, code)
+__device__ __forceinline__ bool traced_wait_warp(Trace &tr, uint64_t *bar_a, uint32_t parity_a, uint64_t *bar_b, uint32_t parity_b,
+                                                 volatile int *abort_flag, unsigned int *status, int code) {
+    const unsigned int t0 = static_cast<unsigned int>(clock());
+    const bool r = mbar_wait_warp(bar_a, parity_a, bar_b, parity_b, abort_flag, status, code);
+    tr.acc[code - 200] += static_cast<unsigned int>(clock()) - t0;
+    return r;
+}
 #else
 #define LT_TRACE_BEGIN()
 #define LT_TRACE_MARK(var)
 #define LT_TRACE_SINCE(slot, var)
 #define LT_TRACE_END(role)
 #define LT_WAIT(bar, parity, code) mbar_wait(bar, parity, abort_flag, p.status, code)
+#define LT_WAIT_BOTH(bar_a, parity_a, bar_b, parity_b, code) mbar_wait_warp(bar_a, parity_a, bar_b, parity_b, abort_flag, p.status, code)
 #endif
-// the same wait by every lane of a warp, with the outcome voted (warp-uniform)
-#define LT_WAIT_ALL(bar, parity, code) __all_sync(0xffffffffu, LT_WAIT(bar, parity, code))
+// the same wait by a whole warp, on one or two barriers (the second one may be NULL), with a warp-uniform outcome
+#define LT_WAIT_ALL(bar, parity, code) LT_WAIT_BOTH(bar, parity, nullptr, 0, code)
 
 // Built only with -DLT_BWD_TIMELINE=<cta> (development aid): clock stamps of that CTA's first 256 iterations.
 #ifdef LT_BWD_TIMELINE
@@ -979,9 +989,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     const int4 item = sm.item_ring[ic % kItemRing];
                     if (item.x < 0) break;
                     const BwdItem w = bwd_item<kSplit>(p, item);
-                    ok = LT_WAIT_ALL(&sm.bar_kv, ic & 1, kWaitKV) &&
-                         LT_WAIT_ALL(&sm.bar_q_full[it & 1], (it >> 1) & 1, kWaitStageFull);
-                    if (!ok) break;
+                    if (!(ok = LT_WAIT_BOTH(&sm.bar_kv, ic & 1, &sm.bar_q_full[it & 1], (it >> 1) & 1, kWaitKV))) break;
                     tc_fence_after_sync();
                     LT_TL(leader, 14, it);
                     if constexpr (!kSavedP) issue_s(it);
@@ -989,8 +997,6 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                         const int s = it & 1;
                         const uint64_t wb = window_base();
                         const uint64_t dQ_mn = wb + s * kQStageStep;
-                        // dO_i and the -delta rows have landed: both dP and dV read them
-                        if (!(ok = LT_WAIT_ALL(&sm.bar_do_full, it & 1, kWaitDoFull))) break;
                         // dP^T = V_j dO_i^T - delta_i   (its columns held the previous dQ partial until the
                         //                                reduce warps drained it)
                         auto issue_dp = [&]() {
@@ -1016,15 +1022,15 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                                         idesc_dv, (n > 0) | (kk > 0));
                         };
                         LT_TL(leader, 0, it);
-                        if (it > 0 && !(ok = LT_WAIT_ALL(&sm.bar_dq_empty, (it - 1) & 1, kWaitDqEmpty))) break;
+                        // dO_i and the -delta rows have landed (both dP and dV read them), the dQ partial has been drained
+                        if (!(ok = LT_WAIT_BOTH(&sm.bar_do_full, it & 1, it > 0 ? &sm.bar_dq_empty : nullptr, (it - 1) & 1, kWaitDqEmpty))) break;
                         tc_fence_after_sync();
                         LT_TL(leader, 1, it);
                         issue_dp();
                         LT_TL(leader, 2, it);
-                        if (!(ok = LT_WAIT_ALL(&sm.bar_p_ready, it & 1, kWaitPReady))) break;
+                        // (the first product of an item overwrites accumulators the previous item's epilogue reads)
+                        if (!(ok = LT_WAIT_BOTH(&sm.bar_p_ready, it & 1, n == 0 && ic > 0 ? &sm.bar_acc_free : nullptr, (ic - 1) & 1, kWaitPReady))) break;
                         LT_TL(leader, 3, it);
-                        // the first product of an item overwrites accumulators the previous item's epilogue reads
-                        if (n == 0 && ic > 0 && !(ok = LT_WAIT_ALL(&sm.bar_acc_free, (ic - 1) & 1, kWaitAccFree))) break;
                         tc_fence_after_sync();
                         issue_dv();
                         if (leader) umma_commit(&sm.bar_do_empty);
@@ -1082,6 +1088,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         uint8_t *ds_tile = sm.ds + half_sel * kBoxBytesBwd;
         uint32_t pv[64];  // bits of this thread's 64 fp32 values of P' = P * 2^c for the current tile pair
         const float p_scale_log2 = static_cast<float>(bwd_p_scale_log2<D>(p, sm.call_max, !kOneTile || !one.own_pre));
+        const uint64_t scale_log2_2 = f32x2(scale_log2, scale_log2), p_scale_log2_2 = f32x2(p_scale_log2, p_scale_log2);
         bool ok = smem_ok;
         int it = 0, ic = 0;
         LT_TRACE_BEGIN();
@@ -1106,7 +1113,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             constexpr bool kMasked = decltype(masked_tag)::value;
             if constexpr (kSavedP) {
                 // P'^T of the previous pair must have been read by its dV product before it is replaced
-                if (t > 0 && !LT_WAIT(&sm.bar_do_empty, (t - 1) & 1, kWaitDoEmpty)) return false;
+                if (t > 0 && !LT_WAIT_ALL(&sm.bar_do_empty, (t - 1) & 1, kWaitDoEmpty)) return false;
                 tc_fence_after_sync();
                 const uint32_t mult = pack_half2(exp2f(p_scale_log2), exp2f(p_scale_log2));  // 2^c <= 2^14
 #pragma unroll
@@ -1122,7 +1129,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if (lane == 0) mbar_arrive(&sm.bar_p_ready);
                 return true;
             }
-            if (!LT_WAIT(&sm.bar_s_full, t & 1, kWaitSFull)) return false;
+            if (!LT_WAIT_ALL(&sm.bar_s_full, t & 1, kWaitSFull)) return false;
             tc_fence_after_sync();
             LT_TL(tid == kComputeWarp0 * 32, 7, t);
             LT_TRACE_MARK(tp0);
@@ -1134,8 +1141,11 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 tmem_wait_ld();
                 // P' = exp2(scale*log2e * (K.Q - LSE/scale) + c)
 #pragma unroll
-                for (int e = 0; e < 32; ++e)
-                    pv[c * 32 + e] = __float_as_uint(fast_exp2(fmaf(__uint_as_float(sv[e]), scale_log2, p_scale_log2)));
+                for (int e = 0; e < 32; e += 2) {
+                    const float2 x = f32x2_parts(f32x2_fma(f32x2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), scale_log2_2, p_scale_log2_2));
+                    pv[c * 32 + e] = __float_as_uint(fast_exp2(x.x));
+                    pv[c * 32 + e + 1] = __float_as_uint(fast_exp2(x.y));
+                }
             }
             if (kMasked || (D == 128 && masked)) {
                 // the key row is hidden from the query columns before it (causal diagonal), or it lies past the end of
@@ -1174,7 +1184,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         };
 
         for (;; ++ic) {
-            if (!ok || !LT_WAIT(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem)) break;
+            if (!ok || !LT_WAIT_ALL(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem)) break;
             const int4 item = sm.item_ring[ic % kItemRing];
             if (item.x < 0) break;
             const BwdItem w = bwd_item<kSplit>(p, item);
@@ -1184,11 +1194,10 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             for (int n = 0; n < w.n_iter && ok; ++n, ++it) {
                 if constexpr (kSavedP)
                     if (n + 1 < w.n_iter) load_saved_p(w, n + 1, pn);
-                if (!(ok = LT_WAIT(&sm.bar_dp_full, it & 1, kWaitDpFull))) break;
+                // (the previous dS^T tile must have been consumed by the dQ product before it is overwritten)
+                if (!(ok = LT_WAIT_BOTH(&sm.bar_dp_full, it & 1, it > 0 ? &sm.bar_ds_free : nullptr, (it - 1) & 1, kWaitDpFull))) break;
                 tc_fence_after_sync();
                 LT_TL(tid == kComputeWarp0 * 32, 9, it);
-                // the previous dS^T tile must have been consumed by the dQ product before it is overwritten
-                if (it > 0 && !(ok = LT_WAIT(&sm.bar_ds_free, (it - 1) & 1, kWaitDsFree))) break;
                 LT_TRACE_MARK(td0);
                 const float saved_mult = kSavedP ? exp2f(p_scale_log2) : 0.f;
 #pragma unroll
@@ -1208,8 +1217,9 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                             o[e] = pack2<kBf16>(f.x * saved_mult * __uint_as_float(dp[2 * e]),
                                                 f.y * saved_mult * __uint_as_float(dp[2 * e + 1]));
                         } else {
-                            o[e] = pack2<kBf16>(__uint_as_float(pv[c * 32 + 2 * e]) * __uint_as_float(dp[2 * e]),
-                                                __uint_as_float(pv[c * 32 + 2 * e + 1]) * __uint_as_float(dp[2 * e + 1]));
+                            const float2 x = f32x2_parts(f32x2_mul(f32x2(__uint_as_float(pv[c * 32 + 2 * e]), __uint_as_float(pv[c * 32 + 2 * e + 1])),
+                                                                   f32x2(__uint_as_float(dp[2 * e]), __uint_as_float(dp[2 * e + 1]))));
+                            o[e] = pack2<kBf16>(x.x, x.y);
                         }
                     }
 #pragma unroll
@@ -1251,14 +1261,14 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         for (;; ++ic) {
             // the four reduction warps share named barriers (D = 128), so after every wait they vote
             // and leave together
-            ok = ok && LT_WAIT(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem);
+            ok = ok && LT_WAIT_ALL(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem);
             ok = named_barrier_and(kBarReduceWarps, kNumReduceWarps * 32, ok);
             if (!ok) break;
             const int4 item = sm.item_ring[ic % kItemRing];
             if (item.x < 0) break;
             const BwdItem w = bwd_item<kSplit>(p, item);
             for (int n = 0; n < w.n_iter; ++n, ++it) {
-                ok = LT_WAIT(&sm.bar_dq_full, it & 1, kWaitDqFull);
+                ok = LT_WAIT_ALL(&sm.bar_dq_full, it & 1, kWaitDqFull);
                 // The four reduction warps share named barriers below, so they leave the loop together.  The
                 // staging buffers form a ring that runs on across tile pairs (running group number gq): at
                 // most the last two reductions of the previous pair are still reading their buffers here,
@@ -1408,7 +1418,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (!ok) break;
             // item epilogue (these warps are idle while the pipeline of the next item fills):
             // dK_j and dV_j leave tensor memory as fp16; thread = key row
-            ok = LT_WAIT(&sm.bar_dkv_full, ic & 1, kWaitDkvFull);
+            ok = LT_WAIT_ALL(&sm.bar_dkv_full, ic & 1, kWaitDkvFull);
             ok = named_barrier_and(kBarReduceWarps, kNumReduceWarps * 32, ok);
             if (!ok) break;
             tc_fence_after_sync();
