@@ -1425,14 +1425,14 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             {
                 const int row = quad * 32 + lane;
                 const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
-#pragma unroll
+#pragma unroll 1  // (runs once per item, out of a cold instruction cache: shorter is faster)
                 for (int which = 0; which < 2; ++which) {
                     const float mult = which == 0 ? dq_mult : inv_p_scale;
                     const uint32_t col0 = which == 0 ? kColdK : kColdV;
                     const int s_row = w.j * kTileRows + row;  // rows past S are never stored
                     const lt_tensor_strides &st = which == 0 ? p.dk_st : p.dv_st;
                     __half *dst = (which == 0 ? p.dK : p.dV) + w.b * st.batch + w.g * st.head + s_row * st.row;
-#pragma unroll
+#pragma unroll 1
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t r[32];
                         tmem_ld32(tmem + lane_base + col0 + c * 32, r);

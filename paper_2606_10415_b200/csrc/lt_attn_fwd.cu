@@ -317,6 +317,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_s_free);
             const int key_tile = kSplitKeys ? 2 * j + t : j;
             if (p.causal ? key_tile == i : key_tile == n_tiles - 1 && tail_keys < kFwdTileRows) {
+                __syncwarp();  // (keeps the selects behind a branch)
                 // keys past `last_key` are invisible
                 const uint32_t hidden = __float_as_uint(scale_log2 >= 0.f ? -INFINITY : INFINITY);
 #pragma unroll

@@ -74,22 +74,30 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 // of time (it then raises *abort_flag and records `code` in the status block) or another
 // thread already raised the flag.  Callers leave their loops and go to the common
 // teardown when they see false.
+// (Every wait is expanded in place, a few dozen of them in a kernel whose loops together about fill the instruction cache:
+// hence the low halves of the clock, and the hint that moves the waiting out of the way.)
+static_assert(kWaitLimitCycles < 4000000000LL, "the limit is compared with a 32-bit difference");
+__device__ __forceinline__ uint32_t clock_low() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%clock;" : "=r"(t));
+    return t;
+}
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
                                           unsigned int *status, int code) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
+    if (__builtin_expect(mbar_try_wait(bar, parity), 1)) return true;
+    const uint32_t t0 = clock_low();
     uint32_t spins = 0;
-    while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
+    while (!mbar_try_wait(bar, parity)) {
         if ((++spins & 63u) == 0u) {
             if (*abort_flag) return false;
-            if (clock64() - t0 > kWaitLimitCycles) {
+            if (clock_low() - t0 > static_cast<uint32_t>(kWaitLimitCycles)) {
                 *abort_flag = 1;
                 atomicCAS(status + kStatusWordTimeout, 0u, static_cast<unsigned int>(code));
                 return false;
             }
         }
     }
+    return true;
 }
 
 // The same wait by a whole warp on one or two barriers, with a warp-uniform outcome.  The first test of both is voted on
@@ -102,12 +110,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar_a, uint32_t parity_
         const bool a = mbar_try_wait(bar_a, parity_a), b = !bar_b || mbar_try_wait(bar_b, parity_b);
         return __all_sync(0xffffffffu, a && b) != 0;
     };
-    if (done()) return true;
-    const long long t0 = clock64();
+    if (__builtin_expect(done(), 1)) return true;
+    const uint32_t t0 = clock_low();
     uint32_t spins = 0;
     while (!done()) {
         if ((++spins & 63u) == 0u) {
-            const bool late = clock64() - t0 > kWaitLimitCycles;
+            const bool late = clock_low() - t0 > static_cast<uint32_t>(kWaitLimitCycles);
             if (late) {
                 *abort_flag = 1;
                 atomicCAS(status + kStatusWordTimeout, 0u, static_cast<unsigned int>(code));
