@@ -697,8 +697,10 @@ template <int D, bool kBf16, bool kSplit, bool kSavedP = false, bool kOneTile = 
 __global__ void __launch_bounds__(kBwdThreads, 1)
 bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_do,
-                const BwdParams p, const __grid_constant__ CUtensorMap map_dq, const BwdOneTileParams one) {
+                const BwdParams p, const __grid_constant__ CUtensorMap map_dq, const __grid_constant__ CUtensorMap map_dk,
+                const __grid_constant__ CUtensorMap map_dv, const BwdOneTileParams one) {
     // map_dq (D = 64 only): the fp32 dQ accumulator as rows of 64 floats, boxes of 128 rows x 32 columns
+    // map_dk, map_dv: the outputs, boxes of 32 rows x 64 columns
     using Smem = BwdSmem<D>;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kTileBytes = kBoxes * kBoxBytesBwd;
@@ -1183,10 +1185,12 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             return form_p(w, t, diag, masked, std::false_type{});
         };
 
+        int last_item = -1;
         for (;; ++ic) {
-            if (!ok || !LT_WAIT_ALL(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem)) break;
+            if (!ok || !(ok = LT_WAIT_ALL(&sm.bar_item[ic % kItemRing], (ic / kItemRing) & 1, kWaitItem))) break;
             const int4 item = sm.item_ring[ic % kItemRing];
             if (item.x < 0) break;
+            last_item = item.x;
             const BwdItem w = bwd_item<kSplit>(p, item);
             if constexpr (kSavedP) load_saved_p(w, 0, ph);
             int tile = kSplit ? w.n_first % w.tiles_per_head : 0;
@@ -1245,6 +1249,47 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if (n + 1 < w.n_iter) ok = compute_p(w, it + 1, tile);
             }
 
+        }
+        // dK_j and dV_j of the CTA's last item leave through these warps, which have nothing else left to do, while the reduction
+        // warps bring the last dQ partial out.  They are laid out in place of K_j and V_j, as a tile load would, for tile stores.
+        // (Behind that partial, by the reduction warps alone and from their registers, each thread its own row 16 bytes at a time,
+        // they took 7 500 cycles from the last product: 45.0 -> 44.0 us for 32 heads of 1 024, 13.2 -> 12.3 for 16 of 64, D = 128.)
+        // (Not where key tiles are split: 40/8 heads of 2 048 139.8 instead of 136.8 us.)
+        if (!kSplit && ok && ic > 0 && (ok = LT_WAIT_ALL(&sm.bar_dkv_full, (ic - 1) & 1, kWaitDkvFull))) {
+            tc_fence_after_sync();
+            const BwdItem w = bwd_item<false>(p, make_int4(last_item, 0, 0, 0));
+            const float inv_p_scale = exp2f(-p_scale_log2);
+            const float mult = half_sel == 0 ? p.scale * inv_p_scale : inv_p_scale;  // half of the warps takes dK, the others dV
+            const uint32_t acc = tmem + lane_base + (half_sel == 0 ? kColdK : kColdV);
+            uint8_t *stage = half_sel == 0 ? sm.k : sm.v;
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t r[32];
+                tmem_ld32(acc + c * 32, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int v8 = 0; v8 < 4; ++v8) {
+                    uint32_t o[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        o[e] = pack2<kBf16>(__uint_as_float(r[8 * v8 + 2 * e]) * mult, __uint_as_float(r[8 * v8 + 2 * e + 1]) * mult);
+                    *reinterpret_cast<uint4 *>(stage + (c >> 1) * kBoxBytesBwd + swz128_offset(row, (c & 1) * 32 + v8 * 8)) =
+                        make_uint4(o[0], o[1], o[2], o[3]);
+                }
+            }
+            const int row0 = w.j * kTileRows + quad * 32;
+            if (row0 < p.S) {  // (rows past S are not written)
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    const CUtensorMap *map = half_sel == 0 ? &map_dk : &map_dv;
+#pragma unroll
+                    for (int x = 0; x < kBoxes; ++x)
+                        tma_store_4d(map, stage + x * kBoxBytesBwd + quad * 4096, x * 64, row0, w.g, w.b);
+                    bulk_commit_group();
+                    bulk_wait_group_read<0>();  // (shared memory stays until the stores have read it)
+                }
+            }
         }
         LT_TRACE_END(kRoleCompute);
     } else {
@@ -1416,11 +1461,12 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 LT_TRACE_SINCE(13, tr0);
             }
             if (!ok) break;
-            // item epilogue (these warps are idle while the pipeline of the next item fills):
+            // item epilogue (these warps are idle while the pipeline of the next item fills; the last item's is the softmax warps'):
             // dK_j and dV_j leave tensor memory as fp16; thread = key row
-            ok = LT_WAIT_ALL(&sm.bar_dkv_full, ic & 1, kWaitDkvFull);
+            ok = LT_WAIT_BOTH(&sm.bar_dkv_full, ic & 1, kSplit ? nullptr : &sm.bar_item[(ic + 1) % kItemRing], ((ic + 1) / kItemRing) & 1, kWaitDkvFull);
             ok = named_barrier_and(kBarReduceWarps, kNumReduceWarps * 32, ok);
             if (!ok) break;
+            if (!kSplit && sm.item_ring[(ic + 1) % kItemRing].x < 0) continue;
             tc_fence_after_sync();
             {
                 const int row = quad * 32 + lane;
@@ -1629,12 +1675,14 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     if (!saved_p) deal = deal_pairs(B, Hq, Hkv, S, D, causal, workspace_bytes - base_bytes);
     const bool split = deal.any();
 
-    CUtensorMap mq, mk, mv, mdo;
+    CUtensorMap mq, mk, mv, mdo, mdk, mdv;
     int rc;
     if ((rc = make_bhsd_map(&mq, Q, B, Hq, S, D, lay.q, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mdo, dO, B, Hq, S, D, lay.d_o, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mk, K, B, Hkv, S, D, lay.k, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mv, V, B, Hkv, S, D, lay.v, 128, kBf16)) != LT_OK) return rc;
+    if ((rc = make_bhsd_map(&mdk, dK, B, Hkv, S, D, lay.dk, 32, kBf16)) != LT_OK) return rc;
+    if ((rc = make_bhsd_map(&mdv, dV, B, Hkv, S, D, lay.dv, 32, kBf16)) != LT_OK) return rc;
 
     // programmatic stream serialisation: each kernel may start before its predecessor has finished and
     // waits inside for it (grid_dependency_wait).  The conversion kernels do not let the next call's preprocess
@@ -1722,7 +1770,7 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     CUtensorMap mdq = mq;  // (D = 128 never touches it)
     if constexpr (D == 64)
         if ((rc = make_f32_tile_map(&mdq, dq_acc, static_cast<uint64_t>(n_rows), 64, 128)) != LT_OK) return rc;
-    e = cudaLaunchKernelEx(&cfg_main, main_kernel, mq, mk, mv, mdo, prm, mdq, one);
+    e = cudaLaunchKernelEx(&cfg_main, main_kernel, mq, mk, mv, mdo, prm, mdq, mdk, mdv, one);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return record_cuda_error("bwd_main_kernel launch", e);
     if (ev_main_end && (e = cudaEventRecord(ev_main_end, stream)) != cudaSuccess)
