@@ -493,26 +493,26 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
 }
 
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
-// makespan in steps of both chains (about 1.9 us), with kFill for a CTA's start, fill and drain, and a margin for the second
-// softmax's merge.  On 860 shapes near the line, both ways measured, it is 0.04 % behind the faster one on average and 7 % at
-// worst (without the margin and the second round 0.9 % and 30 %: 64 heads of 267 12.3 / 16.0).
-// us, pairs of tiles / split keys (heads, S): 8, 2048 33.9 / 21.5; 4, 8000
-// 112.8 / 64.7; 16, 512 13.4 / 10.0; 32, 1024 22.4 / 21.4; 16, 753 unmasked 17.5 / 12.5; on the other side 64, 640
-// 19.4 / 21.2; 40, 1920 53.9 / 60.0; 32, 4096 141.7 / 163.2; 16, 3743 60.4 / 70.3; 64 of 442, D = 64 13.1 / 15.6.
+// makespan in steps of both chains (about 1.6 us), with kFill for a CTA's start, fill and drain, kMerge for putting two
+// softmaxes together, and a margin.  On 260 shapes near the line, both ways measured, it is 0.4 % behind the faster one on
+// average and 18 % at worst (with the constants of the kernel whose chains had a region of scores each, 1.3 % and 31 %).
+// us, pairs of tiles / split keys (heads, S): 8, 2080 31.2 / 20.2; 4, 5248 73.5 / 44.1; 15, 640 12.5 / 11.4; 14, 1038 unmasked
+// 20.8 / 14.7; 32, 1024 19.0 / 19.2; on the other side 31, 640 12.1 / 13.1; 44, 612 12.6 / 16.3; 60, 640 19.8 / 26.3; 19, 2432
+// 35.6 / 39.2; 33, 5329 221 / 250; 54 of 462 unmasked 13.0 / 18.8.
 static bool splits_keys(int B, int Hq, int S, int causal) {
     constexpr int kSms = 148;
-    constexpr double kFill = 2.2;
+    constexpr double kFill = 1.9, kMerge = 0.6;
     const double heads = static_cast<double>(B) * Hq;
     const int n = (S + kFwdTileRows - 1) / kFwdTileRows, pairs = (n + 1) / 2;
     if (n < 2) return false;
     // walk(q): steps of a head's q-th heaviest CTA
-    auto span = [&](int per_head, double head_steps, auto walk) {
-        const double ctas = heads * per_head, longest = walk(0) + kFill;
+    auto span = [&](int per_head, double head_steps, double fill, auto walk) {
+        const double ctas = heads * per_head, longest = walk(0) + fill;
         if (!causal) return ceil(ctas / kSms) * longest;  // walks of one length: whole rounds
-        double t = (heads * head_steps + kFill * ctas) / kSms;
+        double t = (heads * head_steps + fill * ctas) / kSms;
         if (t < longest) t = longest;
         if (ctas > kSms) {  // heavy CTAs first: one SM gets the last of the first round and the first of the second, or lighter ones
-            const double two = walk(static_cast<int>((kSms - 1) / heads)) + walk(static_cast<int>(kSms / heads)) + 2. * kFill;
+            const double two = walk(static_cast<int>((kSms - 1) / heads)) + walk(static_cast<int>(kSms / heads)) + 2. * fill;
             if (t < two) t = two;
         }
         return t;
@@ -521,9 +521,9 @@ static bool splits_keys(int B, int Hq, int S, int causal) {
     const double pair_steps = static_cast<double>(pairs) * (pairs + 1) - (n & 1 ? 1 : 0);
     const double half = (n + 1) / 2, even = n / 2;
     const double split_steps = half * (half + 1) / 2 + even * (even + 1) / 2;
-    const double split = span(n, split_steps, [&](int q) { return static_cast<double>(causal ? (n - q + 1) / 2 : (n + 1) / 2); });
-    const double whole = span(pairs, pair_steps, [&](int q) { return static_cast<double>(causal && q > 0 ? 2 * (pairs - q) : n); });
-    return split < (causal ? 0.92 : 0.95) * whole;
+    const double split = span(n, split_steps, kFill + kMerge, [&](int q) { return static_cast<double>(causal ? (n - q + 1) / 2 : (n + 1) / 2); });
+    const double whole = span(pairs, pair_steps, kFill, [&](int q) { return static_cast<double>(causal && q > 0 ? 2 * (pairs - q) : n); });
+    return split < (causal ? 0.91 : 0.95) * whole;
 }
 
 template <int D, bool kBf16>
