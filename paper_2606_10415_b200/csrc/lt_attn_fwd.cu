@@ -48,7 +48,7 @@ struct __align__(1024) FwdSmem {
     static constexpr int kSlots = D == 128 ? 5 : 8;
     uint8_t kv[kSlots][kTile];   // ring of key and value tiles, in the order of their use
     uint64_t bar_q[2], bar_kv_full[kSlots], bar_kv_empty[kSlots];
-    uint64_t bar_s_full[2], bar_s_free, bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_done, bar_merge;
+    uint64_t bar_s_full[2], bar_s_free, bar_p_ready[2], bar_p_half[2], bar_o_done[2], bar_exp[4], bar_done, bar_merge;
     float2 merge[kFwdTileRows];  // (split keys) maximum and sum of the odd key tiles' half, per query row
     uint32_t tmem_base;
     int abort_flag;
@@ -70,19 +70,20 @@ struct FwdParams {
 // grids that leave multiprocessors idle or wait for a few long walks: splits_keys().
 //
 // What bounds it: the exponential unit, 1 024 cycles per tile of 128 x 128 scores, with the softmax warps' other work (load,
-// maximum, store, hand-offs: about 1 300 cycles a tile) that two warps per scheduler hide only in part; a step of both
-// chains takes about 3 100 cycles, the exponential unit and the tensor cores (2 048 cycles a step at D = 128) are each
-// busy for two thirds of it, and in long runs the power limit.  Hence the layout of tensor memory: the softmax warps hold
+// maximum, store, hand-offs: about 1 300 cycles a tile) that two warps per scheduler hide only in part, although they take
+// turns at it; a step of both chains takes about 3 000 cycles, the exponential unit and the tensor cores (2 048 cycles a step
+// at D = 128) are each busy for two thirds of it, and in long runs the power limit.  Hence the layout of tensor memory: the softmax warps hold
 // a tile's scores in registers as soon as they are there, so the chains share one region of scores and P has columns of its
 // own; a chain's next scores are formed under its softmax instead of behind its product P V.  (With S and P of a chain in one
 // region a step took 3 600 cycles, most of it the chain softmax -> P V -> S.)  Measured, us, a region per chain / this
-// (heads, S, D; causal unless noted; single calls): 32, 4096, 128 145 / 131; 32, 1024, 128 22.4 / 20.1; 32, 3000, 128 92.5 / 82;
-// 64 of 1531, 64 unmasked 79.4 / 77.7; 64/8 heads of 8192 unmasked 1740 / 1690.
+// (heads, S, D; causal unless noted; single calls): 32, 4096, 128 145 / 131; 32, 1024, 128 22.4 / 20.0; 32, 3000, 128 92.5 / 82.6;
+// 64 of 1531, 64 unmasked 79.4 / 77.6; 64/8 heads of 8192 unmasked 1740 / 1662; with turns at the exponential unit 127.3, 18.9, 79.7,
+// 71.5 and 1 604 (40 heads of 1 920 lose by them, 50.1 / 51.1).
 // Tried: two warps per row and tile, 16 softmax warps with a vote on the maximum (11 % slower: they wait for each other);
 // the maximum found during the first quarter's exponentials (3 % slower); both chains started at once (2 %
 // slower: they stay in step and want the exponential unit together); a fifth of the exponentials as polynomials (no gain at
 // this share of the unit's time).
-template <int D, bool kBf16, bool kSplitKeys>
+template <int D, bool kBf16, bool kSplitKeys, bool kOneCopy>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
            const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o, const FwdParams p) {
@@ -116,7 +117,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     // last step of chain t (a key tile; split keys: key tile 2 j + t); -1 when there is no second chain
     const int j_last0 = kSplitKeys ? (n_keys + 1) / 2 - 1 : n_keys - 1;
     const int j_last1 = kSplitKeys ? n_keys / 2 - 1 : has_b ? (p.causal ? i0 + 1 : n_tiles - 1) : -1;
-    const int j_end = j_last0 > j_last1 ? j_last0 : j_last1;
     const int n_q = kSplitKeys ? 1 : has_b ? 2 : 1;              // query tiles
 
     if (tid == 0) {
@@ -134,6 +134,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             mbar_init(&sm.bar_kv_empty[x], 1);
         }
         mbar_init(&sm.bar_s_free, 4);
+        for (int x = 0; x < 4; ++x) mbar_init(&sm.bar_exp[x], 1);
         mbar_init(&sm.bar_done, 1);
         mbar_init(&sm.bar_merge, 128);
         mbar_fence_init();
@@ -157,26 +158,53 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     // The tensor-core work in its order: score products are numbered by (step, chain); number m is issued when the softmax
     // warps hold the scores of number m - 1 in registers, the products with V of number m - 2 come behind it.  on_s and
     // on_pv get (step, chain, whether it is the first and the last to use the step's key or value tile) and return false to leave.
+    // (Behind the end of the first chain of a pair, its last product with V goes ahead, so that its output can be stored.)
+    // Two forms of the same walk (launch_fwd has the rule).  One loop with one copy of either kind of work is a sixth of the code: it is the faster one at
+    // D = 64, and at D = 128 where an SM runs one or two CTAs of short walks out of a cold instruction cache; unrolled over the
+    // chains, with the chain a constant, a product takes fewer instructions to issue, which counts where products are twice as
+    // long and many.  us, one copy / unrolled (heads, S, D): 32, 1024, 128 17.9 / 18.9; 128 of 333, 64 15.8 / 16.8; 32, 4096, 64
+    // 106.7 / 108.0; on the other side 32, 4096, 128 140.5 / 137.5; 128 / 16 of 4 096, 128 534 / 509; 4, 8000, 128 63.6 / 61.4.
     auto walk = [&](auto on_s, auto on_pv) -> bool {
         auto first = [&](int j, int t) { return kSplitKeys || t == (j <= j_last0 ? 0 : 1); };
         auto last = [&](int j, int t) { return kSplitKeys || t == (j <= j_last1 ? 1 : 0); };
-        int m = 0, j1 = 0, t1 = 0, j2 = 0, t2 = 0;  // numbers m - 1 and m - 2
-        for (int j = 0; j <= j_end; ++j) {
+        if constexpr (!kOneCopy) {
+            int m = 0, j1 = 0, t1 = 0, j2 = 0, t2 = 0;  // numbers m - 1 and m - 2
+            const int j_end = j_last0 > j_last1 ? j_last0 : j_last1;
+            for (int j = 0; j <= j_end; ++j) {
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                if (j > (t == 0 ? j_last0 : j_last1)) continue;
-                // (behind the end of the first chain, its last product with V goes ahead, so that its output can be stored)
-                const bool ahead = !kSplitKeys && j > j_last0;
-                if (ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
-                if (!on_s(m, j, t, first(j, t), last(j, t))) return false;
-                if (!ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
-                j2 = j1; t2 = t1;
-                j1 = j; t1 = t;
-                ++m;
+                for (int t = 0; t < 2; ++t) {
+                    if (j > (t == 0 ? j_last0 : j_last1)) continue;
+                    const bool ahead = !kSplitKeys && j > j_last0;
+                    if (ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+                    if (!on_s(m, j, t, first(j, t), last(j, t))) return false;
+                    if (!ahead && m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+                    j2 = j1; t2 = t1;
+                    j1 = j; t1 = t;
+                    ++m;
+                }
+            }
+            if (m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
+            return on_pv(j1, t1, first(j1, t1), last(j1, t1));
+        }
+        const int n = j_last0 + j_last1 + 2;
+        int s = 0, sj = 0, st = 0, v = 0, vj = 0, vt = 0;  // next score product, next product with V
+        auto advance = [&](int &j, int &t) {
+            if (t == 0 && j <= j_last1) { t = 1; return; }
+            ++j;
+            t = j <= j_last0 ? 0 : 1;
+        };
+        while (v < n) {
+            if (s < n && s - v <= (!kSplitKeys && sj > j_last0 ? 1 : 2)) {
+                if (!on_s(s, sj, st, first(sj, st), last(sj, st))) return false;
+                advance(sj, st);
+                ++s;
+            } else {
+                if (!on_pv(vj, vt, first(vj, vt), last(vj, vt))) return false;
+                advance(vj, vt);
+                ++v;
             }
         }
-        if (m >= 2 && !on_pv(j2, t2, first(j2, t2), last(j2, t2))) return false;
-        return on_pv(j1, t1, first(j1, t1), last(j1, t1));
+        return true;
     };
     if (warp < kFwdSoftmaxWarp0) {
         warpgroup_regs_set<kFwdRegsControl, kFwdRegsAtLaunch>();
@@ -221,7 +249,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             auto wait_all = [&](uint64_t *bar, uint32_t parity, uint64_t *bar_b, uint32_t parity_b, int code) {
                 return mbar_wait_warp(bar, parity, bar_b, parity_b, abort_flag, p.status, code);
             };
-            constexpr uint64_t kSlotStep = static_cast<uint64_t>(kTileBytes) >> 4;
+            constexpr uint32_t kSlotStep = kTileBytes >> 4;  // (products with a slot number are 32-bit ones)
             int slot = 0, round = 0;  // the ring's next tile
             int k_slot = 0, k_round = 0, v_slot = 0, v_round = 0;  // the tiles in use
             auto next_tile = [&](bool first, int &mine, int &mine_round) {
@@ -245,7 +273,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                         if (!wait_all(&sm.bar_kv_full[k_slot], k_round & 1, m > 0 ? &sm.bar_s_free : nullptr, (m - 1) & 1, kWaitFwdSFree)) return false;
                         tc_fence_after_sync();
                         if (leader) {
-                            const uint64_t dQ = dQ0 + (kSplitKeys ? 0 : t) * kSlotStep, dK = dK0 + k_slot * kSlotStep;
+                            const uint64_t dQ = dQ0 + static_cast<uint32_t>(kSplitKeys ? 0 : t) * kSlotStep, dK = dK0 + static_cast<uint32_t>(k_slot) * kSlotStep;
 #pragma unroll
                             for (int kk = 0; kk < D / 16; ++kk) umma_ss(tmem + kColS, dQ + koff(kk), dK + koff(kk), idesc_s, kk > 0);
                             umma_commit(&sm.bar_s_full[t]);
@@ -258,7 +286,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                         // first half's products run while the softmax warps exponentiate the second half (quarters were
                         // measured too and lost to the extra hand-offs)
                         next_tile(first, v_slot, v_round);
-                        const uint64_t dV = dV0 + v_slot * kSlotStep;
+                        const uint64_t dV = dV0 + static_cast<uint32_t>(v_slot) * kSlotStep;
 #pragma unroll
                         for (int half = 0; half < 2; ++half) {
                             if (!wait_all(half == 0 ? &sm.bar_p_half[t] : &sm.bar_p_ready[t], j & 1, half == 0 ? &sm.bar_kv_full[v_slot] : nullptr,
@@ -380,10 +408,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             const float neg_m = kSplitKeys ? fminf(-m_used, FLT_MAX) : -m_used;
             const uint64_t scale2 = f32x2(scale_log2, scale_log2), neg_m2 = f32x2(neg_m, neg_m);
             uint64_t rs[2] = {0ull, 0ull};  // independent partial row sums, two each
+            auto exponentials = [&](int e0, int e1) {
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-#pragma unroll
-                for (int e = 64 * half; e < 64 * half + 64; e += 2) {
+                for (int e = e0; e < e1; e += 2) {
                     float2 x = f32x2_parts(f32x2_fma(f32x2(__uint_as_float(sc[e]), __uint_as_float(sc[e + 1])), scale2, neg_m2));
                     x.x = fast_exp2(x.x);
                     x.y = fast_exp2(x.y);
@@ -391,11 +418,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     sc[e] = __float_as_uint(x.x);
                     sc[e + 1] = __float_as_uint(x.y);
                 }
-                if (half == 0 && j > 0) {
-                    // the products with the previous P must have read it
-                    if (!(ok = mbar_wait_warp(&sm.bar_o_done[t], (j - 1) & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO))) break;
-                    tc_fence_after_sync();
-                }
+            };
+            auto store_half = [&](int half) {
 #pragma unroll
                 for (int c = 2 * half; c < 2 * half + 2; ++c) {
                     uint32_t out[16];
@@ -404,13 +428,30 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                         out[e / 2] = pack2<kBf16>(__uint_as_float(sc[c * 32 + e]), __uint_as_float(sc[c * 32 + e + 1]));
                     tmem_st16(tP + c * 16, out);
                 }
-                // a half's probabilities are in place: their products may start
-                tmem_wait_st();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0 && j >= 0) mbar_arrive(half == 0 ? &sm.bar_p_half[t] : &sm.bar_p_ready[t]);
-            }
-            if (!ok) break;
+            };
+            // The two warps of a scheduler take turns at the exponential unit, in the order of the score products, so that one
+            // chain's exponentials run beside the other's loads, maxima and hand-offs; the turn passes on a little before the
+            // last ones (after 112 of 128 keys; 96 measures the same), which covers the hand-off.  (Before the first store the
+            // products with the previous P must have read it, too.)
+            const int m = j + (t == 0 ? min(j, j_last1 + 1) : min(j, j_last0) + 1);
+            if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1, abort_flag, p.status, kWaitFwdO))) break;
+            tc_fence_after_sync();
+            exponentials(0, 64);
+            store_half(0);
+            exponentials(64, 112);
+            __syncwarp();
+            if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_exp[quad]);
+            // a half's probabilities are in place: their products may start
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_p_half[t]);
+            exponentials(112, 128);
+            store_half(1);
+            tmem_wait_st();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_p_ready[t]);
             const float2 rs0 = f32x2_parts(rs[0]), rs1 = f32x2_parts(rs[1]);
             l += (rs0.x + rs0.y) + (rs1.x + rs1.y);
         }
@@ -544,11 +585,15 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     // at least 120 KB, so that one CTA (which takes all 512 tensor-memory columns) lives on an SM
     const size_t smem = std::max<size_t>(sizeof(FwdSmem<D>) + 1024, 120 * 1024);
     const bool split = splits_keys(B, Hq, S, causal);
-    auto kernel = split ? fwd_kernel<D, kBf16, true> : fwd_kernel<D, kBf16, false>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(fwd)", e);
     const int n_tiles = (S + kFwdTileRows - 1) / kFwdTileRows;
     const int grid = B * Hq * (split ? n_tiles : (n_tiles + 1) / 2);
+    // the issuing warp's walk in one copy (figures beside the walk): D = 64, and one or two CTAs of up to 24 products per SM
+    const bool one_copy = D == 64 || (grid <= 2 * 148 && n_tiles * (split ? 1 : 2) <= 24);
+    auto kernel = split ? fwd_kernel<D, kBf16, true, true> : fwd_kernel<D, kBf16, false, true>;
+    if constexpr (D == 128)
+        if (!one_copy) kernel = split ? fwd_kernel<D, kBf16, true, false> : fwd_kernel<D, kBf16, false, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(fwd)", e);
     cudaLaunchAttribute pdl;
     pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl.val.programmaticStreamSerializationAllowed = 1;
