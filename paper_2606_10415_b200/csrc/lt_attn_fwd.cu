@@ -380,7 +380,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             }
             const float row_max = ex[0] * scale_log2;
             if (j <= 0) {
-                m_used = row_max;  // key 0 is never masked, so this is finite for finite inputs
+                m_used = row_max;  // a chain's first key tile has a visible key, so this is finite for finite inputs
                 l = 0.f;
             } else {
                 const bool raise = (row_max - m_used) > kFwdRescaleLog2;
@@ -403,9 +403,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                 }
             }
             // P = exp2(score - m_used) as fp16
-            // (split keys: a chain may begin with a tile whose scores are all -inf, keys hidden by -inf in K; such a tile
-            // gets zeros here, as it does where a tile with a finite maximum came before it)
-            const float neg_m = kSplitKeys ? fminf(-m_used, FLT_MAX) : -m_used;
+            // (a chain may begin with a tile whose scores are all -inf, keys hidden by -inf in K; such a tile gets zeros here, as
+            // it does where a tile with a finite maximum came before it)
+            const float neg_m = fminf(-m_used, FLT_MAX);
             const uint64_t scale2 = f32x2(scale_log2, scale_log2), neg_m2 = f32x2(neg_m, neg_m);
             uint64_t rs[2] = {0ull, 0ull};  // independent partial row sums, two each
             auto exponentials = [&](int e0, int e1) {

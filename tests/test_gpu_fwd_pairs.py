@@ -1,6 +1,6 @@
 """Forward whose CTAs take pairs of query tiles (many heads): a lone last tile, walks shorter and longer than the ring of
-key and value tiles, ragged ends, both masks, maxima that rise late, keys hidden by -inf, and an output between other
-columns and rows that must stay as they are; against fp64 softmax."""
+key and value tiles, ragged ends, both masks, maxima that rise late, keys hidden by -inf (the first tile's among them, as
+left padding has it), and an output between other columns and rows that must stay as they are; against fp64 softmax."""
 import pytest
 import torch
 
@@ -9,7 +9,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("S,D", [(1, 64), (127, 128), (129, 64), (257, 128), (384, 64), (511, 128), (700, 64), (897, 128)])
 @pytest.mark.parametrize("causal", [True, False])
-@pytest.mark.parametrize("dtype,kind", [(torch.float16, "plain"), (torch.bfloat16, "plain"), (torch.float16, "ramp"), (torch.float16, "hidden")])
+@pytest.mark.parametrize("dtype,kind", [(torch.float16, "plain"), (torch.bfloat16, "plain"), (torch.float16, "ramp"), (torch.float16, "hidden"),
+                                        (torch.float16, "hidden first"), (torch.bfloat16, "hidden first")])
 def test_query_pairs(S, D, causal, dtype, kind):
     from paper_2606_10415_b200 import binding as lt
     B, H, Hkv = 3, 64, 16
@@ -20,9 +21,9 @@ def test_query_pairs(S, D, causal, dtype, kind):
     if kind == "ramp":  # scores that grow along the keys: the output is rescaled
         K = K * (0.2 + 0.8 * tile).view(1, 1, S, 1)
     Q, K, V = (t.to(dtype) for t in (Q, K, V))
-    if kind == "hidden":  # every key of the odd key tiles
+    if kind in ("hidden", "hidden first"):  # every key of the odd key tiles, or of the first one
         Q[..., 0] = 1.0
-        K[:, :, tile % 2 == 1, 0] = float("-inf")
+        K[:, :, tile % 2 == 1 if kind == "hidden" else tile == 0, 0] = float("-inf")
     around = torch.full((B, S + 2, (H + 2) * D), 7.0, dtype=dtype, device="cuda")
     O = around.view(B, S + 2, H + 2, D).permute(0, 2, 1, 3)[:, 1:H + 1, 1:S + 1]
     LSE = torch.full((B, H, S), float("nan"), device="cuda")
@@ -37,9 +38,11 @@ def test_query_pairs(S, D, causal, dtype, kind):
         if causal:
             s.masked_fill_(torch.ones(S, S, dtype=torch.bool, device="cuda").triu(1), float("-inf"))
         lse = torch.logsumexp(s, -1)
-        ref = torch.exp(s - lse[..., None]) @ v
+        sees = torch.isfinite(lse)  # (a row without a visible key has no output)
+        ref, lse, got, got_lse = (torch.exp(s - lse[..., None]) @ v)[sees], lse[sees], O[b][sees].double(), LSE[b][sees].double()
+        assert torch.isfinite(got).all()
         # the forward's gates: rounding of P and O, 2^-11 (fp16) or 2^-8 (bf16) each, in the 2-norm
-        assert (O[b].double() - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
-        assert ((LSE[b].double() - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
+        assert (got - ref).norm() <= (2e-3 if dtype == torch.float16 else 4e-3) * ref.norm()
+        assert ((got_lse - lse).abs() <= 1e-3 + 2.0 ** -22 * lse.abs()).all()
     O.fill_(7.0)
     assert (around == 7.0).all()  # nothing but O was written
