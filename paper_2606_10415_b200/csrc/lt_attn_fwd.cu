@@ -330,8 +330,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         float l = 0.f;             // running sum of exp2(score - m_used)
         bool ok = true;
         // Pass -1 works on whatever tensor memory holds and leaves nothing behind: it brings the loop's instructions into the
-        // instruction cache while the first tiles are on their way (a first tile took 3 400 cycles instead of 1 450).
-        for (int j = t == 0 ? -1 : 0; j <= j_last; ++j) {
+        // instruction cache while the first tiles are on their way (a first tile took 3 400 cycles instead of 1 450).  Only where
+        // walks are long and many: it takes longer than the tiles do, and short walks wait for it.  us, with it / without (heads, S,
+        // D): 8, 192, 64 6.02 / 5.46; 128 of 333, 64 15.7 / 15.0; 32, 4096, 64 107.8 / 106.1; 8, 192, 128 6.68 / 6.33; 20, 2048, 128
+        // 32.4 / 31.1; on the other side 32, 3000, 128 86.3 / 87.4; 128 / 16 of 4 096, 128 528 / 534.
+        constexpr bool kWarmUp = !kOneCopy && !kSplitKeys;
+        for (int j = kWarmUp && t == 0 ? -1 : 0; j <= j_last; ++j) {
             if (j >= 0 && !(ok = mbar_wait_warp(&sm.bar_s_full[t], j & 1, nullptr, 0, abort_flag, p.status, kWaitFwdS))) break;
             tc_fence_after_sync();
             // the whole score row of this key tile stays in registers
