@@ -435,16 +435,27 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             };
             // The two warps of a scheduler take turns at the exponential unit, in the order of the score products, so that one
             // chain's exponentials run beside the other's loads, maxima and hand-offs; the turn passes on a little before the
-            // last ones (after 112 of 128 keys; 96 measures the same), which covers the hand-off.  (Before the first store the
-            // products with the previous P must have read it, too.)
-            const int m = j + (t == 0 ? min(j, j_last1 + 1) : min(j, j_last0) + 1);
-            if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1, abort_flag, p.status, kWaitFwdO))) break;
+            // last ones (after 112 of 128 keys; 96 measures the same), which covers the hand-off.  Only for pairs of query tiles at
+            // D = 128, where the power limit makes up for it; elsewhere a turn, which also holds the packing and storing of the first
+            // half, is longer than what it hides.  us, turns / none (heads, S, D; causal unless noted): 128 / 16 of 4 096, 128 521 / 532; on
+            // the other side 64 of 1531, 64 unmasked 66.9 / 65.1; 32, 4096, 64 106.1 / 103.6; 20, 2048, 128 32.3 / 31.5; 8, 4096, 64
+            // unmasked 53.2 / 50.4.  (Short causal calls at D = 64 would gain by them: 128 of 333 15.0 / 15.2; 40, 777 15.0 / 15.4.)
+            // (Before the first store the products with the previous P must have read it, too.)
+            constexpr bool kTurns = D == 128 && !kSplitKeys;
+            if constexpr (kTurns) {
+                const int m = j + (t == 0 ? min(j, j_last1 + 1) : min(j, j_last0) + 1);
+                if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1, abort_flag, p.status, kWaitFwdO))) break;
+            } else if (j > 0 && !(ok = mbar_wait_warp(&sm.bar_o_done[t], (j - 1) & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO))) {
+                break;
+            }
             tc_fence_after_sync();
             exponentials(0, 64);
             store_half(0);
             exponentials(64, 112);
-            __syncwarp();
-            if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_exp[quad]);
+            if constexpr (kTurns) {
+                __syncwarp();
+                if (lane == 0 && j >= 0) mbar_arrive(&sm.bar_exp[quad]);
+            }
             // a half's probabilities are in place: their products may start
             tmem_wait_st();
             tc_fence_before_sync();
