@@ -550,14 +550,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
 
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
 // makespan in steps of both chains (about 1.6 us), with kFill for a CTA's start, fill and drain, kMerge for putting two
-// softmaxes together, and a margin.  On 260 shapes near the line, both ways measured, it is 0.4 % behind the faster one on
-// average and 18 % at worst (with the constants of the kernel whose chains had a region of scores each, 1.3 % and 31 %).
-// us, pairs of tiles / split keys (heads, S): 8, 2080 31.2 / 20.2; 4, 5248 73.5 / 44.1; 15, 640 12.5 / 11.4; 14, 1038 unmasked
-// 20.8 / 14.7; 32, 1024 19.0 / 19.2; on the other side 31, 640 12.1 / 13.1; 44, 612 12.6 / 16.3; 60, 640 19.8 / 26.3; 19, 2432
-// 35.6 / 39.2; 33, 5329 221 / 250; 54 of 462 unmasked 13.0 / 18.8.
+// softmaxes together, and a margin.  Fitted to 400 shapes near the line, both ways measured in graphs: there 0.10 % behind the
+// faster one on average and 6 % at worst, on 300 others 0.05 % and 6 %.  (The constants
+// of the kernel whose softmax warps began with a pass on nothing, 1.9, 0.6, 0.91 and 0.95: 2.0 % and 19 %; 0.8 % and 17 %.)
+// us, pairs of tiles / split keys (heads, S; D = 128 under the causal mask unless noted): 8, 300 8.7 / 7.5; 20, 384 9.1 / 7.9; 32, 400
+// 11.0 / 8.2; 32, 949 18.2 / 17.5; 31, 1455 unmasked 49.3 / 44.1; on the other side 32, 589 12.3 / 12.5; 40, 512 11.6 / 12.4; 33, 2326
+// 58.6 / 61.1; 40, 400 11.0 / 12.3; 60, 1949 unmasked 125 / 130; 48, 5607 unmasked 693 / 744.
 static bool splits_keys(int B, int Hq, int S, int causal) {
     constexpr int kSms = 148;
-    constexpr double kFill = 1.9, kMerge = 0.6;
+    constexpr double kFill = 2.2, kMerge = 0.2;
     const double heads = static_cast<double>(B) * Hq;
     const int n = (S + kFwdTileRows - 1) / kFwdTileRows, pairs = (n + 1) / 2;
     if (n < 2) return false;
@@ -579,7 +580,7 @@ static bool splits_keys(int B, int Hq, int S, int causal) {
     const double split_steps = half * (half + 1) / 2 + even * (even + 1) / 2;
     const double split = span(n, split_steps, kFill + kMerge, [&](int q) { return static_cast<double>(causal ? (n - q + 1) / 2 : (n + 1) / 2); });
     const double whole = span(pairs, pair_steps, kFill, [&](int q) { return static_cast<double>(causal && q > 0 ? 2 * (pairs - q) : n); });
-    return split < (causal ? 0.91 : 0.95) * whole;
+    return split < (causal ? 0.88 : 0.98) * whole;
 }
 
 template <int D, bool kBf16>
