@@ -826,7 +826,15 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
             LT_CUDA(cudaStreamWaitEvent(stream, pipe->ev_do[c], 0), "cudaStreamWaitEvent");
             LT_CUDA(cudaStreamWaitEvent(s_out, pipe->ev_fwd[c], 0), "cudaStreamWaitEvent");
         }
-        if (O) LT_CUDA(cudaMemcpyAsync(O + oq, d_O + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
+        if (O) {
+            // One query head per key/value head: not in the middle of dO's copy in.  The 7B layer then took 3.49 or 3.69 ms, depending
+            // on how the copies of the two directions came to lie beside one another, which a few us of the kernels decide; behind
+            // it 3.45.  Other heads, S, ms at once / behind dO: 32, 2048 1.90 / 1.83; 34, 2600 2.56 / 2.37; 40, 4096 4.48 / 4.36; 20, 4096
+            // 2.31 / 2.32.  With grouped queries dO is a third of a chunk's bytes and more, and too much time passes: 24/12, 8 x 700 2.79 /
+            // 2.84; 40/8, 4096 2.77 / 2.84; 64/8, 2048 2.09 / 2.19.
+            if (pipe && G == 1) LT_CUDA(cudaStreamWaitEvent(s_out, pipe->ev_do[c], 0), "cudaStreamWaitEvent");
+            LT_CUDA(cudaMemcpyAsync(O + oq, d_O + oq, cq, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
+        }
         if (LSE) LT_CUDA(cudaMemcpyAsync(LSE + ol, d_lse + ol, cl, cudaMemcpyDeviceToHost, s_out), "cudaMemcpyAsync");
         rc = lt_attn_bwd(d_Q + oq, d_K + ok_, d_V + ok_, d_O + oq, d_dO + oq, d_lse + ol, d_dQ + oq, d_dK + ok_,
                          d_dV + ok_, 1, hq, hkv, S, D, causal, scale, ws, ws_bytes, stream);
