@@ -446,11 +446,17 @@ __device__ __forceinline__ bool traced_wait(Trace &tr, uint64_t *bar, uint32_t p
 }
 #define LT_WAIT_BOTH(bar_a, parity_a, bar_b, parity_b, code) \
     traced_wait_warp(trace_, bar_a, parity_a, bar_b, parity_b, abort_flag, p.status, code)
+// (two barriers one after the other, so that each gets the cycles that it took)
 __device__ __forceinline__ bool traced_wait_warp(Trace &tr, uint64_t *bar_a, uint32_t parity_a, uint64_t *bar_b, uint32_t parity_b,
                                                  volatile int *abort_flag, unsigned int *status, int code) {
     const unsigned int t0 = static_cast<unsigned int>(clock());
-    const bool r = mbar_wait_warp(bar_a, parity_a, bar_b, parity_b, abort_flag, status, code);
-    tr.acc[code - 200] += static_cast<unsigned int>(clock()) - t0;
+    bool r = mbar_wait_warp(bar_a, parity_a, nullptr, 0, abort_flag, status, code);
+    const unsigned int t1 = static_cast<unsigned int>(clock());
+    tr.acc[(code >= 1000 ? code / 1000 : code) - 200] += t1 - t0;
+    if (r && bar_b) {
+        r = mbar_wait_warp(bar_b, parity_b, nullptr, 0, abort_flag, status, code);
+        tr.acc[code % 1000 - 200] += static_cast<unsigned int>(clock()) - t1;
+    }
     return r;
 }
 #else
@@ -1002,7 +1008,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     const int4 item = sm.item_ring[ic % kItemRing];
                     if (item.x < 0) break;
                     const BwdItem w = bwd_item<kSplit>(p, item);
-                    if (!(ok = LT_WAIT_BOTH(&sm.bar_kv, ic & 1, &sm.bar_q_full[it & 1], (it >> 1) & 1, kWaitKV))) break;
+                    if (!(ok = LT_WAIT_BOTH(&sm.bar_kv, ic & 1, &sm.bar_q_full[it & 1], (it >> 1) & 1,
+                                            both_codes(kWaitKV, kWaitStageFull)))) break;
                     tc_fence_after_sync();
                     LT_TL(leader, 14, it);
                     if constexpr (!kSavedP) issue_s(it);
@@ -1036,13 +1043,15 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                         };
                         LT_TL(leader, 0, it);
                         // dO_i and the -delta rows have landed (both dP and dV read them), the dQ partial has been drained
-                        if (!(ok = LT_WAIT_BOTH(&sm.bar_do_full, it & 1, it > 0 ? &sm.bar_dq_empty : nullptr, (it - 1) & 1, kWaitDqEmpty))) break;
+                        if (!(ok = LT_WAIT_BOTH(&sm.bar_do_full, it & 1, it > 0 ? &sm.bar_dq_empty : nullptr, (it - 1) & 1,
+                                                both_codes(kWaitDoFull, kWaitDqEmpty)))) break;
                         tc_fence_after_sync();
                         LT_TL(leader, 1, it);
                         issue_dp();
                         LT_TL(leader, 2, it);
                         // (the first product of an item overwrites accumulators the previous item's epilogue reads)
-                        if (!(ok = LT_WAIT_BOTH(&sm.bar_p_ready, it & 1, n == 0 && ic > 0 ? &sm.bar_acc_free : nullptr, (ic - 1) & 1, kWaitPReady))) break;
+                        if (!(ok = LT_WAIT_BOTH(&sm.bar_p_ready, it & 1, n == 0 && ic > 0 ? &sm.bar_acc_free : nullptr, (ic - 1) & 1,
+                                                both_codes(kWaitPReady, kWaitAccFree)))) break;
                         LT_TL(leader, 3, it);
                         tc_fence_after_sync();
                         issue_dv();
@@ -1210,7 +1219,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if constexpr (kSavedP)
                     if (n + 1 < w.n_iter) load_saved_p(w, n + 1, pn);
                 // (the previous dS^T tile must have been consumed by the dQ product before it is overwritten)
-                if (!(ok = LT_WAIT_BOTH(&sm.bar_dp_full, it & 1, it > 0 ? &sm.bar_ds_free : nullptr, (it - 1) & 1, kWaitDpFull))) break;
+                if (!(ok = LT_WAIT_BOTH(&sm.bar_dp_full, it & 1, it > 0 ? &sm.bar_ds_free : nullptr, (it - 1) & 1,
+                                        both_codes(kWaitDpFull, kWaitDsFree)))) break;
                 tc_fence_after_sync();
                 LT_TL(tid == kComputeWarp0 * 32, 9, it);
                 LT_TRACE_MARK(td0);
@@ -1474,7 +1484,8 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (!ok) break;
             // item epilogue (these warps are idle while the pipeline of the next item fills; the last item's is the softmax warps'):
             // dK_j and dV_j leave tensor memory as fp16; thread = key row
-            ok = LT_WAIT_BOTH(&sm.bar_dkv_full, ic & 1, kSplit ? nullptr : &sm.bar_item[(ic + 1) % kItemRing], ((ic + 1) / kItemRing) & 1, kWaitDkvFull);
+            ok = LT_WAIT_BOTH(&sm.bar_dkv_full, ic & 1, kSplit ? nullptr : &sm.bar_item[(ic + 1) % kItemRing], ((ic + 1) / kItemRing) & 1,
+                              kSplit ? kWaitDkvFull : both_codes(kWaitDkvFull, kWaitItem));
             ok = named_barrier_and(kBarReduceWarps, kNumReduceWarps * 32, ok);
             if (!ok) break;
             if (!kSplit && sm.item_ring[(ic + 1) % kItemRing].x < 0) continue;

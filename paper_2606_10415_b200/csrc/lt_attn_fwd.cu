@@ -37,7 +37,7 @@ constexpr float kFwdRescaleLog2 = 8.f;        // P <= 2^8 stays far inside fp16 
 
 enum {
     kWaitFwdQ = 301, kWaitFwdKV = 302, kWaitFwdEmpty = 303, kWaitFwdS = 304, kWaitFwdP = 305,
-    kWaitFwdO = 306, kWaitFwdSFree = 307, kWaitFwdDone = 309
+    kWaitFwdO = 306, kWaitFwdSFree = 307, kWaitFwdTurn = 308, kWaitFwdDone = 309, kWaitFwdMerge = 310
 };
 
 template <int D>
@@ -270,7 +270,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                     [&](int m, int j, int t, bool first, bool last) -> bool {
                         // chain t's scores, in the one score region
                         next_tile(first, k_slot, k_round);
-                        if (!wait_all(&sm.bar_kv_full[k_slot], k_round & 1, m > 0 ? &sm.bar_s_free : nullptr, (m - 1) & 1, kWaitFwdSFree)) return false;
+                        if (!wait_all(&sm.bar_kv_full[k_slot], k_round & 1, m > 0 ? &sm.bar_s_free : nullptr, (m - 1) & 1,
+                                      both_codes(kWaitFwdKV, kWaitFwdSFree))) return false;
                         tc_fence_after_sync();
                         if (leader) {
                             const uint64_t dQ = dQ0 + static_cast<uint32_t>(kSplitKeys ? 0 : t) * kSlotStep, dK = dK0 + static_cast<uint32_t>(k_slot) * kSlotStep;
@@ -290,7 +291,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
 #pragma unroll
                         for (int half = 0; half < 2; ++half) {
                             if (!wait_all(half == 0 ? &sm.bar_p_half[t] : &sm.bar_p_ready[t], j & 1, half == 0 ? &sm.bar_kv_full[v_slot] : nullptr,
-                                          v_round & 1, kWaitFwdP)) return false;
+                                          v_round & 1, half == 0 ? both_codes(kWaitFwdP, kWaitFwdKV) : kWaitFwdP)) return false;
                             tc_fence_after_sync();
                             if (leader) {
 #pragma unroll
@@ -444,7 +445,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             constexpr bool kTurns = D == 128 && !kSplitKeys;
             if constexpr (kTurns) {
                 const int m = j + (t == 0 ? min(j, j_last1 + 1) : min(j, j_last0) + 1);
-                if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1, abort_flag, p.status, kWaitFwdO))) break;
+                if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1,
+                                                             abort_flag, p.status, both_codes(kWaitFwdTurn, kWaitFwdO)))) break;
             } else if (j > 0 && !(ok = mbar_wait_warp(&sm.bar_o_done[t], (j - 1) & 1, nullptr, 0, abort_flag, p.status, kWaitFwdO))) {
                 break;
             }
@@ -479,7 +481,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
                 sm.merge[row] = make_float2(m_used, l);  // (no odd key tile: -inf and 0)
                 mbar_arrive(&sm.bar_merge);
             } else if (ok) {
-                ok = mbar_wait(&sm.bar_merge, 0, abort_flag, p.status, kWaitFwdO) &&
+                ok = mbar_wait(&sm.bar_merge, 0, abort_flag, p.status, kWaitFwdMerge) &&
                      (j_last1 < 0 || mbar_wait(&sm.bar_o_done[1], j_last1 & 1, abort_flag, p.status, kWaitFwdO));
                 ok = __all_sync(0xffffffffu, ok);
             }

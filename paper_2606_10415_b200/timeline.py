@@ -16,11 +16,11 @@ import torch
 from . import binding as lt, build, workloads
 
 EVENTS = [
-    "issuer: dO landed", "issuer: dQ drained, dP issue begins", "issuer: dP issued", "issuer: P ready",
+    "issuer: waits for dO and the drained dQ", "issuer: both there, dP issue begins", "issuer: dP issued", "issuer: P ready",
     "issuer: dV and next S issued", "issuer: dS ready", "issuer: dK and dQ issued",
     "softmax: S complete", "softmax: P handed over", "softmax: dP complete", "softmax: dS handed over",
     "reduce: dQ complete", "reduce: dP columns released", "reduce: last group issued",
-    "issuer: first S of a work item issued", "reduce: dK/dV accumulators released",
+    "issuer: first S of a work item issued", "reduce: dK/dV accumulators released",  # (not those of a CTA's last item)
 ]
 N_EVENTS, N_ITER = 20, 256
 
