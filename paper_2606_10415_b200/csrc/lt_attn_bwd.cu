@@ -706,7 +706,7 @@ bwd_main_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 const BwdParams p, const __grid_constant__ CUtensorMap map_dq, const __grid_constant__ CUtensorMap map_dk,
                 const __grid_constant__ CUtensorMap map_dv, const BwdOneTileParams one) {
     // map_dq (D = 64 only): the fp32 dQ accumulator as rows of 64 floats, boxes of 128 rows x 32 columns
-    // map_dk, map_dv: the outputs, boxes of 32 rows x 64 columns
+    // map_dk, map_dv (whole key tiles only): the outputs, boxes of 32 rows x 64 columns
     using Smem = BwdSmem<D>;
     constexpr int kBoxes = D / 64;
     constexpr uint32_t kTileBytes = kBoxes * kBoxBytesBwd;
@@ -1703,8 +1703,9 @@ static int launch_bwd(const lt_half *Q, const lt_half *K, const lt_half *V, cons
     if ((rc = make_bhsd_map(&mdo, dO, B, Hq, S, D, lay.d_o, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mk, K, B, Hkv, S, D, lay.k, 128, kBf16)) != LT_OK) return rc;
     if ((rc = make_bhsd_map(&mv, V, B, Hkv, S, D, lay.v, 128, kBf16)) != LT_OK) return rc;
-    if ((rc = make_bhsd_map(&mdk, dK, B, Hkv, S, D, lay.dk, 32, kBf16)) != LT_OK) return rc;
-    if ((rc = make_bhsd_map(&mdv, dV, B, Hkv, S, D, lay.dv, 32, kBf16)) != LT_OK) return rc;
+    mdk = mdv = mk;  // (split key tiles leave through shares and the reduction warps, never through these)
+    if (!split && (rc = make_bhsd_map(&mdk, dK, B, Hkv, S, D, lay.dk, 32, kBf16)) != LT_OK) return rc;
+    if (!split && (rc = make_bhsd_map(&mdv, dV, B, Hkv, S, D, lay.dv, 32, kBf16)) != LT_OK) return rc;
 
     // programmatic stream serialisation: each kernel may start before its predecessor has finished and
     // waits inside for it (grid_dependency_wait).  The conversion kernels do not let the next call's preprocess
