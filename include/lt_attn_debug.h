@@ -48,6 +48,10 @@ int lt_dbg_wait_timeout(void *workspace, size_t workspace_bytes, lt_stream_t str
  * a tile's contraction (1: nobody does), and whether CTA pairs share tiles.  Nothing is launched, no device is needed. */
 int lt_dbg_gemm_plan(int M, int N, int K, int *tile_columns, int *shares, int *pairs);
 
+/* The kernel the forward chooses for these sizes: whether a CTA takes one query tile with its keys in two chains (otherwise a
+ * pair of query tiles), and whether its issuing warp has the walk in one copy.  Nothing is launched, no device is needed. */
+int lt_dbg_fwd_plan(int B, int Hq, int S, int D, int causal, int *split_keys, int *one_copy);
+
 /* Development builds only (not exported by the product library, hence described, not declared):
  *   -DLT_BWD_TIMELINE=<cta>: `int lt_dbg_bwd_timeline(long long *out)` copies 20 x 256 clock stamps to the
  *     host buffer `out` ([event][tile pair] of that CTA's first 256 tile pairs in the last backward call;

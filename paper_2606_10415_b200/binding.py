@@ -30,7 +30,7 @@ EXPORTS = (
     "lt_last_cuda_error", "lt_attn_bwd_num_launches", "lt_attn_fwd_num_launches", "lt_attn_bwd_noalloc_check_status",
 )
 # test-support entry points (include/lt_attn_debug.h)
-DEBUG_EXPORTS = ("lt_dbg_tile_gemm", "lt_dbg_wait_timeout", "lt_dbg_gemm_plan")
+DEBUG_EXPORTS = ("lt_dbg_tile_gemm", "lt_dbg_wait_timeout", "lt_dbg_gemm_plan", "lt_dbg_fwd_plan")
 
 
 class TensorStrides(ctypes.Structure):
@@ -110,6 +110,8 @@ def _load() -> ctypes.CDLL:
     lib.lt_dbg_wait_timeout.restype = i
     lib.lt_dbg_gemm_plan.argtypes = [i, i, i] + [ctypes.POINTER(i)] * 3
     lib.lt_dbg_gemm_plan.restype = i
+    lib.lt_dbg_fwd_plan.argtypes = [i] * 5 + [ctypes.POINTER(i)] * 2
+    lib.lt_dbg_fwd_plan.restype = i
     return lib
 
 
@@ -393,6 +395,15 @@ def lt_dbg_gemm_plan(M, N, K) -> tuple[int, int, bool]:
     if rc != LT_OK:
         raise LtError("lt_dbg_gemm_plan", rc)
     return out[0].value, out[1].value, bool(out[2].value)
+
+
+def lt_dbg_fwd_plan(B, Hq, S, D, causal) -> tuple[bool, bool]:
+    """(keys of one query tile in two chains, issuing warp's walk in one copy) of the kernel the forward chooses."""
+    out = [ctypes.c_int() for _ in range(2)]
+    rc = _lib.lt_dbg_fwd_plan(B, Hq, S, D, int(bool(causal)), *(ctypes.byref(o) for o in out))
+    if rc != LT_OK:
+        raise LtError("lt_dbg_fwd_plan", rc)
+    return bool(out[0].value), bool(out[1].value)
 
 
 def alloc_workspace(nbytes: int, device="cuda") -> torch.Tensor:

@@ -14,8 +14,8 @@
 
 #include <algorithm>
 #include <mutex>
-#include <type_traits>
 
+#include "../../include/lt_attn_debug.h"
 #include "lt_common.cuh"
 #include "lt_host.h"
 
@@ -53,6 +53,8 @@ struct __align__(1024) FwdSmem {
     uint32_t tmem_base;
     int abort_flag;
 };
+
+static_assert(sizeof(FwdSmem<128>) + 1024 <= 232448, "shared memory (with room to align it) exceeds the 227 KB per-block limit");
 
 struct FwdParams {
     float *lse;
@@ -159,7 +161,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     // warps hold the scores of number m - 1 in registers, the products with V of number m - 2 come behind it.  on_s and
     // on_pv get (step, chain, whether it is the first and the last to use the step's key or value tile) and return false to leave.
     // (Behind the end of the first chain of a pair, its last product with V goes ahead, so that its output can be stored.)
-    // Two forms of the same walk (launch_fwd has the rule).  One loop with one copy of either kind of work is a sixth of the code: it is the faster one at
+    // Two forms of the same walk (fwd_plan has the rule).  One loop with one copy of either kind of work is a sixth of the code: it is the faster one at
     // D = 64, and at D = 128 where an SM runs one or two CTAs of short walks out of a cold instruction cache; unrolled over the
     // chains, with the chain a constant, a product takes fewer instructions to issue, which counts where products are twice as
     // long and many.  us, one copy / unrolled (heads, S, D): 32, 1024, 128 17.9 / 18.9; 128 of 333, 64 15.8 / 16.8; 32, 4096, 64
@@ -550,6 +552,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
+constexpr int kFwdSms = 148;  // (of a B200: the estimates below are fitted to it)
+
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
 // makespan in steps of both chains (about 1.6 us), with kFill for a CTA's start, fill and drain, kMerge for putting two
 // softmaxes together, and a margin.  Fitted to 400 shapes near the line, both ways measured in graphs: there 0.10 % behind the
@@ -559,7 +563,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
 // 11.0 / 8.2; 32, 949 18.2 / 17.5; 31, 1455 unmasked 49.3 / 44.1; on the other side 32, 589 12.3 / 12.5; 40, 512 11.6 / 12.4; 33, 2326
 // 58.6 / 61.1; 40, 400 11.0 / 12.3; 60, 1949 unmasked 125 / 130; 48, 5607 unmasked 693 / 744.
 static bool splits_keys(int B, int Hq, int S, int causal) {
-    constexpr int kSms = 148;
+    constexpr int kSms = kFwdSms;
     constexpr double kFill = 2.2, kMerge = 0.2;
     const double heads = static_cast<double>(B) * Hq;
     const int n = (S + kFwdTileRows - 1) / kFwdTileRows, pairs = (n + 1) / 2;
@@ -585,6 +589,22 @@ static bool splits_keys(int B, int Hq, int S, int causal) {
     return split < (causal ? 0.88 : 0.98) * whole;
 }
 
+// The kernel of a call: how its CTAs split the work, and the form of the issuing warp's walk (figures beside the walk): one copy
+// at D = 64, and for one or two CTAs of up to 24 products per SM.  Measured both ways on 190 shapes at D = 128, from 2 to 64
+// products and 8 to 1 232 CTAs: one copy is the faster one up to 8 products (1-7 %), on up to 24 under the causal mask with more
+// CTAs than SMs (1-7 % up to 12, -3 to 2 % above), equal at 11 and 12 with fewer CTAs, and 1-3 % behind from 16 on without a mask; from
+// 32 on it is 2-8 % behind.  The line is within 3 % of the faster one.
+struct FwdPlan {
+    bool split_keys, one_copy;
+    int grid;
+};
+static FwdPlan fwd_plan(int B, int Hq, int S, int D, int causal) {
+    const bool split = splits_keys(B, Hq, S, causal);
+    const int n_tiles = (S + kFwdTileRows - 1) / kFwdTileRows;
+    const int grid = B * Hq * (split ? n_tiles : (n_tiles + 1) / 2);
+    return {split, D == 64 || (grid <= 2 * kFwdSms && n_tiles * (split ? 1 : 2) <= 24), grid};
+}
+
 template <int D, bool kBf16>
 static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_half *O, float *LSE,
                       const lt_attn_layout &lay, int B, int Hq, int Hkv, int S, int causal, float scale,
@@ -602,21 +622,17 @@ static int launch_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_h
     prm.scale = scale;
     // at least 120 KB, so that one CTA (which takes all 512 tensor-memory columns) lives on an SM
     const size_t smem = std::max<size_t>(sizeof(FwdSmem<D>) + 1024, 120 * 1024);
-    const bool split = splits_keys(B, Hq, S, causal);
-    const int n_tiles = (S + kFwdTileRows - 1) / kFwdTileRows;
-    const int grid = B * Hq * (split ? n_tiles : (n_tiles + 1) / 2);
-    // the issuing warp's walk in one copy (figures beside the walk): D = 64, and one or two CTAs of up to 24 products per SM
-    const bool one_copy = D == 64 || (grid <= 2 * 148 && n_tiles * (split ? 1 : 2) <= 24);
-    auto kernel = split ? fwd_kernel<D, kBf16, true, true> : fwd_kernel<D, kBf16, false, true>;
+    const FwdPlan plan = fwd_plan(B, Hq, S, D, causal);
+    auto kernel = plan.split_keys ? fwd_kernel<D, kBf16, true, true> : fwd_kernel<D, kBf16, false, true>;
     if constexpr (D == 128)
-        if (!one_copy) kernel = split ? fwd_kernel<D, kBf16, true, false> : fwd_kernel<D, kBf16, false, false>;
+        if (!plan.one_copy) kernel = plan.split_keys ? fwd_kernel<D, kBf16, true, false> : fwd_kernel<D, kBf16, false, false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return record_cuda_error("cudaFuncSetAttribute(fwd)", e);
     cudaLaunchAttribute pdl;
     pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3(plan.grid);
     cfg.blockDim = dim3(kFwdThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
@@ -649,6 +665,16 @@ size_t lt_attn_fwd_workspace_bytes(int B, int Hq, int Hkv, int S, int D) {
 }
 
 int lt_attn_fwd_num_launches(void) { return 1; }
+
+int lt_dbg_fwd_plan(int B, int Hq, int S, int D, int causal, int *split_keys, int *one_copy) {
+    const int rc = lt::check_shape(B, Hq, Hq, S, D, 1.0f);
+    if (rc != LT_OK) return rc;
+    if (!split_keys || !one_copy) return LT_ERR_INVALID_ARG;
+    const lt::FwdPlan plan = lt::fwd_plan(B, Hq, S, D, causal);
+    *split_keys = plan.split_keys ? 1 : 0;
+    *one_copy = plan.one_copy ? 1 : 0;
+    return LT_OK;
+}
 
 int lt_attn_fwd(const lt_half *Q, const lt_half *K, const lt_half *V, lt_half *O, float *LSE, int B, int Hq, int Hkv,
                 int S, int D, int causal, float scale, void *workspace, size_t workspace_bytes, lt_stream_t stream) {

@@ -1,4 +1,4 @@
-"""Forward whose CTAs take pairs of query tiles (many heads): a lone last tile, walks shorter and longer than the ring of
+"""Forward whose CTAs take pairs of query tiles (many heads), and the forms of the kernel that fewer or longer walks select: a lone last tile, walks shorter and longer than the ring of
 key and value tiles, ragged ends, both masks, maxima that rise late, keys hidden by -inf (the first tile's among them, as
 left padding has it), and an output between other columns and rows that must stay as they are; against fp64 softmax."""
 import pytest
@@ -12,8 +12,22 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("dtype,kind", [(torch.float16, "plain"), (torch.bfloat16, "plain"), (torch.float16, "ramp"), (torch.float16, "hidden"),
                                         (torch.float16, "hidden first"), (torch.bfloat16, "hidden first")])
 def test_query_pairs(S, D, causal, dtype, kind):
+    check(3, 64, 16, S, D, causal, dtype, kind, (False, D == 64 or S <= 128))
+
+
+# D = 128: pairs with the walk in one copy (few CTAs, several tiles), split keys with the unrolled one (many CTAs, long walks)
+@pytest.mark.parametrize("H,Hkv,S,causal,form", [(64, 8, 512, True, (False, True)), (64, 16, 500, False, (False, True)), (64, 64, 897, False, (False, True)),
+                                                 (44, 4, 897, True, (False, True)), (20, 4, 2048, True, (True, False)),
+                                                 (4, 2, 3201, False, (True, False)), (28, 7, 1290, False, (True, False))])
+@pytest.mark.parametrize("dtype,kind", [(torch.float16, "plain"), (torch.bfloat16, "plain"), (torch.float16, "ramp"), (torch.float16, "hidden"),
+                                        (torch.float16, "hidden first")])
+def test_other_forms(H, Hkv, S, causal, form, dtype, kind):
+    check(1, H, Hkv, S, 128, causal, dtype, kind, form)
+
+
+def check(B, H, Hkv, S, D, causal, dtype, kind, form):
     from paper_2606_10415_b200 import binding as lt
-    B, H, Hkv = 3, 64, 16
+    assert lt.lt_dbg_fwd_plan(B, H, S, D, causal) == form  # (keys split, walk in one copy)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(S + D)
     Q, K, V = (torch.randn((B, h, S, D), generator=gen, device="cuda") for h in (H, Hkv, Hkv))

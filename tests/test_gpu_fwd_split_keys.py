@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
                                                    (torch.float16, -1, False), (torch.float16, 1, True)])
 def test_split_keys(H, Hkv, S, D, causal, dtype, scale_sign, ramp):
     from paper_2606_10415_b200 import binding as lt
+    assert lt.lt_dbg_fwd_plan(1, H, S, D, causal) == (True, True)  # (keys split, walk in one copy)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(S + D)
     Q, K, V = (torch.randn((1, h, S, D), generator=gen, device="cuda") for h in (H, Hkv, Hkv))
@@ -49,6 +50,7 @@ def test_hidden_key_tiles(H, Hkv, S, D, hidden, causal, dtype):
     """Keys hidden by a channel of ones in Q against -inf in K: score -inf, weight zero, also where that is every key of the
     tile a chain starts with, or of all its tiles."""
     from paper_2606_10415_b200 import binding as lt
+    assert lt.lt_dbg_fwd_plan(1, H, S, D, causal) == (True, True)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(S + D)
     Q, K, V = (torch.randn((1, h, S, D), generator=gen, device="cuda").to(dtype) for h in (H, Hkv, Hkv))
@@ -91,6 +93,7 @@ def test_no_further_from_64_bits_than_query_pairs(H, S, D, causal, dtype):
     for B in (1, 512 // H):
         q, k, v = (t.expand(B, -1, -1, -1).contiguous() for t in (Q, K, V))
         O, LSE = torch.empty_like(q), torch.empty((B, H, S), device="cuda")
+        assert lt.lt_dbg_fwd_plan(B, H, S, D, causal)[0] == (B == 1)
         fn(q, k, v, O, LSE, causal, D ** -0.5, lt.alloc_workspace(256))
         assert last is None or not torch.equal(last, O[0])  # the two forms do differ
         last = O[0]
