@@ -72,19 +72,19 @@ struct FwdParams {
 // grids that leave multiprocessors idle or wait for a few long walks: splits_keys().
 //
 // What bounds it: the exponential unit, 1 024 cycles per tile of 128 x 128 scores, with the softmax warps' other work (load,
-// maximum, store, hand-offs: about 1 300 cycles a tile) that two warps per scheduler hide only in part, although they take
-// turns at it; a step of both chains takes about 3 000 cycles, the exponential unit and the tensor cores (2 048 cycles a step
-// at D = 128) are each busy for two thirds of it, and in long runs the power limit.  Hence the layout of tensor memory: the softmax warps hold
-// a tile's scores in registers as soon as they are there, so the chains share one region of scores and P has columns of its
-// own; a chain's next scores are formed under its softmax instead of behind its product P V.  (With S and P of a chain in one
-// region a step took 3 600 cycles, most of it the chain softmax -> P V -> S.)  Measured, us, a region per chain / this
-// (heads, S, D; causal unless noted; single calls): 32, 4096, 128 145 / 131; 32, 1024, 128 22.4 / 20.0; 32, 3000, 128 92.5 / 82.6;
-// 64 of 1531, 64 unmasked 79.4 / 77.6; 64/8 heads of 8192 unmasked 1740 / 1662; with turns at the exponential unit 127.3, 18.9, 79.7,
-// 71.5 and 1 604 (40 heads of 1 920 lose by them, 50.1 / 51.1).
-// Tried: two warps per row and tile, 16 softmax warps with a vote on the maximum (11 % slower: they wait for each other);
-// the maximum found during the first quarter's exponentials (3 % slower); both chains started at once (2 %
-// slower: they stay in step and want the exponential unit together); a fifth of the exponentials as polynomials (no gain at
-// this share of the unit's time).
+// maximum, store, hand-offs: about 1 300 cycles a tile) that two warps per scheduler hide only in part; a step of both chains takes
+// about 3 000 cycles, the exponential unit and the tensor cores (2 048 cycles a step at D = 128) are each busy for two thirds
+// of it, and in long runs the power limit.  Hence the layout of tensor memory: the softmax warps hold a tile's scores in
+// registers as soon as they are there, so the chains share one region of scores and P has columns of its own; a chain's next
+// scores are formed under its softmax instead of behind its product P V.  (With S and P of a chain in one region a step took 3 600
+// cycles, most of it the chain softmax -> P V -> S.)  us, a region per chain / this (heads, S, D; causal unless noted; calls on
+// end): 32, 4096, 128 160 / 147; 32, 1024, 128 21.3 / 17.5; 32, 3000, 128 101 / 86; 8, 300, 128 8.0 / 7.2; 64 of 1531, 64 unmasked 74.8 / 67.7;
+// 128 of 333, 64 17.4 / 15.5; 2, 129, 64 5.46 / 5.22.
+// Tried with this layout: the second chain's first scores in columns of their own, so that both chains' first ones are formed at
+// once (equal for short calls, 2-4 % slower for long ones at D = 128).  Tried before the score region was shared: two warps per row and
+// tile, 16 softmax warps with a vote on the maximum (11 % slower: they wait for each other); the maximum found during the
+// first quarter's exponentials (3 % slower); both chains started at once (2 % slower); a fifth of the exponentials as
+// polynomials (no gain, at a smaller share of the unit's time than now).
 template <int D, bool kBf16, bool kSplitKeys, bool kOneCopy>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -333,12 +333,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
         float l = 0.f;             // running sum of exp2(score - m_used)
         bool ok = true;
         // Pass -1 works on whatever tensor memory holds and leaves nothing behind: it brings the loop's instructions into the
-        // instruction cache while the first tiles are on their way (a first tile took 3 400 cycles instead of 1 450).  Only where
-        // walks are long and many: it takes longer than the tiles do, and short walks wait for it.  us, with it / without (heads, S,
-        // D): 8, 192, 64 6.02 / 5.46; 128 of 333, 64 15.7 / 15.0; 32, 4096, 64 107.8 / 106.1; 8, 192, 128 6.68 / 6.33; 20, 2048, 128
-        // 32.4 / 31.1; on the other side 32, 3000, 128 86.3 / 87.4; 128 / 16 of 4 096, 128 528 / 534.
-        constexpr bool kWarmUp = !kOneCopy && !kSplitKeys;
-        for (int j = kWarmUp && t == 0 ? -1 : 0; j <= j_last; ++j) {
+        // instruction cache while the first tiles are on their way (a first tile took 3 400 cycles instead of 1 450).  It takes longer
+        // than tiles out of L2 do: a forward behind another kernel and on new inputs gains by it, one of many on the same inputs loses,
+        // and short walks of split keys lose either way.  us, with it / without (heads, S, D): forward and backward in turn on
+        // changing inputs: 128 of 333, 64 50.3 / 50.7; 8 of 64, 64 13.8 / 14.0; 32, 1024, 128 65.7 / 66.0; 8, 192, 128 24.0 / 23.7; forward calls alone: 8, 192, 64
+        // 6.02 / 5.46; 32 of 64, 64 5.30 / 5.11; 32, 1024, 64 16.1 / 15.2; 8, 192, 128 6.68 / 6.33; 128 of 333, 64 15.7 / 15.4.
+        const bool warm_up = !kSplitKeys || (D == 128 && n_tiles >= 8);
+        for (int j = warm_up && t == 0 ? -1 : 0; j <= j_last; ++j) {
             if (j >= 0 && !(ok = mbar_wait_warp(&sm.bar_s_full[t], j & 1, nullptr, 0, abort_flag, p.status, kWaitFwdS))) break;
             tc_fence_after_sync();
             // the whole score row of this key tile stays in registers
@@ -438,13 +439,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CU
             };
             // The two warps of a scheduler take turns at the exponential unit, in the order of the score products, so that one
             // chain's exponentials run beside the other's loads, maxima and hand-offs; the turn passes on a little before the
-            // last ones (after 112 of 128 keys; 96 measures the same), which covers the hand-off.  Only for pairs of query tiles at
-            // D = 128, where the power limit makes up for it; elsewhere a turn, which also holds the packing and storing of the first
-            // half, is longer than what it hides.  us, turns / none (heads, S, D; causal unless noted): 128 / 16 of 4 096, 128 521 / 532; on
-            // the other side 64 of 1531, 64 unmasked 66.9 / 65.1; 32, 4096, 64 106.1 / 103.6; 20, 2048, 128 32.3 / 31.5; 8, 4096, 64
-            // unmasked 53.2 / 50.4.  (Short causal calls at D = 64 would gain by them: 128 of 333 15.0 / 15.2; 40, 777 15.0 / 15.4.)
+            // last ones (after 112 of 128 keys; 96 measures the same), which covers the hand-off.  Not with split keys: there a turn,
+            // which also holds the packing and storing of the first half, is longer than what it hides.  us, turns / none (heads, S, D;
+            // causal unless noted): 20, 2048, 128 32.3 / 31.5; 4, 8000, 128 66.5 / 63.8; 4, 4000, 64 unmasked 29.5 / 28.9; pairs: 128 / 16 of 4 096, 128
+            // 521 / 532; 128 of 333, 64 15.0 / 15.2; 40, 777, 64 15.0 / 15.4; but 64 of 1531, 64 unmasked 66.9 / 65.1; 32, 4096, 64 106.1 / 103.6.
             // (Before the first store the products with the previous P must have read it, too.)
-            constexpr bool kTurns = D == 128 && !kSplitKeys;
+            constexpr bool kTurns = !kSplitKeys;
             if constexpr (kTurns) {
                 const int m = j + (t == 0 ? min(j, j_last1 + 1) : min(j, j_last0) + 1);
                 if (m > 0 && j >= 0 && !(ok = mbar_wait_warp(&sm.bar_exp[quad], (m - 1) & 1, j > 0 ? &sm.bar_o_done[t] : nullptr, (j - 1) & 1,
@@ -557,7 +557,7 @@ constexpr int kFwdSms = 148;  // (of a B200: the estimates below are fitted to i
 // Whether a CTA takes one query tile with its key tiles in two chains instead of two query tiles: by the estimated
 // makespan in steps of both chains (about 1.6 us), with kFill for a CTA's start, fill and drain, kMerge for putting two
 // softmaxes together, and a margin.  Fitted to 400 shapes near the line, both ways measured in graphs: there 0.10 % behind the
-// faster one on average and 6 % at worst, on 300 others 0.05 % and 6 %.  (The constants
+// faster one on average and 6 % at worst, on 300 others 0.04 % and 6 %.  (The constants
 // of the kernel whose softmax warps began with a pass on nothing, 1.9, 0.6, 0.91 and 0.95: 2.0 % and 19 %; 0.8 % and 17 %.)
 // us, pairs of tiles / split keys (heads, S; D = 128 under the causal mask unless noted): 8, 300 8.7 / 7.5; 20, 384 9.1 / 7.9; 32, 400
 // 11.0 / 8.2; 32, 949 18.2 / 17.5; 31, 1455 unmasked 49.3 / 44.1; on the other side 32, 589 12.3 / 12.5; 40, 512 11.6 / 12.4; 33, 2326
@@ -586,7 +586,7 @@ static bool splits_keys(int B, int Hq, int S, int causal) {
     const double split_steps = half * (half + 1) / 2 + even * (even + 1) / 2;
     const double split = span(n, split_steps, kFill + kMerge, [&](int q) { return static_cast<double>(causal ? (n - q + 1) / 2 : (n + 1) / 2); });
     const double whole = span(pairs, pair_steps, kFill, [&](int q) { return static_cast<double>(causal && q > 0 ? 2 * (pairs - q) : n); });
-    return split < (causal ? 0.88 : 0.98) * whole;
+    return split < (causal ? 0.88 : 0.96) * whole;
 }
 
 // The kernel of a call: how its CTAs split the work, and the form of the issuing warp's walk (figures beside the walk): one copy
