@@ -777,18 +777,17 @@ int lt_attn_fwd_bwd_host(const lt_half *Q, const lt_half *K, const lt_half *V, c
     // The copies in one direction take as long as those in the other, and the copies back can only begin when the first
     // chunk has come in and been worked on: the smaller that chunk, the better, but every copy beside others in the other
     // direction costs about 15 us on top of its bytes.  Four chunks, the last ones smaller, or six of about equal size.
-    // Measured with O returned on 100 shapes (four / six, ratio of the times, and ms for some): one query head per key/value
-    // head and 20 to 34 units 0.99-1.15, median 1.02 (LLaMA-2-7B layer, 32 units, 3.80 / 3.51; 24 heads of 3 000 2.26 / 2.05); 36 to 64
-    // units 0.94-1.04, median 0.96, at every S from 1 500 to 4 096 (40 heads of 4 096 4.65 / 4.77; of 2 048 2.40 / 2.54; 8 x 8 heads of 2 048
-    // unmasked 3.76 / 3.96); fewer than 20 units, for which six chunks get uneven, 0.97-1.06; grouped queries 0.96-0.99 (Qwen2.5-32B
-    // layer 2.83 / 2.86; 40 / 20 heads of 4 096 3.51 / 3.61).
+    // Measured with O returned on 75 shapes (four / six, ratio of the times, and ms for some): one query head per key/value head and 22
+    // units or more 0.96-1.08, median 1.02 (24 heads of 4 096 2.78 / 2.57; 32 of 3 000 2.83 / 2.73; 40 of 2 048 2.28 / 2.18; 64 of 2 048 3.58 /
+    // 3.32; 8 x 8 heads of 2 048 unmasked 3.58 / 3.35); 20 units 0.98-1.00; fewer, for which six chunks get uneven, 0.93-1.08; grouped
+    // queries 0.88-0.98 (40 / 8 heads of 4 096 2.80 / 2.86; 40 / 20 3.48 / 3.62; 64 / 8 of 2 048 2.11 / 2.25).
     int bounds[kHostMaxChunks + 1];
     int n_chunks = 1;
     bounds[0] = 0;
     bounds[1] = n_units;
     if (unit_iters * n_units >= 3000 && n_units > 1) {  // otherwise not worth the extra streams
         constexpr int kFew[4] = {30, 60, 85, 100}, kMany[6] = {17, 34, 51, 68, 85, 100};  // cumulative shares, %
-        const bool many = G == 1 && n_units >= 20 && n_units <= 34;
+        const bool many = G == 1 && n_units >= 20;
         const int *percent = many ? kMany : kFew;
         const int np = many ? 6 : 4;
         n_chunks = 0;

@@ -1,4 +1,4 @@
-"""The host-buffer call cut into chunks (four of them, or six: 24 heads of 3 000): every unit of every chunk
+"""The host-buffer call cut into chunks (six of them, or four: 16 heads on 8): every unit of every chunk
 against the device entry points on the whole problem, with and without the optional outputs, calls back to back."""
 import pytest
 import torch
@@ -8,7 +8,7 @@ from paper_2606_10415_b200 import workloads
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(4, 16, 16, 1024, 128, False), (1, 24, 24, 3000, 128, True)])
+@pytest.mark.parametrize("B,Hq,Hkv,S,D,causal", [(4, 16, 16, 1024, 128, False), (1, 24, 24, 3000, 128, True), (1, 16, 8, 3000, 128, True)])
 @pytest.mark.parametrize("with_o", [True, False])
 def test_many_chunks(B, Hq, Hkv, S, D, causal, with_o):
     from paper_2606_10415_b200 import binding as lt
